@@ -23,6 +23,7 @@
 
 #include "amdd.h"
 #include "amdd_internal.h"
+#include "fronts.h"
 
 using namespace amdd;
 
@@ -153,8 +154,6 @@ struct amdd_handle {
     double* d_Y = nullptr;
     double* d_Yt = nullptr;
     double* d_Zt = nullptr;
-    double* d_YE = nullptr;
-    double* d_YEt = nullptr;
     GemvDesc* d_gv_l1 = nullptr;
     GemvDesc* d_gv_l2 = nullptr;
     GemvDesc* d_gv_c = nullptr;
@@ -178,20 +177,10 @@ struct amdd_handle {
     float *d_rloc32 = nullptr, *d_tloc32 = nullptr, *d_yloc32 = nullptr;
     GemvDescT<float>* d_gv_l1_32 = nullptr;
     GemvDescT<float>* d_gv_l2_32 = nullptr;
-    double *d_c = nullptr, *d_e = nullptr, *d_ctmp = nullptr;
-    // coarse solve: L_E (d_YE), L_E^T (d_YEt), inverses of its diagonal blocks
-    double *d_Yd = nullptr, *d_Ydt = nullptr;
-    int cSB = 0, cK = 0, coop_blocks = 0;
+    double *d_c = nullptr, *d_e = nullptr;
+    // coarse solve by substructuring (fronts.cu): Ainv, W and W^T of every part
+    FrontSolve fs;
     double csolve_flops = 0.0, csolve_bytes = 0.0;
-    std::vector<int> env_row;     // first non-zero column of each row of E (and L_E)
-    std::vector<int> env_colend;  // one past the last non-zero row of each column of L_E
-    int* d_env_row = nullptr;
-    int32_t* d_cperm = nullptr;  // factorisation order of the coarse unknowns (NULL: subdomain order)
-    double *d_cF = nullptr, *d_cG = nullptr;  // folded coarse solve (CoarseSolveArgs::F, G), NULL: not folded
-    int *d_cfw0 = nullptr, *d_cgw1 = nullptr;
-    int cFW = 0;
-    double *d_cp = nullptr, *d_ep = nullptr;  // coarse vectors in that order (MAXB vectors)
-    int* d_env_colend = nullptr;
     // eigenvectors of partial selections: 0 dense Jacobi, 1 LOBPCG from random
     // rows, 2 LOBPCG from the learned proposal
     int eig_solver = 0, keep_prop = 0;
@@ -206,7 +195,7 @@ struct amdd_handle {
     int mb_cap = 0;
     double *d_m_rloc = nullptr, *d_m_tloc = nullptr, *d_m_yloc = nullptr;
     float *d_m_rloc32 = nullptr, *d_m_tloc32 = nullptr, *d_m_yloc32 = nullptr;
-    double *d_m_c = nullptr, *d_m_ctmp = nullptr, *d_m_e = nullptr, *d_m_zc = nullptr;
+    double *d_m_c = nullptr, *d_m_e = nullptr, *d_m_zc = nullptr;
     GemvDesc* d_m_gv_zp = nullptr;
     double *d_m_q = nullptr, *d_m_r = nullptr, *d_m_z = nullptr, *d_m_p = nullptr, *d_m_part = nullptr;
     PcgScal* d_m_sc = nullptr;
@@ -557,11 +546,6 @@ GemmDescT<T> gd(const T* A, int lda, int ta, const T* B, int ldb, int tb, T* Cm,
 // each stopped at its own column `stop` (the trailing block then holds the
 // Schur complement of the factored leading block).
 //
-// `env` (optional, one entry per matrix, may be null) gives each row's first
-// non-zero column (the envelope).  The Cholesky factor keeps the envelope of
-// the matrix, so panel row tiles and trailing-update tiles whose rows have no
-// entries in the current block column are zero throughout and are skipped.
-//
 // Look-ahead: the trailing update of step k is split into the next block
 // column ("near", on the handle's stream, right after the panel) and the rest
 // ("far", on a second stream).  The far update of step k runs while the
@@ -569,7 +553,7 @@ GemmDescT<T> gd(const T* A, int lda, int ta, const T* B, int ldb, int tb, T* Cm,
 // k+1 waits for it, since both write block column k+2.  The order of the
 // updates of every entry is fixed, so results do not depend on timing.
 template <typename T>
-void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds, const std::vector<const std::vector<int>*>& env = {}) {
+void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds) {
     if (ds.empty()) return;
     amdd_handle* h = C.h;
     cudaStream_t sm = h->s, ss = h->s2;
@@ -577,30 +561,13 @@ void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds, const std::vector
     int maxstop = 0;
     for (const auto& d : ds) maxstop = std::max(maxstop, d.stop);
     bool far_pending = false;  // a far update was issued on ss and not yet joined
-    auto active_rows = [&](int d, int r_begin, int r_end, int kend) {
-        const std::vector<int>* e = (d < (int)env.size()) ? env[d] : nullptr;
-        if (!e) return true;
-        for (int r = r_begin; r < r_end; ++r)
-            if ((*e)[r] < kend) return true;
-        return false;
-    };
-    // tiles of one GEMM descriptor whose row and column blocks are both active
-    auto update_tiles = [&](int gi, const GemmDescT<T>& g, int d, int row_base, int col_base, int kend, int tile,
-                            std::vector<TileRef>& out, double& fl) {
-        const int tm = cdiv(g.m, tile), tn = cdiv(g.n, tile);
-        std::vector<char> ar(tm), ac(tn);
-        for (int a = 0; a < tm; ++a)
-            ar[a] = active_rows(d, row_base + a * tile, std::min(row_base + (a + 1) * tile, row_base + g.m), kend);
-        for (int b = 0; b < tn; ++b)
-            ac[b] = active_rows(d, col_base + b * tile, std::min(col_base + (b + 1) * tile, col_base + g.n), kend);
-        for (int a = 0; a < tm; ++a)
-            for (int b = 0; b < tn; ++b)
-                if (ar[a] && ac[b] && !(g.lower && b > a)) {
-                    out.push_back({gi, a, b});
-                    const double ri = std::min(tile, g.m - a * tile), ci = std::min(tile, g.n - b * tile);
-                    const double outs = (g.lower && a == b) ? ri * (ri + 1) / 2 : ri * ci;
-                    fl += 2.0 * outs * g.k;
-                }
+    auto flops_of = [](const std::vector<GemmDescT<T>>& g) {
+        double fl = 0.0;
+        for (const auto& q : g) {
+            const double m = q.m, w = q.n;
+            fl += 2.0 * q.k * (w <= m ? m * w - w * (w - 1) / 2 : m * (m + 1) / 2);
+        }
+        return fl;
     };
     for (int k0 = 0; k0 < maxstop; k0 += CHOL_NB) {
         {
@@ -616,7 +583,6 @@ void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds, const std::vector
         std::vector<PanelRef> pt;
         double pfl = 0.0;
         std::vector<GemmDescT<T>> gn, gf;  // near / far updates
-        std::vector<int> gn_d, gf_d, gn_kend, gf_kend;
         int tiles64 = 0;
         for (int d = 0; d < (int)ds.size(); ++d) {
             const CholDescT<T>& c = ds[d];
@@ -625,25 +591,18 @@ void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds, const std::vector
             const int rows = c.n - kend;
             if (rows <= 0) continue;
             const int kb = kend - k0;
-            for (int rt = 0; rt < cdiv(rows, PANEL_ROWS); ++rt)
-                if (active_rows(d, kend + rt * PANEL_ROWS, std::min(c.n, kend + (rt + 1) * PANEL_ROWS), kend)) {
-                    pt.push_back({d, rt});
-                    pfl += (double)std::min(PANEL_ROWS, rows - PANEL_ROWS * rt) * kb * (kb + 1);
-                }
+            for (int rt = 0; rt < cdiv(rows, PANEL_ROWS); ++rt) pt.push_back({d, rt});
+            pfl += (double)rows * kb * (kb + 1);
             const T* P = c.A + (size_t)kend * c.ld + k0;  // panel rows [kend, n)
             const int w = std::max(0, std::min(CHOL_NB, c.stop - kend));  // next block column
             if (w > 0) {
                 gn.push_back(gd(P, c.ld, 0, P, c.ld, 1, c.A + (size_t)kend * c.ld + kend, c.ld, rows, w, kb, -1.0, 1.0,
                                 1));
-                gn_d.push_back(d);
-                gn_kend.push_back(kend);
             }
             if (rows - w > 0) {
                 const T* Pf = P + (size_t)w * c.ld;
                 gf.push_back(gd(Pf, c.ld, 0, Pf, c.ld, 1, c.A + (size_t)(kend + w) * c.ld + kend + w, c.ld, rows - w,
                                 rows - w, kb, -1.0, 1.0, 1));
-                gf_d.push_back(d);
-                gf_kend.push_back(kend);
                 tiles64 += cdiv(rows - w, 64) * (cdiv(rows - w, 64) + 1) / 2;
             }
         }
@@ -654,32 +613,17 @@ void chol_batched(Ctx& C, const std::vector<CholDescT<T>>& ds, const std::vector
         }
         // far update on the second stream, after this panel
         int tile = tiles64 < SMALL_LAUNCH_TILES ? 32 : 64;
-        std::vector<TileRef> tf, tn;
-        double ffl = 0.0, nfl = 0.0;
-        auto far_tiles = [&]() {
-            tf.clear();
-            ffl = 0.0;
-            for (int q = 0; q < (int)gf.size(); ++q) {
-                const int kend = gf_kend[q];
-                const int w = (int)(ds[gf_d[q]].n - kend) - gf[q].m;
-                update_tiles(q, gf[q], gf_d[q], kend + w, kend + w, kend, tile, tf, ffl);
-            }
-        };
-        far_tiles();
+        std::vector<TileRef> tf = gemm_tiles(gf, tile), tn = gemm_tiles(gn, 32);
         if (tile == 32 && (int)tf.size() < TINY_LAUNCH_TILES) {
             tile = 16;
-            far_tiles();
+            tf = gemm_tiles(gf, tile);
         }
         int ntile = 32;
-        for (int q = 0; q < (int)gn.size(); ++q)
-            update_tiles(q, gn[q], gn_d[q], gn_kend[q], gn_kend[q], gn_kend[q], ntile, tn, nfl);
         if ((int)tn.size() < TINY_LAUNCH_TILES) {
             ntile = 16;
-            tn.clear();
-            nfl = 0.0;
-            for (int q = 0; q < (int)gn.size(); ++q)
-                update_tiles(q, gn[q], gn_d[q], gn_kend[q], gn_kend[q], gn_kend[q], ntile, tn, nfl);
+            tn = gemm_tiles(gn, ntile);
         }
+        const double ffl = flops_of(gf), nfl = flops_of(gn);
         const GemmDescT<T>* dgf = tf.empty() ? nullptr : C.up(gf);
         const TileRef* dtf = tf.empty() ? nullptr : C.up(tf);
         const GemmDescT<T>* dgn = tn.empty() ? nullptr : C.up(gn);
@@ -1921,79 +1865,165 @@ std::vector<int> learned_eigvecs(Ctx& C, amdd_handle* h, const std::vector<int>&
     return dense;
 }
 
+// Stages of the coarse solve: parts of at most FRONT_LEAF unknowns first, the
+// part sizes growing by at most FRONT_RATIO from stage to stage (plan_fronts).
+// 96 and 20 from the plan's own counts on 24^3 and 64^2 grids: smaller leaves
+// add a launch per direction, larger ones grow the dense blocks (7.8 M entries
+// instead of 5.5 M on 24^3 with 128).
+constexpr int FRONT_LEAF = 96;
+constexpr int FRONT_RATIO = 20;
+
+// Factors E (dense lower triangle, order nC, subdomain order) in the plan's
+// stages: each part's front collects its entries of E and its children's Schur
+// complements, a partial Cholesky eliminates the interior, and the interior's
+// inverse Ainv = Y^T Y (Y = L_II^{-1}) and W^T = L_BI Y are kept for the solve.
+void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, int64_t nC) {
+    cudaStream_t s = h->s;
+    const int nf = (int)P.fronts.size(), S = P.stages();
+    std::vector<FrontDev> fd(nf);
+    std::vector<int64_t> oF(nf + 1, 0), oA(nf + 1, 0), oW(nf + 1, 0), oY(nf + 1, 0), oL(nf + 1, 0);
+    for (int k = 0; k < nf; ++k) {
+        const int64_t m = P.fronts[k].m, b = P.fronts[k].nb;
+        oF[k + 1] = oF[k] + (m + b) * (m + b);
+        oA[k + 1] = oA[k] + m * m;
+        oW[k + 1] = oW[k] + m * b;
+        oL[k + 1] = oL[k] + (int64_t)cdiv(m, CHOL_NB) * CHOL_NB * CHOL_NB;
+    }
+    double* F = C.tnew<double>(oF[nf]);
+    double* Y = C.tnew<double>(oA[nf]);
+    double* linv = C.tnew<double>(oL[nf]);
+    double* Ai = dnew<double>(h, oA[nf]);
+    double* W = dnew<double>(h, oW[nf]);
+    double* Wt = dnew<double>(h, oW[nf]);
+    ck(cudaMemsetAsync(F, 0, oF[nf] * sizeof(double), s));
+
+    // children of each front, with the maps between their boundary and its rows
+    std::vector<std::vector<int>> kids(nf);
+    for (int k = 0; k < nf; ++k)
+        if (P.fronts[k].parent >= 0) kids[P.fronts[k].parent].push_back(k);
+    std::vector<FrontChild> ch;
+    std::vector<int32_t> maps;
+    std::vector<int32_t> at(P.n, -1);
+    for (int k = 0; k < nf; ++k) {
+        const Front& f = P.fronts[k];
+        fd[k] = {F + oF[k], Ai + oA[k], W + oW[k], f.m, f.nb, f.i0, f.b0, (int)ch.size(), 0};
+        if (!kids[k].empty()) {
+            for (int a = 0; a < f.m; ++a) at[f.i0 + a] = a;
+            for (int b = 0; b < f.nb; ++b) at[P.bnd[f.b0 + b]] = f.m + b;
+            for (int c : kids[k]) {
+                const Front& g = P.fronts[c];
+                const int ld = g.m + g.nb;
+                FrontChild q{F + oF[c] + (size_t)g.m * ld + g.m, ld, (int64_t)maps.size(), 0};
+                for (int b = 0; b < g.nb; ++b) maps.push_back(at[P.bnd[g.b0 + b]]);
+                q.inv = (int64_t)maps.size();
+                maps.resize(maps.size() + f.m + f.nb, -1);
+                for (int b = 0; b < g.nb; ++b) maps[q.inv + maps[q.map + b]] = b;
+                ch.push_back(q);
+            }
+        }
+        fd[k].kid1 = (int)ch.size();
+    }
+    // rows of W^T next to each boundary unknown, stage by stage
+    std::vector<int32_t> drow, dptr{0}, rfront(P.n);
+    std::vector<FrontRef> refs;
+    h->fs.down_off.assign(S + 1, 0);
+    std::vector<std::vector<FrontRef>> at_row(P.n);
+    for (int st = 0; st < S; ++st) {
+        std::vector<int32_t> touched;
+        for (int k = P.stage_part[st]; k < P.stage_part[st + 1]; ++k) {
+            const Front& f = P.fronts[k];
+            for (int a = 0; a < f.m; ++a) rfront[f.i0 + a] = k;
+            for (int b = 0; b < f.nb; ++b) {
+                const int32_t t = P.bnd[f.b0 + b];
+                if (at_row[t].empty()) touched.push_back(t);
+                at_row[t].push_back({Wt + oW[k] + (size_t)b * f.m, f.i0, f.m});
+            }
+        }
+        std::sort(touched.begin(), touched.end());
+        for (int32_t t : touched) {
+            drow.push_back(t);
+            refs.insert(refs.end(), at_row[t].begin(), at_row[t].end());
+            dptr.push_back((int32_t)refs.size());
+            at_row[t].clear();
+        }
+        h->fs.down_off[st + 1] = (int64_t)drow.size();
+    }
+    FrontSolve& fs = h->fs;
+    fs.n = P.n;
+    fs.stages = S;
+    fs.row_off = P.stage_off;
+    fs.perm = C.up(P.perm, true);
+    fs.fr = C.up(fd, true);
+    fs.row_front = C.up(rfront, true);
+    fs.bnd = C.up(P.bnd, true);
+    fs.down_rows = C.up(drow, true);
+    fs.down_ptr = C.up(dptr, true);
+    fs.refs = C.up(refs, true);
+    fs.v = dnew<double>(h, (size_t)MAXB * P.n);
+    fs.e = dnew<double>(h, (size_t)MAXB * P.n);
+    const FrontChild* dch = C.up(ch);
+    const int32_t* dmaps = C.up(maps);
+
+    for (int st = 0; st < S; ++st) {
+        const int k0 = P.stage_part[st], k1 = P.stage_part[st + 1];
+        if (k0 == k1) continue;
+        int maxn = 1, maxm = 1;
+        bool add = false;
+        std::vector<CholDesc> cd;
+        std::vector<TrtriDesc> td;
+        std::vector<GemmDesc> ga, gw;
+        std::vector<double*> mats;
+        std::vector<int> mm;
+        std::vector<TransDesc> tr;
+        for (int k = k0; k < k1; ++k) {
+            const int m = P.fronts[k].m, b = P.fronts[k].nb, n = m + b;
+            maxn = std::max(maxn, n);
+            maxm = std::max(maxm, std::max(m, b));
+            add = add || !kids[k].empty();
+            cd.push_back({F + oF[k], n, n, m, nullptr, linv + oL[k]});
+            td.push_back({F + oF[k], Y + oA[k], linv + oL[k], m, n, m});
+            GemmDesc g = gd<double>(Y + oA[k], m, 1, Y + oA[k], m, 0, Ai + oA[k], m, m, m, m, 1.0, 0.0, 1);
+            g.kfrom_row = 1;
+            ga.push_back(g);
+            mats.push_back(Ai + oA[k]);
+            mm.push_back(m);
+            if (b > 0) {
+                gw.push_back(gd<double>(F + oF[k] + (size_t)m * n, n, 0, Y + oA[k], m, 0, Wt + oW[k], m, b, m, m, 1.0,
+                                        0.0, 0));
+                tr.push_back({Wt + oW[k], W + oW[k], b, m, m, b});
+            }
+        }
+        {
+            PScope ps(h, PK_E_ASM, 0.0);
+            launch_front_gather(fs.fr + k0, k1 - k0, fs.bnd, fs.perm, E, nC, maxn, s);
+        }
+        if (add) {
+            PScope ps(h, PK_SMALL);
+            launch_front_extend_add(fs.fr + k0, k1 - k0, dch, dmaps, maxn, s);
+        }
+        chol_batched<double>(C, cd);
+        trtri_batched<double>(C, td);
+        gemm(C, ga);
+        gemm(C, gw);
+        {
+            auto a = C.up(mats);
+            auto b = C.up(mm);
+            PScope ps(h, PK_SMALL);
+            launch_mirror_lower<double>(a, b, b, (int)mats.size(), maxm, s);
+        }
+        if (!tr.empty()) {
+            auto t = C.up(tr);
+            PScope ps(h, PK_SMALL);
+            launch_transpose_rect(t, (int)tr.size(), maxm, s);
+        }
+    }
+    h->csolve_flops = 2.0 * (double)(oA[nf] + 2 * oW[nf]);
+    h->csolve_bytes = 8.0 * (double)(oA[nf] + 2 * oW[nf]) + 48.0 * (double)P.n;
+}
+
 // T: type of the local work (factors of A_ii, T = L_A^{-1} S L_A^{-T}, its
 // eigensolve, Z_i).  TS: type of the splitting (SVD of X_i, Abar_ii and its
 // Schur complement S).
-// Reverse Cuthill-McKee order of a symmetric graph (adjacency lists): per
-// connected component a pseudo-peripheral start (George and Liu: repeated
-// breadth-first searches from a minimum-degree node of the deepest level),
-// then breadth-first numbering with the unnumbered neighbours of each node by
-// increasing degree; the whole sequence reversed.
-std::vector<int32_t> rcm_order(const std::vector<std::vector<int32_t>>& nbr) {
-    const int n = (int)nbr.size();
-    std::vector<int32_t> order;
-    order.reserve(n);
-    std::vector<char> numbered(n, 0);
-    std::vector<int> level(n, -1);
-    auto deg = [&](int v) { return (int)nbr[v].size(); };
-    // levels of the component of root among unnumbered nodes; returns the
-    // depth and leaves the visited nodes in comp (levels reset on exit)
-    std::vector<int32_t> comp, last;
-    auto bfs = [&](int root) {
-        comp.assign(1, root);
-        level[root] = 0;
-        int depth = 0;
-        for (size_t head = 0; head < comp.size(); ++head) {
-            const int v = comp[head];
-            for (int w : nbr[v])
-                if (level[w] < 0 && !numbered[w]) {
-                    level[w] = level[v] + 1;
-                    depth = std::max(depth, level[w]);
-                    comp.push_back(w);
-                }
-        }
-        last.clear();
-        for (int v : comp)
-            if (level[v] == depth) last.push_back(v);
-        for (int v : comp) level[v] = -1;
-        return depth;
-    };
-    for (int s0 = 0; s0 < n; ++s0) {
-        if (numbered[s0]) continue;
-        bfs(s0);
-        int root = s0;
-        for (int v : comp)
-            if (deg(v) < deg(root)) root = v;
-        int depth = bfs(root);
-        for (int it = 0; it < 8; ++it) {
-            int cand = last[0];
-            for (int v : last)
-                if (deg(v) < deg(cand)) cand = v;
-            const int d2 = bfs(cand);
-            if (d2 <= depth) break;
-            root = cand;
-            depth = d2;
-        }
-        const size_t start = order.size();
-        order.push_back(root);
-        numbered[root] = 1;
-        std::vector<int32_t> nb;
-        for (size_t head = start; head < order.size(); ++head) {
-            const int v = order[head];
-            nb.clear();
-            for (int w : nbr[v])
-                if (!numbered[w]) {
-                    numbered[w] = 1;
-                    nb.push_back(w);
-                }
-            std::sort(nb.begin(), nb.end(), [&](int a, int b) { return deg(a) < deg(b) || (deg(a) == deg(b) && a < b); });
-            order.insert(order.end(), nb.begin(), nb.end());
-        }
-    }
-    std::reverse(order.begin(), order.end());
-    return order;
-}
-
 // Sparse local factors (amdd_opts.local_solver): per subdomain the
 // nested-dissection order of the local pattern and the column structure of its
 // Cholesky factor (host, nd_factor_pattern); the permuted A_ii gathered dense on
@@ -2322,17 +2352,11 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         // Cholesky factor and inverse factor
         cudaStream_t s = h->s;  // the stream this call runs on
         const int64_t nC = h->nC;
-        h->d_cperm = nullptr;
-        h->d_YEt = nullptr;
-        h->d_cF = h->d_cG = nullptr;
-        h->d_cfw0 = h->d_cgw1 = nullptr;
-        h->cFW = 0;
         if (nC > 0) {
             std::vector<int64_t> off_az(N + 1, 0);
             for (int i = 0; i < N; ++i) off_az[i + 1] = off_az[i] + (int64_t)h->ni[i] * h->p[i];
             double* AZ = C.tnew<double>(off_az[N]);
-            h->d_YE = dnew<double>(h, (size_t)nC * nC);  // E, then its Cholesky factor L_E (lower)
-            double* E = h->d_YE;
+            double* E = C.tnew<double>((size_t)nC * nC);  // lower triangle
             ck(cudaMemsetAsync(E, 0, (size_t)nC * nC * sizeof(double), s));
             std::vector<GemmDesc> g1, g2;
             std::vector<DiagScaleDesc> dsd;
@@ -2461,183 +2485,48 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 PScope ps(h, PK_SMALL, 0.0, 16.0 * h->E_nnz);
                 launch_gather_idx64(dsrc, h->E_nnz, E, h->d_E_val, s);
             }
-            // ---- sparsity graph of E (coarse unknowns in subdomain order): blocks
-            // of subdomains coupled in A (E_ij = Z_i^T A(Omega_Ii, Omega_Ij) Z_j is
-            // exactly zero otherwise); a diagonal-basis block contributes only the
-            // unknowns whose node touches the other subdomain
-            std::vector<std::vector<int>> adjB(N);
-            for (int64_t g = 0; g < n; ++g)
-                for (int64_t q = rp[g]; q < rp[g + 1]; ++q)
-                    if (part[g] != part[ci[q]]) adjB[part[g]].push_back(part[ci[q]]);
+            // ---- graph of E: a vertex per coarse unknown of a diagonal-basis
+            // subdomain (E has A's own entries there), one vertex for all unknowns
+            // of any other subdomain (its block is dense)
+            std::vector<int32_t> vfirst(N), base, wt;
             for (int i = 0; i < N; ++i) {
-                adjB[i].push_back(i);
-                std::sort(adjB[i].begin(), adjB[i].end());
-                adjB[i].erase(std::unique(adjB[i].begin(), adjB[i].end()), adjB[i].end());
+                vfirst[i] = (int32_t)base.size();
+                const bool fd = diag_basis && h->p[i] == h->nI[i];
+                if (h->p[i] == 0) continue;
+                for (int k = 0; k < (fd ? h->p[i] : 1); ++k) {
+                    base.push_back((int32_t)(h->coff[i] + k));
+                    wt.push_back(fd ? 1 : h->p[i]);
+                }
             }
-            auto full_diag = [&](int i) { return diag_basis && h->p[i] == h->nI[i] && h->p[i] > 0; };
-            std::vector<std::vector<int32_t>> nbr(nC);
+            auto vertex = [&](int64_t g) {
+                const int i = part[g];
+                return vfirst[i] + (diag_basis && h->p[i] == h->nI[i] ? posI[g] : 0);
+            };
+            std::vector<int32_t> aptr(base.size() + 1, 0), adj;
+            std::vector<int32_t> row;
+            auto close_row = [&](int32_t v) {
+                std::sort(row.begin(), row.end());
+                row.erase(std::unique(row.begin(), row.end()), row.end());
+                adj.insert(adj.end(), row.begin(), row.end());
+                aptr[v + 1] = (int32_t)adj.size();
+                row.clear();
+            };
             for (int i = 0; i < N; ++i) {
                 if (h->p[i] == 0) continue;
-                if (full_diag(i)) {
-                    for (int k = 0; k < h->p[i]; ++k) {
-                        const int32_t g = Il[i][k];
-                        auto& L = nbr[h->coff[i] + k];
-                        for (int64_t q = rp[g]; q < rp[g + 1]; ++q) {
-                            const int32_t g2 = ci[q];
-                            const int j = part[g2];
-                            if (h->p[j] == 0) continue;
-                            if (full_diag(j))
-                                L.push_back((int32_t)(h->coff[j] + posI[g2]));
-                            else
-                                for (int l = 0; l < h->p[j]; ++l) L.push_back((int32_t)(h->coff[j] + l));
+                const bool fd = diag_basis && h->p[i] == h->nI[i];
+                for (int a = 0; a < h->nI[i]; ++a) {
+                    const int64_t g = Il[i][a];
+                    const int32_t v = vertex(g);
+                    for (int64_t q = rp[g]; q < rp[g + 1]; ++q)
+                        if (h->p[part[ci[q]]] > 0) {
+                            const int32_t u = vertex(ci[q]);
+                            if (u != v) row.push_back(u);
                         }
-                    }
-                } else {
-                    std::vector<int32_t> row;
-                    for (int j : adjB[i]) {
-                        if (h->p[j] == 0) continue;
-                        if (!full_diag(j) || j == i) {
-                            for (int l = 0; l < h->p[j]; ++l) row.push_back((int32_t)(h->coff[j] + l));
-                        } else {
-                            for (int l = 0; l < h->nI[j]; ++l) {  // nodes of Omega_Ij touching Omega_Ii
-                                const int32_t g2 = Il[j][l];
-                                for (int64_t q = rp[g2]; q < rp[g2 + 1]; ++q)
-                                    if (part[ci[q]] == i) {
-                                        row.push_back((int32_t)(h->coff[j] + l));
-                                        break;
-                                    }
-                            }
-                        }
-                    }
-                    for (int k = 0; k < h->p[i]; ++k) nbr[h->coff[i] + k] = row;
+                    if (fd) close_row(v);
                 }
+                if (!fd) close_row(vfirst[i]);
             }
-            for (auto& L : nbr) {
-                std::sort(L.begin(), L.end());
-                L.erase(std::unique(L.begin(), L.end()), L.end());
-            }
-            // ---- ordering of the coarse unknowns for the factorisation: reverse
-            // Cuthill-McKee when it cuts the factorisation work (the sum over rows
-            // of (r - first(r))^2) by a fifth or more, else the subdomain order.
-            // E is permuted on the device; the coarse solves gather and scatter
-            // through the order.
-            auto envelope = [&](const std::vector<int32_t>& iperm, const std::vector<int32_t>& perm,
-                                std::vector<int>& env) {
-                env.assign(nC, 0);
-                double work = 0.0;
-                for (int64_t rn = 0; rn < nC; ++rn) {
-                    int first = (int)rn;
-                    for (int32_t c : nbr[perm[rn]]) first = std::min(first, (int)iperm[c]);
-                    env[rn] = first;
-                    work += (double)(rn - first) * (double)(rn - first);
-                }
-                return work;
-            };
-            std::vector<int32_t> idp(nC);
-            std::iota(idp.begin(), idp.end(), 0);
-            std::vector<int> env_id, env_rcm;
-            const double prof_id = envelope(idp, idp, env_id);
-            std::vector<int32_t> rperm = rcm_order(nbr);
-            std::vector<int32_t> riperm(nC);
-            for (int64_t q = 0; q < nC; ++q) riperm[rperm[q]] = (int32_t)q;
-            const double prof_rcm = envelope(riperm, rperm, env_rcm);
-            const bool use_rcm = prof_rcm < 0.8 * prof_id;
-            h->env_row = use_rcm ? env_rcm : env_id;
-            h->env_colend.assign(nC, 0);
-            // the factor fills each row's envelope: column c of L_E reaches every
-            // row whose envelope starts at or before c
-            {
-                std::vector<int> mark(nC, 0);
-                for (int64_t r = 0; r < nC; ++r) mark[h->env_row[r]] = std::max(mark[h->env_row[r]], (int)r + 1);
-                int run = 0;
-                for (int64_t c = 0; c < nC; ++c) {
-                    run = std::max(run, mark[c]);
-                    h->env_colend[c] = std::max(run, (int)c + 1);
-                }
-            }
-            double* linvE = C.tnew<double>((size_t)cdiv(nC, CHOL_NB) * CHOL_NB * CHOL_NB);
-            if (use_rcm) {
-                // E (lower triangle, subdomain order) -> Ep[r][c] = E[perm r][perm c]
-                // (lower triangle); the two nC x nC buffers swap roles
-                h->d_cperm = C.up(rperm, true);
-                h->d_cp = dnew<double>(h, (size_t)MAXB * nC);
-                h->d_ep = dnew<double>(h, (size_t)MAXB * nC);
-                h->d_YEt = dnew<double>(h, (size_t)nC * nC);
-                {
-                    PScope ps(h, PK_SMALL, 0.0, 8.0 * (double)nC * nC);
-                    launch_sym_permute(E, h->d_YEt, h->d_cperm, nC, s);
-                }
-                std::swap(h->d_YE, h->d_YEt);
-                E = h->d_YE;
-            }
-            if (!h->d_YEt) h->d_YEt = dnew<double>(h, (size_t)nC * nC);
-            chol_batched<double>(C, {CholDesc{E, (int)nC, (int)nC, (int)nC, nullptr, linvE}}, {&h->env_row});
-            // Inverses of the diagonal blocks of L_E (block size cSB): the coarse
-            // solve is then a blocked forward / backward substitution with L_E and
-            // L_E^T, with no inverse of the whole factor.  About eight blocks, at
-            // most 512 wide: each block costs two grid-wide phases per coarse
-            // solve, and its inverse (stored dense) costs SB^3 / 3 FP64
-            // multiply-adds in the setup, so n_C SB^2 / 3 in all.
-            const int SB = std::min<int>(512, std::max<int>(CHOL_NB, cdiv(cdiv(nC, 8), CHOL_NB) * CHOL_NB));
-            const int K = cdiv(nC, SB);
-            h->cSB = SB;
-            h->cK = K;
-            h->d_Yd = dnew<double>(h, (size_t)K * SB * SB);
-            h->d_Ydt = dnew<double>(h, (size_t)K * SB * SB);
-            std::vector<TrtriDesc> tj;
-            std::vector<const double*> ts;
-            std::vector<double*> tdst;
-            std::vector<int> tn, tl;
-            for (int k = 0; k < K; ++k) {
-                const int r0 = k * SB, sb = (int)std::min<int64_t>(SB, nC - r0);
-                tj.push_back({E + (size_t)r0 * nC + r0, h->d_Yd + (size_t)k * SB * SB,
-                              linvE + (size_t)(r0 / CHOL_NB) * CHOL_NB * CHOL_NB, sb, (int)nC, SB});
-                ts.push_back(h->d_Yd + (size_t)k * SB * SB);
-                tdst.push_back(h->d_Ydt + (size_t)k * SB * SB);
-                tn.push_back(sb);
-                tl.push_back(SB);
-            }
-            trtri_batched(C, tj);
-            transpose_batched(C, ts, tdst, tn, tl, tl);
-            transpose_batched<double>(C, {E}, {h->d_YEt}, {(int)nC}, {(int)nC}, {(int)nC});
-            // folded coarse solve: when every block's rows reach back (and its
-            // columns forward) at most SB entries beyond the block, F_k = Yd_k
-            // L(block k, window) and G_k = Ydt_k L^T(block k, window) let each
-            // block be solved in one grid-wide phase per direction
-            {
-                std::vector<int> fw0(K), gw1(K);
-                int FW = 0;
-                for (int k = 0; k < K; ++k) {
-                    const int r0 = k * SB, r1 = (int)std::min<int64_t>(nC, (int64_t)r0 + SB);
-                    int w0 = r0, w1 = r1;
-                    for (int r = r0; r < r1; ++r) {
-                        w0 = std::min(w0, h->env_row[r]);
-                        w1 = std::max(w1, h->env_colend[r]);
-                    }
-                    fw0[k] = w0;
-                    gw1[k] = w1;
-                    FW = std::max(FW, std::max(r0 - w0, w1 - r1));
-                }
-                if (FW > 0 && FW <= SB) {
-                    h->cFW = FW;
-                    h->d_cF = dnew<double>(h, (size_t)K * SB * FW);
-                    h->d_cG = dnew<double>(h, (size_t)K * SB * FW);
-                    std::vector<GemmDesc> gfg;
-                    for (int k = 0; k < K; ++k) {
-                        const int r0 = k * SB, sb = (int)std::min<int64_t>(SB, nC - r0), r1 = r0 + sb;
-                        const int W = r0 - fw0[k], V = gw1[k] - r1;
-                        if (W > 0)
-                            gfg.push_back(gd(h->d_Yd + (size_t)k * SB * SB, SB, 0, h->d_YE + (size_t)r0 * nC + fw0[k],
-                                             (int)nC, 0, h->d_cF + (size_t)k * SB * FW, FW, sb, W, sb, 1.0, 0.0, 0));
-                        if (V > 0)
-                            gfg.push_back(gd(h->d_Ydt + (size_t)k * SB * SB, SB, 0, h->d_YEt + (size_t)r0 * nC + r1,
-                                             (int)nC, 0, h->d_cG + (size_t)k * SB * FW, FW, sb, V, sb, 1.0, 0.0, 0));
-                    }
-                    gemm(C, gfg);
-                    h->d_cfw0 = C.up(fw0, true);
-                    h->d_cgw1 = C.up(gw1, true);
-                }
-            }
+            factor_fronts(C, h, plan_fronts(aptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO), E, nC);
         } else {
             h->d_zt_off = C.up(std::vector<int64_t>(h->off_zt.begin(), h->off_zt.end() - 1), true);
             h->d_nI = C.up(std::vector<int32_t>(h->nI.begin(), h->nI.end()), true);
@@ -3305,36 +3194,6 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->n_g4 = (int64_t)rd.size();
         h->d_rd_c = C.up(rdc, true);
         h->d_rl_c = C.up(rlc, true);
-        // coarse solve L_E L_E^T e = c: blocked forward / backward substitution
-        // with the stored inverses of the diagonal blocks, one cooperative
-        // launch (profile figures: the envelope of L_E and L_E^T, the diagonal
-        // inverses, once each)
-        if (nC > 0) {
-            h->d_ctmp = dnew<double>(h, nC);
-            h->d_env_row = C.up(h->env_row, true);
-            h->d_env_colend = C.up(h->env_colend, true);
-            h->coop_blocks = coarse_solve_blocks();
-            if (h->coop_blocks <= 0) throw Fail{AMDD_ERR_CUDA};
-            const int SB = h->cSB, K = h->cK;
-            double el = 0.0, dl = 0.0;
-            if (h->cFW == 0)
-                for (int64_t r = 0; r < nC; ++r) el += (double)(r - h->env_row[r]) + (double)(h->env_colend[r] - 1 - r);
-            for (int k = 0; k < K; ++k) {
-                const int r0 = k * SB, r1 = (int)std::min<int64_t>(nC, (int64_t)r0 + SB);
-                const double sb = (double)(r1 - r0);
-                dl += sb * (sb + 1);
-                if (h->cFW > 0) {  // folded: the dense sb x W and sb x V window blocks F_k, G_k
-                    int w0 = r0, w1 = r1;
-                    for (int r = r0; r < r1; ++r) {
-                        w0 = std::min(w0, h->env_row[r]);
-                        w1 = std::max(w1, h->env_colend[r]);
-                    }
-                    el += sb * (double)((r0 - w0) + (w1 - r1));
-                }
-            }
-            h->csolve_flops = 2.0 * el + 2.0 * dl;
-            h->csolve_bytes = 8.0 * el + 8.0 * dl + 8.0 * 6.0 * nC;
-        }
         // prolongation: copies of each unknown in subdomain order, owners
         std::vector<int64_t> scp(n + 1, 0);
         for (int64_t t = 0; t < h->sum_ni; ++t) scp[omega[t] + 1]++;
@@ -3434,15 +3293,6 @@ void local_solves(amdd_handle* h, const double* r) {
 // zc = Z e in owner order (d_zc).  Needs nC > 0.
 void inner_coarse_solve(amdd_handle* h);
 
-// the folded form of the coarse solve when the setup built it
-void fold_args(const amdd_handle* h, CoarseSolveArgs& a) {
-    a.F = h->d_cF;
-    a.G = h->d_cG;
-    a.fw0 = h->d_cfw0;
-    a.gw1 = h->d_cgw1;
-    a.FW = h->cFW;
-}
-
 void coarse_correction(amdd_handle* h) {
     cudaStream_t s = h->s;
     const double zt = (double)h->sum_zt;
@@ -3453,25 +3303,8 @@ void coarse_correction(amdd_handle* h) {
     if (h->next) {
         inner_coarse_solve(h);  // multilevel form: e ~ E^{-1} c by GMRES on the next level
     } else {
-        double* cin = h->d_c;
-        double* eout = h->d_e;
-        if (h->d_cperm) {  // the factorisation order of the coarse unknowns
-            PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->nC);
-            launch_perm_gather(h->nC, h->d_cperm, h->d_c, h->d_cp, 1, h->nC, s);
-            cin = h->d_cp;
-            eout = h->d_ep;
-        }
-        {
-            CoarseSolveArgs a{h->d_YE, h->d_YEt, h->d_Yd, h->d_Ydt, h->d_env_row, h->d_env_colend,
-                              cin, h->d_ctmp, eout, (int)h->nC, (int)h->nC, h->cSB, h->cK};
-            fold_args(h, a);
-            PScope ps(h, PK_CSOLVE, h->csolve_flops, h->csolve_bytes);
-            ck(launch_coarse_solve(a, h->coop_blocks, s));
-        }
-        if (h->d_cperm) {
-            PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->nC);
-            launch_perm_scatter(h->nC, h->d_cperm, h->d_ep, h->d_e, 1, h->nC, s);
-        }
+        PScope ps(h, PK_CSOLVE, h->csolve_flops, h->csolve_bytes);
+        launch_front_solve(h->fs, h->d_c, h->nC, h->d_e, h->nC, 1, s);
     }
     {
         PScope ps(h, PK_GEMV, 2.0 * zt, 8.0 * zt + 8.0 * h->nC + 8.0 * h->n);
@@ -3602,7 +3435,6 @@ void ensure_multi(amdd_handle* h) {
         h->d_m_gv_l2 = make_local_descs<float>(h, h->d_m_rloc32, h->d_m_tloc32, h->d_m_yloc32, 2);
     }
     h->d_m_c = dnew<double>(h, CC);
-    h->d_m_ctmp = dnew<double>(h, CC);
     h->d_m_e = dnew<double>(h, CC);
     if (h->nC > 0) {
         std::vector<GemvDesc> cr(h->N);
@@ -3692,26 +3524,9 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
             PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * L + 16.0 * h->nC) * nb);
             launch_gemv_rows_multi<double>(h->d_m_gv_c, h->d_rd_c, h->d_rl_c, h->nC, nb, L, h->nC, s);
         }
-        double* cin = h->d_m_c;
-        double* eout = h->d_m_e;
-        if (h->d_cperm) {
-            PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->nC * nb);
-            launch_perm_gather(h->nC, h->d_cperm, h->d_m_c, h->d_cp, nb, h->nC, s);
-            cin = h->d_cp;
-            eout = h->d_ep;
-        }
-        CoarseSolveArgs a{h->d_YE, h->d_YEt, h->d_Yd, h->d_Ydt, h->d_env_row, h->d_env_colend,
-                          cin, h->d_m_ctmp, eout, (int)h->nC, (int)h->nC, h->cSB, h->cK};
-        fold_args(h, a);
-        a.nb = nb;
-        a.ldv = h->nC;
         {
             PScope ps(h, PK_CSOLVE, h->csolve_flops * nb, h->csolve_bytes);
-            ck(launch_coarse_solve(a, h->coop_blocks, s));
-        }
-        if (h->d_cperm) {
-            PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->nC * nb);
-            launch_perm_scatter(h->nC, h->d_cperm, h->d_ep, h->d_m_e, nb, h->nC, s);
+            launch_front_solve(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, s);
         }
         PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * h->nC + 8.0 * h->n) * nb);
         launch_gemv_rows_multi<double>(h->d_m_gv_zp, h->d_rd_zp, h->d_rl_zp, h->n_zp, nb, h->nC, h->n, s);

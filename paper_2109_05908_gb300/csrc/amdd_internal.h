@@ -437,32 +437,49 @@ struct ScaleDesc {  // A[r] *= f[r] (or 1 / ||A[r]|| with unit scaling)
 template <typename T>
 void launch_scale_rows(const ScaleDesc<T>* d, int nmat, int unit, cudaStream_t s);
 
-// Coarse solve L_E L_E^T e = c (one cooperative launch; c is overwritten).
-struct CoarseSolveArgs {
-    const double* L;       // factor, n x n row-major (lower), leading dimension ld
-    const double* Lt;      // its transpose, row-major
-    const double* Yd;      // K inverses of the SB x SB diagonal blocks (lower), SB x SB each
-    const double* Ydt;     // their transposes
-    const int* env_row;    // first non-zero column of row r of L
-    const int* env_colend; // one past the last non-zero row of column r of L
-    double* c;             // right-hand side, overwritten
-    double* y;             // work (n)
-    double* e;             // solution (n)
-    int n, ld, SB, K;
-    int nb = 1;            // right-hand sides (c, y, e hold nb vectors ldv apart)
-    int64_t ldv = 0;
-    // Folded form (F != NULL), one grid-wide phase per block and direction:
-    //   y_k = Yd_k c_k - F_k y[fw0_k, r0_k),   F_k = Yd_k L(block k, [fw0_k, r0_k))
-    //   e_k = Ydt_k y_k - G_k e[r1_k, gw1_k),  G_k = Ydt_k L^T(block k, [r1_k, gw1_k))
-    // F_k and G_k are SB x FW row-major blocks (K of each); c is not overwritten.
-    const double* F = nullptr;
-    const double* G = nullptr;
-    const int* fw0 = nullptr;
-    const int* gw1 = nullptr;
-    int FW = 0;
+// Coarse solve by substructuring (front_kernels.cu).  One part: its front F
+// ((m + nb) x (m + nb), lower triangle, setup only), Ainv (m x m, symmetric,
+// full) and W (m x nb), its interior at plan positions i0 .. i0 + m and its
+// boundary bnd[b0 .. b0 + nb).
+struct FrontDev {
+    double* F;
+    double* Ainv;
+    double* W;
+    int m, nb;
+    int64_t i0, b0;
+    int kid0, kid1;  // children (FrontChild) whose Schur complements enter F
 };
-int coarse_solve_blocks();  // cooperative grid size for this device (0 on error)
-cudaError_t launch_coarse_solve(const CoarseSolveArgs& a, int blocks, cudaStream_t s);
+struct FrontChild {
+    const double* S;  // Schur complement on the child's boundary (lower triangle)
+    int ld;
+    int64_t map, inv;  // offsets of the maps child boundary -> parent row, parent row -> child boundary
+};
+struct FrontRef {  // a row of W^T and the interior it multiplies
+    const double* row;
+    int64_t i0;
+    int m;
+};
+struct FrontSolve {
+    int64_t n = 0;
+    int stages = 0;
+    const int32_t* perm = nullptr;  // caller's index of each plan position
+    const FrontDev* fr = nullptr;
+    const int32_t* row_front = nullptr;
+    const int32_t* bnd = nullptr;
+    const int32_t* down_rows = nullptr;  // boundary unknowns of each stage's parts
+    const int32_t* down_ptr = nullptr;   // their refs (one shared list, nrow + 1 pointers over all stages)
+    const FrontRef* refs = nullptr;
+    double* v = nullptr;  // MAXB vectors of n each
+    double* e = nullptr;
+    std::vector<int64_t> down_off, row_off;  // host: per stage
+};
+void launch_front_gather(const FrontDev* fr, int nfr, const int32_t* bnd, const int32_t* perm, const double* E,
+                         int64_t nE, int maxn, cudaStream_t s);
+void launch_front_extend_add(const FrontDev* fr, int nfr, const FrontChild* kids, const int32_t* maps, int maxn,
+                             cudaStream_t s);
+// out = E^{-1} c for nb <= MAXB vectors (c ldc apart, out ldo apart)
+void launch_front_solve(const FrontSolve& a, const double* c, int64_t ldc, double* out, int64_t ldo, int nb,
+                        cudaStream_t s);
 
 struct PcgScal {
     double rz, pq, rr, bb, alpha, beta, rz_new;
@@ -497,14 +514,6 @@ void launch_ras_prolong(int64_t n, const int32_t* order_g, const int32_t* own_id
                         double* z, cudaStream_t s);
 // zg[order_g[t]] = zo[t]
 void launch_owner_to_global(int64_t n, const int32_t* order_g, const double* zo, double* zg, cudaStream_t s);
-// Ep[r][c] = E[perm r][perm c] for c <= r (E and Ep lower triangles of n x n
-// row-major matrices; Ep's upper triangle is zeroed)
-void launch_sym_permute(const double* E, double* Ep, const int32_t* perm, int64_t n, cudaStream_t s);
-// dst[k*ld + r] = src[k*ld + perm[r]] / dst[k*ld + perm[r]] = src[k*ld + r], r < n, k < nb
-void launch_perm_gather(int64_t n, const int32_t* perm, const double* src, double* dst, int nb, int64_t ld,
-                        cudaStream_t s);
-void launch_perm_scatter(int64_t n, const int32_t* perm, const double* src, double* dst, int nb, int64_t ld,
-                         cudaStream_t s);
 // out[t] = val[src[t]] (64-bit indices)
 void launch_gather_idx64(const int64_t* src, int64_t cnt, const double* val, double* out, cudaStream_t s);
 // y = b - A x

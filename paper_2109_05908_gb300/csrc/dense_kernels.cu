@@ -1899,218 +1899,4 @@ void launch_gemv_rows_multi(const GemvDescT<T>* d, const int* row_desc, const in
 template void launch_gemv_rows_multi<double>(const GemvDescT<double>*, const int*, const int*, int64_t, int, int64_t,
                                              int64_t, cudaStream_t);
 
-// ------------------------------------------------------------------ coarse solve
-// L_E L_E^T e = c by blocked substitution in one cooperative launch.  The
-// factor is split into K diagonal blocks of SB rows whose inverses Y_kk are
-// stored.  Forward, for k = 0..K-1: y_k = Y_kk t_k (t = c, updated in
-// place), then every later row r subtracts L[r, block k] y_k.  Backward, for
-// k = K-1..0: e_k = Y_kk^T y_k, then every earlier row r subtracts
-// (L^T)[r, block k] e_k.  Each phase spreads its rows over all warps of the
-// grid (one warp per row, lane-strided products, fixed shuffle tree), and a
-// grid-wide barrier separates the phases; rows outside the envelope of L_E
-// (first column env_row[r], column r ends at env_colend[r]) are skipped.
-// One CTA of 1024 threads per SM keeps the barrier to one arrival per SM.
-// With nb right-hand sides (vectors ldv apart) each matrix entry is read once
-// and applied to all of them.
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-constexpr int CSOLVE_THREADS = 1024;
-
-// NB: the largest number of right-hand sides of the instantiation (1 for a
-// single solve: no per-entry loop over right-hand sides at all).
-template <int NB>
-__global__ void __launch_bounds__(CSOLVE_THREADS) coarse_solve_kernel(CoarseSolveArgs a) {
-    cg::grid_group grid = cg::this_grid();
-    const int lane = threadIdx.x & 31;
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-    const int n = a.n, SB = a.SB, K = a.K, nb = NB == 1 ? 1 : a.nb;
-    const int64_t lv = a.ldv;
-    double* t = a.c;
-    double s[NB];
-    auto reduce_store = [&](double* out, int idx, bool sub) {
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-            if (k >= nb) break;
-            const double v = warp_sum_d(s[k]);
-            if (lane == 0) {
-                if (sub)
-                    out[k * lv + idx] -= v;
-                else
-                    out[k * lv + idx] = v;
-            }
-        }
-    };
-    for (int k0 = 0; k0 < K; ++k0) {
-        const int r0 = k0 * SB, sb = min(SB, n - r0), r1 = r0 + sb;
-        const double* Y = a.Yd + (size_t)k0 * SB * SB;
-        for (int i = gw; i < sb; i += nw) {
-            const double* row = Y + (size_t)i * SB;
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            for (int j = lane; j <= i; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, t[k * lv + r0 + j], s[k]);
-            }
-            reduce_store(a.y, r0 + i, false);
-        }
-        grid.sync();
-        if (k0 + 1 == K) break;
-        for (int r = r1 + gw; r < n; r += nw) {
-            const int j0 = max(a.env_row[r], r0);
-            if (j0 >= r1) continue;
-            const double* row = a.L + (size_t)r * a.ld;
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            for (int j = j0 + lane; j < r1; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, a.y[k * lv + j], s[k]);
-            }
-            reduce_store(t, r, true);
-        }
-        grid.sync();
-    }
-    for (int k0 = K - 1; k0 >= 0; --k0) {
-        const int r0 = k0 * SB, sb = min(SB, n - r0), r1 = r0 + sb;
-        const double* Yt = a.Ydt + (size_t)k0 * SB * SB;
-        for (int i = gw; i < sb; i += nw) {
-            const double* row = Yt + (size_t)i * SB;
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            for (int j = i + lane; j < sb; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, a.y[k * lv + r0 + j], s[k]);
-            }
-            reduce_store(a.e, r0 + i, false);
-        }
-        if (k0 == 0) break;
-        grid.sync();
-        for (int r = gw; r < r0; r += nw) {
-            const int j1 = min(a.env_colend[r], r1);
-            if (j1 <= r0) continue;
-            const double* row = a.Lt + (size_t)r * a.ld;
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            for (int j = r0 + lane; j < j1; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, a.e[k * lv + j], s[k]);
-            }
-            reduce_store(a.y, r, true);
-        }
-        grid.sync();
-    }
-}
-
-template <int NB>
-__global__ void __launch_bounds__(CSOLVE_THREADS) coarse_solve_folded_kernel(CoarseSolveArgs a) {
-    cg::grid_group grid = cg::this_grid();
-    const int lane = threadIdx.x & 31;
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-    const int n = a.n, SB = a.SB, K = a.K, FW = a.FW, nb = NB == 1 ? 1 : a.nb;
-    const int64_t lv = a.ldv;
-    double s[NB];
-    auto store = [&](double* out, int idx) {
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-            if (k >= nb) break;
-            const double v = warp_sum_d(s[k]);
-            if (lane == 0) out[k * lv + idx] = v;
-        }
-    };
-    // forward: y_k = Yd_k c_k - F_k y(window), windows of earlier blocks complete
-    for (int k0 = 0; k0 < K; ++k0) {
-        const int r0 = k0 * SB, sb = min(SB, n - r0);
-        const double* Y = a.Yd + (size_t)k0 * SB * SB;
-        const double* F = a.F + (size_t)k0 * SB * FW;
-        const int w0 = a.fw0[k0], W = r0 - w0;
-        for (int i = gw; i < sb; i += nw) {
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            const double* row = Y + (size_t)i * SB;
-            for (int j = lane; j <= i; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, a.c[k * lv + r0 + j], s[k]);
-            }
-            const double* frow = F + (size_t)i * FW;
-            for (int j = lane; j < W; j += 32) {
-                const double m = frow[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(-m, a.y[k * lv + w0 + j], s[k]);
-            }
-            store(a.y, r0 + i);
-        }
-        grid.sync();
-    }
-    // backward: e_k = Ydt_k y_k - G_k e(window), windows of later blocks complete
-    for (int k0 = K - 1; k0 >= 0; --k0) {
-        const int r0 = k0 * SB, sb = min(SB, n - r0), r1 = r0 + sb;
-        const double* Yt = a.Ydt + (size_t)k0 * SB * SB;
-        const double* G = a.G + (size_t)k0 * SB * FW;
-        const int V = a.gw1[k0] - r1;
-        for (int i = gw; i < sb; i += nw) {
-#pragma unroll
-            for (int k = 0; k < NB; ++k) s[k] = 0.0;
-            const double* row = Yt + (size_t)i * SB;
-            for (int j = i + lane; j < sb; j += 32) {
-                const double m = row[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(m, a.y[k * lv + r0 + j], s[k]);
-            }
-            const double* grow = G + (size_t)i * FW;
-            for (int j = lane; j < V; j += 32) {
-                const double m = grow[j];
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    if (NB == 1 || k < nb) s[k] = fma(-m, a.e[k * lv + r1 + j], s[k]);
-            }
-            store(a.e, r0 + i);
-        }
-        if (k0 > 0) grid.sync();
-    }
-}
-
-int coarse_solve_blocks() {
-    int dev = 0, sms = 0, per = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    int per8 = 0;
-    int pf = 0, pf8 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, coarse_solve_kernel<1>, CSOLVE_THREADS, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per8, coarse_solve_kernel<MAXB>, CSOLVE_THREADS, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf, coarse_solve_folded_kernel<1>, CSOLVE_THREADS, 0) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pf8, coarse_solve_folded_kernel<MAXB>, CSOLVE_THREADS, 0) !=
-            cudaSuccess)
-        return 0;
-    per = std::min(std::min(per, per8), std::min(pf, pf8));
-    // one CTA per SM: the grid barriers between phases then take one arrival per SM
-    return per >= 1 ? sms : 0;
-}
-
-cudaError_t launch_coarse_solve(const CoarseSolveArgs& a, int blocks, cudaStream_t s) {
-    CoarseSolveArgs arg = a;
-    void* params[] = {&arg};
-    const void* fn = a.F ? (a.nb == 1 ? (const void*)coarse_solve_folded_kernel<1>
-                                      : (const void*)coarse_solve_folded_kernel<MAXB>)
-                         : (a.nb == 1 ? (const void*)coarse_solve_kernel<1> : (const void*)coarse_solve_kernel<MAXB>);
-    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(CSOLVE_THREADS), params, 0, s);
-}
-
 }  // namespace amdd

@@ -84,51 +84,6 @@ void launch_gather_idx64(const int64_t* src, int64_t cnt, const double* val, dou
     if (cnt > 0) gather_idx64_kernel<<<grid_for(cnt, 152 * 32), 256, 0, s>>>(src, cnt, val, out);
 }
 
-// ------------------------------------------------------------------ coarse ordering
-__global__ void __launch_bounds__(256) sym_permute_kernel(const double* __restrict__ E, double* __restrict__ Ep,
-                                                          const int32_t* __restrict__ perm, int64_t n) {
-    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
-        const int64_t pr = perm[r];
-        double* out = Ep + r * n;
-        for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-            double v = 0.0;
-            if (c <= r) {
-                const int64_t pc = perm[c];
-                v = pr >= pc ? E[pr * n + pc] : E[pc * n + pr];
-            }
-            out[c] = v;
-        }
-    }
-}
-
-void launch_sym_permute(const double* E, double* Ep, const int32_t* perm, int64_t n, cudaStream_t s) {
-    if (n > 0) sym_permute_kernel<<<(unsigned)(n < 152 * 64 ? n : 152 * 64), 256, 0, s>>>(E, Ep, perm, n);
-}
-
-__global__ void __launch_bounds__(256) perm_move_kernel(int64_t n, const int32_t* __restrict__ perm,
-                                                        const double* __restrict__ src, double* __restrict__ dst,
-                                                        int nb, int64_t ld, int scatter) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t q = perm[r];
-        for (int k = 0; k < nb; ++k) {
-            if (scatter)
-                dst[k * ld + q] = src[k * ld + r];
-            else
-                dst[k * ld + r] = src[k * ld + q];
-        }
-    }
-}
-
-void launch_perm_gather(int64_t n, const int32_t* perm, const double* src, double* dst, int nb, int64_t ld,
-                        cudaStream_t s) {
-    if (n > 0) perm_move_kernel<<<grid_for(n, 152 * 8), 256, 0, s>>>(n, perm, src, dst, nb, ld, 0);
-}
-
-void launch_perm_scatter(int64_t n, const int32_t* perm, const double* src, double* dst, int nb, int64_t ld,
-                         cudaStream_t s) {
-    if (n > 0) perm_move_kernel<<<grid_for(n, 152 * 8), 256, 0, s>>>(n, perm, src, dst, nb, ld, 1);
-}
-
 // ------------------------------------------------------------------ residual SpMV
 // y = b - A x, G lanes per row as in the plain SpMV.
 template <int G>
