@@ -167,9 +167,8 @@ struct amdd_handle {
     std::vector<GemvDesc> gv_zp_h;  // host copy (the batched path rebinds x / y)
     int32_t *d_g4_desc = nullptr, *d_g4_row = nullptr;  // row groups (one warp each) of the local products
     int64_t n_g4 = 0;
-    int32_t *d_order_g = nullptr, *d_own_sub = nullptr, *d_own_a = nullptr, *d_sc_idx = nullptr;
-    int32_t *d_nI = nullptr, *d_p = nullptr;
-    int64_t *d_sc_ptr = nullptr, *d_zt_off = nullptr, *d_coff = nullptr;
+    int32_t *d_order_g = nullptr, *d_sc_idx = nullptr;
+    int64_t* d_sc_ptr = nullptr;
     double *d_rloc = nullptr, *d_tloc = nullptr, *d_yloc = nullptr;
     // mixed form: FP32 local factors and local work vectors
     int precision = 0;
@@ -186,6 +185,10 @@ struct amdd_handle {
     int eig_solver = 0, keep_prop = 0;
     int n_robust = 0;  // subdomains whose Schur complement took the robust form (step 5b)
     bool diag_basis = true;  // full selections use the basis diag(A_II)^{-1/2}
+    // every subdomain has that basis: the coarse restriction and prolongation
+    // are scalings by d_dsc (owner order), and no Z_i is stored
+    bool all_diag = false;
+    double* d_dsc = nullptr;
     amdd_proposal prop{};
     bool have_prop = false;
     std::vector<int> eig_iters;  // per subdomain: LOBPCG iterations, -1 dense path, -2 not partial
@@ -1873,11 +1876,20 @@ std::vector<int> learned_eigvecs(Ctx& C, amdd_handle* h, const std::vector<int>&
 constexpr int FRONT_LEAF = 96;
 constexpr int FRONT_RATIO = 20;
 
-// Factors E (dense lower triangle, order nC, subdomain order) in the plan's
-// stages: each part's front collects its entries of E and its children's Schur
+// Entries of E given through the CSR values of A (every subdomain has the
+// diagonal basis): of unknown t (subdomain order) the position of its diagonal
+// entry, and the lower-triangle entries as (unknown, unknown, position).
+struct SparseE {
+    std::vector<int64_t> diag;
+    std::vector<int32_t> row, col;
+    std::vector<int64_t> src;
+};
+
+// Factors E (dense lower triangle, order nC, subdomain order, or the entries
+// sp) in the plan's stages: each part's front collects its entries of E and its children's Schur
 // complements, a partial Cholesky eliminates the interior, and the interior's
 // inverse Ainv = Y^T Y (Y = L_II^{-1}) and W^T = L_BI Y are kept for the solve.
-void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, int64_t nC) {
+void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, int64_t nC, const SparseE* sp) {
     cudaStream_t s = h->s;
     const int nf = (int)P.fronts.size(), S = P.stages();
     std::vector<FrontDev> fd(nf);
@@ -1953,6 +1965,36 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
     fs.stages = S;
     fs.row_off = P.stage_off;
     fs.perm = C.up(P.perm, true);
+    fs.src = fs.perm;
+    fs.scale = nullptr;
+    if (sp) {
+        // plan-order scales, and each entry into the front of its earlier unknown
+        std::vector<int64_t> pos(P.n), dg(P.n), dst(sp->src.size());
+        std::vector<int32_t> ea(sp->src.size()), eb(sp->src.size()), gsrc(P.n);
+        for (int64_t k = 0; k < P.n; ++k) {
+            pos[P.perm[k]] = k;
+            dg[k] = sp->diag[P.perm[k]];
+        }
+        for (size_t e = 0; e < sp->src.size(); ++e) {
+            const int64_t p = pos[sp->row[e]], q = pos[sp->col[e]];
+            const int64_t a = std::max(p, q), b = std::min(p, q);
+            const Front& f = P.fronts[rfront[b]];
+            const int64_t ld = f.m + f.nb;
+            int64_t r = a - f.i0;
+            if (r >= f.m) {
+                const int32_t* lo = P.bnd.data() + f.b0;
+                r = f.m + (std::lower_bound(lo, lo + f.nb, (int32_t)a) - lo);
+            }
+            dst[e] = oF[rfront[b]] + r * ld + (b - f.i0);
+            ea[e] = (int32_t)a;
+            eb[e] = (int32_t)b;
+        }
+        double* sc = dnew<double>(h, P.n);
+        h->d_dsc = dnew<double>(h, P.n);
+        launch_front_scale(h->val, C.up(dg), fs.perm, sc, h->d_dsc, P.n, s);
+        launch_front_scatter(h->val, C.up(sp->src), C.up(dst), C.up(ea), C.up(eb), sc, F, (int64_t)dst.size(), s);
+        fs.scale = sc;
+    }
     fs.fr = C.up(fd, true);
     fs.row_front = C.up(rfront, true);
     fs.bnd = C.up(P.bnd, true);
@@ -1993,7 +2035,7 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
                 tr.push_back({Wt + oW[k], W + oW[k], b, m, m, b});
             }
         }
-        {
+        if (!sp) {
             PScope ps(h, PK_E_ASM, 0.0);
             launch_front_gather(fs.fr + k0, k1 - k0, fs.bnd, fs.perm, E, nC, maxn, s);
         }
@@ -2139,6 +2181,16 @@ void build_sparse_local(Ctx& C, amdd_handle* h, const std::vector<int64_t>& rp, 
     h->sl_nmax = n_max;
     h->sl_nnz = nnz_tot;
     h->sparse_local = true;
+}
+
+// Global unknown of each plan position when every subdomain has the diagonal
+// basis (coarse unknowns are the unknowns in subdomain order).
+std::vector<int32_t> plan_globals(const FrontPlan& P, const std::vector<std::vector<int32_t>>& Il) {
+    std::vector<int32_t> own, g(P.n);
+    own.reserve(P.n);
+    for (const auto& I : Il) own.insert(own.end(), I.begin(), I.end());
+    for (int64_t k = 0; k < P.n; ++k) g[k] = own[P.perm[k]];
+    return g;
 }
 
 template <typename T, typename TS>
@@ -2352,138 +2404,139 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         // Cholesky factor and inverse factor
         cudaStream_t s = h->s;  // the stream this call runs on
         const int64_t nC = h->nC;
+        h->all_diag = diag_basis && nC > 0 && h->p == h->nI;
         if (nC > 0) {
-            std::vector<int64_t> off_az(N + 1, 0);
-            for (int i = 0; i < N; ++i) off_az[i + 1] = off_az[i] + (int64_t)h->ni[i] * h->p[i];
-            double* AZ = C.tnew<double>(off_az[N]);
-            double* E = C.tnew<double>((size_t)nC * nC);  // lower triangle
-            ck(cudaMemsetAsync(E, 0, (size_t)nC * nC * sizeof(double), s));
-            std::vector<GemmDesc> g1, g2;
-            std::vector<DiagScaleDesc> dsd;
-            int max_ni_d = 1;
-            for (int i = 0; i < N; ++i) {
-                if (h->p[i] == 0) continue;
-                const int ni = h->ni[i], nIi = h->nI[i], pi = h->p[i];
-                if (diag_basis && pi == nIi) {
-                    // Z_i = diag(A_II)^{-1/2}: AZ_i and E_ii are scalings of A_ii
-                    // (the same products as the GEMMs, whose other terms are zeros)
-                    dsd.push_back({Araw + h->off_sq[i], ni, nIi, AZ + off_az[i], E + (size_t)h->coff[i] * nC + h->coff[i],
-                                   (int64_t)nC});
-                    max_ni_d = std::max(max_ni_d, ni);
-                    continue;
-                }
-                // AZ_i = A(Omega_i, Omega_Ii) Z_i   (ni x p_i)
-                g1.push_back(gd(Araw + h->off_sq[i], ni, 0, h->d_Zt + h->off_zt[i], nIi, 1, AZ + off_az[i], pi, ni, pi,
-                                nIi, 1.0, 0.0, 0));
-                // E_ii = Z_i^T A_II Z_i
-                g2.push_back(gd(h->d_Zt + h->off_zt[i], nIi, 0, AZ + off_az[i], pi, 0,
-                                E + (size_t)h->coff[i] * nC + h->coff[i], (int)nC, pi, pi, nIi, 1.0, 0.0, 1));
-            }
-            gemm(C, g1);
-            gemm(C, g2);
-            if (!dsd.empty()) {
-                auto d = C.up(dsd);
-                PScope ps(h, PK_SMALL, 0.0, 0.0);
-                launch_diag_scale(d, (int)dsd.size(), max_ni_d, s);
-            }
-            // E_ij (i > j) = sum over g in Omega_Ii cap Omega_j of Z_i[g]^T (A Z_j)[g]
             std::vector<int32_t> posI(n, -1);
             for (int i = 0; i < N; ++i)
                 for (int a = 0; a < h->nI[i]; ++a) posI[Il[i][a]] = a;
-            std::vector<std::vector<std::pair<int32_t, int32_t>>> lists;  // per pair
-            std::vector<std::pair<int, int>> pairs;
-            {
-                std::vector<int> slot(N, -1);
-                for (int j = 0; j < N; ++j) {
-                    if (h->p[j] == 0) continue;
-                    std::fill(slot.begin(), slot.end(), -1);
-                    std::vector<int> touched;
-                    const int32_t* om = omega.data() + h->off_om[j];
-                    for (int ps = 0; ps < h->ni[j]; ++ps) {
-                        const int32_t g = om[ps];
-                        const int i = part[g];
-                        if (i <= j || h->p[i] == 0) continue;
-                        if (slot[i] < 0) {
-                            slot[i] = (int)pairs.size();
-                            pairs.push_back({i, j});
-                            lists.emplace_back();
-                        }
-                        lists[slot[i]].push_back({posI[g], ps});
-                    }
-                }
-            }
-            std::vector<int32_t> la, lpos;
-            std::vector<EPairRef> et;
-            for (size_t q = 0; q < pairs.size(); ++q) {
-                const int i = pairs[q].first, j = pairs[q].second;
-                const int64_t lo = (int64_t)la.size();
-                for (auto& e : lists[q]) {
-                    la.push_back(e.first);
-                    lpos.push_back(e.second);
-                }
-                for (int tr = 0; tr * 32 < h->p[i]; ++tr)
-                    for (int tc = 0; tc * 32 < h->p[j]; ++tc) {
-                        EPairRef t;
-                        t.i = i;
-                        t.j = j;
-                        t.list_off = lo;
-                        t.list_len = (int)lists[q].size();
-                        t.tr = tr;
-                        t.tc = tc;
-                        et.push_back(t);
-                    }
-            }
-            std::vector<int32_t> nIv(h->nI.begin(), h->nI.end()), pv(h->p.begin(), h->p.end());
-            h->d_zt_off = C.up(std::vector<int64_t>(h->off_zt.begin(), h->off_zt.end() - 1), true);
-            h->d_nI = C.up(nIv, true);
-            h->d_p = C.up(pv, true);
-            h->d_coff = C.up(std::vector<int64_t>(h->coff.begin(), h->coff.end() - 1), true);
-            if (!et.empty()) {
-                auto a = C.up(et);
-                auto b = C.up(la);
-                auto c = C.up(lpos);
-                auto d = C.up(std::vector<int64_t>(off_az.begin(), off_az.end() - 1));
-                double fl = 0.0;
-                for (size_t q = 0; q < pairs.size(); ++q)
-                    fl += 2.0 * h->p[pairs[q].first] * h->p[pairs[q].second] * lists[q].size();
-                PScope ps(h, PK_E_ASM, fl);
-                launch_e_offdiag(a, (int)et.size(), b, c, h->d_Zt, h->d_zt_off, h->d_nI, AZ, d, h->d_p, h->d_coff, E, nC,
-                                 s);
-            }
-            if (h->keep_E) {
-                // a copy of E for a next level (multilevel form), as a sparse matrix
-                // with the block pattern: every entry of E_ij for i == j or for
-                // subdomains coupled in A (a structural non-zero in
-                // A(Omega_Ii, Omega_Ij)); E holds its lower triangle
-                std::vector<std::vector<int>> adj(N);
-                for (int64_t g = 0; g < n; ++g)
-                    for (int64_t k = rp[g]; k < rp[g + 1]; ++k)
-                        if (part[g] != part[ci[k]]) adj[part[g]].push_back(part[ci[k]]);
+            double* E = nullptr;
+            if (!h->all_diag) {
+                std::vector<int64_t> off_az(N + 1, 0);
+                for (int i = 0; i < N; ++i) off_az[i + 1] = off_az[i] + (int64_t)h->ni[i] * h->p[i];
+                double* AZ = C.tnew<double>(off_az[N]);
+                E = C.tnew<double>((size_t)nC * nC);  // lower triangle
+                ck(cudaMemsetAsync(E, 0, (size_t)nC * nC * sizeof(double), s));
+                std::vector<GemmDesc> g1, g2;
+                std::vector<DiagScaleDesc> dsd;
+                int max_ni_d = 1;
                 for (int i = 0; i < N; ++i) {
-                    adj[i].push_back(i);
-                    std::sort(adj[i].begin(), adj[i].end());
-                    adj[i].erase(std::unique(adj[i].begin(), adj[i].end()), adj[i].end());
-                }
-                std::vector<int64_t> erp(nC + 1, 0), esrc;
-                std::vector<int32_t> ecol;
-                for (int i = 0; i < N; ++i)
-                    for (int k = 0; k < h->p[i]; ++k) {
-                        const int64_t r = h->coff[i] + k;
-                        for (int j : adj[i])
-                            for (int l = 0; l < h->p[j]; ++l) {
-                                const int64_t c = h->coff[j] + l;
-                                ecol.push_back((int32_t)c);
-                                esrc.push_back(std::max(r, c) * nC + std::min(r, c));
-                            }
-                        erp[r + 1] = (int64_t)ecol.size();
+                    if (h->p[i] == 0) continue;
+                    const int ni = h->ni[i], nIi = h->nI[i], pi = h->p[i];
+                    if (diag_basis && pi == nIi) {
+                        // Z_i = diag(A_II)^{-1/2}: AZ_i and E_ii are scalings of A_ii
+                        // (the same products as the GEMMs, whose other terms are zeros)
+                        dsd.push_back({Araw + h->off_sq[i], ni, nIi, AZ + off_az[i], E + (size_t)h->coff[i] * nC + h->coff[i],
+                                       (int64_t)nC});
+                        max_ni_d = std::max(max_ni_d, ni);
+                        continue;
                     }
-                h->E_nnz = (int64_t)ecol.size();
-                h->d_E_rowptr = C.up(erp, true);
-                h->d_E_col = C.up(ecol, true);
-                h->d_E_val = dnew<double>(h, h->E_nnz);
-                auto dsrc = C.up(esrc);
-                PScope ps(h, PK_SMALL, 0.0, 16.0 * h->E_nnz);
-                launch_gather_idx64(dsrc, h->E_nnz, E, h->d_E_val, s);
+                    // AZ_i = A(Omega_i, Omega_Ii) Z_i   (ni x p_i)
+                    g1.push_back(gd(Araw + h->off_sq[i], ni, 0, h->d_Zt + h->off_zt[i], nIi, 1, AZ + off_az[i], pi, ni, pi,
+                                    nIi, 1.0, 0.0, 0));
+                    // E_ii = Z_i^T A_II Z_i
+                    g2.push_back(gd(h->d_Zt + h->off_zt[i], nIi, 0, AZ + off_az[i], pi, 0,
+                                    E + (size_t)h->coff[i] * nC + h->coff[i], (int)nC, pi, pi, nIi, 1.0, 0.0, 1));
+                }
+                gemm(C, g1);
+                gemm(C, g2);
+                if (!dsd.empty()) {
+                    auto d = C.up(dsd);
+                    PScope ps(h, PK_SMALL, 0.0, 0.0);
+                    launch_diag_scale(d, (int)dsd.size(), max_ni_d, s);
+                }
+                // E_ij (i > j) = sum over g in Omega_Ii cap Omega_j of Z_i[g]^T (A Z_j)[g]
+                std::vector<std::vector<std::pair<int32_t, int32_t>>> lists;  // per pair
+                std::vector<std::pair<int, int>> pairs;
+                {
+                    std::vector<int> slot(N, -1);
+                    for (int j = 0; j < N; ++j) {
+                        if (h->p[j] == 0) continue;
+                        std::fill(slot.begin(), slot.end(), -1);
+                        std::vector<int> touched;
+                        const int32_t* om = omega.data() + h->off_om[j];
+                        for (int ps = 0; ps < h->ni[j]; ++ps) {
+                            const int32_t g = om[ps];
+                            const int i = part[g];
+                            if (i <= j || h->p[i] == 0) continue;
+                            if (slot[i] < 0) {
+                                slot[i] = (int)pairs.size();
+                                pairs.push_back({i, j});
+                                lists.emplace_back();
+                            }
+                            lists[slot[i]].push_back({posI[g], ps});
+                        }
+                    }
+                }
+                std::vector<int32_t> la, lpos;
+                std::vector<EPairRef> et;
+                for (size_t q = 0; q < pairs.size(); ++q) {
+                    const int i = pairs[q].first, j = pairs[q].second;
+                    const int64_t lo = (int64_t)la.size();
+                    for (auto& e : lists[q]) {
+                        la.push_back(e.first);
+                        lpos.push_back(e.second);
+                    }
+                    for (int tr = 0; tr * 32 < h->p[i]; ++tr)
+                        for (int tc = 0; tc * 32 < h->p[j]; ++tc) {
+                            EPairRef t;
+                            t.i = i;
+                            t.j = j;
+                            t.list_off = lo;
+                            t.list_len = (int)lists[q].size();
+                            t.tr = tr;
+                            t.tc = tc;
+                            et.push_back(t);
+                        }
+                }
+                std::vector<int32_t> nIv(h->nI.begin(), h->nI.end()), pv(h->p.begin(), h->p.end());
+                if (!et.empty()) {
+                    auto a = C.up(et);
+                    auto b = C.up(la);
+                    auto c = C.up(lpos);
+                    auto d = C.up(std::vector<int64_t>(off_az.begin(), off_az.end() - 1));
+                    double fl = 0.0;
+                    for (size_t q = 0; q < pairs.size(); ++q)
+                        fl += 2.0 * h->p[pairs[q].first] * h->p[pairs[q].second] * lists[q].size();
+                    PScope ps(h, PK_E_ASM, fl);
+                    launch_e_offdiag(a, (int)et.size(), b, c, h->d_Zt,
+                                     C.up(std::vector<int64_t>(h->off_zt.begin(), h->off_zt.end() - 1)), C.up(nIv), AZ, d,
+                                     C.up(pv), C.up(std::vector<int64_t>(h->coff.begin(), h->coff.end() - 1)), E, nC, s);
+                }
+                if (h->keep_E) {
+                    // a copy of E for a next level (multilevel form), as a sparse matrix
+                    // with the block pattern: every entry of E_ij for i == j or for
+                    // subdomains coupled in A (a structural non-zero in
+                    // A(Omega_Ii, Omega_Ij)); E holds its lower triangle
+                    std::vector<std::vector<int>> adj(N);
+                    for (int64_t g = 0; g < n; ++g)
+                        for (int64_t k = rp[g]; k < rp[g + 1]; ++k)
+                            if (part[g] != part[ci[k]]) adj[part[g]].push_back(part[ci[k]]);
+                    for (int i = 0; i < N; ++i) {
+                        adj[i].push_back(i);
+                        std::sort(adj[i].begin(), adj[i].end());
+                        adj[i].erase(std::unique(adj[i].begin(), adj[i].end()), adj[i].end());
+                    }
+                    std::vector<int64_t> erp(nC + 1, 0), esrc;
+                    std::vector<int32_t> ecol;
+                    for (int i = 0; i < N; ++i)
+                        for (int k = 0; k < h->p[i]; ++k) {
+                            const int64_t r = h->coff[i] + k;
+                            for (int j : adj[i])
+                                for (int l = 0; l < h->p[j]; ++l) {
+                                    const int64_t c = h->coff[j] + l;
+                                    ecol.push_back((int32_t)c);
+                                    esrc.push_back(std::max(r, c) * nC + std::min(r, c));
+                                }
+                            erp[r + 1] = (int64_t)ecol.size();
+                        }
+                    h->E_nnz = (int64_t)ecol.size();
+                    h->d_E_rowptr = C.up(erp, true);
+                    h->d_E_col = C.up(ecol, true);
+                    h->d_E_val = dnew<double>(h, h->E_nnz);
+                    auto dsrc = C.up(esrc);
+                    PScope ps(h, PK_SMALL, 0.0, 16.0 * h->E_nnz);
+                    launch_gather_idx64(dsrc, h->E_nnz, E, h->d_E_val, s);
+                }
             }
             // ---- graph of E: a vertex per coarse unknown of a diagonal-basis
             // subdomain (E has A's own entries there), one vertex for all unknowns
@@ -2526,12 +2579,26 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 }
                 if (!fd) close_row(vfirst[i]);
             }
-            factor_fronts(C, h, plan_fronts(aptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO), E, nC);
-        } else {
-            h->d_zt_off = C.up(std::vector<int64_t>(h->off_zt.begin(), h->off_zt.end() - 1), true);
-            h->d_nI = C.up(std::vector<int32_t>(h->nI.begin(), h->nI.end()), true);
-            h->d_p = C.up(std::vector<int32_t>(h->p.begin(), h->p.end()), true);
-            h->d_coff = C.up(std::vector<int64_t>(h->coff.begin(), h->coff.end() - 1), true);
+            SparseE sp;
+            if (h->all_diag) {
+                sp.diag.assign(nC, -1);
+                for (int i = 0; i < N; ++i)
+                    for (int a = 0; a < h->nI[i]; ++a) {
+                        const int64_t g = Il[i][a];
+                        const int32_t t = (int32_t)(h->coff[i] + a);
+                        for (int64_t q = rp[g]; q < rp[g + 1]; ++q) {
+                            const int32_t u = (int32_t)(h->coff[part[ci[q]]] + posI[ci[q]]);
+                            if (u == t) sp.diag[t] = q;
+                            if (u > t) continue;
+                            sp.row.push_back(t);
+                            sp.col.push_back(u);
+                            sp.src.push_back(q);
+                        }
+                    }
+            }
+            const FrontPlan plan = plan_fronts(aptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO);
+            factor_fronts(C, h, plan, E, nC, h->all_diag ? &sp : nullptr);
+            if (h->all_diag) h->fs.src = C.up(plan_globals(plan, Il), true);
         }
     };
 
@@ -2569,8 +2636,6 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             std::swap(h->ev_far, h->ev_far3);
         };
         try {
-            h->d_Zt = dnew<double>(h, h->sum_zt);
-            fill_diag_zt();
             factor_coarse();
             ck(cudaEventRecord(h->ev_spec_done, h->s));
         } catch (...) {
@@ -2990,18 +3055,21 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->eig_iters.assign(N, -2);
         if (mf) h->eig_iters = mf_its;
     } else {
-        h->d_Zt = dnew<double>(h, h->sum_zt);
+        const bool all_diag = diag_basis && h->p == h->nI;  // no Z_i is stored then
+        h->d_Zt = all_diag ? nullptr : dnew<double>(h, h->sum_zt);
         T* ZtT = nullptr;
         if constexpr (f64)
             ZtT = h->d_Zt;
-        else
+        else if (!all_diag)
             ZtT = C.tnew<T>(h->sum_zt);
         // full selections: the basis diag(A_II)^{-1/2} keeps every block of E that
         // touches such a subdomain as sparse as A (its envelope-aware Cholesky and
         // the coarse solve then skip most tiles); with a kept E (multilevel form)
         // the A_II-orthonormal rows of L_A^{-1}, so that E is a block-orthogonal
         // congruence of the one any other A_II-orthonormal basis gives
-        if (h->nC > 0) {
+        if (h->nC > 0 && all_diag) {
+            h->eig_iters.assign(N, -2);
+        } else if (h->nC > 0) {
             std::vector<int64_t> ysrc, ydst;
             std::vector<int32_t> ylen;
             for (int i = 0; i < N; ++i) {
@@ -3132,9 +3200,11 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->d_c = dnew<double>(h, nC);
         h->d_e = dnew<double>(h, nC);
         if (nC > 0) {
-            h->d_Zr = dnew<double>(h, h->sum_zt);
             h->d_zc = dnew<double>(h, n);
             ck(cudaMemsetAsync(h->d_zc, 0, n * sizeof(double), s));
+        }
+        if (nC > 0 && !h->all_diag) {
+            h->d_Zr = dnew<double>(h, h->sum_zt);
             std::vector<TransDesc> tdz;
             std::vector<int32_t> rdz, rlz;
             int maxd = 1;
@@ -3170,13 +3240,14 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             h->lm2[i] = Ylt + h->off_sq[i];
             l1[i] = {Yl + h->off_sq[i], ni, ni, ni, 1, rlocT + h->off_om[i], tlocT + h->off_om[i]};
             l2[i] = {Ylt + h->off_sq[i], ni, ni, ni, 2, tlocT + h->off_om[i], ylocT + h->off_om[i]};
-            cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_rloc + h->off_om[i],
-                     h->d_c + h->coff[i]};
+            if (h->d_Zt)
+                cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_rloc + h->off_om[i],
+                         h->d_c + h->coff[i]};
             for (int a = 0; a < ni; a += GEMV_ROWS_PER_WARP) {
                 rd.push_back(i);
                 rl.push_back(a);
             }
-            for (int k = 0; k < h->p[i]; ++k) {
+            for (int k = 0; k < h->p[i] && !h->all_diag; ++k) {
                 rdc.push_back(i);
                 rlc.push_back(k);
             }
@@ -3201,21 +3272,12 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         std::vector<int32_t> sci(h->sum_ni);
         std::vector<int64_t> fill(scp.begin(), scp.end() - 1);
         for (int64_t t = 0; t < h->sum_ni; ++t) sci[fill[omega[t]]++] = (int32_t)t;
-        std::vector<int32_t> og, osub, oa;
+        std::vector<int32_t> og;
         og.reserve(n);
-        osub.reserve(n);
-        oa.reserve(n);
-        for (int i = 0; i < N; ++i)
-            for (int a = 0; a < h->nI[i]; ++a) {
-                og.push_back(Il[i][a]);
-                osub.push_back(i);
-                oa.push_back(a);
-            }
+        for (int i = 0; i < N; ++i) og.insert(og.end(), Il[i].begin(), Il[i].end());
         h->d_sc_ptr = C.up(scp, true);
         h->d_sc_idx = C.up(sci, true);
         h->d_order_g = C.up(og, true);
-        h->d_own_sub = C.up(osub, true);
-        h->d_own_a = C.up(oa, true);
         // PCG vectors
         h->d_r = dnew<double>(h, n);
         h->d_z = dnew<double>(h, n);
@@ -3288,13 +3350,18 @@ void local_solves(amdd_handle* h, const double* r) {
     }
 }
 
-// Coarse correction R_0^T E^{-1} R_0 r of Eq. (two_level_schwarz) from the
-// gathered rloc (its Omega_Ii entries): c = Z^T r, the solve with L_E, and
+// Coarse correction R_0^T E^{-1} R_0 r of Eq. (two_level_schwarz) from r and the
+// gathered rloc (its Omega_Ii entries): c = Z^T r, the solve with E, and
 // zc = Z e in owner order (d_zc).  Needs nC > 0.
 void inner_coarse_solve(amdd_handle* h);
 
-void coarse_correction(amdd_handle* h) {
+void coarse_correction(amdd_handle* h, const double* r) {
     cudaStream_t s = h->s;
+    if (h->all_diag) {  // c and zc are scalings, done where the solve loads and stores its vectors
+        PScope ps(h, PK_CSOLVE, h->csolve_flops, h->csolve_bytes);
+        launch_front_solve(h->fs, r, h->n, h->d_zc, h->n, 1, s);
+        return;
+    }
     const double zt = (double)h->sum_zt;
     {
         PScope ps(h, PK_GEMV, 2.0 * zt, 8.0 * zt + 8.0 * h->sum_ni + 16.0 * h->nC);
@@ -3317,7 +3384,7 @@ void coarse_correction(amdd_handle* h) {
 void apply_one(amdd_handle* h, const double* r, double* z) {
     cudaStream_t s = h->s;
     local_solves(h, r);
-    if (h->nC > 0) coarse_correction(h);
+    if (h->nC > 0) coarse_correction(h, r);
     PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * h->sum_ni + 24.0 * h->n);
     const double* zc = h->nC > 0 ? h->d_zc : nullptr;
     if (h->precision == 0)
@@ -3354,11 +3421,11 @@ void apply_form(amdd_handle* h, int form, const double* r, double* z) {
     const double* x = r;
     if (form != AMDD_FORM_ASM) ensure_forms(h);
     if (coarse) {
-        {
+        if (!h->all_diag) {
             PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->sum_ni);
             launch_gather_vec(h->d_omega, h->sum_ni, r, h->d_rloc, s);
         }
-        coarse_correction(h);
+        coarse_correction(h, r);
         {
             PScope ps(h, PK_GATHER_SCATTER, 0.0, 24.0 * h->n);
             launch_owner_to_global(h->n, h->d_order_g, h->d_zc, h->d_zg, s);
@@ -3437,14 +3504,16 @@ void ensure_multi(amdd_handle* h) {
     h->d_m_c = dnew<double>(h, CC);
     h->d_m_e = dnew<double>(h, CC);
     if (h->nC > 0) {
+        h->d_m_zc = dnew<double>(h, (int64_t)MAXB * h->n);
+        ck(cudaMemsetAsync(h->d_m_zc, 0, (size_t)MAXB * h->n * sizeof(double), h->s));
+    }
+    if (h->nC > 0 && !h->all_diag) {
         std::vector<GemvDesc> cr(h->N);
         for (int i = 0; i < h->N; ++i)
             cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_m_rloc + h->off_om[i],
                      h->d_m_c + h->coff[i]};
         h->d_m_gv_c = dnew<GemvDesc>(h, h->N);
         ck(cudaMemcpyAsync(h->d_m_gv_c, cr.data(), h->N * sizeof(GemvDesc), cudaMemcpyHostToDevice, h->s));
-        h->d_m_zc = dnew<double>(h, (int64_t)MAXB * h->n);
-        ck(cudaMemsetAsync(h->d_m_zc, 0, (size_t)MAXB * h->n * sizeof(double), h->s));
         std::vector<GemvDesc> zp = h->gv_zp_h;
         int q = 0;
         for (int i = 0; i < h->N; ++i) {
@@ -3518,7 +3587,10 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
             launch_gemv_rows4_multi<float>(g2, h->d_g4_desc, h->d_g4_row, h->n_g4, nb, L, L, s);
         }
     }
-    if (h->nC > 0) {
+    if (h->all_diag) {
+        PScope ps(h, PK_CSOLVE, h->csolve_flops * nb, h->csolve_bytes);
+        launch_front_solve(h->fs, r, h->n, h->d_m_zc, h->n, nb, s);
+    } else if (h->nC > 0) {
         const double zt = (double)h->sum_zt;
         {
             PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * L + 16.0 * h->nC) * nb);
@@ -4715,6 +4787,21 @@ amdd_status amdd_get_coarse_block(const amdd_handle* h, int32_t i, double* Zt, i
     if (nI) *nI = h->nI[i];
     if (Zt && cnt > 0) {
         if (cap < cnt) return AMDD_ERR_INVALID;
+        if (h->all_diag) {  // the rows of diag(A_II)^{-1/2}
+            try {
+                const int nIi = h->nI[i];
+                std::vector<double> d(nIi);
+                if (cudaMemcpyAsync(d.data(), h->d_dsc + h->off_I[i], nIi * sizeof(double), cudaMemcpyDeviceToHost,
+                                    h->s) != cudaSuccess ||
+                    cudaStreamSynchronize(h->s) != cudaSuccess)
+                    return AMDD_ERR_CUDA;
+                std::fill(Zt, Zt + cnt, 0.0);
+                for (int k = 0; k < nIi; ++k) Zt[(size_t)k * nIi + k] = d[k];
+            } catch (...) {
+                return guard_exc();
+            }
+            return AMDD_OK;
+        }
         if (cudaMemcpyAsync(Zt, h->d_Zt + h->off_zt[i], cnt * sizeof(double), cudaMemcpyDeviceToHost, h->s) !=
                 cudaSuccess ||
             cudaStreamSynchronize(h->s) != cudaSuccess)

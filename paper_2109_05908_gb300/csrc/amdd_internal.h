@@ -462,7 +462,9 @@ struct FrontRef {  // a row of W^T and the interior it multiplies
 struct FrontSolve {
     int64_t n = 0;
     int stages = 0;
-    const int32_t* perm = nullptr;  // caller's index of each plan position
+    const int32_t* perm = nullptr;  // caller's index of each plan position (output)
+    const int32_t* src = nullptr;   // its index in the input vectors
+    const double* scale = nullptr;  // with it, input and output entries are multiplied by scale[plan position]
     const FrontDev* fr = nullptr;
     const int32_t* row_front = nullptr;
     const int32_t* bnd = nullptr;
@@ -475,6 +477,12 @@ struct FrontSolve {
 };
 void launch_front_gather(const FrontDev* fr, int nfr, const int32_t* bnd, const int32_t* perm, const double* E,
                          int64_t nE, int maxn, cudaStream_t s);
+// scale[k] = own[perm[k]] = 1 / sqrt(val[diag[k]]) (val 0 where diag[k] < 0), k < n
+void launch_front_scale(const double* val, const int64_t* diag, const int32_t* perm, double* scale, double* own,
+                        int64_t n, cudaStream_t s);
+// F[dst[t]] = val[src[t]] scale[a[t]] scale[b[t]], t < cnt
+void launch_front_scatter(const double* val, const int64_t* src, const int64_t* dst, const int32_t* a,
+                          const int32_t* b, const double* scale, double* F, int64_t cnt, cudaStream_t s);
 void launch_front_extend_add(const FrontDev* fr, int nfr, const FrontChild* kids, const int32_t* maps, int maxn,
                              cudaStream_t s);
 // out = E^{-1} c for nb <= MAXB vectors (c ldc apart, out ldo apart)

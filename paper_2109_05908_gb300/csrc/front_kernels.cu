@@ -111,13 +111,55 @@ void launch_front_extend_add(const FrontDev* fr, int nfr, const FrontChild* kids
             fr + k, kids, maps);
 }
 
-// v[k] = c[perm[k]] for every plan position (nb vectors)
-__global__ void __launch_bounds__(256) front_load_kernel(int64_t n, const int32_t* __restrict__ perm,
+// With the basis diag(A_II)^{-1/2} everywhere E is A itself, scaled on both
+// sides: its entries go straight from the CSR values into the fronts.
+__global__ void __launch_bounds__(256) front_scale_kernel(const double* __restrict__ val,
+                                                          const int64_t* __restrict__ diag,
+                                                          const int32_t* __restrict__ perm,
+                                                          double* __restrict__ scale, double* __restrict__ own,
+                                                          int64_t n) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        const double d = 1.0 / sqrt(diag[k] >= 0 ? val[diag[k]] : 0.0);
+        scale[k] = d;
+        own[perm[k]] = d;
+    }
+}
+
+void launch_front_scale(const double* val, const int64_t* diag, const int32_t* perm, double* scale, double* own,
+                        int64_t n, cudaStream_t s) {
+    const int64_t want = (n + 255) / 256;
+    if (n > 0)
+        front_scale_kernel<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(val, diag, perm, scale, own, n);
+}
+
+__global__ void __launch_bounds__(256) front_scatter_kernel(const double* __restrict__ val,
+                                                            const int64_t* __restrict__ src,
+                                                            const int64_t* __restrict__ dst,
+                                                            const int32_t* __restrict__ a,
+                                                            const int32_t* __restrict__ b,
+                                                            const double* __restrict__ scale,
+                                                            double* __restrict__ F, int64_t cnt) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x)
+        F[dst[t]] = val[src[t]] * scale[b[t]] * scale[a[t]];
+}
+
+void launch_front_scatter(const double* val, const int64_t* src, const int64_t* dst, const int32_t* a,
+                          const int32_t* b, const double* scale, double* F, int64_t cnt, cudaStream_t s) {
+    const int64_t want = (cnt + 255) / 256;
+    if (cnt > 0)
+        front_scatter_kernel<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(val, src, dst, a, b, scale,
+                                                                                           F, cnt);
+}
+
+// v[k] = c[src[k]] (times scale[k] when given) for every plan position (nb vectors)
+__global__ void __launch_bounds__(256) front_load_kernel(int64_t n, const int32_t* __restrict__ src,
+                                                         const double* __restrict__ scale,
                                                          const double* __restrict__ c, int64_t ldc,
                                                          double* __restrict__ v, int nb) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t p = perm[k];
-        for (int q = 0; q < nb; ++q) v[q * n + k] = c[q * ldc + p];
+        const int32_t p = src[k];
+        const double d = scale ? scale[k] : 1.0;
+        for (int q = 0; q < nb; ++q) v[q * n + k] = d * c[q * ldc + p];
     }
 }
 
@@ -147,12 +189,13 @@ __global__ void __launch_bounds__(256) front_down_kernel(int64_t nrow, const int
 }
 
 // Up: one warp per interior row of a stage; e in plan order (read by the
-// earlier stages) and, through perm, in the caller's order.
+// earlier stages) and, through perm (times scale), in the caller's order.
 template <int NB>
 __global__ void __launch_bounds__(256) front_up_kernel(const FrontDev* __restrict__ fr,
                                                        const int32_t* __restrict__ row_front, int64_t r0, int64_t r1,
                                                        const int32_t* __restrict__ bnd,
                                                        const int32_t* __restrict__ perm,
+                                                       const double* __restrict__ scale,
                                                        const double* __restrict__ v, double* e,
                                                        double* __restrict__ out, int64_t n, int64_t ldo, int nb) {
     const int64_t i = r0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -175,12 +218,13 @@ __global__ void __launch_bounds__(256) front_up_kernel(const FrontDev* __restric
             if (NB == 1 || k < nb) s[k] = fma(a, e[k * n + b], s[k]);
     }
     const int64_t o = perm[i];
+    const double d = scale ? scale[i] : 1.0;
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
         const double q = warp_sum(s[k]);
         if (lane == 0 && (NB == 1 || k < nb)) {
             e[k * n + i] = q;
-            out[k * ldo + o] = q;
+            out[k * ldo + o] = d * q;
         }
     }
 }
@@ -188,7 +232,8 @@ __global__ void __launch_bounds__(256) front_up_kernel(const FrontDev* __restric
 void launch_front_solve(const FrontSolve& a, const double* c, int64_t ldc, double* out, int64_t ldo, int nb,
                         cudaStream_t s) {
     const int64_t want = (a.n + 255) / 256;
-    front_load_kernel<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(a.n, a.perm, c, ldc, a.v, nb);
+    front_load_kernel<<<(unsigned)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(a.n, a.src, a.scale, c, ldc,
+                                                                                         a.v, nb);
     for (int st = 0; st + 1 < a.stages; ++st) {
         const int64_t nrow = a.down_off[st + 1] - a.down_off[st];
         if (nrow <= 0) continue;
@@ -205,11 +250,11 @@ void launch_front_solve(const FrontSolve& a, const double* c, int64_t ldc, doubl
         if (r1 <= r0) continue;
         const unsigned g = (unsigned)(((r1 - r0) * 32 + 255) / 256);
         if (nb == 1)
-            front_up_kernel<1><<<g, 256, 0, s>>>(a.fr, a.row_front, r0, r1, a.bnd, a.perm, a.v, a.e, out, a.n, ldo,
-                                                 1);
+            front_up_kernel<1><<<g, 256, 0, s>>>(a.fr, a.row_front, r0, r1, a.bnd, a.perm, a.scale, a.v, a.e, out,
+                                                 a.n, ldo, 1);
         else
-            front_up_kernel<MAXB><<<g, 256, 0, s>>>(a.fr, a.row_front, r0, r1, a.bnd, a.perm, a.v, a.e, out, a.n, ldo,
-                                                    nb);
+            front_up_kernel<MAXB><<<g, 256, 0, s>>>(a.fr, a.row_front, r0, r1, a.bnd, a.perm, a.scale, a.v, a.e, out,
+                                                    a.n, ldo, nb);
     }
 }
 
