@@ -4479,7 +4479,7 @@ amdd_status amdd_pcg_solve(amdd_handle* h, const double* b, double* x, int32_t n
                 stats->iterations = its0;
                 stats->converged = conv0 ? 1 : 0;
                 stats->rel_residual = sc0.bb > 0.0 ? std::sqrt(sc0.rr / sc0.bb) : 0.0;
-                stats->true_rel_residual = sc0.bb > 0.0 ? std::sqrt(st.rr / sc0.bb) : 0.0;
+                stats->true_rel_residual = sc0.bb > 0.0 ? std::sqrt(st.rr) / std::sqrt(sc0.bb) : 0.0;
                 lanczos_extremes(al, be, &stats->ritz_min, &stats->ritz_max);
                 stats->cond_est = stats->ritz_max / stats->ritz_min;
             }
@@ -4578,7 +4578,7 @@ amdd_status amdd_pcg_solve(amdd_handle* h, const double* b, double* x, int32_t n
                 stats->iterations = its;
                 stats->converged = conv ? 1 : 0;
                 stats->rel_residual = sc.bb > 0.0 ? std::sqrt(sc.rr / sc.bb) : 0.0;
-                stats->true_rel_residual = sc.bb > 0.0 ? std::sqrt(st.rr / sc.bb) : 0.0;
+                stats->true_rel_residual = sc.bb > 0.0 ? std::sqrt(st.rr) / std::sqrt(sc.bb) : 0.0;
                 lanczos_extremes(al, be, &stats->ritz_min, &stats->ritz_max);
                 stats->cond_est = stats->ritz_max / stats->ritz_min;
             }
