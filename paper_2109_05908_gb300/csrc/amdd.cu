@@ -138,7 +138,6 @@ struct amdd_handle {
     int N = 0, overlap = 0;
     double tau = 0.0, eps = 0.0;
     int max_sweeps = 60;
-    int spmv_group = 4;
     // copy of A
     int64_t* rowptr = nullptr;
     int32_t* col = nullptr;
@@ -2228,7 +2227,6 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         Il[part[g]].push_back((int32_t)g);
     }
     for (int i = 0; i < N; ++i) require(!Il[i].empty());
-    h->spmv_group = spmv_group_for(n, nnz);
 
     // ---- overlap Omega_Gi (distance 1..ov) and extension Omega_Di (ov+1)
     std::vector<std::vector<int32_t>> Gl(N), Dl(N);
@@ -3432,7 +3430,7 @@ void apply_form(amdd_handle* h, int form, const double* r, double* z) {
         }
         {
             PScope ps(h, PK_SPMV, 2.0 * h->nnz, 12.0 * h->nnz + 8.0 * (h->n + 1) + 24.0 * h->n);
-            launch_spmv_resid(h->n, h->rowptr, h->col, h->val, h->d_zg, r, h->d_t, h->spmv_group, s);
+            launch_spmv_resid(h->n, h->nnz, h->rowptr, h->col, h->val, h->d_zg, r, h->d_t, s);
         }
         x = h->d_t;
     }
@@ -3456,7 +3454,7 @@ void apply_form(amdd_handle* h, int form, const double* r, double* z) {
 // Launch wrappers of the PCG loop with their profile accounting.
 void spmv_h(amdd_handle* h, const double* x, double* y) {
     PScope ps(h, PK_SPMV, 2.0 * h->nnz, 12.0 * h->nnz + 8.0 * (h->n + 1) + 16.0 * h->n);
-    launch_spmv(h->n, h->rowptr, h->col, h->val, x, y, h->spmv_group, h->s);
+    launch_spmv(h->n, h->nnz, h->rowptr, h->col, h->val, x, y, h->s);
 }
 void dot_h(amdd_handle* h, const double* x, const double* y, int which, double tol2) {
     {
@@ -3777,7 +3775,7 @@ GmResult gmres_run(amdd_handle* h, int form, const double* b, double* x, int m, 
         // r = b - A x, beta = ||r||, v_0 = r / beta, g = beta e_1
         {
             PScope ps(h, PK_SPMV, 2.0 * h->nnz, 12.0 * h->nnz + 8.0 * (n + 1) + 24.0 * n);
-            launch_spmv_resid(n, h->rowptr, h->col, h->val, x, b, V, h->spmv_group, s);
+            launch_spmv_resid(n, h->nnz, h->rowptr, h->col, h->val, x, b, V, s);
         }
         {
             PScope ps(h, PK_GMRES, 2.0 * n, 8.0 * n);
@@ -3801,7 +3799,7 @@ GmResult gmres_run(amdd_handle* h, int form, const double* b, double* x, int m, 
             apply_form(h, form, vj, zj);
             {
                 PScope ps(h, PK_SPMV, 2.0 * h->nnz, 12.0 * h->nnz + 8.0 * (n + 1) + 16.0 * n);
-                launch_spmv(n, h->rowptr, h->col, h->val, zj, h->d_gm_wA, h->spmv_group, s);
+                launch_spmv(n, h->nnz, h->rowptr, h->col, h->val, zj, h->d_gm_wA, s);
             }
             // CGS2: h1 = V^T w; w1 = w - V h1, h2 = V^T w1; w2 = w1 - V h2, ||w2||
             {
@@ -4074,7 +4072,7 @@ amdd_status amdd_spmv(const amdd_csr* A, const double* x, double* y, void* strea
         return AMDD_ERR_INVALID;
     if (A->n > INT32_MAX) return AMDD_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    launch_spmv(A->n, A->rowptr, A->colind, A->val, x, y, spmv_group_for(A->n, A->nnz), s);
+    launch_spmv(A->n, A->nnz, A->rowptr, A->colind, A->val, x, y, s);
     if (cudaGetLastError() != cudaSuccess) return AMDD_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return AMDD_ERR_CUDA;
     return AMDD_OK;
@@ -4626,7 +4624,7 @@ amdd_status amdd_gmres_solve(amdd_handle* h, int32_t form, const double* b, doub
             if (!g.conv) result = AMDD_ERR_NOCONV;
             if (k == 0 && stats) {
                 // true residual b - A x
-                launch_spmv_resid(n, h->rowptr, h->col, h->val, xk, bk, h->d_gm_wA, h->spmv_group, s);
+                launch_spmv_resid(n, h->nnz, h->rowptr, h->col, h->val, xk, bk, h->d_gm_wA, s);
                 launch_dot_partials(n, h->d_gm_wA, h->d_gm_wA, h->d_gm_part, s);
                 launch_gm_norm(h->d_gm_part, h->d_gm_st, 0, s);
                 double rr = 0.0;

@@ -307,11 +307,13 @@ bool nd_factor_pattern(int n, const int64_t* rowptr, const int32_t* colind, int 
 
 // *flag |= 1 when v[0..n) holds a NaN or an infinity
 void launch_nonfinite(const double* v, int64_t n, int* flag, cudaStream_t s);
-// Lanes per row of launch_spmv for a matrix of n rows and nnz entries: the one
-// choice every SpMV of the library makes, so that equal inputs give equal bits
-int spmv_group_for(int64_t n, int64_t nnz);
-void launch_spmv(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                 double* y, int group, cudaStream_t s);
+// y = A x and y = b - A x: every SpMV of the library goes through these two
+// launchers, which choose the form from n and nnz alone, so that equal inputs
+// give equal bits
+void launch_spmv(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                 const double* x, double* y, cudaStream_t s);
+void launch_spmv_resid(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                       const double* x, const double* b, double* y, cudaStream_t s);
 void launch_gather_values(const int64_t* src, const int64_t* dst, int64_t cnt, const double* val, double* out,
                           cudaStream_t s);
 void launch_gather_vec(const int32_t* idx, int64_t cnt, const double* x, double* out, cudaStream_t s);
@@ -524,10 +526,6 @@ void launch_ras_prolong(int64_t n, const int32_t* order_g, const int32_t* own_id
 void launch_owner_to_global(int64_t n, const int32_t* order_g, const double* zo, double* zg, cudaStream_t s);
 // out[t] = val[src[t]] (64-bit indices)
 void launch_gather_idx64(const int64_t* src, int64_t cnt, const double* val, double* out, cudaStream_t s);
-// y = b - A x
-void launch_spmv_resid(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                       const double* b, double* y, int group, cudaStream_t s);
-
 constexpr int GM_MAXR = 64;   // largest GMRES restart length
 constexpr int GM_CHUNK = 32;  // basis vectors per block row of the fused Gram-Schmidt passes
 struct GmState {

@@ -84,44 +84,6 @@ void launch_gather_idx64(const int64_t* src, int64_t cnt, const double* val, dou
     if (cnt > 0) gather_idx64_kernel<<<grid_for(cnt, 152 * 32), 256, 0, s>>>(src, cnt, val, out);
 }
 
-// ------------------------------------------------------------------ residual SpMV
-// y = b - A x, G lanes per row as in the plain SpMV.
-template <int G>
-__global__ void __launch_bounds__(256) spmv_resid_kernel(int64_t n, const int64_t* __restrict__ rowptr,
-                                                         const int32_t* __restrict__ col,
-                                                         const double* __restrict__ val,
-                                                         const double* __restrict__ x, const double* __restrict__ b,
-                                                         double* __restrict__ y) {
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int sub = threadIdx.x & (G - 1);
-    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
-    const int64_t nround = ((n + groups - 1) / groups) * groups;
-    for (int64_t row = gid / G; row < nround; row += groups) {
-        double s = 0.0;
-        if (row < n) {
-            const int64_t lo = rowptr[row], hi = rowptr[row + 1];
-            for (int64_t k = lo + sub; k < hi; k += G) s = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), s);
-        }
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (row < n && sub == 0) y[row] = b[row] - s;
-    }
-}
-
-void launch_spmv_resid(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                       const double* b, double* y, int group, cudaStream_t s) {
-    if (n <= 0) return;
-    const unsigned blocks = grid_for(n * group, 152 * 64);
-    if (group <= 1)
-        spmv_resid_kernel<1><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
-    else if (group <= 4)
-        spmv_resid_kernel<4><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
-    else if (group <= 8)
-        spmv_resid_kernel<8><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
-    else
-        spmv_resid_kernel<32><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
-}
-
 // ------------------------------------------------------------------ GMRES(m)
 // Classical Gram-Schmidt applied twice (CGS2) against the Arnoldi basis
 // V_0..V_{k-1} (rows ldv apart, ldv even, 16-byte aligned), in three fused

@@ -61,7 +61,7 @@ extern "C" amdd_status amdd_true_residual_noalloc(const amdd_csr* A, const doubl
     const int64_t n = A->n;
     // the record keeps the previous call's values: clear it
     if (cudaMemsetAsync(sc, 0, sizeof(PcgScal), s) != cudaSuccess) return AMDD_ERR_CUDA;
-    launch_spmv(n, A->rowptr, A->colind, A->val, x, q, spmv_group_for(n, A->nnz), s);
+    launch_spmv(n, A->nnz, A->rowptr, A->colind, A->val, x, q, s);
     launch_axpby(n, 1.0, b, -1.0, q, r, s);
     launch_dot_partials(n, b, b, partials, s);
     launch_dot_finalize(partials, sc, 3, 0.0, s);

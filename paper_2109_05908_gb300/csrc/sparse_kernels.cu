@@ -7,13 +7,25 @@
 namespace amdd {
 
 // ------------------------------------------------------------------ SpMV
-// G lanes per row (G in {1, 8, 32}); rows are assigned to lane groups in a
-// grid-stride loop.  G = 1 (rows of at most 8 entries): the entries of a
-// row load in parallel and a warp covers 32 consecutive rows.
-template <int G>
+// y = A x, or y = b - A x (RESID): G lanes per row, rows assigned to lane groups
+// in a grid-stride loop, four entries in flight per lane.  Rows of a few entries
+// take one thread each: a warp then covers 32 consecutive rows, bound by HBM
+// (5-point matrix of 2.1 M rows: 5.4 TB/s).  For longer rows FP64 sets the rate,
+// two multiply-adds per clock and SM whether or not the lanes have work: a warp
+// per row of 72 entries spends more on the shuffle tree than on the row, while
+// with 4 lanes the tree is shared by 8 rows.  27-point matrix with 3 unknowns per
+// node, 98 k rows, call included: 88 -> 47 us.
+template <bool RESID>
+__device__ __forceinline__ void spmv_store(int64_t row, double s, const double* __restrict__ b,
+                                           double* __restrict__ y) {
+    y[row] = RESID ? b[row] - s : s;
+}
+
+template <int G, bool RESID>
 __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ col, const double* __restrict__ val,
-                                                   const double* __restrict__ x, double* __restrict__ y) {
+                                                   const double* __restrict__ x, const double* __restrict__ b,
+                                                   double* __restrict__ y) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int sub = threadIdx.x & (G - 1);
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -23,33 +35,60 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __r
     for (int64_t row = gid / G; row < nround; row += groups) {
         double s = 0.0;
         if (row < n) {
-            const int64_t b = rowptr[row], e = rowptr[row + 1];
-            for (int64_t k = b + sub; k < e; k += G) s = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), s);
+            const int64_t e = rowptr[row + 1];
+            int64_t k = rowptr[row] + sub;
+            for (; k + 3 * G < e; k += 4 * G) {
+                double v[4], xv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    v[u] = __ldg(val + k + u * G);
+                    xv[u] = __ldg(x + __ldg(col + k + u * G));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s = fma(v[u], xv[u], s);
+            }
+            for (; k < e; k += G) s = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), s);
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (row < n && sub == 0) y[row] = s;
+        if (row < n && sub == 0) spmv_store<RESID>(row, s, b, y);
     }
 }
 
-int spmv_group_for(int64_t n, int64_t nnz) {
+// Lanes per row by the average row length, the fastest of 1, 2, 4, 8, 16, 32 at
+// 30 M entries (us; HBM floor 53 to 74): length 7: 78 / 132 / 170 / 286 / 705 /
+// 1670; 16: 176 / 97 / 100 / 166 / 326 / 747; 72: 163 / 87 / 76 / 92 / 125 / 228;
+// 600: 217 / 111 / 79 / 89 / 76 / 79.
+static int spmv_lanes(int64_t n, int64_t nnz) {
     const int64_t per = n > 0 ? nnz / n : 0;
-    return per <= 8 ? 1 : (per <= 24 ? 8 : 32);
+    return per <= 9 ? 1 : (per <= 24 ? 2 : (per <= 250 ? 4 : 16));
 }
 
-void launch_spmv(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                 double* y, int group, cudaStream_t s) {
+template <bool RESID>
+static void spmv_any(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                     const double* x, const double* b, double* y, cudaStream_t s) {
     if (n <= 0) return;
+    const int group = spmv_lanes(n, nnz);
     const int64_t want = (n * group + 255) / 256;
     const int blocks = (int)(want < 152 * 64 ? want : 152 * 64);
-    if (group <= 1)
-        spmv_kernel<1><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, y);
-    else if (group <= 4)
-        spmv_kernel<4><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, y);
-    else if (group <= 8)
-        spmv_kernel<8><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, y);
+    if (group == 1)
+        spmv_kernel<1, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+    else if (group == 2)
+        spmv_kernel<2, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+    else if (group == 4)
+        spmv_kernel<4, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
     else
-        spmv_kernel<32><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, y);
+        spmv_kernel<16, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+}
+
+void launch_spmv(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                 const double* x, double* y, cudaStream_t s) {
+    spmv_any<false>(n, nnz, rowptr, col, val, x, nullptr, y, s);
+}
+
+void launch_spmv_resid(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                       const double* x, const double* b, double* y, cudaStream_t s) {
+    spmv_any<true>(n, nnz, rowptr, col, val, x, b, y, s);
 }
 
 // y_k = A x_k for nb <= MAXB right-hand sides stored ld apart: one thread per
