@@ -88,7 +88,21 @@ struct JacobiDescT {
     int ncols_rot;      // columns rotated (>= ncols_dot)
     T* nrm2;            // rows scratch entries (squared row norms)
     const T* absfloor;  // optional absolute floor on |<p,q>| below which no rotation is made
+    // optional f: no rotation either while <p,q>^2 <= u f max(|p|^2, |q|^2) (u the
+    // unit roundoff of T).  With f = u |M|^2 (launch_row_maxnorm2) a pair is left
+    // alone once its coupling is below the rounding of M itself, u |M|.
+    const T* normfloor = nullptr;
+    // optional c > 0: two rows both longer than sqrt(c) need only be orthogonal to
+    // JAC_LOOSE (their span, not the rows themselves, is wanted)
+    T loose_above = T(0);
 };
+constexpr float JAC_LOOSE = 0x1p-10f;
+// squared relative tolerance for the pair of squared lengths a, b
+template <typename T>
+__host__ __device__ __forceinline__ T jac_tol2(T tol, T a, T b, T loose_above) {
+    const T t = loose_above > T(0) && (a < b ? a : b) > loose_above ? T(JAC_LOOSE) : tol;
+    return t * t;
+}
 using JacobiDesc = JacobiDescT<double>;
 
 // Conversion descriptors of the FP32 preconditioning stage of the Jacobi solvers.
@@ -179,11 +193,12 @@ template <typename T>
 size_t jacobi_block_smem(int rows, int ncols_rot, int cluster);
 // Shared-memory-resident block variant with a cluster of JAC_CLUSTER CTAs per
 // matrix, else (blocks too large) 2 * JAC_CLUSTER; returns false, with nothing
-// launched, when neither fits (smem8 / smem16: bytes per CTA for the two sizes).
+// launched, when neither fits (smem8 / smem16: bytes per CTA for the two sizes;
+// floors: some matrix has absfloor, normfloor or loose_above).
 template <typename T>
 bool launch_jacobi_block(const JacobiDescT<T>* d, int nmat, size_t smem8, size_t smem16, int max_rows,
                          int max_sweeps, T tol, int* sweeps, unsigned long long* rots, int* err, int report_noconv,
-                         cudaStream_t s);
+                         bool floors, cudaStream_t s);
 template <typename T>
 void launch_row_maxnorm2(const JacobiDescT<T>* d, int nmat, T eps, T* out, cudaStream_t s);
 void launch_to_f32_with_identity(const CvtDesc* d, int nmat, int maxrows, cudaStream_t s);

@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(256) jacobi_pair_kernel(const JacobiDescT<T>* 
         return r < d.rows ? r : -1;
     };
     const T absf = d.absfloor ? *d.absfloor : T(0);
+    const T nf = d.normfloor ? (sizeof(T) == 4 ? T(1.1920928955078125e-7) : T(2.220446049250313e-16)) * *d.normfloor : T(0);
     // stats: [0] pair tasks, [1] pairs rotated, [2..4] SM clock cycles of the
     // Gram matrix, the small eigensolve and the rotation of the rows (thread 0),
     // [5] inner sweeps
@@ -523,12 +524,12 @@ __global__ void __launch_bounds__(256) jacobi_pair_kernel(const JacobiDescT<T>* 
             const int p = e / JP_R, q = e % JP_R;
             if (q <= p) continue;
             const T a = G[p * JPI_LDG + p], b = G[q * JPI_LDG + q], g = G[p * JPI_LDG + q];
-            if (g != T(0) && g * g > tol * tol * a * b && fabs(g) > absf) mine = 1;
+            if (g != T(0) && g * g > jac_tol2(tol, a, b, d.loose_above) * a * b && fabs(g) > absf && g * g > nf * fmax(a, b)) mine = 1;
         }
         if (!__syncthreads_or(mine)) return;  // the pair met the stopping test: rows unchanged
     }
     unsigned nrot = 0;
-    const int inner = jpi_solve<T>(G, G1, Qt, jr, tin, absf, inner_max, nrot);
+    const int inner = jpi_solve<T>(G, G1, Qt, jr, tin, absf, nf, d.loose_above, inner_max, nrot);
     if (nrot) atomicAdd(rots + mat, (unsigned long long)nrot);
     const long long t2 = clock64();
     if (tid == 0) {
@@ -614,7 +615,9 @@ void launch_or_flag(int* p, int bits, cudaStream_t s) { or_flag_kernel<<<1, 1, 0
 // visits every row pair once, with one cluster barrier per block round
 // (2 * JAC_CLUSTER - 1 per sweep).  Row norms^2 are recomputed when a block is
 // loaded and updated exactly after each rotation.
-template <typename T, int CL>
+// FL: some matrix of the batch has floors or a loose tolerance; without them the
+// test of a pair stays one comparison (it is on every sub-round's critical path).
+template <typename T, int CL, bool FL>
 __global__ void __launch_bounds__(1024)
     jacobi_block_kernel(const JacobiDescT<T>* __restrict__ descs, int max_sweeps, T tol, int* __restrict__ sweeps,
                         unsigned long long* __restrict__ rots, int* __restrict__ err, int report_noconv) {
@@ -634,7 +637,14 @@ __global__ void __launch_bounds__(1024)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
     const int hbe = hb + (hb & 1);
-    const T absf = d.absfloor ? *d.absfloor : T(0);
+    // in shared memory: read from the descriptor inside the sub-rounds they would
+    // cost a trip to L2 in each
+    __shared__ T floors[3];
+    if (FL && threadIdx.x == 0) {
+        floors[0] = d.absfloor ? *d.absfloor : T(0);
+        floors[1] = d.normfloor ? (sizeof(T) == 4 ? T(1.1920928955078125e-7) : T(2.220446049250313e-16)) * *d.normfloor : T(0);
+        floors[2] = d.loose_above;
+    }
     unsigned long long my_rots = 0;
     int sweep = 0;
     bool done = false;
@@ -696,7 +706,9 @@ __global__ void __launch_bounds__(1024)
                     jflag[k] = 0;
                     if (pair_of(k, sa, sb)) {
                         const T g = jg[k], a = nrm[sa], b = nrm[sb];
-                        if (g != T(0) && g * g > tol * tol * a * b && fabs(g) > absf) {
+                        const T t2 = FL ? jac_tol2(tol, a, b, floors[2]) : tol * tol;
+                        if (g != T(0) && g * g > t2 * a * b &&
+                            (!FL || (fabs(g) > floors[0] && g * g > floors[1] * fmax(a, b)))) {
                             T cs, sn, t;
                             jac_rotation(a, b, g, cs, sn, t);
                             jcs[k] = cs;
@@ -788,13 +800,13 @@ template size_t jacobi_block_smem<double>(int, int, int);
 // (cluster dimension given at launch; CL = 16 is the non-portable size).
 // Returns false, with nothing launched, when the blocks do not fit or the
 // device cannot co-schedule such a cluster.
-template <typename T, int CL>
+template <typename T, int CL, bool FL>
 bool launch_jacobi_block_cl(const JacobiDescT<T>* d, int nmat, size_t smem, int max_rows, int max_sweeps, T tol,
                             int* sweeps, unsigned long long* rots, int* err, int report_noconv, cudaStream_t s) {
     if (smem > JAC_BLOCK_SMEM_MAX) return false;
     const int hb = (max_rows + 2 * CL - 1) / (2 * CL);
     if (hb + 2 > JAC_MAX_PAIRS) return false;
-    auto kern = jacobi_block_kernel<T, CL>;
+    auto kern = jacobi_block_kernel<T, CL, FL>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         (CL > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         cudaGetLastError();
@@ -826,21 +838,30 @@ bool launch_jacobi_block_cl(const JacobiDescT<T>* d, int nmat, size_t smem, int 
     return true;
 }
 
+template <typename T, bool FL>
+bool launch_jacobi_block_any(const JacobiDescT<T>* d, int nmat, size_t smem8, size_t smem16, int max_rows,
+                             int max_sweeps, T tol, int* sweeps, unsigned long long* rots, int* err,
+                             int report_noconv, cudaStream_t s) {
+    return launch_jacobi_block_cl<T, JAC_CLUSTER, FL>(d, nmat, smem8, max_rows, max_sweeps, tol, sweeps, rots, err,
+                                                      report_noconv, s) ||
+           launch_jacobi_block_cl<T, 2 * JAC_CLUSTER, FL>(d, nmat, smem16, max_rows, max_sweeps, tol, sweeps, rots,
+                                                          err, report_noconv, s);
+}
+
 template <typename T>
 bool launch_jacobi_block(const JacobiDescT<T>* d, int nmat, size_t smem8, size_t smem16, int max_rows,
                          int max_sweeps, T tol, int* sweeps, unsigned long long* rots, int* err, int report_noconv,
-                         cudaStream_t s) {
+                         bool floors, cudaStream_t s) {
     if (nmat <= 0) return true;
-    if (launch_jacobi_block_cl<T, JAC_CLUSTER>(d, nmat, smem8, max_rows, max_sweeps, tol, sweeps, rots, err,
-                                               report_noconv, s))
-        return true;
-    return launch_jacobi_block_cl<T, 2 * JAC_CLUSTER>(d, nmat, smem16, max_rows, max_sweeps, tol, sweeps, rots, err,
-                                                      report_noconv, s);
+    return floors ? launch_jacobi_block_any<T, true>(d, nmat, smem8, smem16, max_rows, max_sweeps, tol, sweeps, rots,
+                                                     err, report_noconv, s)
+                  : launch_jacobi_block_any<T, false>(d, nmat, smem8, smem16, max_rows, max_sweeps, tol, sweeps, rots,
+                                                      err, report_noconv, s);
 }
 template bool launch_jacobi_block<float>(const JacobiDescT<float>*, int, size_t, size_t, int, int, float, int*,
-                                         unsigned long long*, int*, int, cudaStream_t);
+                                         unsigned long long*, int*, int, bool, cudaStream_t);
 template bool launch_jacobi_block<double>(const JacobiDescT<double>*, int, size_t, size_t, int, int, double, int*,
-                                          unsigned long long*, int*, int, cudaStream_t);
+                                          unsigned long long*, int*, int, bool, cudaStream_t);
 
 // absfloor[mat] = eps * max_r ||row r||^2 over ncols_dot (one CTA per matrix).
 template <typename T>
@@ -1621,6 +1642,14 @@ __device__ __forceinline__ int sturm_count(const T* __restrict__ d, const T* __r
     return cnt;
 }
 
+// BIS_L lanes per eigenvalue: each pass takes the Sturm counts at BIS_L interior
+// points and keeps the subinterval that holds eigenvalue j, so the interval
+// shrinks (BIS_L + 1)-fold per pass.  A pass is a chain of n dependent steps
+// bound by latency, whatever the number of lanes: 8 lanes need a third of the
+// passes of plain bisection.  FP64, 1872 eigenvalues of matrices of 233 to 272
+// rows: 11.4 -> 3.7 ms; FP32, 4096 of 256 rows: 0.38 -> 0.15 ms.
+constexpr int BIS_L = 8;
+
 template <typename T>
 __global__ void __launch_bounds__(32) bisect_kernel(const TridiagDescT<T>* __restrict__ descs,
                                                      const int* __restrict__ eig_mat,
@@ -1674,14 +1703,6 @@ __global__ void bisect_prepare_kernel(const TridiagDescT<T>* __restrict__ descs)
     const TridiagDescT<T> t = descs[blockIdx.x];
     for (int i = threadIdx.x; i < t.n; i += blockDim.x) t.e[i] = t.e[i] * t.e[i];
 }
-
-// BIS_L lanes per eigenvalue: each pass takes the Sturm counts at BIS_L interior
-// points and keeps the subinterval that holds eigenvalue j, so the interval
-// shrinks (BIS_L + 1)-fold per pass.  A pass is a chain of n dependent steps
-// bound by latency, whatever the number of lanes: 8 lanes need a third of the
-// passes of plain bisection.  FP64, 1872 eigenvalues of matrices of 233 to 272
-// rows: 11.4 -> 3.7 ms; FP32, 4096 of 256 rows: 0.38 -> 0.15 ms.
-constexpr int BIS_L = 8;
 
 template <typename T>
 void launch_bisect(const TridiagDescT<T>* d, int nmat, const int* eig_mat, const int* eig_idx, int64_t total,

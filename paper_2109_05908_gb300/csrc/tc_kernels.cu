@@ -361,6 +361,7 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
             return r < d.rows ? r : -1;
         };
         const float absf = d.absfloor ? *d.absfloor : 0.0f;
+        const float nf = d.normfloor ? 1.1920928955078125e-7f * *d.normfloor : 0.0f;
         const long long t0 = clock64();
         bool rot_pair = false;
 
@@ -473,13 +474,13 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 const int p = e >> 6, q = e & 63;
                 if (q <= p) continue;
                 const float a = G0[p * JPI_LDG + p], b = G0[q * JPI_LDG + q], g = G0[p * JPI_LDG + q];
-                if (g != 0.0f && g * g > tol * tol * a * b && fabsf(g) > absf) mine = 1;
+                if (g != 0.0f && g * g > jac_tol2(tol, a, b, d.loose_above) * a * b && fabsf(g) > absf && g * g > nf * fmaxf(a, b)) mine = 1;
             }
             rot_pair = __syncthreads_or(mine) != 0;
         }
         if (ok && rot_pair) {
             unsigned nrot = 0;
-            const int inner = jpi_solve<float>(G0, G1, Qt, jr, tin, absf, inner_max, nrot);
+            const int inner = jpi_solve<float>(G0, G1, Qt, jr, tin, absf, nf, d.loose_above, inner_max, nrot);
             if (nrot) atomicAdd(rots + mat, (unsigned long long)nrot);
             const long long t2 = clock64();
             if (tid == 0) {
