@@ -1616,64 +1616,6 @@ void mf_local_eigs(Ctx& C, amdd_handle* h, const double* X1, const std::vector<i
     }
 }
 
-// MLP forward on n standardised feature rows X (n x 32): Q (n x 16 x 16,
-// symmetrised).  Work: Z1, H1, Z2, H2, Y (n x 256 each).
-void mlp_forward(Ctx& C, const float* Wb, const float* X, int n, float* work, float* Q) {
-    amdd_handle* h = C.h;
-    float* Z1 = work;
-    float* H1 = Z1 + (size_t)n * PROP_NH;
-    float* Z2 = H1 + (size_t)n * PROP_NH;
-    float* H2 = Z2 + (size_t)n * PROP_NH;
-    float* Y = H2 + (size_t)n * PROP_NH;
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(X, PROP_NF, 0, Wb + MLP_OFF_W1, PROP_NH, 0, Z1, PROP_NH, n, PROP_NH,
-                                                    PROP_NF, 1.0, 0.0, 0)});
-    launch_bias_act(Z1, Wb + MLP_OFF_B1, H1, n, PROP_NH, h->s);
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(H1, PROP_NH, 0, Wb + MLP_OFF_W2, PROP_NH, 0, Z2, PROP_NH, n, PROP_NH,
-                                                    PROP_NH, 1.0, 0.0, 0)});
-    launch_bias_act(Z2, Wb + MLP_OFF_B2, H2, n, PROP_NH, h->s);
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(H2, PROP_NH, 0, Wb + MLP_OFF_W3, PROP_NO, 0, Y, PROP_NO, n, PROP_NO,
-                                                    PROP_NH, 1.0, 0.0, 0)});
-    launch_bias_act(Y, Wb + MLP_OFF_B3, nullptr, n, PROP_NO, h->s);
-    launch_symmetrise(Y, Q, n, h->s);
-}
-
-// Gradient of the mean squared Frobenius error (forward with Wb, work as in
-// mlp_forward plus Q, dY, dH, dZ (n x 256) and n partial sums).
-void mlp_backward(Ctx& C, const float* Wb, const float* X, const float* Qt, int n, float* work, float* grad,
-                  float* loss) {
-    amdd_handle* h = C.h;
-    const size_t L = (size_t)n * PROP_NH;
-    float* Z1 = work;
-    float* H1 = Z1 + L;
-    float* Z2 = H1 + L;
-    float* H2 = Z2 + L;
-    float* Q = H2 + 2 * L;  // after Y
-    float* dY = Q + L;
-    float* dH = dY + L;
-    float* dZ = dH + L;
-    float* part = dZ + L;
-    mlp_forward(C, Wb, X, n, work, Q);
-    launch_loss_grad(Q, Qt, dY, part, loss, n, h->s);
-    // output layer
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(H2, PROP_NH, 1, dY, PROP_NO, 0, grad + MLP_OFF_W3, PROP_NO, PROP_NH,
-                                                    PROP_NO, n, 1.0, 0.0, 0)});
-    launch_colsum(dY, grad + MLP_OFF_B3, n, PROP_NO, h->s);
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(dY, PROP_NO, 0, Wb + MLP_OFF_W3, PROP_NO, 1, dH, PROP_NH, n, PROP_NH,
-                                                    PROP_NO, 1.0, 0.0, 0)});
-    launch_relu_back(dH, Z2, dZ, n * PROP_NH, h->s);
-    // second hidden layer
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(H1, PROP_NH, 1, dZ, PROP_NH, 0, grad + MLP_OFF_W2, PROP_NH, PROP_NH,
-                                                    PROP_NH, n, 1.0, 0.0, 0)});
-    launch_colsum(dZ, grad + MLP_OFF_B2, n, PROP_NH, h->s);
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(dZ, PROP_NH, 0, Wb + MLP_OFF_W2, PROP_NH, 1, dH, PROP_NH, n, PROP_NH,
-                                                    PROP_NH, 1.0, 0.0, 0)});
-    launch_relu_back(dH, Z1, dZ, n * PROP_NH, h->s);
-    // first layer
-    gemm(C, std::vector<GemmDescT<float>>{gd<float>(X, PROP_NF, 1, dZ, PROP_NH, 0, grad + MLP_OFF_W1, PROP_NH, PROP_NF,
-                                                    PROP_NH, n, 1.0, 0.0, 0)});
-    launch_colsum(dZ, grad + MLP_OFF_B1, n, PROP_NH, h->s);
-}
-
 // Eigenvectors of the partial selections without the dense Jacobi: the
 // features and Krylov bases of those subdomains (kept in the handle for
 // amdd_proposal_export when asked), then, with eig_solver >= 1, block LOBPCG
@@ -1743,9 +1685,8 @@ std::vector<int> learned_eigvecs(Ctx& C, amdd_handle* h, const std::vector<int>&
     if (warm) {
         float* Xn = C.tnew<float>((int64_t)np * PROP_NF);
         launch_normalize_features(feat, h->prop.mean, h->prop.sd, Xn, np, s);
-        float* work = C.tnew<float>((int64_t)5 * np * PROP_NH);
         float* Qh = C.tnew<float>((int64_t)np * PROP_NO);
-        mlp_forward(C, h->prop.weights, Xn, np, work, Qh);
+        launch_mlp_forward(h->prop.weights, Xn, np, Qh, s);
         std::vector<int64_t> go(np);
         std::vector<int> mm(np, PROP_NB), lg(np, PROP_NB);
         for (int q = 0; q < np; ++q) go[q] = (int64_t)q * PROP_NO;
@@ -4393,19 +4334,9 @@ amdd_status amdd_mlp_normalize(const float* feat, const float* mean, const float
 
 amdd_status amdd_mlp_forward(const float* wb, const float* x, int32_t n, float* q, float* work, void* stream) {
     if (n < 1 || !wb || !x || !q || !work) return AMDD_ERR_INVALID;
-    try {
-        amdd_handle tmp;
-        tmp.s = static_cast<cudaStream_t>(stream);
-        {
-            Ctx C(&tmp);
-            mlp_forward(C, wb, x, n, work, q);
-            ck(cudaGetLastError());
-            ck(cudaStreamSynchronize(tmp.s));
-        }
-        ck(cudaStreamSynchronize(tmp.s));
-    } catch (...) {
-        return guard_exc();
-    }
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    launch_mlp_forward(wb, x, n, q, s);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return AMDD_ERR_CUDA;
     return AMDD_OK;
 }
 
@@ -4413,20 +4344,9 @@ amdd_status amdd_mlp_train_step(float* w, float* wb, float* m, float* v, int32_t
                                 const float* qt, int32_t n, float* grad, float* work, float* loss, void* stream) {
     if (n < 1 || !wb || !x || !qt || !grad || !work || !loss || !(lr >= 0.0f)) return AMDD_ERR_INVALID;
     if (lr > 0.0f && (!w || !m || !v || t < 1)) return AMDD_ERR_INVALID;
-    try {
-        amdd_handle tmp;
-        tmp.s = static_cast<cudaStream_t>(stream);
-        {
-            Ctx C(&tmp);
-            mlp_backward(C, wb, x, qt, n, work, grad, loss);
-            if (lr > 0.0f) launch_adam(w, wb, m, v, grad, (int)MLP_NPARAM, lr, t, tmp.s);
-            ck(cudaGetLastError());
-            ck(cudaStreamSynchronize(tmp.s));
-        }
-        ck(cudaStreamSynchronize(tmp.s));
-    } catch (...) {
-        return guard_exc();
-    }
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    launch_mlp_step(w, wb, m, v, t, lr, x, qt, n, grad, work, loss, s);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return AMDD_ERR_CUDA;
     return AMDD_OK;
 }
 

@@ -411,12 +411,11 @@ void launch_krylov(const KrylovDesc* d, int nmat, cudaStream_t s);
 void launch_feature_stats(const float* feat, int n, float* mean, float* sd, cudaStream_t s);
 void launch_normalize_features(const float* feat, const float* mean, const float* sd, float* X, int n,
                                cudaStream_t s);
-void launch_bias_act(float* Z, const float* bias, float* H, int rows, int cols, cudaStream_t s);
-void launch_symmetrise(const float* Y, float* Q, int n, cudaStream_t s);
-void launch_loss_grad(const float* Q, const float* Qt, float* dY, float* part, float* loss, int n, cudaStream_t s);
-void launch_relu_back(const float* dH, const float* Z, float* dZ, int n, cudaStream_t s);
-void launch_colsum(const float* dZ, float* db, int rows, int cols, cudaStream_t s);
-void launch_adam(float* W, float* Wb, float* m, float* v, const float* g, int n, float lr, int t, cudaStream_t s);
+// The proposal network (mlp_kernels.cu): q (n x 256) of n samples; one training
+// step (work as amdd_mlp_sizes; lr = 0: gradient and loss only)
+void launch_mlp_forward(const float* wb, const float* x, int n, float* q, cudaStream_t s);
+void launch_mlp_step(float* w, float* wb, float* m, float* v, int t, float lr, const float* x, const float* qt, int n,
+                     float* grad, float* work, float* loss, cudaStream_t s);
 void launch_bf16_round(const float* W, float* Wb, int n, cudaStream_t s);
 
 template <typename T>

@@ -280,124 +280,6 @@ void launch_normalize_features(const float* feat, const float* mean, const float
     if (n > 0) normalize_features_kernel<<<(n * PROP_NF + 255) / 256, 256, 0, s>>>(feat, mean, sd, X, n);
 }
 
-// Z[b][j] += bias[j]; H = relu(Z) when H is given (Z keeps the pre-activation)
-__global__ void bias_act_kernel(float* __restrict__ Z, const float* __restrict__ bias, float* __restrict__ H, int rows,
-                                int cols) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < rows * cols; t += gridDim.x * blockDim.x) {
-        const float z = Z[t] + bias[t % cols];
-        Z[t] = z;
-        if (H) H[t] = fmaxf(z, 0.0f);
-    }
-}
-
-void launch_bias_act(float* Z, const float* bias, float* H, int rows, int cols, cudaStream_t s) {
-    const int n = rows * cols;
-    if (n > 0) bias_act_kernel<<<(n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096, 256, 0, s>>>(Z, bias, H, rows, cols);
-}
-
-// Q[b] = (Y[b] + Y[b]^T) / 2 as 16 x 16 matrices
-__global__ void symmetrise_kernel(const float* __restrict__ Y, float* __restrict__ Q, int n) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * PROP_NO; t += gridDim.x * blockDim.x) {
-        const int b = t / PROP_NO, e = t % PROP_NO, r = e / PROP_NB, c = e % PROP_NB;
-        const float* y = Y + (size_t)b * PROP_NO;
-        Q[t] = 0.5f * (y[r * PROP_NB + c] + y[c * PROP_NB + r]);
-    }
-}
-
-void launch_symmetrise(const float* Y, float* Q, int n, cudaStream_t s) {
-    if (n > 0) symmetrise_kernel<<<(n * PROP_NO + 255) / 256, 256, 0, s>>>(Y, Q, n);
-}
-
-// Loss sum_b ||Q_b - Qt_b||_F^2 / n (partial sums per CTA, row b) and the
-// gradient with respect to the unsymmetrised outputs:
-// dY = (dQ + dQ^T) / 2 with dQ = 2 (Q - Qt) / n.
-__global__ void __launch_bounds__(256) loss_grad_kernel(const float* __restrict__ Q, const float* __restrict__ Qt,
-                                                        float* __restrict__ dY, float* __restrict__ part, int n) {
-    __shared__ float sh[8];
-    const int b = blockIdx.x;
-    const float* q = Q + (size_t)b * PROP_NO;
-    const float* qt = Qt + (size_t)b * PROP_NO;
-    float acc = 0.0f;
-    for (int e = threadIdx.x; e < PROP_NO; e += blockDim.x) {
-        const int r = e / PROP_NB, c = e % PROP_NB;
-        const float dqe = q[e] - qt[e];
-        const float dqt = q[c * PROP_NB + r] - qt[c * PROP_NB + r];
-        acc = fmaf(dqe, dqe, acc);
-        dY[(size_t)b * PROP_NO + e] = (dqe + dqt) / (float)n;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.0f;
-        for (int w = 0; w < 8; ++w) t += sh[w];
-        part[b] = t;
-    }
-}
-
-// loss = sum of the per-sample partials / n, in sample order
-__global__ void loss_finalize_kernel(const float* __restrict__ part, float* __restrict__ out, int n) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int b = 0; b < n; ++b) t += part[b];
-        out[0] = (float)(t / n);
-    }
-}
-
-void launch_loss_grad(const float* Q, const float* Qt, float* dY, float* part, float* loss, int n, cudaStream_t s) {
-    if (n <= 0) return;
-    loss_grad_kernel<<<n, 256, 0, s>>>(Q, Qt, dY, part, n);
-    loss_finalize_kernel<<<1, 32, 0, s>>>(part, loss, n);
-}
-
-// dZ = dH * (Z > 0)
-__global__ void relu_back_kernel(const float* __restrict__ dH, const float* __restrict__ Z, float* __restrict__ dZ,
-                                 int n) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-        dZ[t] = Z[t] > 0.0f ? dH[t] : 0.0f;
-}
-
-void launch_relu_back(const float* dH, const float* Z, float* dZ, int n, cudaStream_t s) {
-    if (n > 0) relu_back_kernel<<<(n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096, 256, 0, s>>>(dH, Z, dZ, n);
-}
-
-// db[j] = sum_b dZ[b][j], summed in sample order
-__global__ void colsum_kernel(const float* __restrict__ dZ, float* __restrict__ db, int rows, int cols) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
-    float s = 0.0f;
-    for (int b = 0; b < rows; ++b) s += dZ[(size_t)b * cols + j];
-    db[j] = s;
-}
-
-void launch_colsum(const float* dZ, float* db, int rows, int cols, cudaStream_t s) {
-    if (cols > 0) colsum_kernel<<<(cols + 127) / 128, 128, 0, s>>>(dZ, db, rows, cols);
-}
-
-// Adam (Kingma & Ba) on the FP32 master weights, then the bfloat16-rounded copy
-__global__ void adam_kernel(float* __restrict__ W, float* __restrict__ Wb, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, int n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const float gt = g[t];
-        const float mt = b1 * m[t] + (1.0f - b1) * gt;
-        const float vt = b2 * v[t] + (1.0f - b2) * gt * gt;
-        m[t] = mt;
-        v[t] = vt;
-        const float w = W[t] - lr * (mt / c1) / (sqrtf(vt / c2) + eps);
-        W[t] = w;
-        Wb[t] = bf16_round(w);
-    }
-}
-
-void launch_adam(float* W, float* Wb, float* m, float* v, const float* g, int n, float lr, int t, cudaStream_t s) {
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    adam_kernel<<<(n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096, 256, 0, s>>>(W, Wb, m, v, g, n, lr, b1, b2, 1e-8f,
-                                                                                c1, c2);
-}
-
 __global__ void bf16_round_kernel(const float* __restrict__ W, float* __restrict__ Wb, int n) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) Wb[t] = bf16_round(W[t]);
 }
