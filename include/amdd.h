@@ -145,7 +145,8 @@ typedef struct {
                              error is of the order of an FP32 multiply-add loop's; 0: CUDA-core FMA;
                              default 1                                                              */
     int32_t local_solver; /* local solves of the Schwarz methods (Sec. 4.1: exact local Cholesky):
-                             0: the explicit inverse factors L_i^{-1}, L_i^{-T} (dense triangles);
+                             0: substructuring: nested-dissection parts of every A_ii with dense
+                             inverses and couplings, eliminated in FP64;
                              1: sparse Cholesky factors in a nested-dissection order (the same exact
                              factor of the permuted A_ii, with the symbolic fill only), solved by
                              forward and backward substitution with each factor staged in shared

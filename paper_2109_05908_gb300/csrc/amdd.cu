@@ -147,14 +147,9 @@ struct amdd_handle {
     std::vector<int64_t> off_om, off_sq, off_zt, off_I, coff;
     int64_t sum_ni = 0, sum_sq = 0, sum_nI = 0, sum_nt = 0, nC = 0, sum_zt = 0;
     int max_ni = 0, max_nt = 0;
-    int64_t apply_tri_elems = 0;  // sum_i ni (ni + 1): elements read by the two local triangular products
     // persistent device data of the apply
     int32_t* d_omega = nullptr;
-    double* d_Y = nullptr;
-    double* d_Yt = nullptr;
     double* d_Zt = nullptr;
-    GemvDesc* d_gv_l1 = nullptr;
-    GemvDesc* d_gv_l2 = nullptr;
     GemvDesc* d_gv_c = nullptr;
     int32_t *d_rd_c = nullptr, *d_rl_c = nullptr;
     // coarse prolongation zc = Z e as row GEMVs over Z_i = Zt_i^T (nI x p_i)
@@ -164,21 +159,19 @@ struct amdd_handle {
     int32_t *d_rd_zp = nullptr, *d_rl_zp = nullptr;
     int64_t n_zp = 0;
     std::vector<GemvDesc> gv_zp_h;  // host copy (the batched path rebinds x / y)
-    int32_t *d_g4_desc = nullptr, *d_g4_row = nullptr;  // row groups (one warp each) of the local products
-    int64_t n_g4 = 0;
     int32_t *d_order_g = nullptr, *d_sc_idx = nullptr;
     int64_t* d_sc_ptr = nullptr;
-    double *d_rloc = nullptr, *d_tloc = nullptr, *d_yloc = nullptr;
+    double *d_rloc = nullptr, *d_yloc = nullptr;
     // mixed form: FP32 local factors and local work vectors
     int precision = 0;
-    float *d_Y32 = nullptr, *d_Yt32 = nullptr;
-    float *d_rloc32 = nullptr, *d_tloc32 = nullptr, *d_yloc32 = nullptr;
-    GemvDescT<float>* d_gv_l1_32 = nullptr;
-    GemvDescT<float>* d_gv_l2_32 = nullptr;
+    float *d_rloc32 = nullptr, *d_yloc32 = nullptr;  // (sparse local factors only, as d_yloc)
     double *d_c = nullptr, *d_e = nullptr;
     // coarse solve by substructuring (fronts.cu): Ainv, W and W^T of every part
-    FrontSolve fs;
-    double csolve_flops = 0.0, csolve_bytes = 0.0;
+    FrontSolveT<double> fs;
+    // local solves by the same construction on all A_ii at once (one tree per
+    // subdomain), in FP64 or FP32 (mixed form)
+    FrontSolveT<double> lfs;
+    FrontSolveT<float> lfs32;
     // eigenvectors of partial selections: 0 dense Jacobi, 1 LOBPCG from random
     // rows, 2 LOBPCG from the learned proposal
     int eig_solver = 0, keep_prop = 0;
@@ -195,16 +188,13 @@ struct amdd_handle {
     int64_t lob_total = 0;
     // batched right-hand sides (up to MAXB per pass), allocated on first use
     int mb_cap = 0;
-    double *d_m_rloc = nullptr, *d_m_tloc = nullptr, *d_m_yloc = nullptr;
-    float *d_m_rloc32 = nullptr, *d_m_tloc32 = nullptr, *d_m_yloc32 = nullptr;
+    double *d_m_rloc = nullptr, *d_m_yloc = nullptr;
+    float *d_m_rloc32 = nullptr, *d_m_yloc32 = nullptr;
     double *d_m_c = nullptr, *d_m_e = nullptr, *d_m_zc = nullptr;
     GemvDesc* d_m_gv_zp = nullptr;
     double *d_m_q = nullptr, *d_m_r = nullptr, *d_m_z = nullptr, *d_m_p = nullptr, *d_m_part = nullptr;
     PcgScal* d_m_sc = nullptr;
-    void* d_m_gv_l1 = nullptr;  // GemvDescT<double or float> per subdomain, on the batched buffers
-    void* d_m_gv_l2 = nullptr;
     GemvDesc* d_m_gv_c = nullptr;
-    std::vector<const void*> lm1, lm2;  // per subdomain: L_i^{-1} and L_i^{-T} (FP64 or FP32)
     // kept for amdd_proposal_export: features and Krylov bases of the partial subdomains
     float* prop_feat = nullptr;
     double* prop_bt = nullptr;
@@ -214,6 +204,7 @@ struct amdd_handle {
     // in the local vectors of each unknown's own copy (owner order), and work
     // vectors in global order
     int32_t* d_own_idx = nullptr;
+    std::vector<int32_t> own_pos;  // the same on the host
     double *d_zg = nullptr, *d_t = nullptr;
     // multilevel form: kept copy of E with its block pattern (CSR), the
     // second level and the counters of its inner solves
@@ -333,6 +324,13 @@ struct Ctx {
     std::vector<void*> temps;
     std::vector<std::shared_ptr<void>> keep;
     size_t tbytes = 0;  // bytes of the temporaries
+    std::function<void()> overlap;  // work of the setup's other streams, run once where the host is free
+    void run_overlap() {
+        if (!overlap) return;
+        const std::function<void()> f = std::move(overlap);
+        overlap = nullptr;
+        f();
+    }
     explicit Ctx(amdd_handle* hh) : h(hh) {}
     ~Ctx() {
         // work on the other setup streams may still read temporaries (after an error)
@@ -690,20 +688,6 @@ void trtri_batched(Ctx& C, const std::vector<TrtriDescT<T>>& ds) {
     }
 }
 
-template <typename T>
-void transpose_batched(Ctx& C, const std::vector<const T*>& src, const std::vector<T*>& dst,
-                       const std::vector<int>& n, const std::vector<int>& lds, const std::vector<int>& ldd) {
-    if (src.empty()) return;
-    int maxn = *std::max_element(n.begin(), n.end());
-    auto a = C.up(src);
-    auto b = C.up(dst);
-    auto c = C.up(n);
-    auto d = C.up(lds);
-    auto e = C.up(ldd);
-    PScope ps(C.h, PK_SMALL);
-    launch_transpose<T>(a, b, c, d, e, (int)src.size(), maxn, C.h->s);
-}
-
 // Block-pair one-sided Jacobi (rows in global memory): the host runs the
 // sweeps, each either as one launch per round over every matrix still
 // rotating or, in FP32 with amdd_opts.tensor_cores, as one persistent launch
@@ -772,6 +756,7 @@ void jacobi_pairs(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDes
                 launch_jacobi_pair_round<T>(djd, dt, (int)tasks.size(), r, tol, h->jacobi_inner, d_rot, rots, d_st,
                                             h->s);
         ck(cudaGetLastError());
+        C.run_overlap();  // the first sweep runs meanwhile
         ck(cudaMemcpyAsync(rot_h.data(), d_rot, nm * sizeof(int), cudaMemcpyDeviceToHost, h->s));
         ck(cudaStreamSynchronize(h->s));
         std::vector<int> still;
@@ -808,9 +793,10 @@ void run_jacobi(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDescT
         maxr = std::max(maxr, j.rows);
         floors = floors || j.absfloor || j.normfloor || j.loose_above > T(0);
     }
-    if (!launch_jacobi_block<T>(djd, (int)jd.size(), smem8, smem16, maxr, max_sweeps, tol, sweeps, rots, h->d_err,
-                                report_noconv, floors, h->s))
-        jacobi_pairs<T>(C, jd, djd, max_sweeps, tol, sweeps, rots, report_noconv);
+    const bool launched = launch_jacobi_block<T>(djd, (int)jd.size(), smem8, smem16, maxr, max_sweeps, tol, sweeps,
+                                                 rots, h->d_err, report_noconv, floors, h->s);
+    if (launched) C.run_overlap();
+    if (!launched) jacobi_pairs<T>(C, jd, djd, max_sweeps, tol, sweeps, rots, report_noconv);
 }
 
 // FP32 stage of the Jacobi solvers.  For each R x L matrix A_b (FP64, lda),
@@ -1818,24 +1804,61 @@ std::vector<int> learned_eigvecs(Ctx& C, amdd_handle* h, const std::vector<int>&
 constexpr int FRONT_LEAF = 96;
 constexpr int FRONT_RATIO = 20;
 
-// Entries of E given through the CSR values of A (every subdomain has the
-// diagonal basis): of unknown t (subdomain order) the position of its diagonal
-// entry, and the lower-triangle entries as (unknown, unknown, position).
-struct SparseE {
-    std::vector<int64_t> diag;
+// Symmetric adjacency of nv vertices from edges given in one direction (self
+// loops dropped; repeated edges removed when dups).
+void front_graph(int nv, const std::vector<int32_t>& a, const std::vector<int32_t>& b, bool dups,
+                 std::vector<int32_t>& ptr, std::vector<int32_t>& adj) {
+    ptr.assign(nv + 1, 0);
+    for (size_t e = 0; e < a.size(); ++e)
+        if (a[e] != b[e]) {
+            ++ptr[a[e] + 1];
+            ++ptr[b[e] + 1];
+        }
+    for (int v = 0; v < nv; ++v) ptr[v + 1] += ptr[v];
+    adj.resize(ptr[nv]);
+    std::vector<int32_t> at(ptr.begin(), ptr.end() - 1);
+    for (size_t e = 0; e < a.size(); ++e)
+        if (a[e] != b[e]) {
+            adj[at[a[e]]++] = b[e];
+            adj[at[b[e]]++] = a[e];
+        }
+    if (!dups) return;
+    int32_t w = 0;
+    for (int v = 0; v < nv; ++v) {
+        const int32_t lo = ptr[v], hi = at[v];
+        std::sort(adj.begin() + lo, adj.begin() + hi);
+        ptr[v] = w;
+        for (int32_t k = lo; k < hi; ++k)
+            if (k == lo || adj[k] != adj[k - 1]) adj[w++] = adj[k];
+    }
+    ptr[nv] = w;
+    adj.resize(w);
+}
+
+// Lower-triangle entries of a matrix given through the CSR values of A: (row
+// unknown, column unknown, position in the values); with diag (position of each
+// unknown's diagonal entry) the matrix is scaled to unit diagonal on both sides.
+struct FrontEntries {
     std::vector<int32_t> row, col;
-    std::vector<int64_t> src;
+    std::vector<int64_t> src, diag;
 };
 
-// Factors E (dense lower triangle, order nC, subdomain order, or the entries
-// sp) in the plan's stages: each part's front collects its entries of E and its children's Schur
-// complements, a partial Cholesky eliminates the interior, and the interior's
-// inverse Ainv = Y^T Y (Y = L_II^{-1}) and W^T = L_BI Y are kept for the solve.
-void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, int64_t nC, const SparseE* sp) {
+// Factors a matrix (the entries sp, or the dense lower triangle E of order nE in
+// the caller's order) in the plan's stages: each part's front collects its
+// entries and its children's Schur complements, a partial Cholesky eliminates the
+// interior, and the interior's inverse Ainv = Y^T Y (Y = L_II^{-1}) and W^T =
+// L_BI Y are kept for the solve.  All of this in FP64; with T = float (the local
+// solves of the mixed form) Ainv and W are rounded once at the end, so that the
+// solve carries only that rounding and its own FP32 sums (one-level apply on 24^3,
+// relative error 7e-8; with FP32 factors 4e-7 to 7e-7).
+template <typename T>
+void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& P, const FrontEntries* sp,
+                   const double* E, int64_t nE) {
     cudaStream_t s = h->s;
     const int nf = (int)P.fronts.size(), S = P.stages();
-    std::vector<FrontDev> fd(nf);
-    std::vector<int64_t> oF(nf + 1, 0), oA(nf + 1, 0), oW(nf + 1, 0), oY(nf + 1, 0), oL(nf + 1, 0);
+    std::vector<FrontDevT<double>> fd(nf);  // of the factorisation
+    std::vector<FrontDevT<T>> fk(nf);       // kept for the solve
+    std::vector<int64_t> oF(nf + 1, 0), oA(nf + 1, 0), oW(nf + 1, 0), oL(nf + 1, 0);
     for (int k = 0; k < nf; ++k) {
         const int64_t m = P.fronts[k].m, b = P.fronts[k].nb;
         oF[k + 1] = oF[k] + (m + b) * (m + b);
@@ -1843,12 +1866,23 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
         oW[k + 1] = oW[k] + m * b;
         oL[k + 1] = oL[k] + (int64_t)cdiv(m, CHOL_NB) * CHOL_NB * CHOL_NB;
     }
+    constexpr bool f64 = std::is_same<T, double>::value;
     double* F = C.tnew<double>(oF[nf]);
     double* Y = C.tnew<double>(oA[nf]);
     double* linv = C.tnew<double>(oL[nf]);
-    double* Ai = dnew<double>(h, oA[nf]);
-    double* W = dnew<double>(h, oW[nf]);
-    double* Wt = dnew<double>(h, oW[nf]);
+    T* Aik = dnew<T>(h, oA[nf]);
+    T* Wk = dnew<T>(h, oW[nf]);
+    T* Wtk = dnew<T>(h, oW[nf]);
+    double *Ai, *W, *Wt;
+    if constexpr (f64) {
+        Ai = Aik;
+        W = Wk;
+        Wt = Wtk;
+    } else {
+        Ai = C.tnew<double>(oA[nf]);
+        W = C.tnew<double>(oW[nf]);
+        Wt = C.tnew<double>(oW[nf]);
+    }
     ck(cudaMemsetAsync(F, 0, oF[nf] * sizeof(double), s));
 
     // children of each front, with the maps between their boundary and its rows
@@ -1876,33 +1910,32 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
             }
         }
         fd[k].kid1 = (int)ch.size();
+        fk[k] = {nullptr, Aik + oA[k], Wk + oW[k], f.m, f.nb, f.i0, f.b0, 0, 0};
     }
     // rows of W^T next to each boundary unknown, stage by stage
     std::vector<int32_t> drow, dptr{0}, rfront(P.n);
-    std::vector<FrontRef> refs;
-    h->fs.down_off.assign(S + 1, 0);
-    std::vector<std::vector<FrontRef>> at_row(P.n);
+    std::vector<FrontRefT<T>> refs;
+    refs.reserve(P.bnd.size());
+    fs.down_off.assign(S + 1, 0);
     for (int st = 0; st < S; ++st) {
-        std::vector<int32_t> touched;
+        std::vector<std::pair<int32_t, std::pair<int32_t, int32_t>>> touch;  // unknown, (front, boundary row)
         for (int k = P.stage_part[st]; k < P.stage_part[st + 1]; ++k) {
             const Front& f = P.fronts[k];
             for (int a = 0; a < f.m; ++a) rfront[f.i0 + a] = k;
-            for (int b = 0; b < f.nb; ++b) {
-                const int32_t t = P.bnd[f.b0 + b];
-                if (at_row[t].empty()) touched.push_back(t);
-                at_row[t].push_back({Wt + oW[k] + (size_t)b * f.m, f.i0, f.m});
+            for (int b = 0; b < f.nb; ++b) touch.push_back({P.bnd[f.b0 + b], {k, b}});
+        }
+        std::sort(touch.begin(), touch.end());
+        for (size_t q = 0; q < touch.size(); ++q) {
+            const Front& f = P.fronts[touch[q].second.first];
+            if (q == 0 || touch[q].first != touch[q - 1].first) {
+                if (q > 0) dptr.push_back((int32_t)refs.size());
+                drow.push_back(touch[q].first);
             }
+            refs.push_back({Wtk + oW[touch[q].second.first] + (size_t)touch[q].second.second * f.m, f.i0, f.m});
         }
-        std::sort(touched.begin(), touched.end());
-        for (int32_t t : touched) {
-            drow.push_back(t);
-            refs.insert(refs.end(), at_row[t].begin(), at_row[t].end());
-            dptr.push_back((int32_t)refs.size());
-            at_row[t].clear();
-        }
-        h->fs.down_off[st + 1] = (int64_t)drow.size();
+        if (!touch.empty()) dptr.push_back((int32_t)refs.size());
+        fs.down_off[st + 1] = (int64_t)drow.size();
     }
-    FrontSolve& fs = h->fs;
     fs.n = P.n;
     fs.stages = S;
     fs.row_off = P.stage_off;
@@ -1911,12 +1944,10 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
     fs.scale = nullptr;
     if (sp) {
         // plan-order scales, and each entry into the front of its earlier unknown
-        std::vector<int64_t> pos(P.n), dg(P.n), dst(sp->src.size());
-        std::vector<int32_t> ea(sp->src.size()), eb(sp->src.size()), gsrc(P.n);
-        for (int64_t k = 0; k < P.n; ++k) {
-            pos[P.perm[k]] = k;
-            dg[k] = sp->diag[P.perm[k]];
-        }
+        std::vector<int64_t> pos(P.n), dg(sp->diag.size()), dst(sp->src.size());
+        std::vector<int32_t> ea(sp->src.size()), eb(sp->src.size());
+        for (int64_t k = 0; k < P.n; ++k) pos[P.perm[k]] = k;
+        for (size_t k = 0; k < dg.size(); ++k) dg[k] = sp->diag[P.perm[k]];
         for (size_t e = 0; e < sp->src.size(); ++e) {
             const int64_t p = pos[sp->row[e]], q = pos[sp->col[e]];
             const int64_t a = std::max(p, q), b = std::min(p, q);
@@ -1931,83 +1962,93 @@ void factor_fronts(Ctx& C, amdd_handle* h, const FrontPlan& P, const double* E, 
             ea[e] = (int32_t)a;
             eb[e] = (int32_t)b;
         }
-        double* sc = dnew<double>(h, P.n);
-        h->d_dsc = dnew<double>(h, P.n);
-        launch_front_scale(h->val, C.up(dg), fs.perm, sc, h->d_dsc, P.n, s);
-        launch_front_scatter(h->val, C.up(sp->src), C.up(dst), C.up(ea), C.up(eb), sc, F, (int64_t)dst.size(), s);
-        fs.scale = sc;
+        const double* scale = nullptr;
+        if (!sp->diag.empty()) {
+            double* sc = dnew<double>(h, P.n);
+            h->d_dsc = dnew<double>(h, P.n);
+            launch_front_scale(h->val, C.up(dg), fs.perm, sc, h->d_dsc, P.n, s);
+            scale = sc;
+        }
+        launch_front_scatter(h->val, C.up(sp->src), C.up(dst), C.up(ea), C.up(eb), scale, F, (int64_t)dst.size(),
+                                s);
+        fs.scale = scale;
     }
-    fs.fr = C.up(fd, true);
+    fs.fr = C.up(fk, true);
+    const FrontDevT<double>* dfd = C.up(fd);
     fs.row_front = C.up(rfront, true);
     fs.bnd = C.up(P.bnd, true);
     fs.down_rows = C.up(drow, true);
     fs.down_ptr = C.up(dptr, true);
     fs.refs = C.up(refs, true);
-    fs.v = dnew<double>(h, (size_t)MAXB * P.n);
-    fs.e = dnew<double>(h, (size_t)MAXB * P.n);
+    fs.v = dnew<T>(h, (size_t)MAXB * P.n);
+    fs.e = dnew<T>(h, (size_t)MAXB * P.n);
+    fs.entries = (double)(oA[nf] + 2 * oW[nf]);
     const FrontChild* dch = C.up(ch);
     const int32_t* dmaps = C.up(maps);
 
-    for (int st = 0; st < S; ++st) {
-        const int k0 = P.stage_part[st], k1 = P.stage_part[st + 1];
-        if (k0 == k1) continue;
-        int maxn = 1, maxm = 1;
-        bool add = false;
-        std::vector<CholDesc> cd;
-        std::vector<TrtriDesc> td;
-        std::vector<GemmDesc> ga, gw;
-        std::vector<double*> mats;
-        std::vector<int> mm;
-        std::vector<TransDesc> tr;
-        for (int k = k0; k < k1; ++k) {
-            const int m = P.fronts[k].m, b = P.fronts[k].nb, n = m + b;
-            maxn = std::max(maxn, n);
-            maxm = std::max(maxm, std::max(m, b));
-            add = add || !kids[k].empty();
-            cd.push_back({F + oF[k], n, n, m, nullptr, linv + oL[k]});
-            td.push_back({F + oF[k], Y + oA[k], linv + oL[k], m, n, m});
-            GemmDesc g = gd<double>(Y + oA[k], m, 1, Y + oA[k], m, 0, Ai + oA[k], m, m, m, m, 1.0, 0.0, 1);
-            g.kfrom_row = 1;
-            ga.push_back(g);
-            mats.push_back(Ai + oA[k]);
-            mm.push_back(m);
-            if (b > 0) {
-                gw.push_back(gd<double>(F + oF[k] + (size_t)m * n, n, 0, Y + oA[k], m, 0, Wt + oW[k], m, b, m, m, 1.0,
-                                        0.0, 0));
-                tr.push_back({Wt + oW[k], W + oW[k], b, m, m, b});
+    for (int st = 0; st < S; ++st)
+        // (at most 32768 fronts a launch: some kernels count the matrices in a
+        // 16-bit grid dimension)
+        for (int k0 = P.stage_part[st]; k0 < P.stage_part[st + 1]; k0 += 32768) {
+            const int k1 = std::min(P.stage_part[st + 1], k0 + 32768);
+            int maxn = 1, maxm = 1;
+            bool add = false;
+            std::vector<CholDesc> cd;
+            std::vector<TrtriDesc> td;
+            std::vector<GemmDesc> ga, gw;
+            std::vector<double*> mats;
+            std::vector<int> mm;
+            std::vector<TransDesc> tr;
+            for (int k = k0; k < k1; ++k) {
+                const int m = P.fronts[k].m, b = P.fronts[k].nb, n = m + b;
+                maxn = std::max(maxn, n);
+                maxm = std::max(maxm, std::max(m, b));
+                add = add || !kids[k].empty();
+                cd.push_back({F + oF[k], n, n, m, nullptr, linv + oL[k]});
+                td.push_back({F + oF[k], Y + oA[k], linv + oL[k], m, n, m});
+                GemmDesc g = gd<double>(Y + oA[k], m, 1, Y + oA[k], m, 0, Ai + oA[k], m, m, m, m, 1.0, 0.0, 1);
+                g.kfrom_row = 1;
+                ga.push_back(g);
+                mats.push_back(Ai + oA[k]);
+                mm.push_back(m);
+                if (b > 0) {
+                    gw.push_back(gd<double>(F + oF[k] + (size_t)m * n, n, 0, Y + oA[k], m, 0, Wt + oW[k], m, b, m, m, 1.0,
+                                       0.0, 0));
+                    tr.push_back({Wt + oW[k], W + oW[k], b, m, m, b});
+                }
+            }
+            if (!sp) {
+                PScope ps(h, PK_E_ASM, 0.0);
+                launch_front_gather(dfd + k0, k1 - k0, fs.bnd, fs.perm, E, nE, maxn, s);
+            }
+            if (add) {
+                PScope ps(h, PK_SMALL);
+                launch_front_extend_add(dfd + k0, k1 - k0, dch, dmaps, maxn, s);
+            }
+            chol_batched<double>(C, cd);
+            trtri_batched<double>(C, td);
+            gemm(C, ga);
+            gemm(C, gw);
+            {
+                auto a = C.up(mats);
+                auto b = C.up(mm);
+                PScope ps(h, PK_SMALL);
+                launch_mirror_lower<double>(a, b, b, (int)mats.size(), maxm, s);
+            }
+            if (!tr.empty()) {
+                auto t = C.up(tr);
+                PScope ps(h, PK_SMALL);
+                launch_transpose_rect(t, (int)tr.size(), maxm, s);
             }
         }
-        if (!sp) {
-            PScope ps(h, PK_E_ASM, 0.0);
-            launch_front_gather(fs.fr + k0, k1 - k0, fs.bnd, fs.perm, E, nC, maxn, s);
-        }
-        if (add) {
-            PScope ps(h, PK_SMALL);
-            launch_front_extend_add(fs.fr + k0, k1 - k0, dch, dmaps, maxn, s);
-        }
-        chol_batched<double>(C, cd);
-        trtri_batched<double>(C, td);
-        gemm(C, ga);
-        gemm(C, gw);
-        {
-            auto a = C.up(mats);
-            auto b = C.up(mm);
-            PScope ps(h, PK_SMALL);
-            launch_mirror_lower<double>(a, b, b, (int)mats.size(), maxm, s);
-        }
-        if (!tr.empty()) {
-            auto t = C.up(tr);
-            PScope ps(h, PK_SMALL);
-            launch_transpose_rect(t, (int)tr.size(), maxm, s);
-        }
+    if constexpr (!f64) {
+        PScope ps(h, PK_SMALL);
+        launch_convert<double, float>(Ai, Aik, oA[nf], s);
+        launch_convert<double, float>(W, Wk, oW[nf], s);
+        launch_convert<double, float>(Wt, Wtk, oW[nf], s);
     }
-    h->csolve_flops = 2.0 * (double)(oA[nf] + 2 * oW[nf]);
-    h->csolve_bytes = 8.0 * (double)(oA[nf] + 2 * oW[nf]) + 48.0 * (double)P.n;
 }
 
-// T: type of the local work (factors of A_ii, T = L_A^{-1} S L_A^{-T}, its
-// eigensolve, Z_i).  TS: type of the splitting (SVD of X_i, Abar_ii and its
-// Schur complement S).
 // Sparse local factors (amdd_opts.local_solver): per subdomain the
 // nested-dissection order of the local pattern and the column structure of its
 // Cholesky factor (host, nd_factor_pattern); the permuted A_ii gathered dense on
@@ -2125,6 +2166,14 @@ void build_sparse_local(Ctx& C, amdd_handle* h, const std::vector<int64_t>& rp, 
     h->sparse_local = true;
 }
 
+template <typename T>
+FrontSolveT<T>& local_fronts(amdd_handle* h) {
+    if constexpr (std::is_same<T, double>::value)
+        return h->lfs;
+    else
+        return h->lfs32;
+}
+
 // Global unknown of each plan position when every subdomain has the diagonal
 // basis (coarse unknowns are the unknowns in subdomain order).
 std::vector<int32_t> plan_globals(const FrontPlan& P, const std::vector<std::vector<int32_t>>& Il) {
@@ -2135,6 +2184,9 @@ std::vector<int32_t> plan_globals(const FrontPlan& P, const std::vector<std::vec
     return g;
 }
 
+// T: type of the local work (factors of A_ii, T = L_A^{-1} S L_A^{-T}, its
+// eigensolve, Z_i).  TS: type of the splitting (SVD of X_i, Abar_ii and its
+// Schur complement S).
 template <typename T, typename TS>
 void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     constexpr bool f64 = std::is_same<T, double>::value;
@@ -2215,13 +2267,13 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     h->sum_nt = 0;
     for (int i = 0; i < N; ++i) {
         h->sum_nt += h->nt[i];
-        h->apply_tri_elems += (int64_t)h->ni[i] * (h->ni[i] + 1);
     }
 
     // ---- gather plans for A_ii = R_i A R_i^T (order [I, G]) and for
     // X_i = R_i A tilde R_i^T with columns ordered [G, D, I] (Eq. (Xi)).
     std::vector<int32_t> omega(h->sum_ni);
     std::vector<int64_t> pa_src, pa_dst, px_src, px_dst;
+    FrontEntries le;  // lower triangles of all A_ii (unknown: position in omega)
     {
         std::vector<int32_t> stamp(n, -1), posA(n, -1), posX(n, -1);
         for (int i = 0; i < N; ++i) {
@@ -2256,6 +2308,11 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                     if (posA[c] >= 0) {
                         pa_src.push_back(k);
                         pa_dst.push_back(h->off_sq[i] + (int64_t)a * ni + posA[c]);
+                        if (posA[c] <= a) {
+                            le.row.push_back((int32_t)(h->off_om[i] + a));
+                            le.col.push_back((int32_t)(h->off_om[i] + posA[c]));
+                            le.src.push_back(k);
+                        }
                     }
                     px_src.push_back(k);
                     px_dst.push_back(off_x[i] + (int64_t)a * nt + posX[c]);
@@ -2285,15 +2342,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     unsigned long long* rots = C.tnew<unsigned long long>(4 * N);
     ck(cudaMemsetAsync(rots, 0, 4 * N * sizeof(unsigned long long), s));
     TS* nrmT = C.tnew<TS>(h->sum_ni);
-    T* Yl = dnew<T>(h, h->sum_sq);   // L_i^{-1}
-    T* Ylt = dnew<T>(h, h->sum_sq);  // L_i^{-T}
-    if constexpr (f64) {
-        h->d_Y = Yl;
-        h->d_Yt = Ylt;
-    } else {
-        h->d_Y32 = Yl;
-        h->d_Yt32 = Ylt;
-    }
+    T* Yl = C.tnew<T>(h->sum_sq);  // L_A^{-1}, the leading nI x nI block of an ni x ni array
     ck(cudaMemsetAsync(Araw, 0, h->sum_sq * sizeof(double), s));
     ck(cudaMemsetAsync(Xp, 0, off_x[N] * sizeof(double), s));
     {
@@ -2496,31 +2545,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 const int i = part[g];
                 return vfirst[i] + (diag_basis && h->p[i] == h->nI[i] ? posI[g] : 0);
             };
-            std::vector<int32_t> aptr(base.size() + 1, 0), adj;
-            std::vector<int32_t> row;
-            auto close_row = [&](int32_t v) {
-                std::sort(row.begin(), row.end());
-                row.erase(std::unique(row.begin(), row.end()), row.end());
-                adj.insert(adj.end(), row.begin(), row.end());
-                aptr[v + 1] = (int32_t)adj.size();
-                row.clear();
-            };
-            for (int i = 0; i < N; ++i) {
-                if (h->p[i] == 0) continue;
-                const bool fd = diag_basis && h->p[i] == h->nI[i];
-                for (int a = 0; a < h->nI[i]; ++a) {
-                    const int64_t g = Il[i][a];
-                    const int32_t v = vertex(g);
-                    for (int64_t q = rp[g]; q < rp[g + 1]; ++q)
-                        if (h->p[part[ci[q]]] > 0) {
-                            const int32_t u = vertex(ci[q]);
-                            if (u != v) row.push_back(u);
-                        }
-                    if (fd) close_row(v);
-                }
-                if (!fd) close_row(vfirst[i]);
-            }
-            SparseE sp;
+            FrontEntries sp;
+            std::vector<int32_t> ea, eb;  // edges (with every unknown a vertex, the entries themselves)
             if (h->all_diag) {
                 sp.diag.assign(nC, -1);
                 for (int i = 0; i < N; ++i)
@@ -2536,9 +2562,21 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                             sp.src.push_back(q);
                         }
                     }
+            } else {
+                for (int64_t g = 0; g < n; ++g) {
+                    if (h->p[part[g]] == 0) continue;
+                    const int32_t v = vertex(g);
+                    for (int64_t q = rp[g]; q < rp[g + 1]; ++q)
+                        if (h->p[part[ci[q]]] > 0) {
+                            ea.push_back(v);
+                            eb.push_back(vertex(ci[q]));
+                        }
+                }
             }
+            std::vector<int32_t> aptr, adj;
+            front_graph((int)base.size(), h->all_diag ? sp.row : ea, h->all_diag ? sp.col : eb, !h->all_diag, aptr, adj);
             const FrontPlan plan = plan_fronts(aptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO);
-            factor_fronts(C, h, plan, E, nC, h->all_diag ? &sp : nullptr);
+            factor_fronts<double>(C, h, h->fs, plan, h->all_diag ? &sp : nullptr, E, nC);
             if (h->all_diag) h->fs.src = C.up(plan_globals(plan, Il), true);
         }
     };
@@ -2564,7 +2602,14 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->nC = h->coff[N];
         h->sum_zt = h->off_zt[N];
         spec_p = h->p;
-        ck(cudaEventRecord(h->ev_spec_in, h->s));  // A_ii gathered
+    }
+    // the copies of A and the plans' inputs are in place on the handle's stream
+    ck(cudaEventRecord(h->ev_spec_in, h->s));
+    // That coarse work and the factors of the local solves, on the third and fourth
+    // streams.  run_jacobi calls it (C.overlap) where the host would otherwise wait
+    // for the SVD: none of it is needed before the apply.
+    std::vector<int32_t> local_pos;  // plan position of each local unknown (omega order)
+    C.overlap = [&]() {
         ck(cudaStreamWaitEvent(h->s3, h->ev_spec_in, 0));
         std::swap(h->s, h->s3);
         std::swap(h->s2, h->s4);
@@ -2577,40 +2622,47 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             std::swap(h->ev_far, h->ev_far3);
         };
         try {
-            factor_coarse();
+            if (spec) factor_coarse();
+            if (!h->sparse_local) {
+                std::vector<int32_t> ptr, adj, wt(h->sum_ni, 1), base(h->sum_ni), src(h->sum_ni);
+                std::iota(base.begin(), base.end(), 0);
+                front_graph((int)h->sum_ni, le.row, le.col, false, ptr, adj);
+                const FrontPlan P = plan_fronts(ptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO);
+                local_pos.resize(h->sum_ni);
+                for (int64_t k = 0; k < P.n; ++k) {
+                    local_pos[P.perm[k]] = (int32_t)k;
+                    src[k] = omega[P.perm[k]];
+                }
+                FrontSolveT<T>& lf = local_fronts<T>(h);
+                factor_fronts<T>(C, h, lf, P, &le, nullptr, 0);
+                lf.src = C.up(src, true);
+            }
             ck(cudaEventRecord(h->ev_spec_done, h->s));
         } catch (...) {
             restore();
             throw;
         }
         restore();
-    }
+    };
 
-    // ---- (1) exact Cholesky of A_ii (local solver) and its inverse factor
+    // ---- (1) Cholesky factor L_A of A_II (the leading block of A_ii) and its
+    // inverse, for the eigenproblem of eq. (Zi)
     {
         std::vector<CholDescT<T>> cd(N);
         std::vector<TrtriDescT<T>> td(N);
-        std::vector<const T*> src(N);
-        std::vector<T*> dst(N);
-        std::vector<int> nn(N), ld(N);
         for (int i = 0; i < N; ++i) {
-            const int ni = h->ni[i];
-            cd[i] = {Lb + h->off_sq[i], ni, ni, ni, nullptr, linvA + off_la[i]};
-            td[i] = {Lb + h->off_sq[i], Yl + h->off_sq[i], linvA + off_la[i], ni, ni, ni};
-            src[i] = Yl + h->off_sq[i];
-            dst[i] = Ylt + h->off_sq[i];
-            nn[i] = ni;
-            ld[i] = ni;
+            const int ni = h->ni[i], nIi = h->nI[i];
+            cd[i] = {Lb + h->off_sq[i], nIi, ni, nIi, nullptr, linvA + off_la[i]};
+            td[i] = {Lb + h->off_sq[i], Yl + h->off_sq[i], linvA + off_la[i], nIi, ni, ni};
         }
         chol_batched(C, cd);
         trtri_batched(C, td);
-        transpose_batched(C, src, dst, nn, ld, ld);
     }
 
     // ---- (1b) sparse Cholesky factors of the A_ii in a nested-dissection order
     // (Sec. 4.1: exact local Cholesky; the same factor of the permuted matrix,
     // with the fill of the symbolic factorisation only): local solves then read
-    // the factor's entries instead of the dense triangles of L_i^{-1}.
+    // the factor's entries by substitution.
     if (h->local_solver != 0) build_sparse_local<T>(C, h, rp, ci, omega);
 
     // ---- (2) SVD of X_i (Sec. 3.2) by one-sided Jacobi on its rows: an
@@ -2676,6 +2728,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         PScope ps(h, PK_SMALL);
         launch_rownorms<float>(djd, N, dsp, delta, eps, 1, s);
     }
+
+    C.run_overlap();
 
     // steps (3)-(6): the splitting, its Schur complement, T_i and its eigenvalues
     if (!mf) {
@@ -2976,13 +3030,12 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     h->sum_zt = h->off_zt[N];
     if (spec) {
         spec_ok = h->p == spec_p;
-        if (spec_ok) {
-            ck(cudaStreamWaitEvent(s, h->ev_spec_done, 0));
-        } else {  // the speculative buffers stay owned by the handle until amdd_destroy
+        if (!spec_ok) {  // the speculative buffers stay owned by the handle until amdd_destroy
             ck(cudaStreamSynchronize(h->s3));
             ck(cudaStreamSynchronize(h->s4));
         }
     }
+    ck(cudaStreamWaitEvent(s, h->ev_spec_done, 0));
 
     // ---- (8) coarse block Z_i on Omega_Ii as A_II-orthonormal rows.  When
     // every eigenvalue is selected, span(Z_i) = R^{|Omega_Ii|} and any
@@ -3140,19 +3193,18 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
 
     // ---- (10) apply plan
     {
-        std::vector<GemvDescT<T>> l1(N), l2(N);
         std::vector<GemvDesc> cr(N);
         h->d_rloc = dnew<double>(h, h->sum_ni);
-        T* rlocT = f64 ? (T*)h->d_rloc : dnew<T>(h, h->sum_ni);
-        T* tlocT = dnew<T>(h, h->sum_ni);
-        T* ylocT = dnew<T>(h, h->sum_ni);
-        if constexpr (f64) {
-            h->d_tloc = tlocT;
-            h->d_yloc = ylocT;
+        if (h->sparse_local) {
+            if constexpr (f64) {
+                h->d_yloc = dnew<T>(h, h->sum_ni);
+            } else {
+                h->d_rloc32 = dnew<T>(h, h->sum_ni);
+                h->d_yloc32 = dnew<T>(h, h->sum_ni);
+            }
         } else {
-            h->d_rloc32 = rlocT;
-            h->d_tloc32 = tlocT;
-            h->d_yloc32 = ylocT;
+            h->d_yloc = h->lfs.e;
+            h->d_yloc32 = h->lfs32.e;
         }
         h->d_c = dnew<double>(h, nC);
         h->d_e = dnew<double>(h, nC);
@@ -3188,38 +3240,17 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             h->d_rl_zp = C.up(rlz, true);
             h->n_zp = (int64_t)rdz.size();
         }
-        std::vector<int32_t> rd, rl, rdc, rlc;  // rd / rl: row groups of the local products (matrix, first row)
-        h->lm1.assign(N, nullptr);
-        h->lm2.assign(N, nullptr);
+        std::vector<int32_t> rdc, rlc;
         for (int i = 0; i < N; ++i) {
-            const int ni = h->ni[i];
-            h->lm1[i] = Yl + h->off_sq[i];
-            h->lm2[i] = Ylt + h->off_sq[i];
-            l1[i] = {Yl + h->off_sq[i], ni, ni, ni, 1, rlocT + h->off_om[i], tlocT + h->off_om[i]};
-            l2[i] = {Ylt + h->off_sq[i], ni, ni, ni, 2, tlocT + h->off_om[i], ylocT + h->off_om[i]};
             if (h->d_Zt)
                 cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_rloc + h->off_om[i],
                          h->d_c + h->coff[i]};
-            for (int a = 0; a < ni; a += GEMV_ROWS_PER_WARP) {
-                rd.push_back(i);
-                rl.push_back(a);
-            }
             for (int k = 0; k < h->p[i] && !h->all_diag; ++k) {
                 rdc.push_back(i);
                 rlc.push_back(k);
             }
         }
-        if constexpr (f64) {
-            h->d_gv_l1 = C.up(l1, true);
-            h->d_gv_l2 = C.up(l2, true);
-        } else {
-            h->d_gv_l1_32 = C.up(l1, true);
-            h->d_gv_l2_32 = C.up(l2, true);
-        }
         h->d_gv_c = C.up(cr, true);
-        h->d_g4_desc = C.up(rd, true);
-        h->d_g4_row = C.up(rl, true);
-        h->n_g4 = (int64_t)rd.size();
         h->d_rd_c = C.up(rdc, true);
         h->d_rl_c = C.up(rlc, true);
         // prolongation: copies of each unknown in subdomain order, owners
@@ -3228,7 +3259,15 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         for (int64_t g = 0; g < n; ++g) scp[g + 1] += scp[g];
         std::vector<int32_t> sci(h->sum_ni);
         std::vector<int64_t> fill(scp.begin(), scp.end() - 1);
-        for (int64_t t = 0; t < h->sum_ni; ++t) sci[fill[omega[t]]++] = (int32_t)t;
+        // (copies in subdomain order; where each lies in the local solution)
+        if (h->sparse_local) {
+            local_pos.resize(h->sum_ni);
+            std::iota(local_pos.begin(), local_pos.end(), 0);
+        }
+        for (int64_t t = 0; t < h->sum_ni; ++t) sci[fill[omega[t]]++] = local_pos[t];
+        h->own_pos.resize(n);  // [I, G] order: a subdomain's own unknowns come first
+        for (int i = 0; i < N; ++i)
+            for (int a = 0; a < h->nI[i]; ++a) h->own_pos[h->off_I[i] + a] = local_pos[h->off_om[i] + a];
         std::vector<int32_t> og;
         og.reserve(n);
         for (int i = 0; i < N; ++i) og.insert(og.end(), Il[i].begin(), Il[i].end());
@@ -3248,9 +3287,9 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     if (e) throw Fail{err_status(e)};
 }
 
-// Local solves of the Schwarz methods: rloc = R_i r for every subdomain,
-// then y_i = L_i^{-T} L_i^{-1} rloc_i (into d_yloc, or d_yloc32 in the mixed
-// form, whose local solves run in FP32).
+// Local solves of the Schwarz methods: y_i = A_ii^{-1} R_i r for every subdomain
+// (d_yloc, or d_yloc32 in the mixed form, whose local solves run in FP32), by
+// substructuring or with the sparse factors (amdd_opts.local_solver).
 // The sparse local solves on nb gathered vectors (ld apart) of precision T.
 template <typename T>
 void sparse_local_solves(amdd_handle* h, const T* rloc, T* yloc, int nb, int64_t ld) {
@@ -3262,64 +3301,56 @@ void sparse_local_solves(amdd_handle* h, const T* rloc, T* yloc, int nb, int64_t
                                  static_cast<const T*>(h->d_sl_val), h->d_sl_perm, rloc, yloc, nb, ld, h->s);
 }
 
+// One pass of the local solves by substructuring on nb vectors r (n apart),
+// results in the plan order of lf.e.
+template <typename T>
+void front_local_solves(amdd_handle* h, const FrontSolveT<T>& lf, const double* r, int nb) {
+    PScope ps(h, pk<T>(PK_GEMV, PK_GEMV_F32), 2.0 * lf.entries * nb,
+              sizeof(T) * lf.entries + (12.0 + 4.0 * sizeof(T)) * h->sum_ni * nb);
+    launch_front_solve<T>(lf, r, h->n, (T*)nullptr, 0, nb, h->s);
+}
+
 void local_solves(amdd_handle* h, const double* r) {
     cudaStream_t s = h->s;
-    const double tri = (double)h->apply_tri_elems;  // elements of the lower + upper local factors
+    if (!h->sparse_local) {
+        if (h->precision == 0)
+            front_local_solves<double>(h, h->lfs, r, 1);
+        else
+            front_local_solves<float>(h, h->lfs32, r, 1);
+        return;
+    }
     {
         PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->sum_ni);
         launch_gather_vec(h->d_omega, h->sum_ni, r, h->d_rloc, s);
     }
-    if (h->sparse_local) {
-        if (h->precision == 0) {
-            sparse_local_solves<double>(h, h->d_rloc, h->d_yloc, 1, h->sum_ni);
-        } else {
-            {
-                PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * h->sum_ni);
-                launch_convert<double, float>(h->d_rloc, h->d_rloc32, h->sum_ni, s);
-            }
-            sparse_local_solves<float>(h, h->d_rloc32, h->d_yloc32, 1, h->sum_ni);
-        }
-        return;
-    }
     if (h->precision == 0) {
-        {
-            PScope ps(h, PK_GEMV, tri, 8.0 * tri / 2 + 24.0 * h->sum_ni);
-            launch_gemv_rows4<double>(h->d_gv_l1, h->d_g4_desc, h->d_g4_row, h->n_g4, s);
-        }
-        {
-            PScope ps(h, PK_GEMV, tri, 8.0 * tri / 2 + 24.0 * h->sum_ni);
-            launch_gemv_rows4<double>(h->d_gv_l2, h->d_g4_desc, h->d_g4_row, h->n_g4, s);
-        }
+        sparse_local_solves<double>(h, h->d_rloc, h->d_yloc, 1, h->sum_ni);
     } else {
-        // mixed form: local solves in FP32 (FP32 factors, FP32 accumulation)
         {
             PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * h->sum_ni);
             launch_convert<double, float>(h->d_rloc, h->d_rloc32, h->sum_ni, s);
         }
-        {
-            PScope ps(h, PK_GEMV_F32, tri, 4.0 * tri / 2 + 12.0 * h->sum_ni);
-            launch_gemv_rows4<float>(h->d_gv_l1_32, h->d_g4_desc, h->d_g4_row, h->n_g4, s);
-        }
-        {
-            PScope ps(h, PK_GEMV_F32, tri, 4.0 * tri / 2 + 12.0 * h->sum_ni);
-            launch_gemv_rows4<float>(h->d_gv_l2_32, h->d_g4_desc, h->d_g4_row, h->n_g4, s);
-        }
+        sparse_local_solves<float>(h, h->d_rloc32, h->d_yloc32, 1, h->sum_ni);
     }
 }
 
-// Coarse correction R_0^T E^{-1} R_0 r of Eq. (two_level_schwarz) from r and the
-// gathered rloc (its Omega_Ii entries): c = Z^T r, the solve with E, and
-// zc = Z e in owner order (d_zc).  Needs nC > 0.
+// Coarse correction R_0^T E^{-1} R_0 r of Eq. (two_level_schwarz): c = Z^T r from
+// the gathered r (rloc, its Omega_Ii entries), the solve with E, and zc = Z e in
+// owner order (d_zc).  Needs nC > 0.
 void inner_coarse_solve(amdd_handle* h);
 
 void coarse_correction(amdd_handle* h, const double* r) {
     cudaStream_t s = h->s;
     if (h->all_diag) {  // c and zc are scalings, done where the solve loads and stores its vectors
-        PScope ps(h, PK_CSOLVE, h->csolve_flops, h->csolve_bytes);
-        launch_front_solve(h->fs, r, h->n, h->d_zc, h->n, 1, s);
+        PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries, 8.0 * h->fs.entries + 48.0 * h->nC);
+        launch_front_solve<double>(h->fs, r, h->n, h->d_zc, h->n, 1, s);
         return;
     }
     const double zt = (double)h->sum_zt;
+    {
+        PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->sum_ni);
+        launch_gather_vec(h->d_omega, h->sum_ni, r, h->d_rloc, s);
+    }
     {
         PScope ps(h, PK_GEMV, 2.0 * zt, 8.0 * zt + 8.0 * h->sum_ni + 16.0 * h->nC);
         launch_gemv_rows<double>(h->d_gv_c, h->d_rd_c, h->d_rl_c, h->nC, s);
@@ -3327,8 +3358,8 @@ void coarse_correction(amdd_handle* h, const double* r) {
     if (h->next) {
         inner_coarse_solve(h);  // multilevel form: e ~ E^{-1} c by GMRES on the next level
     } else {
-        PScope ps(h, PK_CSOLVE, h->csolve_flops, h->csolve_bytes);
-        launch_front_solve(h->fs, h->d_c, h->nC, h->d_e, h->nC, 1, s);
+        PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries, 8.0 * h->fs.entries + 48.0 * h->nC);
+        launch_front_solve<double>(h->fs, h->d_c, h->nC, h->d_e, h->nC, 1, s);
     }
     {
         PScope ps(h, PK_GEMV, 2.0 * zt, 8.0 * zt + 8.0 * h->nC + 8.0 * h->n);
@@ -3353,11 +3384,8 @@ void apply_one(amdd_handle* h, const double* r, double* z) {
 // Buffers of the deflated and restricted forms, on first use.
 void ensure_forms(amdd_handle* h) {
     if (h->d_own_idx) return;
-    std::vector<int32_t> own(h->n);
-    for (int i = 0; i < h->N; ++i)
-        for (int a = 0; a < h->nI[i]; ++a) own[h->off_I[i] + a] = (int32_t)(h->off_om[i] + a);  // [I, G] order
     h->d_own_idx = dnew<int32_t>(h, h->n);
-    ck(cudaMemcpyAsync(h->d_own_idx, own.data(), h->n * sizeof(int32_t), cudaMemcpyHostToDevice, h->s));
+    ck(cudaMemcpyAsync(h->d_own_idx, h->own_pos.data(), h->n * sizeof(int32_t), cudaMemcpyHostToDevice, h->s));
     h->d_zg = dnew<double>(h, h->n);
     h->d_t = dnew<double>(h, h->n);
     ck(cudaStreamSynchronize(h->s));
@@ -3378,10 +3406,6 @@ void apply_form(amdd_handle* h, int form, const double* r, double* z) {
     const double* x = r;
     if (form != AMDD_FORM_ASM) ensure_forms(h);
     if (coarse) {
-        if (!h->all_diag) {
-            PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * h->sum_ni);
-            launch_gather_vec(h->d_omega, h->sum_ni, r, h->d_rloc, s);
-        }
         coarse_correction(h, r);
         {
             PScope ps(h, PK_GATHER_SCATTER, 0.0, 24.0 * h->n);
@@ -3425,38 +3449,20 @@ void dot_h(amdd_handle* h, const double* x, const double* y, int which, double t
 }
 
 // Buffers and descriptors of the batched path (MAXB right-hand sides), on first use.
-template <typename T>
-void* make_local_descs(amdd_handle* h, T* rloc, T* tloc, T* yloc, int which) {
-    const int N = h->N;
-    std::vector<GemvDescT<T>> g(N);
-    for (int i = 0; i < N; ++i) {
-        const int ni = h->ni[i];
-        if (which == 1)
-            g[i] = {static_cast<const T*>(h->lm1[i]), ni, ni, ni, 1, rloc + h->off_om[i], tloc + h->off_om[i]};
-        else
-            g[i] = {static_cast<const T*>(h->lm2[i]), ni, ni, ni, 2, tloc + h->off_om[i], yloc + h->off_om[i]};
-    }
-    GemvDescT<T>* d = dnew<GemvDescT<T>>(h, N);
-    ck(cudaMemcpyAsync(d, g.data(), N * sizeof(GemvDescT<T>), cudaMemcpyHostToDevice, h->s));
-    ck(cudaStreamSynchronize(h->s));
-    return d;
-}
-
 void ensure_multi(amdd_handle* h) {
     if (h->mb_cap >= MAXB) return;
     const int64_t L = (int64_t)MAXB * h->sum_ni, V = (int64_t)MAXB * h->n, CC = (int64_t)MAXB * std::max<int64_t>(h->nC, 1);
-    h->d_m_rloc = dnew<double>(h, L);
-    if (h->precision == 0) {
-        h->d_m_tloc = dnew<double>(h, L);
-        h->d_m_yloc = dnew<double>(h, L);
-        h->d_m_gv_l1 = make_local_descs<double>(h, h->d_m_rloc, h->d_m_tloc, h->d_m_yloc, 1);
-        h->d_m_gv_l2 = make_local_descs<double>(h, h->d_m_rloc, h->d_m_tloc, h->d_m_yloc, 2);
+    if (h->sparse_local || (h->nC > 0 && !h->all_diag)) h->d_m_rloc = dnew<double>(h, L);
+    if (h->sparse_local) {
+        if (h->precision == 0) {
+            h->d_m_yloc = dnew<double>(h, L);
+        } else {
+            h->d_m_rloc32 = dnew<float>(h, L);
+            h->d_m_yloc32 = dnew<float>(h, L);
+        }
     } else {
-        h->d_m_rloc32 = dnew<float>(h, L);
-        h->d_m_tloc32 = dnew<float>(h, L);
-        h->d_m_yloc32 = dnew<float>(h, L);
-        h->d_m_gv_l1 = make_local_descs<float>(h, h->d_m_rloc32, h->d_m_tloc32, h->d_m_yloc32, 1);
-        h->d_m_gv_l2 = make_local_descs<float>(h, h->d_m_rloc32, h->d_m_tloc32, h->d_m_yloc32, 2);
+        h->d_m_yloc = h->lfs.e;
+        h->d_m_yloc32 = h->lfs32.e;
     }
     h->d_m_c = dnew<double>(h, CC);
     h->d_m_e = dnew<double>(h, CC);
@@ -3502,51 +3508,27 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
     ensure_multi(h);
     cudaStream_t s = h->s;
     const int64_t L = h->sum_ni;
-    const double tri = (double)h->apply_tri_elems;
-    {
+    if (h->d_m_rloc) {
         PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * L * nb);
         launch_gather_vec_multi(h->d_omega, L, r, h->n, h->d_m_rloc, nb, s);
     }
-    if (h->sparse_local) {
-        if (h->precision == 0) {
-            sparse_local_solves<double>(h, h->d_m_rloc, h->d_m_yloc, nb, L);
-        } else {
-            {
-                PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * L * nb);
-                launch_convert<double, float>(h->d_m_rloc, h->d_m_rloc32, L * nb, s);
-            }
-            sparse_local_solves<float>(h, h->d_m_rloc32, h->d_m_yloc32, nb, L);
-        }
+    if (!h->sparse_local) {
+        if (h->precision == 0)
+            front_local_solves<double>(h, h->lfs, r, nb);
+        else
+            front_local_solves<float>(h, h->lfs32, r, nb);
     } else if (h->precision == 0) {
-        auto g1 = static_cast<const GemvDesc*>(h->d_m_gv_l1);
-        auto g2 = static_cast<const GemvDesc*>(h->d_m_gv_l2);
-        {
-            PScope ps(h, PK_GEMV, tri * nb, 8.0 * tri / 2 + 24.0 * L * nb);
-            launch_gemv_rows4_multi<double>(g1, h->d_g4_desc, h->d_g4_row, h->n_g4, nb, L, L, s);
-        }
-        {
-            PScope ps(h, PK_GEMV, tri * nb, 8.0 * tri / 2 + 24.0 * L * nb);
-            launch_gemv_rows4_multi<double>(g2, h->d_g4_desc, h->d_g4_row, h->n_g4, nb, L, L, s);
-        }
+        sparse_local_solves<double>(h, h->d_m_rloc, h->d_m_yloc, nb, L);
     } else {
-        auto g1 = static_cast<const GemvDescT<float>*>(h->d_m_gv_l1);
-        auto g2 = static_cast<const GemvDescT<float>*>(h->d_m_gv_l2);
         {
             PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * L * nb);
             launch_convert<double, float>(h->d_m_rloc, h->d_m_rloc32, L * nb, s);
         }
-        {
-            PScope ps(h, PK_GEMV_F32, tri * nb, 4.0 * tri / 2 + 12.0 * L * nb);
-            launch_gemv_rows4_multi<float>(g1, h->d_g4_desc, h->d_g4_row, h->n_g4, nb, L, L, s);
-        }
-        {
-            PScope ps(h, PK_GEMV_F32, tri * nb, 4.0 * tri / 2 + 12.0 * L * nb);
-            launch_gemv_rows4_multi<float>(g2, h->d_g4_desc, h->d_g4_row, h->n_g4, nb, L, L, s);
-        }
+        sparse_local_solves<float>(h, h->d_m_rloc32, h->d_m_yloc32, nb, L);
     }
     if (h->all_diag) {
-        PScope ps(h, PK_CSOLVE, h->csolve_flops * nb, h->csolve_bytes);
-        launch_front_solve(h->fs, r, h->n, h->d_m_zc, h->n, nb, s);
+        PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
+        launch_front_solve<double>(h->fs, r, h->n, h->d_m_zc, h->n, nb, s);
     } else if (h->nC > 0) {
         const double zt = (double)h->sum_zt;
         {
@@ -3554,8 +3536,8 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
             launch_gemv_rows_multi<double>(h->d_m_gv_c, h->d_rd_c, h->d_rl_c, h->nC, nb, L, h->nC, s);
         }
         {
-            PScope ps(h, PK_CSOLVE, h->csolve_flops * nb, h->csolve_bytes);
-            launch_front_solve(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, s);
+            PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
+            launch_front_solve<double>(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, s);
         }
         PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * h->nC + 8.0 * h->n) * nb);
         launch_gemv_rows_multi<double>(h->d_m_gv_zp, h->d_rd_zp, h->d_rl_zp, h->n_zp, nb, h->nC, h->n, s);

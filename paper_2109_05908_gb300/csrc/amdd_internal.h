@@ -21,7 +21,6 @@ enum : int {
 constexpr int CHOL_NB = 32;     // diagonal block of the blocked Cholesky / inverse
 constexpr int GEMM_T = 64;      // GEMM output tile
 constexpr int PANEL_ROWS = 16;  // rows per CTA of the Cholesky panel solve
-constexpr int GEMV_ROWS_PER_WARP = 4;  // rows per warp of the local triangular products
 constexpr int MAXB = 8;                // right-hand sides per batched apply / PCG pass
 constexpr int JAC_CLUSTER = 8;  // CTAs per matrix in the Jacobi solvers
 constexpr int JAC_MAX_PAIRS = 64;  // largest sub-round of the shared-memory block Jacobi
@@ -265,17 +264,8 @@ void launch_add_diag(T* const* mats, const int* n, const int* ld, const T* delta
 template <typename T>
 void launch_mirror_lower(T* const* mats, const int* n, const int* ld, int nmat, int maxn, cudaStream_t s);
 template <typename T>
-void launch_transpose(const T* const* src, T* const* dst, const int* n, const int* lds, const int* ldd, int nmat,
-                      int maxn, cudaStream_t s);
-template <typename T>
 void launch_gemv_rows(const GemvDescT<T>* d, const int* row_desc, const int* row_local, int64_t nrows,
                       cudaStream_t s);
-template <typename T>
-void launch_gemv_rows4(const GemvDescT<T>* d, const int* grp_desc, const int* grp_row, int64_t ngroups,
-                       cudaStream_t s);
-template <typename T>
-void launch_gemv_rows4_multi(const GemvDescT<T>* d, const int* grp_desc, const int* grp_row, int64_t ngroups, int nb,
-                             int64_t xs, int64_t ys, cudaStream_t s);
 template <typename T>
 void launch_gemv_rows_multi(const GemvDescT<T>* d, const int* row_desc, const int* row_local, int64_t nrows, int nb,
                             int64_t xs, int64_t ys, cudaStream_t s);
@@ -453,14 +443,15 @@ struct ScaleDesc {  // A[r] *= f[r] (or 1 / ||A[r]|| with unit scaling)
 template <typename T>
 void launch_scale_rows(const ScaleDesc<T>* d, int nmat, int unit, cudaStream_t s);
 
-// Coarse solve by substructuring (front_kernels.cu).  One part: its front F
+// Exact solves by substructuring (front_kernels.cu).  One part: its front F
 // ((m + nb) x (m + nb), lower triangle, setup only), Ainv (m x m, symmetric,
 // full) and W (m x nb), its interior at plan positions i0 .. i0 + m and its
 // boundary bnd[b0 .. b0 + nb).
-struct FrontDev {
-    double* F;
-    double* Ainv;
-    double* W;
+template <typename T>
+struct FrontDevT {
+    T* F;
+    T* Ainv;
+    T* W;
     int m, nb;
     int64_t i0, b0;
     int kid0, kid1;  // children (FrontChild) whose Schur complements enter F
@@ -470,39 +461,44 @@ struct FrontChild {
     int ld;
     int64_t map, inv;  // offsets of the maps child boundary -> parent row, parent row -> child boundary
 };
-struct FrontRef {  // a row of W^T and the interior it multiplies
-    const double* row;
+template <typename T>
+struct FrontRefT {  // a row of W^T and the interior it multiplies
+    const T* row;
     int64_t i0;
     int m;
 };
-struct FrontSolve {
+template <typename T>
+struct FrontSolveT {
     int64_t n = 0;
     int stages = 0;
     const int32_t* perm = nullptr;  // caller's index of each plan position (output)
     const int32_t* src = nullptr;   // its index in the input vectors
     const double* scale = nullptr;  // with it, input and output entries are multiplied by scale[plan position]
-    const FrontDev* fr = nullptr;
+    const FrontDevT<T>* fr = nullptr;
     const int32_t* row_front = nullptr;
     const int32_t* bnd = nullptr;
     const int32_t* down_rows = nullptr;  // boundary unknowns of each stage's parts
     const int32_t* down_ptr = nullptr;   // their refs (one shared list, nrow + 1 pointers over all stages)
-    const FrontRef* refs = nullptr;
-    double* v = nullptr;  // MAXB vectors of n each
-    double* e = nullptr;
+    const FrontRefT<T>* refs = nullptr;
+    T* v = nullptr;  // MAXB vectors of n each
+    T* e = nullptr;
     std::vector<int64_t> down_off, row_off;  // host: per stage
+    double entries = 0.0;                    // host: stored entries (multiply-adds of one solve)
 };
-void launch_front_gather(const FrontDev* fr, int nfr, const int32_t* bnd, const int32_t* perm, const double* E,
-                         int64_t nE, int maxn, cudaStream_t s);
+void launch_front_gather(const FrontDevT<double>* fr, int nfr, const int32_t* bnd, const int32_t* perm,
+                         const double* E, int64_t nE, int maxn, cudaStream_t s);
 // scale[k] = own[perm[k]] = 1 / sqrt(val[diag[k]]) (val 0 where diag[k] < 0), k < n
 void launch_front_scale(const double* val, const int64_t* diag, const int32_t* perm, double* scale, double* own,
                         int64_t n, cudaStream_t s);
-// F[dst[t]] = val[src[t]] scale[a[t]] scale[b[t]], t < cnt
+// F[dst[t]] = val[src[t]] (times scale[a[t]] scale[b[t]] when given), t < cnt
 void launch_front_scatter(const double* val, const int64_t* src, const int64_t* dst, const int32_t* a,
                           const int32_t* b, const double* scale, double* F, int64_t cnt, cudaStream_t s);
-void launch_front_extend_add(const FrontDev* fr, int nfr, const FrontChild* kids, const int32_t* maps, int maxn,
-                             cudaStream_t s);
-// out = E^{-1} c for nb <= MAXB vectors (c ldc apart, out ldo apart)
-void launch_front_solve(const FrontSolve& a, const double* c, int64_t ldc, double* out, int64_t ldo, int nb,
+void launch_front_extend_add(const FrontDevT<double>* fr, int nfr, const FrontChild* kids, const int32_t* maps,
+                             int maxn, cudaStream_t s);
+// the solution for nb <= MAXB vectors (c ldc apart) in a.e (plan order, n apart)
+// and, when out is given, in the caller's order (ldo apart)
+template <typename T>
+void launch_front_solve(const FrontSolveT<T>& a, const double* c, int64_t ldc, T* out, int64_t ldo, int nb,
                         cudaStream_t s);
 
 struct PcgScal {

@@ -1103,46 +1103,7 @@ void launch_mirror_lower(T* const* mats, const int* n, const int* ld, int nmat, 
 template void launch_mirror_lower<float>(float* const*, const int*, const int*, int, int, cudaStream_t);
 template void launch_mirror_lower<double>(double* const*, const int*, const int*, int, int, cudaStream_t);
 
-// dst = src^T for square n x n matrices, 32 x 32 tiles through shared memory.
-template <typename T>
-__global__ void transpose_kernel(const T* const* __restrict__ src, T* const* __restrict__ dst,
-                                 const int* __restrict__ n, const int* __restrict__ lds,
-                                 const int* __restrict__ ldd) {
-    const int b = blockIdx.z;
-    const int nn = n[b];
-    const int nt = (nn + 31) / 32;
-    __shared__ T tile[32][33];
-    for (int t = blockIdx.x; t < nt * nt; t += gridDim.x) {
-        const int tr = t / nt, tc = t % nt;
-        for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-            const int r = e / 32, c = e % 32;
-            const int gr = tr * 32 + r, gc = tc * 32 + c;
-            tile[r][c] = (gr < nn && gc < nn) ? src[b][(size_t)gr * lds[b] + gc] : T(0);
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-            const int r = e / 32, c = e % 32;
-            const int gr = tc * 32 + r, gc = tr * 32 + c;
-            if (gr < nn && gc < nn) dst[b][(size_t)gr * ldd[b] + gc] = tile[c][r];
-        }
-        __syncthreads();
-    }
-}
-
-template <typename T>
-void launch_transpose(const T* const* src, T* const* dst, const int* n, const int* lds, const int* ldd, int nmat,
-                      int maxn, cudaStream_t s) {
-    if (nmat <= 0 || maxn <= 0) return;
-    const int nt = (maxn + 31) / 32;
-    dim3 grid(min(nt * nt, 4096), 1, nmat);
-    transpose_kernel<T><<<grid, 256, 0, s>>>(src, dst, n, lds, ldd);
-}
-template void launch_transpose<float>(const float* const*, float* const*, const int*, const int*, const int*, int,
-                                      int, cudaStream_t);
-template void launch_transpose<double>(const double* const*, double* const*, const int*, const int*, const int*,
-                                       int, int, cudaStream_t);
-
-// dst = src^T for a batch of rectangular FP64 matrices, 32 x 32 tiles through
+// dst = src^T for a batch of rectangular matrices, 32 x 32 tiles through
 // shared memory (blockIdx.z = matrix)
 __global__ void transpose_rect_kernel(const TransDesc* __restrict__ descs) {
     const TransDesc d = descs[blockIdx.z];
@@ -1574,7 +1535,7 @@ void launch_tridiag(const TridiagDescT<T>* d, int nmat, int maxn, cudaStream_t s
 template void launch_tridiag<float>(const TridiagDescT<float>*, int, int, cudaStream_t);
 template void launch_tridiag<double>(const TridiagDescT<double>*, int, int, cudaStream_t);
 
-// All eigenvalues of symmetric tridiagonal matrices by multisection, BIS_L lanes
+// All eigenvalues of symmetric tridiagonal matrices by multisection, L lanes
 // per eigenvalue j (ascending): eigenvalue j is the x where the Sturm count
 // (number of eigenvalues below x = number of negative pivots of T - x I)
 // passes j.  The count uses the leading principal minors
@@ -1642,15 +1603,15 @@ __device__ __forceinline__ int sturm_count(const T* __restrict__ d, const T* __r
     return cnt;
 }
 
-// BIS_L lanes per eigenvalue: each pass takes the Sturm counts at BIS_L interior
-// points and keeps the subinterval that holds eigenvalue j, so the interval
-// shrinks (BIS_L + 1)-fold per pass.  A pass is a chain of n dependent steps
-// bound by latency, whatever the number of lanes: 8 lanes need a third of the
-// passes of plain bisection.  FP64, 1872 eigenvalues of matrices of 233 to 272
+// L lanes per eigenvalue: each pass takes the Sturm counts at L interior points
+// and keeps the subinterval that holds eigenvalue j, so the interval shrinks
+// (L + 1)-fold per pass.  A pass is a chain of n dependent steps, bound by latency
+// while the chip has room: 8 lanes then need a third of the passes of plain
+// bisection.  Once the FP64 units are full the 2.5 times larger number of counts
+// decides, so many eigenvalues take one lane each (FP64, 262,144 of 256 rows: 77
+// ms with one lane, 167 with eight).  FP64, 1872 eigenvalues of matrices of 233 to 272
 // rows: 11.4 -> 3.7 ms; FP32, 4096 of 256 rows: 0.38 -> 0.15 ms.
-constexpr int BIS_L = 8;
-
-template <typename T>
+template <typename T, int BIS_L>
 __global__ void __launch_bounds__(32) bisect_kernel(const TridiagDescT<T>* __restrict__ descs,
                                                      const int* __restrict__ eig_mat,
                                                      const int* __restrict__ eig_idx, int64_t total,
@@ -1658,7 +1619,7 @@ __global__ void __launch_bounds__(32) bisect_kernel(const TridiagDescT<T>* __res
     const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / BIS_L;
     if (gid >= total) return;  // uniform over the BIS_L lanes of an eigenvalue
     const int lane = threadIdx.x & 31, sub = lane & (BIS_L - 1);
-    const unsigned gmask = ((1u << BIS_L) - 1u) << (lane - sub);
+    const unsigned gmask = (BIS_L == 32 ? 0xffffffffu : (1u << BIS_L) - 1u) << (lane - sub);
     const TridiagDescT<T> t = descs[eig_mat[gid]];
     const int j = eig_idx[gid];
     const int n = t.n;
@@ -1710,7 +1671,10 @@ void launch_bisect(const TridiagDescT<T>* d, int nmat, const int* eig_mat, const
     if (total <= 0) return;
     bisect_prepare_kernel<T><<<nmat, 256, 0, s>>>(d);
     // one warp per block so that the eigenvalues spread over every SM
-    bisect_kernel<T><<<(unsigned)((total * BIS_L + 31) / 32), 32, 0, s>>>(d, eig_mat, eig_idx, total, out);
+    if (total <= (sizeof(T) == 8 ? 152 * 256 : 152 * 2048))
+        bisect_kernel<T, 8><<<(unsigned)((total * 8 + 31) / 32), 32, 0, s>>>(d, eig_mat, eig_idx, total, out);
+    else
+        bisect_kernel<T, 1><<<(unsigned)((total + 31) / 32), 32, 0, s>>>(d, eig_mat, eig_idx, total, out);
 }
 template void launch_bisect<float>(const TridiagDescT<float>*, int, const int*, const int*, int64_t, double* const*,
                                    cudaStream_t);
@@ -1757,153 +1721,6 @@ void launch_gemv_rows(const GemvDescT<T>* d, const int* row_desc, const int* row
 }
 template void launch_gemv_rows<float>(const GemvDescT<float>*, const int*, const int*, int64_t, cudaStream_t);
 template void launch_gemv_rows<double>(const GemvDescT<double>*, const int*, const int*, int64_t, cudaStream_t);
-
-// Local triangular products of the apply: one warp per group of RW
-// consecutive rows of one matrix (mode 1: row r uses columns [0, r]; mode 2:
-// [r, ncols)).  The descriptor is read once per group; each loop iteration
-// issues 2 x RW independent coalesced row loads; x (one subdomain's vector)
-// stays in L1.  Per row: lane-strided partial sums (two interleaved
-// accumulators) and a fixed shuffle tree.
-constexpr int GEMV_RW = GEMV_ROWS_PER_WARP;
-
-template <typename T>
-__global__ void __launch_bounds__(256) gemv_rows4_kernel(const GemvDescT<T>* __restrict__ descs,
-                                                         const int* __restrict__ grp_desc,
-                                                         const int* __restrict__ grp_row, int64_t ngroups) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= ngroups) return;
-    const GemvDescT<T> d = descs[grp_desc[w]];
-    const int r0 = grp_row[w];
-    const int nr = min(GEMV_RW, d.rows - r0);
-    int lo[GEMV_RW], hi[GEMV_RW];
-    int cmin = d.ncols, cmax = 0;
-#pragma unroll
-    for (int k = 0; k < GEMV_RW; ++k) {
-        const int r = r0 + k;
-        lo[k] = (d.mode == 2) ? r : 0;
-        hi[k] = (d.mode == 1) ? min(r + 1, d.ncols) : d.ncols;
-        if (k >= nr) hi[k] = lo[k];
-        if (k < nr) {
-            cmin = min(cmin, lo[k]);
-            cmax = max(cmax, hi[k]);
-        }
-    }
-    const T* M0 = d.M + (size_t)r0 * d.ld;
-    T s[GEMV_RW], t[GEMV_RW];
-#pragma unroll
-    for (int k = 0; k < GEMV_RW; ++k) s[k] = t[k] = T(0);
-    int c = cmin + lane;
-    for (; c + 32 < cmax; c += 64) {
-        const T x0 = d.x[c], x1 = d.x[c + 32];
-#pragma unroll
-        for (int k = 0; k < GEMV_RW; ++k) {
-            if (c >= lo[k] && c < hi[k]) s[k] = fma(M0[(size_t)k * d.ld + c], x0, s[k]);
-            if (c + 32 >= lo[k] && c + 32 < hi[k]) t[k] = fma(M0[(size_t)k * d.ld + c + 32], x1, t[k]);
-        }
-    }
-    if (c < cmax) {
-        const T x0 = d.x[c];
-#pragma unroll
-        for (int k = 0; k < GEMV_RW; ++k)
-            if (c >= lo[k] && c < hi[k]) s[k] = fma(M0[(size_t)k * d.ld + c], x0, s[k]);
-    }
-    T mine = T(0);
-#pragma unroll
-    for (int k = 0; k < GEMV_RW; ++k) {
-        T v = s[k] + t[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == k) mine = v;
-    }
-    if (lane < nr) {
-        const int r = r0 + lane;
-        d.y[r] = d.b ? fma(d.alpha, mine, d.b[r]) : d.alpha * mine;
-    }
-}
-
-template <typename T>
-void launch_gemv_rows4(const GemvDescT<T>* d, const int* grp_desc, const int* grp_row, int64_t ngroups,
-                       cudaStream_t s) {
-    if (ngroups <= 0) return;
-    const int64_t blocks = (ngroups * 32 + 255) / 256;
-    gemv_rows4_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(d, grp_desc, grp_row, ngroups);
-}
-template void launch_gemv_rows4<float>(const GemvDescT<float>*, const int*, const int*, int64_t, cudaStream_t);
-template void launch_gemv_rows4<double>(const GemvDescT<double>*, const int*, const int*, int64_t, cudaStream_t);
-
-// The same products for nb <= MAXB right-hand sides (x_k = x + k xs, y_k = y
-// + k ys; no b term): each factor entry is read once and applied to every
-// x_k.  With GEMV_RW x MAXB = 32 the reduced sum of (row r, rhs k) is
-// written by lane r MAXB + k.
-template <typename T>
-__global__ void __launch_bounds__(256) gemv_rows4_multi_kernel(const GemvDescT<T>* __restrict__ descs,
-                                                               const int* __restrict__ grp_desc,
-                                                               const int* __restrict__ grp_row, int64_t ngroups,
-                                                               int nb, int64_t xs, int64_t ys) {
-    static_assert(GEMV_RW * MAXB == 32, "one output per lane");
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= ngroups) return;
-    const GemvDescT<T> d = descs[grp_desc[w]];
-    const int r0 = grp_row[w];
-    const int nr = min(GEMV_RW, d.rows - r0);
-    int lo[GEMV_RW], hi[GEMV_RW];
-    int cmin = d.ncols, cmax = 0;
-#pragma unroll
-    for (int k = 0; k < GEMV_RW; ++k) {
-        const int r = r0 + k;
-        lo[k] = (d.mode == 2) ? r : 0;
-        hi[k] = (d.mode == 1) ? min(r + 1, d.ncols) : d.ncols;
-        if (k >= nr) hi[k] = lo[k];
-        if (k < nr) {
-            cmin = min(cmin, lo[k]);
-            cmax = max(cmax, hi[k]);
-        }
-    }
-    const T* M0 = d.M + (size_t)r0 * d.ld;
-    T s[GEMV_RW][MAXB];
-#pragma unroll
-    for (int r = 0; r < GEMV_RW; ++r)
-#pragma unroll
-        for (int k = 0; k < MAXB; ++k) s[r][k] = T(0);
-    for (int c = cmin + lane; c < cmax; c += 32) {
-        T xv[MAXB];
-#pragma unroll
-        for (int k = 0; k < MAXB; ++k) xv[k] = k < nb ? d.x[k * xs + c] : T(0);
-#pragma unroll
-        for (int r = 0; r < GEMV_RW; ++r)
-            if (c >= lo[r] && c < hi[r]) {
-                const T m = M0[(size_t)r * d.ld + c];
-#pragma unroll
-                for (int k = 0; k < MAXB; ++k) s[r][k] = fma(m, xv[k], s[r][k]);
-            }
-    }
-    T mine = T(0);
-#pragma unroll
-    for (int r = 0; r < GEMV_RW; ++r)
-#pragma unroll
-        for (int k = 0; k < MAXB; ++k) {
-            T v = s[r][k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == r * MAXB + k) mine = v;
-        }
-    const int rr = lane / MAXB, kk = lane % MAXB;
-    if (rr < nr && kk < nb) d.y[kk * ys + r0 + rr] = d.alpha * mine;
-}
-
-template <typename T>
-void launch_gemv_rows4_multi(const GemvDescT<T>* d, const int* grp_desc, const int* grp_row, int64_t ngroups, int nb,
-                             int64_t xs, int64_t ys, cudaStream_t s) {
-    if (ngroups <= 0) return;
-    const int64_t blocks = (ngroups * 32 + 255) / 256;
-    gemv_rows4_multi_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(d, grp_desc, grp_row, ngroups, nb, xs, ys);
-}
-template void launch_gemv_rows4_multi<float>(const GemvDescT<float>*, const int*, const int*, int64_t, int, int64_t,
-                                             int64_t, cudaStream_t);
-template void launch_gemv_rows4_multi<double>(const GemvDescT<double>*, const int*, const int*, int64_t, int, int64_t,
-                                              int64_t, cudaStream_t);
 
 // One warp per row of a batch of row-major matrices (mode 0: all columns),
 // nb right-hand sides: y_k[row] = alpha (M x_k)[row].
