@@ -2957,7 +2957,17 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 double fl = 0.0;
                 for (int i = 0; i < N; ++i) fl += 8.0 / 3.0 * std::pow((double)h->nI[i], 3);
                 PScope ps(h, pk<T>(PK_TRIDIAG, PK_TRIDIAG_F32), fl);
-                launch_tridiag<T>(dtd, N, maxn, s);
+                // the matrices that fit on the chip together, the larger ones apart
+                std::vector<TridiagDescT<T>> fit, big;
+                int maxf = 0;
+                for (int i = 0; i < N; ++i) {
+                    (tridiag_fits<T>(h->nI[i]) ? fit : big).push_back(td[i]);
+                    if (tridiag_fits<T>(h->nI[i])) maxf = std::max(maxf, h->nI[i]);
+                }
+                // a cluster of 16 takes most of a GPC, so eight run at a time: longest first
+                std::stable_sort(fit.begin(), fit.end(), [](const auto& x, const auto& y) { return x.n > y.n; });
+                if (!fit.empty()) launch_tridiag<T>(C.up(fit), (int)fit.size(), maxf, s);
+                if (!big.empty()) launch_tridiag<T>(C.up(big), (int)big.size(), maxn, s);
             }
             PScope ps(h, pk<T>(PK_BISECT, PK_BISECT_F32));
             launch_bisect<T>(dtd, N, dem, dej, (int64_t)em.size(), dout, s);

@@ -269,6 +269,9 @@ void launch_gemv_rows(const GemvDescT<T>* d, const int* row_desc, const int* row
 template <typename T>
 void launch_gemv_rows_multi(const GemvDescT<T>* d, const int* row_desc, const int* row_local, int64_t nrows, int nb,
                             int64_t xs, int64_t ys, cudaStream_t s);
+// whether a matrix of order n fits the distributed shared memory of a cluster
+template <typename T>
+bool tridiag_fits(int n);
 template <typename T>
 void launch_tridiag(const TridiagDescT<T>* d, int nmat, int maxn, cudaStream_t s);
 template <typename T>

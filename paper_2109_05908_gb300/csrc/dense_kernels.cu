@@ -1293,20 +1293,27 @@ __global__ void __cluster_dims__(JAC_CLUSTER, 1, 1) __launch_bounds__(256)
 // cluster of TD_CL CTAs per matrix, CTA c keeping the lower-triangle part
 // (columns 0..r) of the rows r = c mod TD_CL, packed row after row.  Per step
 // k (m = n - k - 1 trailing rows):
-//   A. the owned entries of column k go to colk and their squares to a partial
-//      sum; the owner of row k writes d[k];                 (cluster barrier 1)
-//   B. the norm, alpha and beta from the TD_CL partials in rank order; v
-//      gathered from the owners' colk; for every owned row r (one warp) the
-//      row part sum_{j <= r} A_rj v_j of (A22 v)_r and, for j < r, the column
-//      part A_rj v_r, accumulated per warp (in row order) and then summed over
-//      the warps into pcs;                                  (cluster barrier 2)
+//   A. the owned entries of column k go to colb;               (cluster barrier 1)
+//   B. every CTA gathers the whole column, takes its norm and forms the
+//      reflector v (the same sums in the same order in every CTA); then the
+//      products with A22 of the owned rows: a warp per row for the row parts
+//      sum_{j <= r} A_rj v_j, a thread per column for the column parts
+//      sum_{r > j} A_rj v_r, both straight from the packed rows;
+//                                                              (cluster barrier 2)
 //   C. p_r = beta (row part + the TD_CL column parts of r in rank order) for
-//      the owned rows, and a partial sum of p^T v;          (cluster barrier 3)
-//   D. K = beta/2 p^T v, w = p - K v gathered from the owners, and the rank-2
-//      update A_rj -= v_r w_j + w_r v_j of the owned rows.
-// colk, pcs, pv and the partials are double-buffered by step parity, so the
-// three barriers of a step also order it against the next one.  Every
-// reduction has a fixed order: the result does not depend on the schedule.
+//      the owned rows;                                         (cluster barrier 3)
+//   D. every CTA gathers p, forms K = beta/2 p^T v and w = p - K v, and updates
+//      the owned rows, A_rj -= v_r w_j + w_r v_j, a thread per column with v_j and
+//      w_j in registers.
+// colb alternates by step parity (a step whose column is already reduced skips
+// barriers 2 and 3); what else other CTAs read is rewritten only a barrier after
+// they have read it.  Every reduction has a fixed order: the result does not
+// depend on the schedule.
+// Bound by the latency of the three barriers and gathers; the sums the threads
+// used to exchange through per-warp buffers (8 n entries, two more cluster sums
+// per step) are what limited it before, in time and in n.  FP32, 16 matrices of
+// 614 to 1105 rows: 97 ms (the largest did not fit, so all streamed from L2) ->
+// 18 ms; of 256 rows: 1.20 -> 1.13 ms; FP64, 256 rows: 3.9 -> 3.5 ms.
 constexpr int TD_CL = 16;
 
 __host__ __device__ inline int64_t td_rows_entries(int c, int n, int* nown_out = nullptr) {
@@ -1326,8 +1333,9 @@ __host__ __device__ inline int64_t td_region(int n) {
     }
     return (mx + 1) / 2 * 2;
 }
-// the packed rows, then colk, pcs, pv (2n each), v, w (n each), pcw (8n)
-constexpr int TD_VECS = 16;
+// the packed rows, then (v, w) pairs (2n), colb (2n), pcb and pvb (n each)
+constexpr int TD_VECS = 6;
+constexpr size_t TD_SMEM_MAX = 226 * 1024;  // of 227 KB; the rest is static
 
 template <typename T>
 size_t tridiag_dsm_smem(int n) {
@@ -1344,135 +1352,142 @@ __global__ void __launch_bounds__(256) tridiag_dsm_kernel(const TridiagDescT<T>*
     extern __shared__ __align__(16) unsigned char td_raw[];
     int nown = 0;
     (void)td_rows_entries(c, n, &nown);
-    T* L = reinterpret_cast<T*>(td_raw);
-    T* colk = L + td_region(n);  // 2n, by global row
-    T* pcs = colk + 2 * n;            // 2n, by global row
-    T* pv = pcs + 2 * n;              // 2n, by global row
-    T* v = pv + 2 * n;                // n, by trailing index
-    T* w = v + n;                     // n
-    T* pcw = w + n;                   // 8n: column parts per warp
-    __shared__ T part[2][2];
-    __shared__ T red[8];
-    __shared__ T scal[4];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    auto off = [&](int l) -> int64_t { return (int64_t)l * (c + 1) + (int64_t)(TD_CL / 2) * l * (l - 1); };
-    // sum of the TD_CL partials part[b][q] in rank order, by warp 0, into scal[slot]
-    auto cluster_sum = [&](int b, int q, int slot) {
-        if (warp == 0) {
-            T x = T(0);
-            if (lane < TD_CL) x = *cluster.map_shared_rank(&part[b][q], lane);
-            T acc = T(0);
-            for (int i = 0; i < TD_CL; ++i) acc += __shfl_sync(0xffffffffu, x, i);
-            if (lane == 0) scal[slot] = acc;
-        }
-        __syncthreads();
+    struct Pair {
+        T v, w;
     };
-    auto block_sum = [&](T x, int b, int q) {
+    T* L = reinterpret_cast<T*>(td_raw);
+    Pair* vw = reinterpret_cast<Pair*>(L + td_region(n));  // n, by trailing index
+    T* colk = reinterpret_cast<T*>(vw + n);                // 2n, by global row
+    T* pcb = colk + 2 * n;                                 // n, by global row: column parts
+    T* pvb = pcb + n;                                      // n, by global row: row parts, then p
+    __shared__ T red[8];
+    __shared__ T scal[2];
+    __shared__ T x0s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    auto off = [&](int l) -> int { return l * (c + 1) + (TD_CL / 2) * l * (l - 1); };
+    // the sum over the CTA into red; every thread adds the eight warp sums in order
+    auto block_sum = [&](T x) -> T {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) red[warp] = x;
         __syncthreads();
-        if (tid == 0) {
-            T acc = T(0);
-            for (int ww = 0; ww < 8; ++ww) acc += red[ww];
-            part[b][q] = acc;
-        }
+        T acc = red[0];
+#pragma unroll
+        for (int ww = 1; ww < 8; ++ww) acc += red[ww];
+        return acc;
     };
 
-    for (int l = 0; l < nown; ++l) {
+    for (int l = warp; l < nown; l += 8) {
         const int r = c + TD_CL * l;
         T* dst = L + off(l);
-        for (int j = tid; j <= r; j += blockDim.x) dst[j] = t.A[(size_t)r * t.ld + j];
+        for (int j = lane; j <= r; j += 32) dst[j] = t.A[(size_t)r * t.ld + j];
     }
     if (c == 0 && tid == 0) t.e[0] = T(0);
     __syncthreads();
 
     for (int k = 0; k + 2 < n; ++k) {
-        const int b = k & 1, m = n - k - 1;
+        const int m = n - k - 1;
         const int l0 = (k + 1 - c) > 0 ? (k + 1 - c + TD_CL - 1) / TD_CL : 0;
-        T* colb = colk + (size_t)b * n;
-        T* pcb = pcs + (size_t)b * n;
-        T* pvb = pv + (size_t)b * n;
+        T* colb = colk + (size_t)(k & 1) * n;
         // A
-        T sl = T(0);
-        for (int l = l0 + tid; l < nown; l += blockDim.x) {
-            const int r = c + TD_CL * l;
-            const T x = L[off(l) + k];
-            colb[r] = x;
-            sl = fma(x, x, sl);
-        }
+        for (int l = l0 + tid; l < nown; l += 256) colb[c + TD_CL * l] = L[off(l) + k];
         if (c == k % TD_CL && tid == 0) t.d[k] = L[off((k - c) / TD_CL) + k];
-        block_sum(sl, b, 0);
         cluster.sync();  // 1
-        // B
-        cluster_sum(b, 0, 0);
-        const T s2 = scal[0];
-        const T x0 = *cluster.map_shared_rank(colb + (k + 1), (k + 1) % TD_CL);
-        const T tail = s2 - x0 * x0;
-        if (!(tail > T(0))) {
+        // B: column and reflector
+        T tl = T(0);
+        for (int i = tid; i < m; i += 256) {
+            const int r = k + 1 + i;
+            const T x = *cluster.map_shared_rank(colb + r, r & (TD_CL - 1));
+            vw[i].v = x;
+            if (i > 0)
+                tl = fma(x, x, tl);
+            else
+                x0s = x;
+        }
+        const T tail = block_sum(tl);
+        const T x0 = x0s;  // (vw[0].v becomes v_0 below)
+        if (!(tail > T(0))) {  // the same decision in every CTA
             if (c == 0 && tid == 0) t.e[k + 1] = x0;
             __syncthreads();
             continue;
         }
-        const T alpha = -copysign(sqrt(s2), x0);
-        const T v0 = x0 - alpha;
-        const T beta = T(2) / fma(v0, v0, tail);
-        for (int i = tid; i < m; i += blockDim.x) {
-            const int r = k + 1 + i;
-            v[i] = i == 0 ? v0 : *cluster.map_shared_rank(colb + r, r % TD_CL);
-        }
-        T* pw = pcw + (size_t)warp * n;
-        for (int j = lane; j < m; j += 32) pw[j] = T(0);
-        __syncthreads();
-        for (int l = l0 + warp; l < nown; l += 8) {
-            const int r = c + TD_CL * l, i = r - k - 1;
-            const T* row = L + off(l) + (k + 1);
-            const T vi = v[i];
-            T acc = T(0);
-            for (int j = lane; j <= i; j += 32) {
-                const T a = row[j];
-                acc = fma(a, v[j], acc);
-                if (j < i) pw[j] = fma(a, vi, pw[j]);
+        // scalars by one warp: the FP64 square root and division would otherwise
+        // occupy the FP64 units eight times over
+        if (warp == 0) {
+            const T alpha = -copysign(sqrt(fma(x0, x0, tail)), x0);
+            const T v0 = x0 - alpha;
+            if (lane == 0) {
+                scal[0] = alpha;
+                scal[1] = T(2) / fma(v0, v0, tail);
+                vw[0].v = v0;
             }
+        }
+        __syncthreads();
+        const T beta = scal[1];
+        // row parts
+        for (int l = l0 + warp; l < nown; l += 8) {
+            const int i = c + TD_CL * l - k - 1;
+            const T* row = L + off(l) + (k + 1);
+            T a0 = T(0), a1 = T(0);
+            int j = lane;
+            for (; j + 32 <= i; j += 64) {
+                a0 = fma(row[j], vw[j].v, a0);
+                a1 = fma(row[j + 32], vw[j + 32].v, a1);
+            }
+            if (j <= i) a0 = fma(row[j], vw[j].v, a0);
+            T acc = a0 + a1;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) pvb[r] = acc;
+            if (lane == 0) pvb[i + k + 1] = acc;
         }
-        __syncthreads();
-        for (int j = tid; j < m; j += blockDim.x) {
-            T acc = T(0);
-#pragma unroll
-            for (int ww = 0; ww < 8; ++ww) acc += pcw[(size_t)ww * n + j];
-            pcb[k + 1 + j] = acc;
+        // column parts: rows below j only
+        for (int j = tid; j < m; j += 256) {
+            const int g = k + 1 + j;  // first owned row below g
+            int l = g + 1 - c > 0 ? (g + 1 - c + TD_CL - 1) / TD_CL : 0;
+            T a0 = T(0), a1 = T(0);
+            for (; l + 1 < nown; l += 2) {
+                const int i = c + TD_CL * l - k - 1;
+                a0 = fma(L[off(l) + g], vw[i].v, a0);
+                a1 = fma(L[off(l + 1) + g], vw[i + TD_CL].v, a1);
+            }
+            if (l < nown) a0 = fma(L[off(l) + g], vw[c + TD_CL * l - k - 1].v, a0);
+            pcb[g] = a0 + a1;
         }
         cluster.sync();  // 2
         // C
-        T kl = T(0);
-        for (int l = l0 + tid; l < nown; l += blockDim.x) {
+        for (int l = l0 + tid; l < nown; l += 256) {
             const int r = c + TD_CL * l;
+            T part[TD_CL];
+#pragma unroll
+            for (int cc = 0; cc < TD_CL; ++cc) part[cc] = *cluster.map_shared_rank(pcb + r, cc);
             T acc = pvb[r];
-            for (int cc = 0; cc < TD_CL; ++cc) acc += *cluster.map_shared_rank(pcb + r, cc);
-            const T pr = beta * acc;
-            pvb[r] = pr;
-            kl = fma(pr, v[r - k - 1], kl);
+#pragma unroll
+            for (int cc = 0; cc < TD_CL; ++cc) acc += part[cc];
+            pvb[r] = beta * acc;
         }
-        block_sum(kl, b, 1);
         cluster.sync();  // 3
         // D
-        cluster_sum(b, 1, 1);
-        const T K = T(0.5) * beta * scal[1];
-        for (int i = tid; i < m; i += blockDim.x) {
+        T kl = T(0);
+        for (int i = tid; i < m; i += 256) {
             const int r = k + 1 + i;
-            w[i] = fma(-K, v[i], *cluster.map_shared_rank(pvb + r, r % TD_CL));
+            const T pr = *cluster.map_shared_rank(pvb + r, r & (TD_CL - 1));
+            vw[i].w = pr;
+            kl = fma(pr, vw[i].v, kl);
         }
+        const T K = T(0.5) * beta * block_sum(kl);
+        for (int i = tid; i < m; i += 256) vw[i].w = fma(-K, vw[i].v, vw[i].w);
         __syncthreads();
-        for (int l = l0 + warp; l < nown; l += 8) {
-            const int r = c + TD_CL * l, i = r - k - 1;
-            T* row = L + off(l) + (k + 1);
-            const T vi = v[i], wi = w[i];
-            for (int j = lane; j <= i; j += 32) row[j] = fma(-vi, w[j], fma(-wi, v[j], row[j]));
+        for (int j = tid; j < m; j += 256) {
+            const int g = k + 1 + j;
+            const Pair q = vw[j];
+#pragma unroll 4
+            for (int l = g - c > 0 ? (g - c + TD_CL - 1) / TD_CL : 0; l < nown; ++l) {
+                const Pair pr = vw[c + TD_CL * l - k - 1];
+                T* a = L + off(l) + g;
+                *a = fma(-pr.v, q.w, fma(-pr.w, q.v, *a));
+            }
         }
-        if (c == 0 && tid == 0) t.e[k + 1] = alpha;
+        if (c == 0 && tid == 0) t.e[k + 1] = scal[0];
         __syncthreads();
     }
     if (tid == 0) {
@@ -1492,7 +1507,7 @@ __global__ void __launch_bounds__(256) tridiag_dsm_kernel(const TridiagDescT<T>*
 template <typename T>
 bool launch_tridiag_dsm(const TridiagDescT<T>* d, int nmat, int maxn, cudaStream_t s) {
     const size_t smem = tridiag_dsm_smem<T>(maxn);
-    if (smem > JAC_BLOCK_SMEM_MAX) return false;
+    if (smem > TD_SMEM_MAX) return false;
     auto kern = tridiag_dsm_kernel<T>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -1522,6 +1537,13 @@ bool launch_tridiag_dsm(const TridiagDescT<T>* d, int nmat, int maxn, cudaStream
     }
     return true;
 }
+
+template <typename T>
+bool tridiag_fits(int n) {
+    return tridiag_dsm_smem<T>(n) <= TD_SMEM_MAX;
+}
+template bool tridiag_fits<float>(int);
+template bool tridiag_fits<double>(int);
 
 template <typename T>
 void launch_tridiag(const TridiagDescT<T>* d, int nmat, int maxn, cudaStream_t s) {
