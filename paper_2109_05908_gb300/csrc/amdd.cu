@@ -3289,7 +3289,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->d_z = dnew<double>(h, n);
         h->d_pv = dnew<double>(h, n);
         h->d_q = dnew<double>(h, n);
-        h->d_part = dnew<double>(h, DOT_BLOCKS);
+        h->d_part = dnew<double>(h, DOT_MAX_BLOCKS);
         h->d_sc = dnew<PcgScal>(h, 1);
     }
     ck(cudaGetLastError());
@@ -3377,18 +3377,52 @@ void coarse_correction(amdd_handle* h, const double* r) {
     }
 }
 
+// Runs f with the handle's stream set to its second one, behind the work issued so
+// far; the handle's stream continues beside it until join().
+struct Fork {
+    amdd_handle* h;
+    bool on;
+    explicit Fork(amdd_handle* hh, bool use) : h(hh), on(use) {
+        if (!on) return;
+        ck(cudaEventRecord(h->ev_panel, h->s));
+        ck(cudaStreamWaitEvent(h->s2, h->ev_panel, 0));
+    }
+    template <class F>
+    void run(F f) {
+        if (!on) return f();
+        std::swap(h->s, h->s2);
+        try {
+            f();
+        } catch (...) {
+            std::swap(h->s, h->s2);
+            throw;
+        }
+        std::swap(h->s, h->s2);
+        ck(cudaEventRecord(h->ev_far, h->s2));
+    }
+    void join() {
+        if (on) ck(cudaStreamWaitEvent(h->s, h->ev_far, 0));
+    }
+};
+
 // z = M^{-1} r, Eq. (two_level_schwarz): one-level sum plus the coarse term,
-// summed per unknown in a fixed order.
-void apply_one(amdd_handle* h, const double* r, double* z) {
-    cudaStream_t s = h->s;
+// summed per unknown in a fixed order; with d also r.z into the PCG scalars.  The
+// coarse solve (a chain of small launches) runs beside the local solves.
+void apply_one(amdd_handle* h, const double* r, double* z, const DotArgs& d = DotArgs{}) {
+    // (the sparse local solves and a dense coarse basis share the gathered r)
+    Fork side(h, h->nC > 0 && !h->next && (h->all_diag || !h->sparse_local));
+    if (h->nC > 0) side.run([&] { coarse_correction(h, r); });
     local_solves(h, r);
-    if (h->nC > 0) coarse_correction(h, r);
+    side.join();
     PScope ps(h, PK_GATHER_SCATTER, 0.0, 12.0 * h->sum_ni + 24.0 * h->n);
     const double* zc = h->nC > 0 ? h->d_zc : nullptr;
+    const DotArgs* dp = d.sc ? &d : nullptr;
     if (h->precision == 0)
-        launch_scatter_prolong<double>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_yloc, zc, z, s);
+        launch_scatter_prolong<double>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_yloc, zc, z, h->s, 1, 0, 0, 0,
+                                       r, dp);
     else
-        launch_scatter_prolong<float>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_yloc32, zc, z, s);
+        launch_scatter_prolong<float>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_yloc32, zc, z, h->s, 1, 0, 0, 0,
+                                      r, dp);
 }
 
 // Buffers of the deflated and restricted forms, on first use.
@@ -3450,12 +3484,14 @@ void spmv_h(amdd_handle* h, const double* x, double* y) {
     launch_spmv(h->n, h->nnz, h->rowptr, h->col, h->val, x, y, h->s);
 }
 void dot_h(amdd_handle* h, const double* x, const double* y, int which, double tol2) {
-    {
-        PScope ps(h, PK_PCG_VEC, 2.0 * h->n, 16.0 * h->n);
-        launch_dot_partials(h->n, x, y, h->d_part, h->s);
-    }
-    PScope ps(h, PK_PCG_VEC);
-    launch_dot_finalize(h->d_part, h->d_sc, which, tol2, h->s);
+    PScope ps(h, PK_PCG_VEC, 2.0 * h->n, 16.0 * h->n);
+    launch_dot(h->n, x, y, DotArgs{h->d_part, h->d_sc, which, tol2, 0}, h->s);
+}
+// q = A p with p.q, and x += alpha p, r -= alpha q with r.r
+void spmv_pq_h(amdd_handle* h) {
+    PScope ps(h, PK_SPMV, 2.0 * h->nnz + 2.0 * h->n, 12.0 * h->nnz + 8.0 * (h->n + 1) + 16.0 * h->n);
+    launch_spmv_dot(h->n, h->nnz, h->rowptr, h->col, h->val, h->d_pv, h->d_q, DotArgs{h->d_part, h->d_sc, 0, 0.0, 0},
+                    h->s);
 }
 
 // Buffers and descriptors of the batched path (MAXB right-hand sides), on first use.
@@ -3502,7 +3538,7 @@ void ensure_multi(amdd_handle* h) {
     h->d_m_r = dnew<double>(h, V);
     h->d_m_z = dnew<double>(h, V);
     h->d_m_p = dnew<double>(h, V);
-    h->d_m_part = dnew<double>(h, (int64_t)MAXB * DOT_BLOCKS);
+    h->d_m_part = dnew<double>(h, (int64_t)MAXB * DOT_MAX_BLOCKS);
     h->d_m_sc = dnew<PcgScal>(h, MAXB);
     ck(cudaStreamSynchronize(h->s));
     h->mb_cap = MAXB;
@@ -3510,9 +3546,10 @@ void ensure_multi(amdd_handle* h) {
 
 // z_k = M^{-1} r_k for nb <= MAXB right-hand sides (vectors n apart): every
 // factor, Z_i and L_E entry is read once per pass for all of them.
-void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
+void apply_multi(amdd_handle* h, const double* r, double* z, int nb, const DotArgs& d = DotArgs{}) {
     if (h->next) {  // inexact coarse solves run one right-hand side at a time
         for (int k = 0; k < nb; ++k) apply_one(h, r + (size_t)k * h->n, z + (size_t)k * h->n);
+        if (d.sc) launch_dot(h->n, r, z, d, h->s, nb, h->n);
         return;
     }
     ensure_multi(h);
@@ -3522,6 +3559,26 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
         PScope ps(h, PK_GATHER_SCATTER, 0.0, 20.0 * L * nb);
         launch_gather_vec_multi(h->d_omega, L, r, h->n, h->d_m_rloc, nb, s);
     }
+    Fork side(h, h->nC > 0);
+    if (h->nC > 0)
+        side.run([&] {
+            if (h->all_diag) {
+                PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
+                launch_front_solve<double>(h->fs, r, h->n, h->d_m_zc, h->n, nb, h->s);
+                return;
+            }
+            const double zt = (double)h->sum_zt;
+            {
+                PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * L + 16.0 * h->nC) * nb);
+                launch_gemv_rows_multi<double>(h->d_m_gv_c, h->d_rd_c, h->d_rl_c, h->nC, nb, L, h->nC, h->s);
+            }
+            {
+                PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
+                launch_front_solve<double>(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, h->s);
+            }
+            PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * h->nC + 8.0 * h->n) * nb);
+            launch_gemv_rows_multi<double>(h->d_m_gv_zp, h->d_rd_zp, h->d_rl_zp, h->n_zp, nb, h->nC, h->n, h->s);
+        });
     if (!h->sparse_local) {
         if (h->precision == 0)
             front_local_solves<double>(h, h->lfs, r, nb);
@@ -3536,44 +3593,25 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb) {
         }
         sparse_local_solves<float>(h, h->d_m_rloc32, h->d_m_yloc32, nb, L);
     }
-    if (h->all_diag) {
-        PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
-        launch_front_solve<double>(h->fs, r, h->n, h->d_m_zc, h->n, nb, s);
-    } else if (h->nC > 0) {
-        const double zt = (double)h->sum_zt;
-        {
-            PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * L + 16.0 * h->nC) * nb);
-            launch_gemv_rows_multi<double>(h->d_m_gv_c, h->d_rd_c, h->d_rl_c, h->nC, nb, L, h->nC, s);
-        }
-        {
-            PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
-            launch_front_solve<double>(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, s);
-        }
-        PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * h->nC + 8.0 * h->n) * nb);
-        launch_gemv_rows_multi<double>(h->d_m_gv_zp, h->d_rd_zp, h->d_rl_zp, h->n_zp, nb, h->nC, h->n, s);
-    }
+    side.join();
     PScope ps(h, PK_GATHER_SCATTER, 0.0, (12.0 * L + 24.0 * h->n) * nb);
     const double* zc = h->nC > 0 ? h->d_m_zc : nullptr;
     if (h->precision == 0)
         launch_scatter_prolong<double>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_m_yloc, zc, z, s, nb, L,
-                                       h->n, h->n);
+                                       h->n, h->n, r, d.sc ? &d : nullptr);
     else
         launch_scatter_prolong<float>(h->n, h->d_order_g, h->d_sc_ptr, h->d_sc_idx, h->d_m_yloc32, zc, z, s, nb, L,
-                                      h->n, h->n);
+                                      h->n, h->n, r, d.sc ? &d : nullptr);
 }
 
-void spmv_multi_h(amdd_handle* h, const double* x, double* y, int nb) {
+void spmv_multi_h(amdd_handle* h, const double* x, double* y, int nb, const DotArgs* d = nullptr) {
     PScope ps(h, PK_SPMV, 2.0 * h->nnz * nb, 12.0 * h->nnz + 8.0 * (h->n + 1) + 16.0 * h->n * nb);
-    launch_spmv_multi(h->n, h->rowptr, h->col, h->val, x, y, nb, h->n, h->s);
+    launch_spmv_multi(h->n, h->rowptr, h->col, h->val, x, y, nb, h->n, h->s, d);
 }
 
 void dot_multi_h(amdd_handle* h, const double* x, const double* y, int which, double tol2, int nb, int skip) {
-    {
-        PScope ps(h, PK_PCG_VEC, 2.0 * h->n * nb, 16.0 * h->n * nb);
-        launch_dot_partials(h->n, x, y, h->d_m_part, h->s, nb, h->n);
-    }
-    PScope ps(h, PK_PCG_VEC);
-    launch_dot_finalize(h->d_m_part, h->d_m_sc, which, tol2, h->s, nb, skip);
+    PScope ps(h, PK_PCG_VEC, 2.0 * h->n * nb, 16.0 * h->n * nb);
+    launch_dot(h->n, x, y, DotArgs{h->d_m_part, h->d_m_sc, which, tol2, skip}, h->s, nb, h->n);
 }
 
 // nb <= MAXB independent PCG solves advanced together (one SpMV and one
@@ -3613,19 +3651,14 @@ bool pcg_multi(amdd_handle* h, const double* b, double* x, int nb, double rtol, 
     }
     int its = 0;
     if (!all) {
-        apply_multi(h, h->d_m_r, h->d_m_z, nb);
-        dot_multi_h(h, h->d_m_r, h->d_m_z, 4, tol2, nb, 0);
+        apply_multi(h, h->d_m_r, h->d_m_z, nb, DotArgs{h->d_m_part, h->d_m_sc, 4, tol2, 0});
         ck(cudaMemcpyAsync(h->d_m_p, h->d_m_z, V * sizeof(double), cudaMemcpyDeviceToDevice, s));
         for (its = 1; its <= maxit; ++its) {
-            spmv_multi_h(h, h->d_m_p, h->d_m_q, nb);
-            dot_multi_h(h, h->d_m_p, h->d_m_q, 0, tol2, nb, 1);
+            const DotArgs pq{h->d_m_part, h->d_m_sc, 0, tol2, 1}, rr{h->d_m_part, h->d_m_sc, 2, tol2, 1};
+            spmv_multi_h(h, h->d_m_p, h->d_m_q, nb, &pq);
             {
                 PScope ps(h, PK_PCG_VEC, 6.0 * V, 48.0 * V);
-                launch_pcg_update_xr(n, x, h->d_m_r, h->d_m_p, h->d_m_q, h->d_m_sc, h->d_m_part, s, nb, n, 1);
-            }
-            {
-                PScope ps(h, PK_PCG_VEC);
-                launch_dot_finalize(h->d_m_part, h->d_m_sc, 2, tol2, s, nb, 1);
+                launch_pcg_update_xr(n, x, h->d_m_r, h->d_m_p, h->d_m_q, rr, s, nb, n);
             }
             ck(cudaMemcpyAsync(sc.data(), h->d_m_sc, nb * sizeof(PcgScal), cudaMemcpyDeviceToHost, s));
             ck(cudaStreamSynchronize(s));
@@ -3637,8 +3670,7 @@ bool pcg_multi(amdd_handle* h, const double* b, double* x, int nb, double rtol, 
             for (int k = 0; k < nb; ++k)
                 if (!(sc[k].bb == 0.0 || sc[k].conv)) all = false;
             if (all || its == maxit) break;
-            apply_multi(h, h->d_m_r, h->d_m_z, nb);
-            dot_multi_h(h, h->d_m_r, h->d_m_z, 1, tol2, nb, 1);
+            apply_multi(h, h->d_m_r, h->d_m_z, nb, DotArgs{h->d_m_part, h->d_m_sc, 1, tol2, 1});
             PScope ps(h, PK_PCG_VEC, 2.0 * V, 24.0 * V);
             launch_pcg_update_p(n, h->d_m_p, h->d_m_z, h->d_m_sc, s, nb, n, 1);
         }
@@ -3832,7 +3864,7 @@ bool graph_ok(const amdd_handle* h) {
 //       q = A p;  alpha = rz / p.q;  x += alpha p, r -= alpha q;  rr = r.r
 //   }
 // on the handle's vectors (x accumulates in d_px), the condition set on the
-// device after each pass (pcg_loop_cond_kernel), so a whole solve is one
+// device after each pass (pcg_update_xr_kernel), so a whole solve is one
 // graph launch and one synchronisation.  The same kernels in the same order
 // as the per-iteration loop, so the results are the same bits.  Returns false
 // when the runtime cannot capture or instantiate it (the solve then launches
@@ -3880,14 +3912,11 @@ bool pcg_graph(amdd_handle* h, double tol2, int maxit) {
         h->s = h->s_cap;
         s = h->s_cap;
         try {
-            apply_one(h, h->d_r, h->d_z);
-            dot_h(h, h->d_r, h->d_z, 1, tol2);
+            apply_one(h, h->d_r, h->d_z, DotArgs{h->d_part, h->d_sc, 1, tol2, 0});
             launch_pcg_update_p(n, h->d_pv, h->d_z, h->d_sc, s);
-            spmv_h(h, h->d_pv, h->d_q);
-            dot_h(h, h->d_pv, h->d_q, 0, tol2);
-            launch_pcg_update_xr(n, h->d_px, h->d_r, h->d_pv, h->d_q, h->d_sc, h->d_part, s);
-            launch_dot_finalize(h->d_part, h->d_sc, 2, tol2, s);
-            launch_pcg_loop_cond(h->d_sc, h->d_maxit, h->d_alog, h->d_blog, loop, s);
+            spmv_pq_h(h);
+            launch_pcg_update_xr(n, h->d_px, h->d_r, h->d_pv, h->d_q, DotArgs{h->d_part, h->d_sc, 2, tol2, 0}, s, 1, 0,
+                                 h->d_maxit, h->d_alog, h->d_blog, loop);
         } catch (...) {
             launched = false;
         }
@@ -4462,19 +4491,13 @@ amdd_status amdd_pcg_solve(amdd_handle* h, const double* b, double* x, int32_t n
                     ck(cudaStreamSynchronize(s));
                 }
             } else if (!conv) {
-                apply_one(h, h->d_r, h->d_z);
-                dot_h(h, h->d_r, h->d_z, 4, tol2);
+                apply_one(h, h->d_r, h->d_z, DotArgs{h->d_part, h->d_sc, 4, tol2, 0});
                 ck(cudaMemcpyAsync(h->d_pv, h->d_z, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
                 for (its = 1; its <= maxit; ++its) {
-                    spmv_h(h, h->d_pv, h->d_q);
-                    dot_h(h, h->d_pv, h->d_q, 0, tol2);
+                    spmv_pq_h(h);
                     {
                         PScope ps(h, PK_PCG_VEC, 6.0 * n, 48.0 * n);
-                        launch_pcg_update_xr(n, xk, h->d_r, h->d_pv, h->d_q, h->d_sc, h->d_part, s);
-                    }
-                    {
-                        PScope ps(h, PK_PCG_VEC);
-                        launch_dot_finalize(h->d_part, h->d_sc, 2, tol2, s);
+                        launch_pcg_update_xr(n, xk, h->d_r, h->d_pv, h->d_q, DotArgs{h->d_part, h->d_sc, 2, tol2, 0}, s);
                     }
                     ck(cudaMemcpyAsync(&sc, h->d_sc, sizeof(PcgScal), cudaMemcpyDeviceToHost, s));
                     ck(cudaStreamSynchronize(s));
@@ -4487,8 +4510,7 @@ amdd_status amdd_pcg_solve(amdd_handle* h, const double* b, double* x, int32_t n
                         break;
                     }
                     if (its == maxit) break;
-                    apply_one(h, h->d_r, h->d_z);
-                    dot_h(h, h->d_r, h->d_z, 1, tol2);
+                    apply_one(h, h->d_r, h->d_z, DotArgs{h->d_part, h->d_sc, 1, tol2, 0});
                     PScope ps(h, PK_PCG_VEC, 2.0 * n, 24.0 * n);
                     launch_pcg_update_p(n, h->d_pv, h->d_z, h->d_sc, s);
                 }

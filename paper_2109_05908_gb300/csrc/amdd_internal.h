@@ -285,6 +285,26 @@ void launch_convert_blocks(const Ti* const* src, const int* lds, To* const* dst,
                            int nmat, int maxn, cudaStream_t s);
 
 // ---------------------------------------------------------------- sparse / vectors
+struct PcgScal {
+    double rz, pq, rr, bb, alpha, beta;
+    int conv, iters;
+    unsigned ticket;  // CTAs of the running reduction that have finished (0 between kernels)
+    unsigned pad;
+};
+// A dot product computed at the end of a kernel: nb sums into the scalars sc[k].
+// which: 0 -> pq (alpha = rz/pq), 1 -> rz (beta = new rz / old rz), 2 -> rr (conv = rr
+// <= tol2 * bb, iters + 1), 3 -> bb, 4 -> rz (initial), 5 -> rr (conv).  part: nb x CTAs
+// of the kernel partial sums (at most DOT_MAX_BLOCKS each); skip: a right-hand side
+// that has converged keeps its scalars.
+struct DotArgs {
+    double* part = nullptr;
+    PcgScal* sc = nullptr;
+    int which = 0;
+    double tol2 = 0.0;
+    int skip = 0;
+};
+constexpr int DOT_BLOCKS = 264;            // CTAs of the plain vector kernels
+constexpr int DOT_MAX_BLOCKS = 152 * 16;   // CTAs of a kernel with a fused dot product, at most
 // Sparse local Cholesky factors: per subdomain its order n, factor entries
 // nnz, the offset of its column pointers (n + 1 local offsets), of its entries
 // and of its rows in the local vectors.
@@ -322,20 +342,24 @@ void launch_spmv(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* c
                  const double* x, double* y, cudaStream_t s);
 void launch_spmv_resid(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
                        const double* x, const double* b, double* y, cudaStream_t s);
+// y = A x and x.y into the PCG scalars
+void launch_spmv_dot(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                     const double* x, double* y, const DotArgs& d, cudaStream_t s);
 void launch_gather_values(const int64_t* src, const int64_t* dst, int64_t cnt, const double* val, double* out,
                           cudaStream_t s);
 void launch_gather_vec(const int32_t* idx, int64_t cnt, const double* x, double* out, cudaStream_t s);
 void launch_gather_vec_multi(const int32_t* idx, int64_t cnt, const double* x, int64_t ldx, double* out, int nb,
                              cudaStream_t s);
 void launch_spmv_multi(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                       double* y, int nb, int64_t ld, cudaStream_t s);
+                       double* y, int nb, int64_t ld, cudaStream_t s, const DotArgs* d = nullptr);
 template <typename T>
 void launch_gather_rows(const T* src, const int64_t* src_off, T* dst, const int64_t* dst_off, const int32_t* len,
                         int64_t nrows, cudaStream_t s);
 template <typename TY>
 void launch_scatter_prolong(int64_t n, const int32_t* order_g, const int64_t* sc_ptr, const int32_t* sc_idx,
                             const TY* yloc, const double* zc, double* z, cudaStream_t s, int nb = 1, int64_t ldy = 0,
-                            int64_t ldzc = 0, int64_t ldz = 0);
+                            int64_t ldzc = 0, int64_t ldz = 0, const double* r = nullptr,
+                            const DotArgs* d = nullptr);
 // batched rectangular transposes: dst (cols x rows, leading dimension ldd) = src^T
 struct TransDesc {
     const double* src;
@@ -354,9 +378,6 @@ void launch_e_offdiag(const EPairRef* tiles, int ntiles, const int32_t* la, cons
                       const int64_t* az_off, const int32_t* p, const int64_t* coff, double* E, int64_t ldE,
                       cudaStream_t s);
 
-// Deterministic dot products: fixed grid of DOT_BLOCKS partial sums reduced in
-// a fixed order by one block.
-constexpr int DOT_BLOCKS = 264;
 // ---------------------------------------------------------------------------
 // Learned warm start of the local eigensolve and block LOBPCG
 // ---------------------------------------------------------------------------
@@ -504,30 +525,21 @@ template <typename T>
 void launch_front_solve(const FrontSolveT<T>& a, const double* c, int64_t ldc, T* out, int64_t ldo, int nb,
                         cudaStream_t s);
 
-struct PcgScal {
-    double rz, pq, rr, bb, alpha, beta, rz_new;
-    int conv, iters;
-};
-// Vector operations of PCG on nb right-hand sides stored ld apart (scalars sc[k],
-// partial sums DOT_BLOCKS apart); with skip_done a converged right-hand side
-// (sc[k].conv) keeps x, r, p and its scalars.
+// Vector operations of PCG on nb right-hand sides stored ld apart; with d.skip (or
+// skip_done) a converged right-hand side (sc[k].conv) keeps x, r, p and its scalars.
 void launch_dot_partials(int64_t n, const double* x, const double* y, double* partials, cudaStream_t s, int nb = 1,
                          int64_t ld = 0);
-// which: 0 -> pq (alpha = rz/pq), 1 -> rz_new (beta = rz_new/rz, rz = rz_new),
-// 2 -> rr (conv = rr <= tol2 * bb), 3 -> bb, 4 -> rz (initial)
-void launch_dot_finalize(const double* partials, PcgScal* sc, int which, double tol2, cudaStream_t s, int nb = 1,
-                         int skip_done = 0);
-void launch_pcg_update_xr(int64_t n, double* x, double* r, const double* p, const double* q, const PcgScal* sc,
-                          double* partials, cudaStream_t s, int nb = 1, int64_t ld = 0, int skip_done = 0);
+void launch_dot(int64_t n, const double* x, const double* y, const DotArgs& d, cudaStream_t s, int nb = 1,
+                int64_t ld = 0);
+// x += alpha p, r -= alpha q, r.r (d); inside a graph's while-loop (maxit given) also
+// alog[k-1] = alpha, blog[k-2] = beta (k = iterations done, entries below *maxit only)
+// and the loop's condition !conv && k < *maxit
+void launch_pcg_update_xr(int64_t n, double* x, double* r, const double* p, const double* q, const DotArgs& d,
+                          cudaStream_t s, int nb = 1, int64_t ld = 0, const int* maxit = nullptr,
+                          double* alog = nullptr, double* blog = nullptr, cudaGraphConditionalHandle loop = 0);
 void launch_pcg_update_p(int64_t n, double* p, const double* z, const PcgScal* sc, cudaStream_t s, int nb = 1,
                          int64_t ld = 0, int skip_done = 0);
 void launch_axpby(int64_t n, double a, const double* x, double b, const double* y, double* out, cudaStream_t s);
-// One thread: alog[k-1] = sc->alpha, blog[k-2] = sc->beta (k = sc->iters, entries
-// below *maxit only), then the while-loop condition of the graph that replays
-// PCG iterations: !sc->conv && k < *maxit.
-void launch_pcg_loop_cond(const PcgScal* sc, const int* maxit, double* alog, double* blog,
-                          cudaGraphConditionalHandle loop, cudaStream_t s);
-
 // ---------------------------------------------------------------------------
 // Deflated / restricted additive Schwarz forms and GMRES(m) (Sec. 4.1)
 // ---------------------------------------------------------------------------

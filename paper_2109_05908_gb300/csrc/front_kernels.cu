@@ -241,9 +241,10 @@ namespace {
 
 // Lanes per row: 4 while that fills the chip (FP64 runs at two multiply-adds per
 // clock and SM, idle lanes or not, so the shuffle tree is best shared by 8 rows),
-// a warp when the rows of the stage are few.
-int lanes_for(int64_t rows) {
-    const int64_t fill = 152 * 448;
+// a warp when the rows of the stage are few.  With several vectors each load feeds
+// eight independent sums, so fewer threads fill it.
+int lanes_for(int64_t rows, int nb) {
+    const int64_t fill = 152 * (nb == 1 ? 448 : 128);
     return rows * 4 >= fill ? 4 : (rows * 8 >= fill ? 8 : 32);
 }
 
@@ -265,7 +266,7 @@ void solve_nb(const FrontSolveT<T>& a, T* out, int64_t ldo, int nb, cudaStream_t
     for (int st = 0; st + 1 < a.stages; ++st) {
         const int64_t nrow = a.down_off[st + 1] - a.down_off[st];
         if (nrow <= 0) continue;
-        const int g = lanes_for(nrow);
+        const int g = lanes_for(nrow, nb);
         if (g == 4)
             stage_down<T, NB, 4>(a, st, nb, s);
         else if (g == 8)
@@ -275,7 +276,7 @@ void solve_nb(const FrontSolveT<T>& a, T* out, int64_t ldo, int nb, cudaStream_t
     }
     for (int st = a.stages - 1; st >= 0; --st) {
         if (a.row_off[st + 1] <= a.row_off[st]) continue;
-        const int g = lanes_for(a.row_off[st + 1] - a.row_off[st]);
+        const int g = lanes_for(a.row_off[st + 1] - a.row_off[st], nb);
         if (g == 4)
             stage_up<T, NB, 4>(a, st, out, ldo, nb, s);
         else if (g == 8)

@@ -63,10 +63,8 @@ extern "C" amdd_status amdd_true_residual_noalloc(const amdd_csr* A, const doubl
     if (cudaMemsetAsync(sc, 0, sizeof(PcgScal), s) != cudaSuccess) return AMDD_ERR_CUDA;
     launch_spmv(n, A->nnz, A->rowptr, A->colind, A->val, x, q, s);
     launch_axpby(n, 1.0, b, -1.0, q, r, s);
-    launch_dot_partials(n, b, b, partials, s);
-    launch_dot_finalize(partials, sc, 3, 0.0, s);
-    launch_dot_partials(n, r, r, partials, s);
-    launch_dot_finalize(partials, sc, 5, 0.0, s);
+    launch_dot(n, b, b, DotArgs{partials, sc, 3, 0.0, 0}, s);
+    launch_dot(n, r, r, DotArgs{partials, sc, 5, 0.0, 0}, s);
     PcgScal h{};
     if (cudaMemcpyAsync(&h, sc, sizeof(PcgScal), cudaMemcpyDeviceToHost, s) != cudaSuccess) return AMDD_ERR_CUDA;
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return AMDD_ERR_CUDA;

@@ -6,8 +6,97 @@
 
 namespace amdd {
 
+// ------------------------------------------------------------------ reductions
+// Every reduction has a fixed grid for a given n, fixed per-thread strides and
+// fixed trees: the result is bitwise reproducible.
+__device__ __forceinline__ double block_sum_256(double v) {
+    __shared__ double red[256];
+    red[threadIdx.x] = v;
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+        __syncthreads();
+    }
+    const double r = red[0];
+    __syncthreads();
+    return r;
+}
+
+// what a finished sum v does to the scalars of one right-hand side
+__device__ __forceinline__ void dot_finish(PcgScal* sc, int which, double v, double tol2) {
+    switch (which) {
+        case 0:
+            sc->pq = v;
+            sc->alpha = sc->rz / v;
+            break;
+        case 1:
+            sc->beta = v / sc->rz;
+            sc->rz = v;
+            break;
+        case 2:
+            sc->rr = v;
+            sc->iters += 1;
+            sc->conv = (v <= tol2 * sc->bb) ? 1 : 0;
+            break;
+        case 3:
+            sc->bb = v;
+            break;
+        case 4:
+            sc->rz = v;
+            break;
+        default:
+            sc->rr = v;
+            sc->conv = (v <= tol2 * sc->bb) ? 1 : 0;
+            break;
+    }
+}
+
+// The end of a kernel of 256 threads per CTA whose threads hold their parts s[k]
+// of nb sums: CTA sums to d.part, and the CTA that finishes last adds them up in
+// order (a warp per sum) and updates the scalars, so a dot product needs no second
+// launch.  The ticket returns to zero by itself.  True in the last CTA, after its
+// warps' updates.
+template <int NB>
+__device__ __forceinline__ bool dot_tail(double (&s)[NB], int nb, const DotArgs& d) {
+    __shared__ double red[8][NB];
+    __shared__ int last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        double v = s[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[warp][k] = v;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < nb) {
+        double v = red[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) v += red[w][threadIdx.x];
+        d.part[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = v;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(&d.sc->ticket, gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return false;
+    if (warp < nb) {
+        double v = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32) v += __ldcg(d.part + (int64_t)warp * gridDim.x + b);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && !(d.skip && d.sc[warp].conv)) dot_finish(d.sc + warp, d.which, v, d.tol2);
+    }
+    __syncthreads();
+    return true;
+}
+
 // ------------------------------------------------------------------ SpMV
-// y = A x, or y = b - A x (RESID): G lanes per row, rows assigned to lane groups
+// y = A x (MODE 0), y = b - A x (1), or y = A x with x.y into the PCG scalars (2):
+// G lanes per row, rows assigned to lane groups
 // in a grid-stride loop, four entries in flight per lane.  Rows of a few entries
 // take one thread each: a warp then covers 32 consecutive rows, bound by HBM
 // (5-point matrix of 2.1 M rows: 5.4 TB/s).  For longer rows FP64 sets the rate,
@@ -15,23 +104,18 @@ namespace amdd {
 // per row of 72 entries spends more on the shuffle tree than on the row, while
 // with 4 lanes the tree is shared by 8 rows.  27-point matrix with 3 unknowns per
 // node, 98 k rows, call included: 88 -> 47 us.
-template <bool RESID>
-__device__ __forceinline__ void spmv_store(int64_t row, double s, const double* __restrict__ b,
-                                           double* __restrict__ y) {
-    y[row] = RESID ? b[row] - s : s;
-}
-
-template <int G, bool RESID>
+template <int G, int MODE>
 __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ col, const double* __restrict__ val,
                                                    const double* __restrict__ x, const double* __restrict__ b,
-                                                   double* __restrict__ y) {
+                                                   double* __restrict__ y, DotArgs d) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int sub = threadIdx.x & (G - 1);
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
     // every lane of the grid runs the same number of iterations, so the full
     // warp takes part in each shuffle
     const int64_t nround = ((n + groups - 1) / groups) * groups;
+    double dot[1] = {0.0};
     for (int64_t row = gid / G; row < nround; row += groups) {
         double s = 0.0;
         if (row < n) {
@@ -51,8 +135,12 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __r
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (row < n && sub == 0) spmv_store<RESID>(row, s, b, y);
+        if (row < n && sub == 0) {
+            y[row] = MODE == 1 ? b[row] - s : s;
+            if (MODE == 2) dot[0] = fma(x[row], s, dot[0]);
+        }
     }
+    if (MODE == 2) dot_tail<1>(dot, 1, d);
 }
 
 // Lanes per row by the average row length, the fastest of 1, 2, 4, 8, 16, 32 at
@@ -64,39 +152,50 @@ static int spmv_lanes(int64_t n, int64_t nnz) {
     return per <= 9 ? 1 : (per <= 24 ? 2 : (per <= 250 ? 4 : 16));
 }
 
-template <bool RESID>
+template <int MODE>
 static void spmv_any(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
-                     const double* x, const double* b, double* y, cudaStream_t s) {
+                     const double* x, const double* b, double* y, const DotArgs& d, cudaStream_t s) {
     if (n <= 0) return;
     const int group = spmv_lanes(n, nnz);
     const int64_t want = (n * group + 255) / 256;
-    const int blocks = (int)(want < 152 * 64 ? want : 152 * 64);
+    const int most = MODE == 2 ? DOT_MAX_BLOCKS : 152 * 64;
+    const int blocks = (int)(want < most ? want : most);
     if (group == 1)
-        spmv_kernel<1, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+        spmv_kernel<1, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
     else if (group == 2)
-        spmv_kernel<2, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+        spmv_kernel<2, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
     else if (group == 4)
-        spmv_kernel<4, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+        spmv_kernel<4, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
     else
-        spmv_kernel<16, RESID><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y);
+        spmv_kernel<16, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
 }
 
 void launch_spmv(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
                  const double* x, double* y, cudaStream_t s) {
-    spmv_any<false>(n, nnz, rowptr, col, val, x, nullptr, y, s);
+    spmv_any<0>(n, nnz, rowptr, col, val, x, nullptr, y, DotArgs{}, s);
 }
 
 void launch_spmv_resid(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
                        const double* x, const double* b, double* y, cudaStream_t s) {
-    spmv_any<true>(n, nnz, rowptr, col, val, x, b, y, s);
+    spmv_any<1>(n, nnz, rowptr, col, val, x, b, y, DotArgs{}, s);
+}
+
+void launch_spmv_dot(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
+                     const double* x, double* y, const DotArgs& d, cudaStream_t s) {
+    spmv_any<2>(n, nnz, rowptr, col, val, x, nullptr, y, d, s);
 }
 
 // y_k = A x_k for nb <= MAXB right-hand sides stored ld apart: one thread per
-// row reads the row's entries once and applies them to every x_k.
+// row reads the row's entries once and applies them to every x_k; with DOT also
+// x_k.y_k into the PCG scalars.
+template <bool DOT>
 __global__ void __launch_bounds__(256) spmv_multi_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                          const int32_t* __restrict__ col,
                                                          const double* __restrict__ val, const double* __restrict__ x,
-                                                         double* __restrict__ y, int nb, int64_t ld) {
+                                                         double* __restrict__ y, int nb, int64_t ld, DotArgs d) {
+    double dot[MAXB];
+#pragma unroll
+    for (int k = 0; k < MAXB; ++k) dot[k] = 0.0;
     for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
          row += (int64_t)gridDim.x * blockDim.x) {
         double acc[MAXB];
@@ -111,15 +210,24 @@ __global__ void __launch_bounds__(256) spmv_multi_kernel(int64_t n, const int64_
         }
 #pragma unroll
         for (int k = 0; k < MAXB; ++k)
-            if (k < nb) y[k * ld + row] = acc[k];
+            if (k < nb) {
+                y[k * ld + row] = acc[k];
+                if (DOT) dot[k] = fma(x[k * ld + row], acc[k], dot[k]);
+            }
     }
+    if (DOT) dot_tail<MAXB>(dot, nb, d);
 }
 
 void launch_spmv_multi(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
-                       double* y, int nb, int64_t ld, cudaStream_t s) {
+                       double* y, int nb, int64_t ld, cudaStream_t s, const DotArgs* d) {
     if (n <= 0) return;
     const int64_t want = (n + 255) / 256;
-    spmv_multi_kernel<<<(unsigned)(want < 152 * 64 ? want : 152 * 64), 256, 0, s>>>(n, rowptr, col, val, x, y, nb, ld);
+    if (d)
+        spmv_multi_kernel<true><<<(unsigned)(want < DOT_MAX_BLOCKS ? want : DOT_MAX_BLOCKS), 256, 0, s>>>(
+            n, rowptr, col, val, x, y, nb, ld, *d);
+    else
+        spmv_multi_kernel<false><<<(unsigned)(want < 152 * 64 ? want : 152 * 64), 256, 0, s>>>(n, rowptr, col, val, x, y,
+                                                                                              nb, ld, DotArgs{});
 }
 
 // ------------------------------------------------------------------ sparse local factors
@@ -330,35 +438,58 @@ template void launch_gather_rows<double>(const double*, const int64_t*, double*,
 //                 a = position of g in Omega_Ii, t = off_I[i] + a: thread t
 //                 runs in that owner order).  nb right-hand sides: yloc, zc
 //                 and z hold nb vectors ldy, ldzc and ldz apart.
-template <typename TY>
+// With DOT also r_k.z_k into the PCG scalars (r: nb vectors ldz apart).
+template <typename TY, int NB, bool DOT>
 __global__ void __launch_bounds__(256) scatter_prolong_kernel(
     int64_t n, const int32_t* __restrict__ order_g, const int64_t* __restrict__ sc_ptr,
     const int32_t* __restrict__ sc_idx, const TY* __restrict__ yloc, const double* __restrict__ zc,
-    double* __restrict__ z, int nb, int64_t ldy, int64_t ldzc, int64_t ldz) {
+    double* __restrict__ z, int nb, int64_t ldy, int64_t ldzc, int64_t ldz, const double* __restrict__ r, DotArgs d) {
+    double dot[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) dot[k] = 0.0;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const int g = order_g[t];
-        for (int r = 0; r < nb; ++r) {
+        const int64_t k0 = sc_ptr[g], k1 = sc_ptr[g + 1];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            if (NB > 1 && q >= nb) break;
             double s = 0.0;
-            for (int64_t k = sc_ptr[g]; k < sc_ptr[g + 1]; ++k) s += (double)yloc[r * ldy + sc_idx[k]];
-            if (zc) s += zc[r * ldzc + t];
-            z[r * ldz + g] = s;
+            for (int64_t k = k0; k < k1; ++k) s += (double)yloc[q * ldy + sc_idx[k]];
+            if (zc) s += zc[q * ldzc + t];
+            z[q * ldz + g] = s;
+            if (DOT) dot[q] = fma(r[q * ldz + g], s, dot[q]);
         }
     }
+    if (DOT) dot_tail<NB>(dot, nb, d);
 }
 
 template <typename TY>
 void launch_scatter_prolong(int64_t n, const int32_t* order_g, const int64_t* sc_ptr, const int32_t* sc_idx,
                             const TY* yloc, const double* zc, double* z, cudaStream_t s, int nb, int64_t ldy,
-                            int64_t ldzc, int64_t ldz) {
+                            int64_t ldzc, int64_t ldz, const double* r, const DotArgs* d) {
     if (n <= 0) return;
     const int64_t want = (n + 255) / 256;
-    scatter_prolong_kernel<TY><<<(unsigned)(want < 152 * 32 ? want : 152 * 32), 256, 0, s>>>(
-        n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy, ldzc, ldz);
+    const unsigned g = (unsigned)(want < DOT_MAX_BLOCKS ? want : DOT_MAX_BLOCKS);
+    const DotArgs da = d ? *d : DotArgs{};
+    if (nb == 1 && d)
+        scatter_prolong_kernel<TY, 1, true><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, 1, ldy, ldzc, ldz, r,
+                                                              da);
+    else if (nb == 1)
+        scatter_prolong_kernel<TY, 1, false><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, 1, ldy, ldzc, ldz,
+                                                               r, da);
+    else if (d)
+        scatter_prolong_kernel<TY, MAXB, true><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy, ldzc,
+                                                                 ldz, r, da);
+    else
+        scatter_prolong_kernel<TY, MAXB, false><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy, ldzc,
+                                                                  ldz, r, da);
 }
 template void launch_scatter_prolong<float>(int64_t, const int32_t*, const int64_t*, const int32_t*, const float*,
-                                            const double*, double*, cudaStream_t, int, int64_t, int64_t, int64_t);
+                                            const double*, double*, cudaStream_t, int, int64_t, int64_t, int64_t,
+                                            const double*, const DotArgs*);
 template void launch_scatter_prolong<double>(int64_t, const int32_t*, const int64_t*, const int32_t*, const double*,
-                                             const double*, double*, cudaStream_t, int, int64_t, int64_t, int64_t);
+                                             const double*, double*, cudaStream_t, int, int64_t, int64_t, int64_t,
+                                             const double*, const DotArgs*);
 
 // ------------------------------------------------------------------ coarse blocks
 // E[coff_i + r][coff_j + c] = sum_l Zt_i[r][la[l]] * AZ_j[lpos[l]][c], 32 x 32
@@ -407,22 +538,8 @@ void launch_e_offdiag(const EPairRef* tiles, int ntiles, const int32_t* la, cons
         e_offdiag_kernel<<<ntiles, 256, 0, s>>>(tiles, la, lpos, Zt, zt_off, nI, AZ, az_off, p, coff, E, ldE);
 }
 
-// ------------------------------------------------------------------ reductions
-// Fixed grid (DOT_BLOCKS x 256) and fixed per-thread strides, then a fixed
-// tree in shared memory: the result is bitwise reproducible for a given n.
-__device__ __forceinline__ double block_sum_256(double v) {
-    __shared__ double red[256];
-    red[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
-    const double r = red[0];
-    __syncthreads();
-    return r;
-}
-
+// ------------------------------------------------------------------ vectors of PCG
+// x.y for blockIdx.y = right-hand side: partial sums only
 __global__ void __launch_bounds__(256) dot_partials_kernel(int64_t n, const double* __restrict__ x,
                                                             const double* __restrict__ y,
                                                             double* __restrict__ partials, int64_t ld) {
@@ -441,78 +558,64 @@ void launch_dot_partials(int64_t n, const double* x, const double* y, double* pa
     dot_partials_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, y, partials, ld);
 }
 
-__global__ void __launch_bounds__(256) dot_finalize_kernel(const double* __restrict__ partials, PcgScal* sc,
-                                                            int which, double tol2, int skip_done) {
-    partials += (int64_t)blockIdx.x * DOT_BLOCKS;
-    sc += blockIdx.x;
-    if (skip_done && sc->conv) return;  // a converged right-hand side keeps its state
-    double v = 0.0;
-    for (int i = threadIdx.x; i < DOT_BLOCKS; i += 256) v += partials[i];
-    v = block_sum_256(v);
-    if (threadIdx.x == 0) {
-        switch (which) {
-            case 0:
-                sc->pq = v;
-                sc->alpha = sc->rz / v;
-                break;
-            case 1:
-                sc->rz_new = v;
-                sc->beta = v / sc->rz;
-                sc->rz = v;
-                break;
-            case 2:
-                sc->rr = v;
-                sc->iters += 1;
-                sc->conv = (v <= tol2 * sc->bb) ? 1 : 0;
-                break;
-            case 3:
-                sc->bb = v;
-                break;
-            case 4:
-                sc->rz = v;
-                break;
-            default:
-                sc->rr = v;
-                sc->conv = (v <= tol2 * sc->bb) ? 1 : 0;
-                break;
-        }
-    }
+// x_k.y_k into the scalars (blockIdx.y = right-hand side)
+__global__ void __launch_bounds__(256) dot_kernel(int64_t n, const double* __restrict__ x,
+                                                  const double* __restrict__ y, int64_t ld, DotArgs d) {
+    const int k = blockIdx.y;
+    x += (int64_t)k * ld;
+    y += (int64_t)k * ld;
+    double s[1] = {0.0};
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
+        s[0] = fma(x[i], y[i], s[0]);
+    d.part += (int64_t)k * gridDim.x;
+    d.sc += k;
+    dot_tail<1>(s, 1, d);
 }
 
-void launch_dot_finalize(const double* partials, PcgScal* sc, int which, double tol2, cudaStream_t s, int nb,
-                         int skip_done) {
-    dot_finalize_kernel<<<nb, 256, 0, s>>>(partials, sc, which, tol2, skip_done);
+void launch_dot(int64_t n, const double* x, const double* y, const DotArgs& d, cudaStream_t s, int nb, int64_t ld) {
+    dot_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, y, ld, d);
 }
 
-// x += alpha p; r -= alpha q; partial sums of r.r
+// x += alpha p; r -= alpha q; r.r into the scalars.  With a loop handle (the
+// iterations replayed inside a CUDA graph's while-loop) the last CTA also logs the
+// step length alpha of the iteration just finished (and the ratio beta that built
+// its direction, from the second iteration on) for the Lanczos condition estimate,
+// and continues the loop while the recursive residual is above the tolerance and
+// fewer than *maxit iterations have run.
 __global__ void __launch_bounds__(256) pcg_update_xr_kernel(int64_t n, double* __restrict__ x,
                                                              double* __restrict__ r, const double* __restrict__ p,
-                                                             const double* __restrict__ q,
-                                                             const PcgScal* __restrict__ sc,
-                                                             double* __restrict__ partials, int64_t ld,
-                                                             int skip_done) {
+                                                             const double* __restrict__ q, int64_t ld, DotArgs d,
+                                                             const int* __restrict__ maxit, double* __restrict__ alog,
+                                                             double* __restrict__ blog,
+                                                             cudaGraphConditionalHandle loop) {
     const int k = blockIdx.y;
-    if (skip_done && sc[k].conv) return;
+    d.sc += k;
+    if (d.skip && d.sc->conv) return;
     x += (int64_t)k * ld;
     r += (int64_t)k * ld;
     p += (int64_t)k * ld;
     q += (int64_t)k * ld;
-    partials += (int64_t)k * DOT_BLOCKS;
-    const double a = sc[k].alpha;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)DOT_BLOCKS * 256) {
+    d.part += (int64_t)k * gridDim.x;
+    const double a = d.sc->alpha;
+    double s[1] = {0.0};
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         x[i] = fma(a, p[i], x[i]);
         const double ri = fma(-a, q[i], r[i]);
         r[i] = ri;
-        s = fma(ri, ri, s);
+        s[0] = fma(ri, ri, s[0]);
     }
-    s = block_sum_256(s);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    if (dot_tail<1>(s, 1, d) && maxit && threadIdx.x == 0) {
+        const int it = d.sc->iters;
+        if (it >= 1 && it <= *maxit) alog[it - 1] = d.sc->alpha;
+        if (it >= 2 && it <= *maxit) blog[it - 2] = d.sc->beta;
+        cudaGraphSetConditional(loop, (!d.sc->conv && it < *maxit) ? 1u : 0u);
+    }
 }
 
-void launch_pcg_update_xr(int64_t n, double* x, double* r, const double* p, const double* q, const PcgScal* sc,
-                          double* partials, cudaStream_t s, int nb, int64_t ld, int skip_done) {
-    pcg_update_xr_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, r, p, q, sc, partials, ld, skip_done);
+void launch_pcg_update_xr(int64_t n, double* x, double* r, const double* p, const double* q, const DotArgs& d,
+                          cudaStream_t s, int nb, int64_t ld, const int* maxit, double* alog, double* blog,
+                          cudaGraphConditionalHandle loop) {
+    pcg_update_xr_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, r, p, q, ld, d, maxit, alog, blog, loop);
 }
 
 // p = z + beta p
@@ -530,26 +633,6 @@ __global__ void pcg_update_p_kernel(int64_t n, double* __restrict__ p, const dou
 void launch_pcg_update_p(int64_t n, double* p, const double* z, const PcgScal* sc, cudaStream_t s, int nb,
                          int64_t ld, int skip_done) {
     pcg_update_p_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, p, z, sc, ld, skip_done);
-}
-
-// End of one PCG iteration replayed inside a CUDA graph's while-loop: log the
-// step length alpha of the iteration just finished (and the ratio beta that
-// built its direction, from the second iteration on) for the Lanczos
-// condition estimate, and continue the loop while the recursive residual is
-// above the tolerance and fewer than *maxit iterations have run.
-__global__ void pcg_loop_cond_kernel(const PcgScal* __restrict__ sc, const int* __restrict__ maxit,
-                                     double* __restrict__ alog, double* __restrict__ blog,
-                                     cudaGraphConditionalHandle loop) {
-    if (threadIdx.x != 0) return;
-    const int k = sc->iters;
-    if (k >= 1 && k <= *maxit) alog[k - 1] = sc->alpha;
-    if (k >= 2 && k <= *maxit) blog[k - 2] = sc->beta;
-    cudaGraphSetConditional(loop, (!sc->conv && k < *maxit) ? 1u : 0u);
-}
-
-void launch_pcg_loop_cond(const PcgScal* sc, const int* maxit, double* alog, double* blog,
-                          cudaGraphConditionalHandle loop, cudaStream_t s) {
-    pcg_loop_cond_kernel<<<1, 32, 0, s>>>(sc, maxit, alog, blog, loop);
 }
 
 // out = a x + b y
