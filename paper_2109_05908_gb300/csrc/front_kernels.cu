@@ -172,10 +172,13 @@ __global__ void __launch_bounds__(256) front_load_kernel(int64_t n, const int32_
     }
 }
 
+// Small CTAs: the rows of a stage are few, and their work should reach every SM.
+constexpr int FRONT_THREADS = 64;
+
 // Down: G lanes per boundary unknown t of a stage, over the parts next to it
 // (refs[ptr[t] .. ptr[t + 1]): a row of W^T and the part's interior).
 template <typename T, int NB, int G>
-__global__ void __launch_bounds__(256) front_down_kernel(int64_t nrow, const int32_t* __restrict__ rows,
+__global__ void __launch_bounds__(FRONT_THREADS) front_down_kernel(int64_t nrow, const int32_t* __restrict__ rows,
                                                          const int32_t* __restrict__ ptr,
                                                          const FrontRefT<T>* __restrict__ refs, T* v, int64_t n,
                                                          int nb) {
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(256) front_down_kernel(int64_t nrow, const int
 // Up: G lanes per interior row of a stage; e in plan order (read by the earlier
 // stages) and, when out is given, through perm (times scale) in the caller's order.
 template <typename T, int NB, int G>
-__global__ void __launch_bounds__(256) front_up_kernel(const FrontDevT<T>* __restrict__ fr,
+__global__ void __launch_bounds__(FRONT_THREADS) front_up_kernel(const FrontDevT<T>* __restrict__ fr,
                                                        const int32_t* __restrict__ row_front, int64_t r0, int64_t r1,
                                                        const int32_t* __restrict__ bnd,
                                                        const int32_t* __restrict__ perm,
@@ -251,13 +254,13 @@ int lanes_for(int64_t rows, int nb) {
 template <typename T, int NB, int G>
 void stage_down(const FrontSolveT<T>& a, int st, int nb, cudaStream_t s) {
     const int64_t nrow = a.down_off[st + 1] - a.down_off[st];
-    front_down_kernel<T, NB, G><<<(unsigned)((nrow * G + 255) / 256), 256, 0, s>>>(
+    front_down_kernel<T, NB, G><<<(unsigned)((nrow * G + FRONT_THREADS - 1) / FRONT_THREADS), FRONT_THREADS, 0, s>>>(
         nrow, a.down_rows + a.down_off[st], a.down_ptr + a.down_off[st], a.refs, a.v, a.n, nb);
 }
 template <typename T, int NB, int G>
 void stage_up(const FrontSolveT<T>& a, int st, T* out, int64_t ldo, int nb, cudaStream_t s) {
     const int64_t r0 = a.row_off[st], r1 = a.row_off[st + 1];
-    front_up_kernel<T, NB, G><<<(unsigned)(((r1 - r0) * G + 255) / 256), 256, 0, s>>>(
+    front_up_kernel<T, NB, G><<<(unsigned)(((r1 - r0) * G + FRONT_THREADS - 1) / FRONT_THREADS), FRONT_THREADS, 0, s>>>(
         a.fr, a.row_front, r0, r1, a.bnd, a.perm, a.scale, a.v, a.e, out, a.n, ldo, nb);
 }
 

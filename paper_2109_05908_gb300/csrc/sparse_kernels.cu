@@ -185,49 +185,77 @@ void launch_spmv_dot(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_
     spmv_any<2>(n, nnz, rowptr, col, val, x, nullptr, y, d, s);
 }
 
-// y_k = A x_k for nb <= MAXB right-hand sides stored ld apart: one thread per
-// row reads the row's entries once and applies them to every x_k; with DOT also
-// x_k.y_k into the PCG scalars.
-template <bool DOT>
+// y_k = A x_k for nb <= MAXB right-hand sides stored ld apart, with DOT also
+// x_k.y_k into the PCG scalars.  ROWS = 256: one thread per row reads the row's
+// entries once and applies them to every x_k.  ROWS = 32: warp k of a CTA takes x_k,
+// over the CTA's 32 rows (the eight warps share the entries through L1); eight times
+// the CTAs, for matrices too small to fill the chip otherwise (n = 8000, eight
+// vectors: 22 -> 17 us).
+template <int ROWS, bool DOT>
 __global__ void __launch_bounds__(256) spmv_multi_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                          const int32_t* __restrict__ col,
                                                          const double* __restrict__ val, const double* __restrict__ x,
                                                          double* __restrict__ y, int nb, int64_t ld, DotArgs d) {
+    static_assert(MAXB == 8, "a warp per right-hand side");
     double dot[MAXB];
 #pragma unroll
     for (int k = 0; k < MAXB; ++k) dot[k] = 0.0;
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
-         row += (int64_t)gridDim.x * blockDim.x) {
-        double acc[MAXB];
-#pragma unroll
-        for (int k = 0; k < MAXB; ++k) acc[k] = 0.0;
-        for (int64_t e = rowptr[row]; e < rowptr[row + 1]; ++e) {
-            const double v = __ldg(val + e);
-            const int64_t c = __ldg(col + e);
-#pragma unroll
-            for (int k = 0; k < MAXB; ++k)
-                if (k < nb) acc[k] = fma(v, __ldg(x + k * ld + c), acc[k]);
+    if (ROWS == 32) {
+        const int k = threadIdx.x >> 5;
+        double s = 0.0;
+        for (int64_t row = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31); row < n && k < nb;
+             row += (int64_t)gridDim.x * 32) {
+            double acc = 0.0;
+            for (int64_t e = rowptr[row]; e < rowptr[row + 1]; ++e)
+                acc = fma(__ldg(val + e), __ldg(x + k * ld + __ldg(col + e)), acc);
+            y[k * ld + row] = acc;
+            if (DOT) s = fma(x[k * ld + row], acc, s);
         }
 #pragma unroll
-        for (int k = 0; k < MAXB; ++k)
-            if (k < nb) {
-                y[k * ld + row] = acc[k];
-                if (DOT) dot[k] = fma(x[k * ld + row], acc[k], dot[k]);
+        for (int q = 0; q < MAXB; ++q) dot[q] = q == k ? s : 0.0;
+    } else {
+        for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
+             row += (int64_t)gridDim.x * blockDim.x) {
+            double acc[MAXB];
+#pragma unroll
+            for (int k = 0; k < MAXB; ++k) acc[k] = 0.0;
+            for (int64_t e = rowptr[row]; e < rowptr[row + 1]; ++e) {
+                const double v = __ldg(val + e);
+                const int64_t c = __ldg(col + e);
+#pragma unroll
+                for (int k = 0; k < MAXB; ++k)
+                    if (k < nb) acc[k] = fma(v, __ldg(x + k * ld + c), acc[k]);
             }
+#pragma unroll
+            for (int k = 0; k < MAXB; ++k)
+                if (k < nb) {
+                    y[k * ld + row] = acc[k];
+                    if (DOT) dot[k] = fma(x[k * ld + row], acc[k], dot[k]);
+                }
+        }
     }
     if (DOT) dot_tail<MAXB>(dot, nb, d);
 }
 
+// Up to this many rows the kernels for several right-hand sides give each its own warp.
+constexpr int64_t MULTI_SMALL = 152 * 512;
+
 void launch_spmv_multi(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val, const double* x,
                        double* y, int nb, int64_t ld, cudaStream_t s, const DotArgs* d) {
     if (n <= 0) return;
-    const int64_t want = (n + 255) / 256;
-    if (d)
-        spmv_multi_kernel<true><<<(unsigned)(want < DOT_MAX_BLOCKS ? want : DOT_MAX_BLOCKS), 256, 0, s>>>(
-            n, rowptr, col, val, x, y, nb, ld, *d);
+    const bool small = n <= MULTI_SMALL;
+    const int64_t want = small ? (n + 31) / 32 : (n + 255) / 256;
+    const int64_t most = d ? DOT_MAX_BLOCKS : 152 * 64;
+    const unsigned g = (unsigned)(want < most ? want : most);
+    const DotArgs da = d ? *d : DotArgs{};
+    if (small && d)
+        spmv_multi_kernel<32, true><<<g, 256, 0, s>>>(n, rowptr, col, val, x, y, nb, ld, da);
+    else if (small)
+        spmv_multi_kernel<32, false><<<g, 256, 0, s>>>(n, rowptr, col, val, x, y, nb, ld, da);
+    else if (d)
+        spmv_multi_kernel<256, true><<<g, 256, 0, s>>>(n, rowptr, col, val, x, y, nb, ld, da);
     else
-        spmv_multi_kernel<false><<<(unsigned)(want < 152 * 64 ? want : 152 * 64), 256, 0, s>>>(n, rowptr, col, val, x, y,
-                                                                                              nb, ld, DotArgs{});
+        spmv_multi_kernel<256, false><<<g, 256, 0, s>>>(n, rowptr, col, val, x, y, nb, ld, da);
 }
 
 // ------------------------------------------------------------------ sparse local factors
@@ -444,23 +472,26 @@ __global__ void __launch_bounds__(256) scatter_prolong_kernel(
     int64_t n, const int32_t* __restrict__ order_g, const int64_t* __restrict__ sc_ptr,
     const int32_t* __restrict__ sc_idx, const TY* __restrict__ yloc, const double* __restrict__ zc,
     double* __restrict__ z, int nb, int64_t ldy, int64_t ldzc, int64_t ldz, const double* __restrict__ r, DotArgs d) {
-    double dot[NB];
-#pragma unroll
-    for (int k = 0; k < NB; ++k) dot[k] = 0.0;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    // one thread per unknown; with several right-hand sides warp q of the CTA takes
+    // the q-th, over the CTA's 32 unknowns
+    constexpr int PER = NB > 1 ? 32 : 256;
+    const int q = NB > 1 ? threadIdx.x >> 5 : 0;
+    double dsum = 0.0;
+    for (int64_t t = (int64_t)blockIdx.x * PER + (threadIdx.x & (PER - 1)); t < n && q < nb;
+         t += (int64_t)gridDim.x * PER) {
         const int g = order_g[t];
-        const int64_t k0 = sc_ptr[g], k1 = sc_ptr[g + 1];
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            if (NB > 1 && q >= nb) break;
-            double s = 0.0;
-            for (int64_t k = k0; k < k1; ++k) s += (double)yloc[q * ldy + sc_idx[k]];
-            if (zc) s += zc[q * ldzc + t];
-            z[q * ldz + g] = s;
-            if (DOT) dot[q] = fma(r[q * ldz + g], s, dot[q]);
-        }
+        double s = 0.0;
+        for (int64_t k = sc_ptr[g]; k < sc_ptr[g + 1]; ++k) s += (double)yloc[q * ldy + sc_idx[k]];
+        if (zc) s += zc[q * ldzc + t];
+        z[q * ldz + g] = s;
+        if (DOT) dsum = fma(r[q * ldz + g], s, dsum);
     }
-    if (DOT) dot_tail<NB>(dot, nb, d);
+    if (DOT) {
+        double dot[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) dot[k] = k == q ? dsum : 0.0;
+        dot_tail<NB>(dot, nb, d);
+    }
 }
 
 template <typename TY>
@@ -468,7 +499,7 @@ void launch_scatter_prolong(int64_t n, const int32_t* order_g, const int64_t* sc
                             const TY* yloc, const double* zc, double* z, cudaStream_t s, int nb, int64_t ldy,
                             int64_t ldzc, int64_t ldz, const double* r, const DotArgs* d) {
     if (n <= 0) return;
-    const int64_t want = (n + 255) / 256;
+    const int64_t want = nb == 1 ? (n + 255) / 256 : (n + 31) / 32;
     const unsigned g = (unsigned)(want < DOT_MAX_BLOCKS ? want : DOT_MAX_BLOCKS);
     const DotArgs da = d ? *d : DotArgs{};
     if (nb == 1 && d)
@@ -558,6 +589,12 @@ void launch_dot_partials(int64_t n, const double* x, const double* y, double* pa
     dot_partials_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, y, partials, ld);
 }
 
+// CTAs of a vector kernel: what n fills, at most DOT_BLOCKS
+static unsigned vec_blocks(int64_t n) {
+    const int64_t want = (n + 255) / 256;
+    return (unsigned)(want < 1 ? 1 : (want < DOT_BLOCKS ? want : DOT_BLOCKS));
+}
+
 // x_k.y_k into the scalars (blockIdx.y = right-hand side)
 __global__ void __launch_bounds__(256) dot_kernel(int64_t n, const double* __restrict__ x,
                                                   const double* __restrict__ y, int64_t ld, DotArgs d) {
@@ -573,7 +610,7 @@ __global__ void __launch_bounds__(256) dot_kernel(int64_t n, const double* __res
 }
 
 void launch_dot(int64_t n, const double* x, const double* y, const DotArgs& d, cudaStream_t s, int nb, int64_t ld) {
-    dot_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, y, ld, d);
+    dot_kernel<<<dim3(vec_blocks(n), nb), 256, 0, s>>>(n, x, y, ld, d);
 }
 
 // x += alpha p; r -= alpha q; r.r into the scalars.  With a loop handle (the
@@ -615,7 +652,7 @@ __global__ void __launch_bounds__(256) pcg_update_xr_kernel(int64_t n, double* _
 void launch_pcg_update_xr(int64_t n, double* x, double* r, const double* p, const double* q, const DotArgs& d,
                           cudaStream_t s, int nb, int64_t ld, const int* maxit, double* alog, double* blog,
                           cudaGraphConditionalHandle loop) {
-    pcg_update_xr_kernel<<<dim3(DOT_BLOCKS, nb), 256, 0, s>>>(n, x, r, p, q, ld, d, maxit, alog, blog, loop);
+    pcg_update_xr_kernel<<<dim3(vec_blocks(n), nb), 256, 0, s>>>(n, x, r, p, q, ld, d, maxit, alog, blog, loop);
 }
 
 // p = z + beta p
