@@ -703,6 +703,21 @@ void jacobi_pairs(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDes
                   int* sweeps, unsigned long long* rots, int report_noconv) {
     amdd_handle* h = C.h;
     const int nm = (int)jd.size();
+    // the tensor-core kernel reads 16 bytes at a time: matrices whose rows do not start
+    // on 16-byte boundaries work on an aligned copy
+    std::vector<JacobiDescT<T>> jal;
+    if (std::is_same<T, float>::value && h->tensor_cores) {
+        for (int m = 0; m < nm; ++m) {
+            const JacobiDescT<T>& j = jd[m];
+            if ((j.ld % 4 == 0 && reinterpret_cast<uintptr_t>(j.A) % 16 == 0) || j.rows < 2) continue;
+            if (jal.empty()) jal = jd;
+            jal[m].ld = jacobi_ld(j.ncols_rot);
+            jal[m].A = C.tnew<T>((size_t)j.rows * jal[m].ld);
+            ck(cudaMemcpy2DAsync(jal[m].A, jal[m].ld * sizeof(T), j.A, j.ld * sizeof(T), j.ncols_rot * sizeof(T), j.rows,
+                                 cudaMemcpyDeviceToDevice, h->s));
+        }
+        if (!jal.empty()) djd = C.up(jal);
+    }
     std::vector<int> nblk(nm), active;
     auto sw = std::make_shared<std::vector<int>>(nm, max_sweeps);
     for (int m = 0; m < nm; ++m) {
@@ -768,6 +783,10 @@ void jacobi_pairs(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDes
         }
         active.swap(still);
     }
+    for (int m = 0; m < (int)jal.size(); ++m)
+        if (jal[m].A != jd[m].A)
+            ck(cudaMemcpy2DAsync(jd[m].A, jd[m].ld * sizeof(T), jal[m].A, jal[m].ld * sizeof(T),
+                                 jd[m].ncols_rot * sizeof(T), jd[m].rows, cudaMemcpyDeviceToDevice, h->s));
     C.keep.push_back(sw);
     ck(cudaMemcpyAsync(sweeps, sw->data(), nm * sizeof(int), cudaMemcpyHostToDevice, h->s));
     unsigned long long st[9];
@@ -2239,6 +2258,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     h->off_om.assign(N + 1, 0);
     h->off_sq.assign(N + 1, 0);
     h->off_I.assign(N + 1, 0);
+    std::vector<int> ldx(N);  // leading dimensions of the X_i
     std::vector<int64_t> off_x(N + 1, 0), off_m(N + 1, 0), off_ti(N + 1, 0), off_P(N + 1, 0), off_la(N + 1, 0),
         off_lm(N + 1, 0);
     for (int i = 0; i < N; ++i) {
@@ -2252,7 +2272,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->off_om[i + 1] = h->off_om[i] + ni;
         h->off_sq[i + 1] = h->off_sq[i] + ni * ni;
         h->off_I[i + 1] = h->off_I[i] + a;
-        off_x[i + 1] = off_x[i] + ni * nt;
+        ldx[i] = s64 ? (int)nt : jacobi_ld((int)nt);
+        off_x[i + 1] = off_x[i] + ni * ldx[i];
         off_m[i + 1] = off_m[i] + nt * nt;
         off_ti[i + 1] = off_ti[i] + (int64_t)a * 2 * a;
         off_P[i + 1] = off_P[i] + (int64_t)a * a;
@@ -2315,7 +2336,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                         }
                     }
                     px_src.push_back(k);
-                    px_dst.push_back(off_x[i] + (int64_t)a * nt + posX[c]);
+                    px_dst.push_back(off_x[i] + (int64_t)a * ldx[i] + posX[c]);
                 }
             }
         }
@@ -2714,7 +2735,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         std::vector<double*> sp(N);
         int maxc = 1;
         for (int i = 0; i < N; ++i) {
-            jd[i] = {X1 + off_x[i], h->ni[i], h->nt[i], h->nt[i], h->nt[i], nrmT + h->off_om[i], nullptr};
+            jd[i] = {X1 + off_x[i], h->ni[i], ldx[i], h->nt[i], h->nt[i], nrmT + h->off_om[i], nullptr};
             sp[i] = sig + h->off_om[i];
             maxc = std::max(maxc, h->nt[i]);
         }
@@ -2741,7 +2762,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             for (int i = 0; i < N; ++i) {
                 const int ni = h->ni[i], nt = h->nt[i];
                 TS* Xi = X1 + off_x[i];
-                g[i] = gd(Xi, nt, 1, Xi, nt, 0, M + off_m[i], nt, nt, nt, ni, 1.0, 0.0, 1);
+                g[i] = gd(Xi, ldx[i], 1, Xi, ldx[i], 0, M + off_m[i], nt, nt, nt, ni, 1.0, 0.0, 1);
                 mats[i] = M + off_m[i];
                 nn[i] = nt;
                 ld[i] = nt;
@@ -2864,7 +2885,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 int maxr = 1, maxc = 1;
                 for (int q = 0; q < nf; ++q) {
                     const int i = F[q], ni = h->ni[i], nt = h->nt[i], nR = h->nG[i] + h->nD[i], lj = nR + ni;
-                    kd[q] = {X1 + off_x[i], J + oj[q], ni, nR, nt, lj, delta + i};
+                    kd[q] = {X1 + off_x[i], J + oj[q], ni, nR, ldx[i], lj, delta + i};
                     jd[q] = {J + oj[q], ni, lj, nR, lj, nrm + h->off_om[i], nullptr};
                     maxr = std::max(maxr, ni);
                     maxc = std::max(maxc, nR);
@@ -2895,7 +2916,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 std::vector<GemmDescT<TS>> gw(nf);
                 for (int q = 0; q < nf; ++q) {
                     const int i = F[q], ni = h->ni[i], nt = h->nt[i], nR = h->nG[i] + h->nD[i], nIi = h->nI[i];
-                    gw[q] = gd<TS>(J + oj[q] + nR, nR + ni, 0, X1 + off_x[i] + nR, nt, 0, W + ow[q], nIi, ni, nIi, ni,
+                    gw[q] = gd<TS>(J + oj[q] + nR, nR + ni, 0, X1 + off_x[i] + nR, ldx[i], 0, W + ow[q], nIi, ni, nIi, ni,
                                    1.0, 0.0, 0);
                 }
                 gemm(C, gw);

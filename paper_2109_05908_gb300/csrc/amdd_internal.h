@@ -157,6 +157,9 @@ void launch_set_identity(const TrtriDescT<T>* d, int nmat, int maxn, cudaStream_
 // cycles of the three phases (Gram matrix, small eigensolve, rotation of the
 // rows) and the inner sweeps.  The host runs the rounds of a sweep and the sweeps.
 constexpr int JP_ROWS = 32;
+// leading dimension with every row on a 128-byte boundary: the tensor-core kernel's
+// 16-byte loads need 16, and its stores of 32 columns then fill whole lines
+inline int jacobi_ld(int ncols) { return (ncols + 31) / 32 * 32; }
 template <typename T>
 size_t jacobi_pair_smem();
 template <typename T>

@@ -23,7 +23,7 @@
 // 32 w .. 32 w + 31, i.e. output rows) into their registers.  The epilogue
 // applies alpha, beta and the lower-triangle mask.
 #include "amdd_internal.h"
-#include "jacobi_pair_inner.cuh"
+#include "jacobi_pair_blocks.cuh"
 
 namespace amdd {
 
@@ -59,6 +59,11 @@ __device__ __forceinline__ float tf32_rna(float x) {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return __uint_as_float(r);
+}
+
+__device__ __forceinline__ void split4(const float4& v, float4& hi, float4& lo) {
+    hi = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
+    lo = make_float4(tf32_rna(v.x - hi.x), tf32_rna(v.y - hi.y), tf32_rna(v.z - hi.z), tf32_rna(v.w - hi.w));
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const GemmDescT<float>* __
 
 // ------------------------------------------------------------------ block-pair Jacobi on tensor cores
 // One round of the block-pair one-sided Jacobi (the FP32 form of
-// jacobi_pair_kernel, the same schedule, tests and inner eigensolve) with its
+// jacobi_pair_kernel, the same schedule and tests, the inner eigensolve by 8 x 8 blocks) with its
 // two contractions on the tensor cores, in the same split as the GEMM above:
 //   * Gram matrix of the pair's 64 rows Y over ncols_dot columns, in chunks of
 //     64: the tile [hi(Y); lo(Y)] (128 rows, K-major, 128-byte swizzle, two
@@ -272,6 +277,11 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const GemmDescT<float>* __
 //     become the k index); in tensor memory lane c then holds column c of the
 //     new rows, so every thread stores its column's entries and each warp
 //     store covers 32 consecutive columns of one row.
+// Rows start on 16-byte boundaries, so that both contractions stage with 16-byte
+// loads and stores (the rotation transposes 4 x 4 blocks in registers).  On the 3D
+// workload (24^3, 16 subdomains, orders to 1903) a visit's Gram matrix went from
+// 135 k to 82 k cycles and its rotation from 238 k to 185 k, and the sweeps,
+// with the inner solve by blocks, from 235 to 174 ms.
 // Every wait on the tensor core is bounded; on a timeout the CTA latches
 // DERR_TIMEOUT, waits once more for its last commit and frees its tensor
 // memory.  Shared memory: region X (the two Gram staging tiles, then the
@@ -284,8 +294,9 @@ constexpr int JT_X = 64 * 1024;             // region X
 constexpr int JT_Q = 32 * 1024;             // region Q
 constexpr int JT_QT_OFF = 33 * 1024;        // Qt (FP32) inside region X, after G0 and G1
 constexpr int JT_TMEM_COLS = 128;
+constexpr int JT_W_OFF = 52 * 1024;         // the inner eigensolve's rotations, after Qt
 static_assert(2 * JPI_N * JPI_LDG * 4 <= JT_QT_OFF, "Gram buffers before Qt");
-static_assert(JT_QT_OFF + JPI_N * JPI_LDQ * 4 <= JT_X, "Qt in region X");
+static_assert(JT_QT_OFF + JPI_N * JPI_LDQ * 4 <= JT_W_OFF && JT_W_OFF + 2 * JB_R * 4 <= JT_X, "Qt and W in region X");
 }  // namespace
 
 __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>* __restrict__ descs,
@@ -303,7 +314,8 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
     float* G0 = reinterpret_cast<float*>(rx);
     float* G1 = G0 + JPI_N * JPI_LDG;
     float* Qt = reinterpret_cast<float*>(rx + JT_QT_OFF);
-    __shared__ JpRound<float> jr[2];
+    float* const W = reinterpret_cast<float*>(rx + JT_W_OFF);
+    __shared__ __align__(16) JbShared jb;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
 
@@ -367,18 +379,19 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
 
         // ---- 1. Gram matrix over ncols_dot columns
         {
-            // staging: column scol of the chunk in rows srow0 + 4 j (j < 8: block bp,
-            // else bq), so that a warp's load reads 32 consecutive columns of one row
-            const int scol = tid & 63, srow0 = tid >> 6;
-            const int rp0 = bp * 32 + srow0, rq0 = bq * 32 + srow0;
-            float pre[16];
+            // staging: columns scol .. scol + 3 of the chunk in rows srow0 + 16 j (j < 2:
+            // block bp, else bq), 16-byte loads and stores: a warp's load reads 64
+            // columns of two rows, and eight lanes' stores fill the 128 bytes of a row
+            const int scol = (tid & 15) * 4, srow0 = tid >> 4;
+            float4 pre[4];
             auto load = [&](int c0) {
                 const int c = c0 + scol;
-                const bool cok = c < d.ncols_dot;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int r = (j < 8 ? rp0 : rq0) + 4 * (j & 7);
-                    pre[j] = (cok && r < d.rows) ? __ldcg(d.A + (size_t)r * d.ld + c) : 0.0f;
+                for (int j = 0; j < 4; ++j) {
+                    const int r = (j < 2 ? bp : bq) * 32 + srow0 + 16 * (j & 1);
+                    pre[j] = (c < d.ncols_dot && r < d.rows)
+                                 ? __ldcg(reinterpret_cast<const float4*>(d.A + (size_t)r * d.ld + c))
+                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 }
             };
             const int nch = (d.ncols_dot + JT_KC - 1) / JT_KC;
@@ -394,13 +407,22 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 // tile i & 1: 128 rows x 64 k, two k atoms of 16 KB (rows 0..63 hi, 64..127 lo)
                 unsigned char* S = rx + (i & 1) * 32768;
                 unsigned char* Sa = S + (scol >> 5) * 16384;
+                const int nc = d.ncols_dot - i * JT_KC - scol;  // columns left: cleared past the end here,
+                if (nc < 4) {                                    // where the loads have arrived
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float v = pre[j];
-                    const float hi = tf32_rna(v);
-                    const int row = srow0 + 4 * j;
-                    *reinterpret_cast<float*>(Sa + sw128_off(row, scol & 31)) = hi;
-                    *reinterpret_cast<float*>(Sa + sw128_off(row + 64, scol & 31)) = tf32_rna(v - hi);
+                    for (int j = 0; j < 4; ++j) {
+                        pre[j].w = 0.0f;
+                        if (nc < 3) pre[j].z = 0.0f;
+                        if (nc < 2) pre[j].y = 0.0f;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int row = srow0 + 16 * j;
+                    float4 hi, lo;
+                    split4(pre[j], hi, lo);
+                    *reinterpret_cast<float4*>(Sa + sw128_off(row, scol & 31)) = hi;
+                    *reinterpret_cast<float4*>(Sa + sw128_off(row + 64, scol & 31)) = lo;
                 }
                 if (i + 1 < nch) load((i + 1) * JT_KC);
                 // the previous chunk's MMAs are done (its staging tile and product buffer are free)
@@ -450,10 +472,9 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 for (int j = 0; j < 32; ++j) dst[colh + j] = acc[j];
                 for (int e = tid; e < JPI_N * JPI_N; e += 256) Qt[(e >> 6) * JPI_LDQ + (e & 63)] = (e >> 6) == (e & 63) ? 1.0f : 0.0f;
                 __syncthreads();
-                // G = hh + lh + lh^T on the upper triangle and the diagonal
+                // G = hh + lh + lh^T
                 for (int e = tid; e < JPI_N * JPI_N; e += 256) {
                     const int r = e >> 6, c = e & 63;
-                    if (c < r) continue;
                     G0[r * JPI_LDG + c] += G1[r * JPI_LDG + c] + G1[c * JPI_LDG + r];
                 }
                 __syncthreads();
@@ -480,8 +501,8 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
         }
         if (ok && rot_pair) {
             unsigned nrot = 0;
-            const int inner = jpi_solve<float>(G0, G1, Qt, jr, tin, absf, nf, d.loose_above, inner_max, nrot);
-            if (nrot) atomicAdd(rots + mat, (unsigned long long)nrot);
+            const int inner = jb_solve(G0, Qt, W, jb, JbTest{tin, absf, nf, d.loose_above, 0.0f}, inner_max, nrot);
+            if (nrot && lane == 0) atomicAdd(rots + mat, (unsigned long long)nrot);
             const long long t2 = clock64();
             if (tid == 0) {
                 rotated[mat] = 1;
@@ -502,23 +523,30 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 *reinterpret_cast<float*>(rq + 16384 + o) = tf32_rna(v - hi);
             }
             // staging of Y_c^T (A operand, 128 rows c x 64 k, hi at X, lo at X + 32 KB,
-            // two k atoms of 16 KB): warp w takes 32 tiles of 8 columns x 4 rows, lane
-            // l the entry (column 8 cb + (l & 7), row 4 kb + (l >> 3)); a warp's load
-            // reads four 32-byte segments and its stores hit 32 distinct banks
-            // (tile j of warp w: id = 32 w + j, cb = id & 15, kb = id >> 4 = 2 w + (j >> 4))
-            const int cl = lane & 7, kl = lane >> 3;
-            const int gy0 = grow(8 * warp + kl), gy1 = grow(8 * warp + 4 + kl);
-            const float* yrow0 = gy0 >= 0 ? d.A + (size_t)gy0 * d.ld : nullptr;
-            const float* yrow1 = gy1 >= 0 ? d.A + (size_t)gy1 * d.ld : nullptr;
-            float pre[32];
+            // two k atoms of 16 KB): a thread takes 4 x 4 blocks (four rows of Y, four
+            // columns), 16-byte loads, transposed in registers, 16-byte stores.  Warp w's
+            // tiles j = 0, 1 are 16 rows (row group w >> 1) x 32 columns (column group
+            // 2 (w & 1) + j); of a tile's 4 x 8 blocks, lane l takes row block (l >> 1) & 3
+            // and column block (l & 1) | (l >> 3) << 1, so that a load reads 128 bytes of four
+            // rows and eight consecutive lanes store to the eight 16-byte chunks of a swizzled row
+            const int k0 = 16 * (warp >> 1) + 4 * ((lane >> 1) & 3);       // the thread's four rows of Y
+            const int cb0 = 64 * (warp & 1) + 4 * ((lane & 1) | ((lane >> 3) << 1));  // and columns (tile 0)
+            const int gy = (k0 < 32 ? bp : bq) * 32 + (k0 & 31);
+            const int nrow = d.rows - gy;                                  // rows of the four inside the matrix
+            const float* yrow = d.A + (size_t)gy * d.ld;
+            float4 pre[2][4];
             auto load = [&](int c0) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int c = c0 + 8 * (j & 15) + cl;
-                    const float* rp = j < 16 ? yrow0 : yrow1;
-                    pre[j] = (rp && c < d.ncols_rot) ? __ldcg(rp + c) : 0.0f;
+                for (int j = 0; j < 2; ++j) {
+                    const int c = c0 + cb0 + 32 * j;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        pre[j][r] = (r < nrow && c < d.ncols_rot)
+                                        ? __ldcg(reinterpret_cast<const float4*>(yrow + (size_t)r * d.ld + c))
+                                        : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 }
             };
+            unsigned char* const st = rx + (k0 >> 5) * 16384;
             const int nch = (d.ncols_rot + JT_NC - 1) / JT_NC;
             // D f32, A and B tf32, both K-major, N = 64, M = 128
             const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -562,13 +590,20 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                     asm volatile("tcgen05.fence::after_thread_sync;");
                 }
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int c = 8 * (j & 15) + cl, k = 8 * warp + 4 * (j >> 4) + kl;
-                    const float v = pre[j];
-                    const float hi = tf32_rna(v);
-                    const uint32_t o = (uint32_t)(k >> 5) * 16384 + sw128_off(c, k & 31);
-                    *reinterpret_cast<float*>(rx + o) = hi;
-                    *reinterpret_cast<float*>(rx + 32768 + o) = tf32_rna(v - hi);
+                for (int j = 0; j < 2; ++j) {
+                    const float4 *y = pre[j];
+                    const float4 col[4] = {make_float4(y[0].x, y[1].x, y[2].x, y[3].x),
+                                           make_float4(y[0].y, y[1].y, y[2].y, y[3].y),
+                                           make_float4(y[0].z, y[1].z, y[2].z, y[3].z),
+                                           make_float4(y[0].w, y[1].w, y[2].w, y[3].w)};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float4 hi, lo;
+                        split4(col[e], hi, lo);
+                        unsigned char* const o = st + sw128_off(cb0 + 32 * j + e, k0 & 31);
+                        *reinterpret_cast<float4*>(o) = hi;
+                        *reinterpret_cast<float4*>(o + 32768) = lo;
+                    }
                 }
                 if (i + 1 < nch) load((i + 1) * JT_NC);
                 asm volatile("fence.proxy.async.shared::cta;");
@@ -577,13 +612,22 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 if (tid == 0) {
                     const uint32_t dcol = tmem + (uint32_t)((i & 1) * 64);
+                    // the corrections first: the tensor core truncates each accumulation at
+                    // the size of the sum so far, which shortens the rows a little every
+                    // visit (singular values of a 32 x 32 grid half: 5.2e-4 too small with
+                    // the terms interleaved, 1.1e-4 off now)
 #pragma unroll
                     for (int ks = 0; ks < JPI_N / 8; ++ks) {
                         const uint64_t ao = (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4);
                         const uint64_t bo = (uint64_t)(((ks >> 2) * 8192 + (ks & 3) * 32) >> 4);
-                        mma_tf32(dcol, adesc + ao, bdesc + bo, idesc, ks > 0 ? 1u : 0u);
-                        mma_tf32(dcol, adesc + ao, bdesc + bo + (16384 >> 4), idesc, 1u);
+                        mma_tf32(dcol, adesc + ao, bdesc + bo + (16384 >> 4), idesc, ks > 0 ? 1u : 0u);
                         mma_tf32(dcol, adesc + ao + (32768 >> 4), bdesc + bo, idesc, 1u);
+                    }
+#pragma unroll
+                    for (int ks = 0; ks < JPI_N / 8; ++ks) {
+                        const uint64_t ao = (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4);
+                        const uint64_t bo = (uint64_t)(((ks >> 2) * 8192 + (ks & 3) * 32) >> 4);
+                        mma_tf32(dcol, adesc + ao, bdesc + bo, idesc, 1u);
                     }
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mb));
                 }
