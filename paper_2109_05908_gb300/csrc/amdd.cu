@@ -2386,8 +2386,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         launch_convert<double, float>(Araw, Lb, h->sum_sq, s);
 
     // full selections: the basis diag(A_II)^{-1/2} keeps every block of E that
-    // touches such a subdomain as sparse as A (its envelope-aware Cholesky and
-    // the coarse solve then skip most tiles); with a kept E (multilevel form)
+    // touches such a subdomain as sparse as A (and the separators of its
+    // substructuring as small); with a kept E (multilevel form)
     // the A_II-orthonormal rows of L_A^{-1}, so that E is a block-orthogonal
     // congruence of the one any other A_II-orthonormal basis gives
     const bool diag_basis = !h->keep_E;
@@ -3088,8 +3088,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         else if (!all_diag)
             ZtT = C.tnew<T>(h->sum_zt);
         // full selections: the basis diag(A_II)^{-1/2} keeps every block of E that
-        // touches such a subdomain as sparse as A (its envelope-aware Cholesky and
-        // the coarse solve then skip most tiles); with a kept E (multilevel form)
+        // touches such a subdomain as sparse as A (and the separators of its
+        // substructuring as small); with a kept E (multilevel form)
         // the A_II-orthonormal rows of L_A^{-1}, so that E is a block-orthogonal
         // congruence of the one any other A_II-orthonormal basis gives
         if (h->nC > 0 && all_diag) {
