@@ -99,7 +99,8 @@ __device__ __forceinline__ bool dot_tail(double (&s)[NB], int nb, const DotArgs&
 // G lanes per row, rows assigned to lane groups
 // in a grid-stride loop, four entries in flight per lane.  Rows of a few entries
 // take one thread each: a warp then covers 32 consecutive rows, bound by HBM
-// (5-point matrix of 2.1 M rows: 5.4 TB/s).  For longer rows FP64 sets the rate,
+// (5-point matrix of 2.1 M rows: 5.4 TB/s).  There the four-entry loop does not pay:
+// 54.6 us a call with it, 51.7 without.  For longer rows FP64 sets the rate,
 // two multiply-adds per clock and SM whether or not the lanes have work: a warp
 // per row of 72 entries spends more on the shuffle tree than on the row, while
 // with 4 lanes the tree is shared by 8 rows.  27-point matrix with 3 unknowns per
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __r
         if (row < n) {
             const int64_t e = rowptr[row + 1];
             int64_t k = rowptr[row] + sub;
-            for (; k + 3 * G < e; k += 4 * G) {
+            for (; G > 1 && k + 3 * G < e; k += 4 * G) {
                 double v[4], xv[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
