@@ -810,7 +810,7 @@ void run_jacobi(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDescT
         smem8 = std::max(smem8, jacobi_block_smem<T>(j.rows, j.ncols_rot, JAC_CLUSTER));
         smem16 = std::max(smem16, jacobi_block_smem<T>(j.rows, j.ncols_rot, 2 * JAC_CLUSTER));
         maxr = std::max(maxr, j.rows);
-        floors = floors || j.absfloor || j.normfloor || j.loose_above > T(0);
+        floors = floors || j.absfloor || j.normfloor || j.loose.above > T(0);
     }
     const bool launched = launch_jacobi_block<T>(djd, (int)jd.size(), smem8, smem16, maxr, max_sweeps, tol, sweeps,
                                                  rots, h->d_err, report_noconv, floors, h->s);
@@ -3140,21 +3140,28 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 // u |T_i|.  The other eigenvalues crowd below 1 (differences down to u),
                 // where making the rows orthogonal to each other to the relative test
                 // took most of the 33 to 36 sweeps: rows both longer than 1.25 tau are
-                // only kept apart from the kept ones (loose_above), and couplings below
-                // u |T_i| are left (normfloor).  On a 16 x 16 box of the Laplacian the
-                // kept span is as close to the eigenvectors' as before (8.6e-15 against
+                // only kept apart from the kept ones (loose), and couplings below
+                // u |T_i| are left (normfloor).  The long rows, pairwise within t of
+                // orthogonal, have a Gram matrix whose eigenvalues are at least
+                // (1.25 tau)^2 (1 - (n_I - 1) t), with t <= 1 / (4 n_I) above
+                // (1.08 tau)^2: no kept eigenvector can lie among them, however it
+                // spreads over the unknowns, and the p_i shortest rows are the kept
+                // ones.  On a 16 x 16 box of the Laplacian the kept span is as close to
+                // the eigenvectors' as with the strict test throughout (8.6e-15 against
                 // 8.4e-15) in 15 sweeps instead of 26.  FP64 13 x 12 x 12 diffusion,
-                // tau 0.5, eight subdomains: 148 -> 114 ms.
+                // tau 0.5, eight subdomains, this eigensolve alone: 148 -> 114 ms.
                 T* nfl = C.tnew<T>(np);
                 T cut2 = (T)(1.25 * h->tau) * (T)(1.25 * h->tau);
                 if (!(cut2 >= std::numeric_limits<T>::min())) cut2 = T(0);  // no cut below the type's range
                 int maxc = 1;
                 for (int q = 0; q < np; ++q) {
                     const int i = partial_d[q], nIi = h->nI[i];
-                    jd[q] = {TI + off_ti[i], nIi, 2 * nIi, nIi, 2 * nIi, nrmE + h->off_I[i], nullptr, nfl + q, cut2};
+                    jd[q] = {TI + off_ti[i], nIi, 2 * nIi, nIi, 2 * nIi, nrmE + h->off_I[i], nullptr, nfl + q};
                     mp[q] = mu_j + h->off_I[i];
                     maxc = std::max(maxc, nIi);
                 }
+                const T tol = (f64 ? T(2) : T(8)) * std::sqrt((T)maxc) * std::numeric_limits<T>::epsilon();
+                for (auto& j : jd) j.loose = {cut2, std::max(tol, std::min(T(0x1p-10), T(0.25) / (T)j.rows))};
                 JacobiDescT<T>* djd = C.up(jd);
                 {
                     PScope ps(h, PK_SMALL);
@@ -3163,7 +3170,6 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 double* const* dmp = C.up(mp);
                 {
                     PScope ps(h, PK_JAC_EIG);
-                    const T tol = (f64 ? T(2) : T(8)) * std::sqrt((T)maxc) * std::numeric_limits<T>::epsilon();
                     run_jacobi<T>(C, jd, djd, h->max_sweeps, tol, sweeps + N, rots + N, f64 ? 1 : 0);
                 }
                 {

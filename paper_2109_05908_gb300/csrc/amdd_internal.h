@@ -79,6 +79,11 @@ struct ChunkRef {
     int desc, ct;  // column chunk (64 columns)
 };
 
+// a looser tolerance for long rows (above: squared length, 0: none)
+template <typename T>
+struct JacLoose {
+    T above, tol;
+};
 template <typename T>
 struct JacobiDescT {
     T* A;               // rows x ld, rows orthogonalised in place
@@ -91,15 +96,14 @@ struct JacobiDescT {
     // unit roundoff of T).  With f = u |M|^2 (launch_row_maxnorm2) a pair is left
     // alone once its coupling is below the rounding of M itself, u |M|.
     const T* normfloor = nullptr;
-    // optional c > 0: two rows both longer than sqrt(c) need only be orthogonal to
-    // JAC_LOOSE (their span, not the rows themselves, is wanted)
-    T loose_above = T(0);
+    // optional: two rows both longer than sqrt(loose.above) need only be orthogonal
+    // to loose.tol (their span, not the rows themselves, is wanted)
+    JacLoose<T> loose = {};
 };
-constexpr float JAC_LOOSE = 0x1p-10f;
 // squared relative tolerance for the pair of squared lengths a, b
 template <typename T>
-__host__ __device__ __forceinline__ T jac_tol2(T tol, T a, T b, T loose_above) {
-    const T t = loose_above > T(0) && (a < b ? a : b) > loose_above ? T(JAC_LOOSE) : tol;
+__host__ __device__ __forceinline__ T jac_tol2(T tol, T a, T b, JacLoose<T> l) {
+    const T t = l.above > T(0) && (a < b ? a : b) > l.above ? l.tol : tol;
     return t * t;
 }
 using JacobiDesc = JacobiDescT<double>;
@@ -196,7 +200,7 @@ size_t jacobi_block_smem(int rows, int ncols_rot, int cluster);
 // Shared-memory-resident block variant with a cluster of JAC_CLUSTER CTAs per
 // matrix, else (blocks too large) 2 * JAC_CLUSTER; returns false, with nothing
 // launched, when neither fits (smem8 / smem16: bytes per CTA for the two sizes;
-// floors: some matrix has absfloor, normfloor or loose_above).
+// floors: some matrix has absfloor, normfloor or loose).
 template <typename T>
 bool launch_jacobi_block(const JacobiDescT<T>* d, int nmat, size_t smem8, size_t smem16, int max_rows,
                          int max_sweeps, T tol, int* sweeps, unsigned long long* rots, int* err, int report_noconv,

@@ -524,12 +524,12 @@ __global__ void __launch_bounds__(256) jacobi_pair_kernel(const JacobiDescT<T>* 
             const int p = e / JP_R, q = e % JP_R;
             if (q <= p) continue;
             const T a = G[p * JPI_LDG + p], b = G[q * JPI_LDG + q], g = G[p * JPI_LDG + q];
-            if (g != T(0) && g * g > jac_tol2(tol, a, b, d.loose_above) * a * b && fabs(g) > absf && g * g > nf * fmax(a, b)) mine = 1;
+            if (g != T(0) && g * g > jac_tol2(tol, a, b, d.loose) * a * b && fabs(g) > absf && g * g > nf * fmax(a, b)) mine = 1;
         }
         if (!__syncthreads_or(mine)) return;  // the pair met the stopping test: rows unchanged
     }
     unsigned nrot = 0;
-    const int inner = jpi_solve<T>(G, G1, Qt, jr, tin, absf, nf, d.loose_above, inner_max, nrot);
+    const int inner = jpi_solve<T>(G, G1, Qt, jr, tin, absf, nf, d.loose, inner_max, nrot);
     if (nrot) atomicAdd(rots + mat, (unsigned long long)nrot);
     const long long t2 = clock64();
     if (tid == 0) {
@@ -639,11 +639,12 @@ __global__ void __launch_bounds__(1024)
     const int hbe = hb + (hb & 1);
     // in shared memory: read from the descriptor inside the sub-rounds they would
     // cost a trip to L2 in each
-    __shared__ T floors[3];
+    __shared__ T floors[2];
+    __shared__ JacLoose<T> loose;
     if (FL && threadIdx.x == 0) {
         floors[0] = d.absfloor ? *d.absfloor : T(0);
         floors[1] = d.normfloor ? (sizeof(T) == 4 ? T(1.1920928955078125e-7) : T(2.220446049250313e-16)) * *d.normfloor : T(0);
-        floors[2] = d.loose_above;
+        loose = d.loose;
     }
     unsigned long long my_rots = 0;
     int sweep = 0;
@@ -706,7 +707,7 @@ __global__ void __launch_bounds__(1024)
                     jflag[k] = 0;
                     if (pair_of(k, sa, sb)) {
                         const T g = jg[k], a = nrm[sa], b = nrm[sb];
-                        const T t2 = FL ? jac_tol2(tol, a, b, floors[2]) : tol * tol;
+                        const T t2 = FL ? jac_tol2(tol, a, b, loose) : tol * tol;
                         if (g != T(0) && g * g > t2 * a * b &&
                             (!FL || (fabs(g) > floors[0] && g * g > floors[1] * fmax(a, b)))) {
                             T cs, sn, t;

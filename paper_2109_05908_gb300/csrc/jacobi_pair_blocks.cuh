@@ -35,7 +35,9 @@ struct JbShared {
 };
 
 struct JbTest {
-    float tin, absf, nf, loose, rel;  // rel: couplings below rel max(a, b) are left alone
+    float tin, absf, nf;
+    JacLoose<float> loose;
+    float rel;  // couplings below rel max(a, b) are left alone
 };
 
 // the two indices blocks of pair g (0..3) of round ir (0..6)

@@ -92,7 +92,7 @@ __device__ __forceinline__ void jpi_rotation(T a, T b, T g, T& cs, T& sn, T& t) 
 // rotates.
 template <typename T>
 __device__ __forceinline__ bool jpi_next(const T* G, const JpRound<T>& cur, bool pend, int rrn, int swn, T tin,
-                                         T absf, T nf, T loose_above, T ueps, JpRound<T>& nx, int lane) {
+                                         T absf, T nf, JacLoose<T> loose, T ueps, JpRound<T>& nx, int lane) {
     int p, q;
     jpi_pair(lane, rrn, p, q);
     nx.pq[lane] = p | (q << 8);
@@ -119,7 +119,7 @@ __device__ __forceinline__ bool jpi_next(const T* G, const JpRound<T>& cur, bool
         const T r0 = (iy & 0x80) ? n[1] : n[0], r1 = (iy & 0x80) ? n[3] : n[2];
         g = (ix & 0x80) ? r1 : r0;
     }
-    const bool doit = g != T(0) && g * g > jac_tol2(tin, a, b, loose_above) * a * b && fabs(g) > absf &&
+    const bool doit = g != T(0) && g * g > jac_tol2(tin, a, b, loose) * a * b && fabs(g) > absf &&
                       g * g > nf * fmax(a, b) &&
                       (swn == 0 || fabs(g) > T(8) * ueps * fmax(a, b));
     nx.on[lane] = doit ? 1 : 0;
@@ -258,7 +258,7 @@ __device__ __forceinline__ void jpi_apply(const T* Gc, T* Gn, T* Qt, const JpRou
 // (to every thread) the number of inner sweeps; *nrot_out (warp 0) counts the
 // rotations.
 template <typename T>
-__device__ int jpi_solve(T* G0, T* G1, T* Qt, JpRound<T>* jr, T tin, T absf, T nf, T loose_above, int max_sweeps,
+__device__ int jpi_solve(T* G0, T* G1, T* Qt, JpRound<T>* jr, T tin, T absf, T nf, JacLoose<T> loose, int max_sweeps,
                          unsigned& nrot_out) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const T ueps = sizeof(T) == 4 ? T(1.1920928955078125e-7) : T(2.220446049250313e-16);
@@ -266,7 +266,7 @@ __device__ int jpi_solve(T* G0, T* G1, T* Qt, JpRound<T>* jr, T tin, T absf, T n
     bool swrot = false;
     const JpiWork work = jpi_work(tid - 32);  // used by warps 1..7
     if (warp == 0) {
-        const bool d = jpi_next<T>(G0, jr[1], false, 0, 0, tin, absf, nf, loose_above, ueps, jr[0], lane);
+        const bool d = jpi_next<T>(G0, jr[1], false, 0, 0, tin, absf, nf, loose, ueps, jr[0], lane);
         nrot += d ? 1u : 0u;
         swrot = __any_sync(0xffffffffu, d);
         if (lane == 0) {
@@ -290,7 +290,7 @@ __device__ int jpi_solve(T* G0, T* G1, T* Qt, JpRound<T>* jr, T tin, T absf, T n
                 stop = !swrot || swn >= max_sweeps;
                 swrot = false;
             }
-            const bool d = jpi_next<T>(Gc, cur, pend, rrn, swn, tin, absf, nf, loose_above, ueps, nx, lane);
+            const bool d = jpi_next<T>(Gc, cur, pend, rrn, swn, tin, absf, nf, loose, ueps, nx, lane);
             nrot += d ? 1u : 0u;
             const bool any = __any_sync(0xffffffffu, d);
             swrot = swrot || any;

@@ -495,13 +495,13 @@ __global__ void __maxnreg__(120) jacobi_pair_tc_kernel(const JacobiDescT<float>*
                 const int p = e >> 6, q = e & 63;
                 if (q <= p) continue;
                 const float a = G0[p * JPI_LDG + p], b = G0[q * JPI_LDG + q], g = G0[p * JPI_LDG + q];
-                if (g != 0.0f && g * g > jac_tol2(tol, a, b, d.loose_above) * a * b && fabsf(g) > absf && g * g > nf * fmaxf(a, b)) mine = 1;
+                if (g != 0.0f && g * g > jac_tol2(tol, a, b, d.loose) * a * b && fabsf(g) > absf && g * g > nf * fmaxf(a, b)) mine = 1;
             }
             rot_pair = __syncthreads_or(mine) != 0;
         }
         if (ok && rot_pair) {
             unsigned nrot = 0;
-            const int inner = jb_solve(G0, Qt, W, jb, JbTest{tin, absf, nf, d.loose_above, 0.0f}, inner_max, nrot);
+            const int inner = jb_solve(G0, Qt, W, jb, JbTest{tin, absf, nf, d.loose, 0.0f}, inner_max, nrot);
             if (nrot && lane == 0) atomicAdd(rots + mat, (unsigned long long)nrot);
             const long long t2 = clock64();
             if (tid == 0) {
