@@ -95,6 +95,23 @@ __device__ __forceinline__ bool dot_tail(double (&s)[NB], int nb, const DotArgs&
 }
 
 // ------------------------------------------------------------------ SpMV
+// s += entries k, k + G, ... < e of a row times x, four in flight when FOUR
+template <int G, bool FOUR>
+__device__ __forceinline__ void spmv_row(double& s, int64_t k, int64_t e, const int32_t* __restrict__ col,
+                                         const double* __restrict__ val, const double* __restrict__ x) {
+    for (; FOUR && k + 3 * G < e; k += 4 * G) {
+        double v[4], xv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = __ldg(val + k + u * G);
+            xv[u] = __ldg(x + __ldg(col + k + u * G));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s = fma(v[u], xv[u], s);
+    }
+    for (; k < e; k += G) s = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), s);
+}
+
 // y = A x (MODE 0), y = b - A x (1), or y = A x with x.y into the PCG scalars (2):
 // G lanes per row, rows assigned to lane groups
 // in a grid-stride loop, four entries in flight per lane.  Rows of a few entries
@@ -105,11 +122,14 @@ __device__ __forceinline__ bool dot_tail(double (&s)[NB], int nb, const DotArgs&
 // per row of 72 entries spends more on the shuffle tree than on the row, while
 // with 4 lanes the tree is shared by 8 rows.  27-point matrix with 3 unknowns per
 // node, 98 k rows, call included: 88 -> 47 us.
+// A row of more than lng entries is left to the whole warp after its groups' other
+// rows, so that a few long rows among short ones do not set the time: 300 k rows of
+// 9 with eight of 20,000, 2704 us by one lane, 799 by eight, 102 so.
 template <int G, int MODE>
 __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ col, const double* __restrict__ val,
                                                    const double* __restrict__ x, const double* __restrict__ b,
-                                                   double* __restrict__ y, DotArgs d) {
+                                                   double* __restrict__ y, int64_t lng, DotArgs d) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int sub = threadIdx.x & (G - 1);
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -119,23 +139,21 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __r
     double dot[1] = {0.0};
     for (int64_t row = gid / G; row < nround; row += groups) {
         double s = 0.0;
-        if (row < n) {
-            const int64_t e = rowptr[row + 1];
-            int64_t k = rowptr[row] + sub;
-            for (; G > 1 && k + 3 * G < e; k += 4 * G) {
-                double v[4], xv[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    v[u] = __ldg(val + k + u * G);
-                    xv[u] = __ldg(x + __ldg(col + k + u * G));
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) s = fma(v[u], xv[u], s);
-            }
-            for (; k < e; k += G) s = fma(__ldg(val + k), __ldg(x + __ldg(col + k)), s);
-        }
+        const int64_t k0 = row < n ? rowptr[row] : 0, e = row < n ? rowptr[row + 1] : 0;
+        const bool wide = G < 32 && e - k0 > lng;
+        if (!wide) spmv_row<G, (G > 1)>(s, k0 + sub, e, col, val, x);
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (G < 32)
+            for (unsigned m = __ballot_sync(0xffffffffu, wide && sub == 0); m; m &= m - 1) {
+                const int from = __ffs(m) - 1, lane = threadIdx.x & 31;
+                double w = 0.0;
+                spmv_row<32, true>(w, __shfl_sync(0xffffffffu, k0, from) + lane, __shfl_sync(0xffffffffu, e, from), col,
+                                   val, x);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+                if (lane == from) s = w;
+            }
         if (row < n && sub == 0) {
             y[row] = MODE == 1 ? b[row] - s : s;
             if (MODE == 2) dot[0] = fma(x[row], s, dot[0]);
@@ -144,13 +162,19 @@ __global__ void __launch_bounds__(256) spmv_kernel(int64_t n, const int64_t* __r
     if (MODE == 2) dot_tail<1>(dot, 1, d);
 }
 
-// Lanes per row by the average row length, the fastest of 1, 2, 4, 8, 16, 32 at
-// 30 M entries (us; HBM floor 53 to 74): length 7: 78 / 132 / 170 / 286 / 705 /
-// 1670; 16: 176 / 97 / 100 / 166 / 326 / 747; 72: 163 / 87 / 76 / 92 / 125 / 228;
-// 600: 217 / 111 / 79 / 89 / 76 / 79.
+// Lanes per row: by the average row length the fastest of 1, 2, 4, 8, 16, 32 once
+// the chip is full (kernel us with 1 / 2 / 4 / 8 / 16 / 32 lanes, lane count of the rule
+// marked; 2.1 M rows of 7: 42.6* / 66 / 88 / 139 / 338 / 771; 300 k rows of 24: 34.9 /
+// 20.7* / 22.7 / 30.9 / 68 / 117; 100 k rows of 81: 49.7 / 26.9 / 24.4* / 25.0 / 37 / 69;
+// 30 k rows of 600: 142 / 87 / 59 / 45 / 47* / 52), and from 9 entries on twice as many while
+// that still takes at most 64,000 threads, since a smaller matrix is bound by the chain
+// of loads of its rows (1000 rows of 81: 18.5 / 10.3 / 6.2 / 6.2 / 6.2 / 4.1*; 3000 rows of 24: 8.2 / 6.2 /
+// 4.1 / 4.1* / 4.2 / 6.1; 10 k rows of 9: 5.5 / 4.1 / 4.1* / 5.1 / 6.2 / 8.2; launch alone 4.1).
 static int spmv_lanes(int64_t n, int64_t nnz) {
-    const int64_t per = n > 0 ? nnz / n : 0;
-    return per <= 9 ? 1 : (per <= 24 ? 2 : (per <= 250 ? 4 : 16));
+    const int64_t per = nnz / n;
+    int g = per <= 9 ? 1 : (per <= 24 ? 2 : (per <= 250 ? 4 : 16));
+    while (per > 8 && g < 32 && 2 * g <= per && 2 * g * n <= 64000) g *= 2;
+    return g;
 }
 
 template <int MODE>
@@ -161,14 +185,16 @@ static void spmv_any(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_
     const int64_t want = (n * group + 255) / 256;
     const int most = MODE == 2 ? DOT_MAX_BLOCKS : 152 * 64;
     const int blocks = (int)(want < most ? want : most);
-    if (group == 1)
-        spmv_kernel<1, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
-    else if (group == 2)
-        spmv_kernel<2, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
-    else if (group == 4)
-        spmv_kernel<4, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
-    else
-        spmv_kernel<16, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, d);
+    // far above the average: rows of about equal length stay with their groups
+    const int64_t lng = std::max<int64_t>(64, 4 * (nnz / n));
+    switch (group) {
+        case 1: spmv_kernel<1, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d); break;
+        case 2: spmv_kernel<2, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d); break;
+        case 4: spmv_kernel<4, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d); break;
+        case 8: spmv_kernel<8, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d); break;
+        case 16: spmv_kernel<16, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d); break;
+        default: spmv_kernel<32, MODE><<<blocks, 256, 0, s>>>(n, rowptr, col, val, x, b, y, lng, d);
+    }
 }
 
 void launch_spmv(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const double* val,
