@@ -494,31 +494,67 @@ template void launch_gather_rows<double>(const double*, const int64_t*, double*,
 //                 runs in that owner order).  nb right-hand sides: yloc, zc
 //                 and z hold nb vectors ldy, ldzc and ldz apart.
 // With DOT also r_k.z_k into the PCG scalars (r: nb vectors ldz apart).
-template <typename TY, int NB, bool DOT>
+// With several right-hand sides: ROWS = 32, warp q of the CTA takes the q-th, over
+// the CTA's 32 unknowns, where they would not fill the chip otherwise (5184, eight
+// vectors: 22.5 -> 7.3 us); ROWS = 256, one thread per unknown for all of them, in large
+// systems, where the warps without a right-hand side would be in the way (409,600, two
+// vectors: 14.5 us, with ROWS = 32 27.5).  Whole one-level applies put the line at about
+// 80 k unknowns for two or three vectors and 300 k for more: 262,144 with 2 / 8
+// vectors 127 / 176 us against 133 / 173 with ROWS = 32, 1,048,576 376 / 560 against 408 / 570.
+template <typename TY, int NB, int ROWS, bool DOT>
 __global__ void __launch_bounds__(256) scatter_prolong_kernel(
     int64_t n, const int32_t* __restrict__ order_g, const int64_t* __restrict__ sc_ptr,
     const int32_t* __restrict__ sc_idx, const TY* __restrict__ yloc, const double* __restrict__ zc,
     double* __restrict__ z, int nb, int64_t ldy, int64_t ldzc, int64_t ldz, const double* __restrict__ r, DotArgs d) {
-    // one thread per unknown; with several right-hand sides warp q of the CTA takes
-    // the q-th, over the CTA's 32 unknowns
-    constexpr int PER = NB > 1 ? 32 : 256;
-    const int q = NB > 1 ? threadIdx.x >> 5 : 0;
+    double dot[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) dot[k] = 0.0;
+    const int q = ROWS == 32 ? threadIdx.x >> 5 : 0;
     double dsum = 0.0;
-    for (int64_t t = (int64_t)blockIdx.x * PER + (threadIdx.x & (PER - 1)); t < n && q < nb;
-         t += (int64_t)gridDim.x * PER) {
+    for (int64_t t = (int64_t)blockIdx.x * ROWS + (threadIdx.x & (ROWS - 1)); t < n && q < nb;
+         t += (int64_t)gridDim.x * ROWS) {
         const int g = order_g[t];
-        double s = 0.0;
-        for (int64_t k = sc_ptr[g]; k < sc_ptr[g + 1]; ++k) s += (double)yloc[q * ldy + sc_idx[k]];
-        if (zc) s += zc[q * ldzc + t];
-        z[q * ldz + g] = s;
-        if (DOT) dsum = fma(r[q * ldz + g], s, dsum);
+        const int64_t k0 = sc_ptr[g], k1 = sc_ptr[g + 1];
+        auto value = [&](int v) {
+            double s = 0.0;
+            for (int64_t k = k0; k < k1; ++k) s += (double)yloc[v * ldy + sc_idx[k]];
+            if (zc) s += zc[v * ldzc + t];
+            z[v * ldz + g] = s;
+            return s;
+        };
+        if (ROWS == 32 || NB == 1) {
+            const double s = value(q);
+            if (DOT) dsum = fma(r[q * ldz + g], s, dsum);
+        } else {
+#pragma unroll
+            for (int v = 0; v < NB; ++v)
+                if (v < nb) {
+                    const double s = value(v);
+                    if (DOT) dot[v] = fma(r[v * ldz + g], s, dot[v]);
+                }
+        }
     }
     if (DOT) {
-        double dot[NB];
+        if (ROWS == 32 || NB == 1) {
 #pragma unroll
-        for (int k = 0; k < NB; ++k) dot[k] = k == q ? dsum : 0.0;
+            for (int k = 0; k < NB; ++k) dot[k] = k == q ? dsum : 0.0;
+        }
         dot_tail<NB>(dot, nb, d);
     }
+}
+
+template <typename TY, int NB, int ROWS>
+static void scatter_any(int64_t n, const int32_t* order_g, const int64_t* sc_ptr, const int32_t* sc_idx,
+                        const TY* yloc, const double* zc, double* z, cudaStream_t s, int nb, int64_t ldy, int64_t ldzc,
+                        int64_t ldz, const double* r, const DotArgs* d) {
+    const int64_t want = (n + ROWS - 1) / ROWS, most = d ? DOT_MAX_BLOCKS : 152 * 32;
+    const unsigned g = (unsigned)(want < most ? want : most);
+    if (d)
+        scatter_prolong_kernel<TY, NB, ROWS, true><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy,
+                                                                     ldzc, ldz, r, *d);
+    else
+        scatter_prolong_kernel<TY, NB, ROWS, false><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy,
+                                                                      ldzc, ldz, r, DotArgs{});
 }
 
 template <typename TY>
@@ -526,21 +562,12 @@ void launch_scatter_prolong(int64_t n, const int32_t* order_g, const int64_t* sc
                             const TY* yloc, const double* zc, double* z, cudaStream_t s, int nb, int64_t ldy,
                             int64_t ldzc, int64_t ldz, const double* r, const DotArgs* d) {
     if (n <= 0) return;
-    const int64_t want = nb == 1 ? (n + 255) / 256 : (n + 31) / 32;
-    const unsigned g = (unsigned)(want < DOT_MAX_BLOCKS ? want : DOT_MAX_BLOCKS);
-    const DotArgs da = d ? *d : DotArgs{};
-    if (nb == 1 && d)
-        scatter_prolong_kernel<TY, 1, true><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, 1, ldy, ldzc, ldz, r,
-                                                              da);
-    else if (nb == 1)
-        scatter_prolong_kernel<TY, 1, false><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, 1, ldy, ldzc, ldz,
-                                                               r, da);
-    else if (d)
-        scatter_prolong_kernel<TY, MAXB, true><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy, ldzc,
-                                                                 ldz, r, da);
+    if (nb == 1)
+        scatter_any<TY, 1, 256>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, s, 1, ldy, ldzc, ldz, r, d);
+    else if (n <= MULTI_SMALL * (nb < 4 ? 1 : 4))
+        scatter_any<TY, MAXB, 32>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, s, nb, ldy, ldzc, ldz, r, d);
     else
-        scatter_prolong_kernel<TY, MAXB, false><<<g, 256, 0, s>>>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, nb, ldy, ldzc,
-                                                                  ldz, r, da);
+        scatter_any<TY, MAXB, 256>(n, order_g, sc_ptr, sc_idx, yloc, zc, z, s, nb, ldy, ldzc, ldz, r, d);
 }
 template void launch_scatter_prolong<float>(int64_t, const int32_t*, const int64_t*, const int32_t*, const float*,
                                             const double*, double*, cudaStream_t, int, int64_t, int64_t, int64_t,
