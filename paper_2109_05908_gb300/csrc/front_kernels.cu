@@ -245,9 +245,17 @@ namespace {
 // Lanes per row: 4 while that fills the chip (FP64 runs at two multiply-adds per
 // clock and SM, idle lanes or not, so the shuffle tree is best shared by 8 rows),
 // a warp when the rows of the stage are few.  With several vectors each load feeds
-// eight independent sums, so fewer threads fill it.
-int lanes_for(int64_t rows, int nb) {
-    const int64_t fill = 152 * (nb == 1 ? 448 : 128);
+// eight independent sums: in FP64 fewer threads then fill the chip, in FP32, whose
+// rate is not the limit, more are wanted to hide the loads (local solves in FP32 on
+// 19,000 rows of a 27-point matrix with three unknowns a node, one-level apply with
+// 2 / 8 vectors: 161 / 199 us with the FP64 line, 90 / 107 so; dense triangles 158 / 174).
+template <typename T, int NB>
+int lanes_for(int64_t rows) {
+    if (sizeof(T) == 4 && NB > 1) {
+        const int64_t fill = 152 * 768;
+        return rows * 4 >= fill ? 4 : (rows * 8 >= fill ? 8 : (rows * 16 >= fill ? 16 : 32));
+    }
+    const int64_t fill = 152 * (NB == 1 ? 448 : 128);
     return rows * 4 >= fill ? 4 : (rows * 8 >= fill ? 8 : 32);
 }
 
@@ -269,21 +277,25 @@ void solve_nb(const FrontSolveT<T>& a, T* out, int64_t ldo, int nb, cudaStream_t
     for (int st = 0; st + 1 < a.stages; ++st) {
         const int64_t nrow = a.down_off[st + 1] - a.down_off[st];
         if (nrow <= 0) continue;
-        const int g = lanes_for(nrow, nb);
+        const int g = lanes_for<T, NB>(nrow);
         if (g == 4)
             stage_down<T, NB, 4>(a, st, nb, s);
         else if (g == 8)
             stage_down<T, NB, 8>(a, st, nb, s);
+        else if (g == 16)
+            stage_down<T, NB, 16>(a, st, nb, s);
         else
             stage_down<T, NB, 32>(a, st, nb, s);
     }
     for (int st = a.stages - 1; st >= 0; --st) {
         if (a.row_off[st + 1] <= a.row_off[st]) continue;
-        const int g = lanes_for(a.row_off[st + 1] - a.row_off[st], nb);
+        const int g = lanes_for<T, NB>(a.row_off[st + 1] - a.row_off[st]);
         if (g == 4)
             stage_up<T, NB, 4>(a, st, out, ldo, nb, s);
         else if (g == 8)
             stage_up<T, NB, 8>(a, st, out, ldo, nb, s);
+        else if (g == 16)
+            stage_up<T, NB, 16>(a, st, out, ldo, nb, s);
         else
             stage_up<T, NB, 32>(a, st, out, ldo, nb, s);
     }
