@@ -72,7 +72,7 @@ __device__ __forceinline__ void mlp_fma(float (&acc)[2][8], float w0, float w1, 
 }  // namespace
 
 // Thread t owns columns t % 128 and t % 128 + 128 for samples 8 (t / 128) .. + 8.
-// TRAIN: writes H1, H2, dY, dZ2, dZ1 (n x 256) and the CTA's loss sum; else Q.
+// TRAIN: writes H1, H2, dY, dZ2, dZ1 (n x 256) and each sample's loss; else Q.
 template <bool TRAIN>
 __global__ void __launch_bounds__(256) mlp_rows_kernel(const float* __restrict__ wb, const float* __restrict__ x,
                                                        const float* __restrict__ qt, int n, float* __restrict__ H1,
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) mlp_rows_kernel(const float* __restrict__
     float* h1 = xs + MT * MR;
     float* h2 = h1 + MW * MR;
     float* ys = h2 + MW * MR;
-    __shared__ float red[8];
+    __shared__ float red[8][8];
     const int tid = threadIdx.x, c0 = tid & 127, rg = (tid >> 7) * 8;
     const int row0 = blockIdx.x * MR;
     mlp_issue(0, wb, wt[0], vec);
@@ -146,7 +146,9 @@ __global__ void __launch_bounds__(256) mlp_rows_kernel(const float* __restrict__
             }
             clear();
             __syncthreads();
-            float d[2][8], loss = 0.0f;
+            float d[2][8], loss[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) loss[r] = 0.0f;
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int j = c0 + 128 * c, jt = (j % PROP_NB) * PROP_NB + j / PROP_NB;
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(256) mlp_rows_kernel(const float* __restrict__
                     if (row < n) {
                         if (TRAIN) {
                             const float de = q - qt[(size_t)row * MW + j], dt = q - qt[(size_t)row * MW + jt];
-                            loss = fmaf(de, de, loss);
+                            loss[r] = fmaf(de, de, loss[r]);
                             d[c][r] = (de + dt) / (float)n;
                             dY[(size_t)row * MW + j] = d[c][r];
                         } else {
@@ -173,14 +175,25 @@ __global__ void __launch_bounds__(256) mlp_rows_kernel(const float* __restrict__
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
                     for (int r = 0; r < 8; ++r) ys[(c0 + 128 * c) * MR + rg + r] = d[c][r];
+                // each sample's sum over the warp's columns: the lanes first halve the
+                // eight samples among them, lane l ends with sample (l >> 2) in bit
+                // order 16, 8, 4
+                const int lane = tid & 31;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-                if ((tid & 31) == 0) red[tid >> 5] = loss;
+                for (int o = 16, h = 4; h > 0; o >>= 1, h >>= 1)
+#pragma unroll
+                    for (int r = 0; r < h; ++r) {
+                        const bool up = (lane & o) != 0;
+                        const float give = up ? loss[r] : loss[r + h];
+                        loss[r] = (up ? loss[r + h] : loss[r]) + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                loss[0] += __shfl_xor_sync(0xffffffffu, loss[0], 2);
+                loss[0] += __shfl_xor_sync(0xffffffffu, loss[0], 1);
+                if ((lane & 3) == 0) red[tid >> 5][lane >> 2] = loss[0];
                 __syncthreads();
-                if (tid == 0) {
-                    float s = 0.0f;
-                    for (int k = 0; k < 8; ++k) s += red[k];
-                    part[blockIdx.x] = s;
+                if (tid < MR && row0 + tid < n) {
+                    const float(*w4)[8] = red + 4 * (tid >> 3);  // the four warps of the sample's columns
+                    part[row0 + tid] = (w4[0][tid & 7] + w4[1][tid & 7]) + (w4[2][tid & 7] + w4[3][tid & 7]);
                 }
             }
         } else if (t == 24 || t == 32) {  // dZ = dH where the unit was on
@@ -273,14 +286,14 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(const float* __restrict__
 }
 
 // grad = sum of the splits (in order), then, with W, one Adam step (Kingma and Ba)
-// on the FP32 master weights and their bfloat16-rounded copy; the first CTA also
-// sums the loss.
+// on the FP32 master weights and their bfloat16-rounded copy; the last CTA sums the
+// samples' losses in FP64.
 __global__ void __launch_bounds__(256) mlp_update_kernel(const float* __restrict__ parts, int splits,
                                                          float* __restrict__ grad, float* __restrict__ W,
                                                          float* __restrict__ Wb, float* __restrict__ m,
                                                          float* __restrict__ v, float lr, float b1, float b2, float eps,
-                                                         float c1, float c2, const float* __restrict__ lpart, int nl,
-                                                         int n, float* __restrict__ loss) {
+                                                         float c1, float c2, const float* __restrict__ lpart, int n,
+                                                         float* __restrict__ loss) {
     const int t = blockIdx.x * 256 + threadIdx.x;
     if (t < (int)MLP_NPARAM) {
         float g = parts[t];
@@ -296,12 +309,18 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(const float* __restrict
             Wb[t] = mlp_bf16_round(w);
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
+    if (blockIdx.x + 1 == gridDim.x) {  // a CTA of its own: the loss
+        __shared__ double red[8];
         double s = 0.0;
-        for (int k = threadIdx.x; k < nl; k += 32) s += lpart[k];
+        for (int k = threadIdx.x; k < n; k += 256) s += lpart[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) loss[0] = (float)(s / n);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < 8; ++k) s += red[k];
+            loss[0] = (float)(s / n);
+        }
     }
 }
 
@@ -317,7 +336,7 @@ void launch_mlp_forward(const float* wb, const float* x, int n, float* q, cudaSt
                                                                          mlp_vec(wb, nullptr, nullptr));
 }
 
-// work: 9 n 256 + n floats (amdd_mlp_sizes): H1, H2, dY, dZ2, dZ1, the loss sums,
+// work: 9 n 256 + n floats (amdd_mlp_sizes): H1, H2, dY, dZ2, dZ1, the samples' losses,
 // then the gradient splits, as many as fit (at most 8, at least 128 samples each)
 void launch_mlp_step(float* w, float* wb, float* m, float* v, int t, float lr, const float* x, const float* qt, int n,
                      float* grad, float* work, float* loss, cudaStream_t s) {
@@ -337,8 +356,8 @@ void launch_mlp_step(float* w, float* wb, float* m, float* v, int t, float lr, c
     mlp_grad_kernel<<<dim3(36, splits), 256, 0, s>>>(x, H1, H2, dY, dZ2, dZ1, n, per, out, vec);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    mlp_update_kernel<<<((int)MLP_NPARAM + 255) / 256, 256, 0, s>>>(out, splits, grad, lr > 0.0f ? w : nullptr, wb, m, v,
-                                                                    lr, b1, b2, 1e-8f, c1, c2, lpart, nl, n, loss);
+    mlp_update_kernel<<<((int)MLP_NPARAM + 255) / 256 + 1, 256, 0, s>>>(out, splits, grad, lr > 0.0f ? w : nullptr, wb, m, v,
+                                                                    lr, b1, b2, 1e-8f, c1, c2, lpart, n, loss);
 }
 
 }  // namespace amdd
