@@ -144,7 +144,7 @@ struct amdd_handle {
     double* val = nullptr;
     // per-subdomain sizes
     std::vector<int32_t> nI, nG, nD, ni, nt, p;
-    std::vector<int64_t> off_om, off_sq, off_zt, off_I, coff;
+    std::vector<int64_t> off_om, off_sq, off_ii, off_zt, off_I, coff;  // off_sq, off_ii: n_i^2, n_I^2 summed
     int64_t sum_ni = 0, sum_sq = 0, sum_nI = 0, sum_nt = 0, nC = 0, sum_zt = 0;
     int max_ni = 0, max_nt = 0;
     // persistent device data of the apply
@@ -172,6 +172,9 @@ struct amdd_handle {
     // subdomain), in FP64 or FP32 (mixed form)
     FrontSolveT<double> lfs;
     FrontSolveT<float> lfs32;
+    // the same with the work vectors of the batched solves (ensure_multi)
+    FrontSolveT<double> m_fs, m_lfs;
+    FrontSolveT<float> m_lfs32;
     // eigenvectors of partial selections: 0 dense Jacobi, 1 LOBPCG from random
     // rows, 2 LOBPCG from the learned proposal
     int eig_solver = 0, keep_prop = 0;
@@ -321,7 +324,7 @@ struct PScope {
 // back asynchronous uploads are kept until the final synchronisation.
 struct Ctx {
     amdd_handle* h;
-    std::vector<void*> temps;
+    std::vector<std::pair<void*, size_t>> temps;  // with their bytes
     std::vector<std::shared_ptr<void>> keep;
     size_t tbytes = 0;  // bytes of the temporaries
     std::function<void()> overlap;  // work of the setup's other streams, run once where the host is free
@@ -337,7 +340,7 @@ struct Ctx {
         if (h->s2) cudaStreamSynchronize(h->s2);
         if (h->s3) cudaStreamSynchronize(h->s3);
         if (h->s4) cudaStreamSynchronize(h->s4);
-        for (void* p : temps) cudaFreeAsync(p, h->s);
+        for (const auto& t : temps) cudaFreeAsync(t.first, h->s);
         h->bytes_now -= std::min(h->bytes_now, tbytes);
     }
     template <class T>
@@ -345,9 +348,21 @@ struct Ctx {
         void* p = nullptr;
         account(h, std::max<size_t>(count, 1) * sizeof(T));
         ck(cudaMallocAsync(&p, std::max<size_t>(count, 1) * sizeof(T), h->s));
-        temps.push_back(p);
-        tbytes += std::max<size_t>(count, 1) * sizeof(T);
+        temps.push_back({p, std::max<size_t>(count, 1) * sizeof(T)});
+        tbytes += temps.back().second;
         return static_cast<T*>(p);
+    }
+    // frees a temporary behind the work issued so far on the handle's stream, which
+    // alone may use it
+    void release(const void* p) {
+        for (size_t k = 0; k < temps.size(); ++k)
+            if (temps[k].first == p) {
+                ck(cudaFreeAsync(temps[k].first, h->s));
+                h->bytes_now -= temps[k].second;
+                tbytes -= temps[k].second;
+                temps.erase(temps.begin() + k);
+                return;
+            }
     }
     template <class T>
     T* up(const std::vector<T>& v, bool persistent = false) {
@@ -826,6 +841,13 @@ void run_jacobi(Ctx& C, const std::vector<JacobiDescT<T>>& jd, const JacobiDescT
 // which then start from pairs that are orthogonal to ~1e-5 and converge in a
 // few sweeps.  `floor` adds the absolute rotation floor eps32 * max row norm^2
 // (used where only absolute accuracy of the rows is needed).
+// Whether the rows of a rows x ncols FP32 matrix are too large for the shared memory of
+// a cluster: the batch then takes the block-pair form, whose rows want jacobi_ld.
+bool jacobi_beyond_cluster(int rows, int ncols) {
+    return jacobi_block_smem<float>(rows, ncols, 2 * JAC_CLUSTER) > JAC_BLOCK_SMEM_MAX ||
+           cdiv(rows, 4 * JAC_CLUSTER) + 2 > JAC_MAX_PAIRS;
+}
+
 struct PrecondJob {
     const double* A;
     int R, L, lda;
@@ -838,10 +860,14 @@ void fp32_precondition(Ctx& C, const std::vector<PrecondJob>& jobs, bool floor, 
     const int nb = (int)jobs.size();
     if (nb == 0) return;
     std::vector<int64_t> o32(nb + 1, 0), oR(nb + 1, 0), oQ(nb + 1, 0), oL(nb + 1, 0);
+    std::vector<int> ld32(nb);
     int maxR = 1, maxL = 1;
+    bool pad = false;
+    for (const PrecondJob& j : jobs) pad = pad || jacobi_beyond_cluster(j.R, j.L + j.R);
     for (int b = 0; b < nb; ++b) {
         const int64_t R = jobs[b].R, L = jobs[b].L;
-        o32[b + 1] = o32[b] + R * (L + R);
+        ld32[b] = pad ? jacobi_ld((int)(L + R)) : (int)(L + R);
+        o32[b + 1] = o32[b] + R * ld32[b];
         oR[b + 1] = oR[b] + R;
         oQ[b + 1] = oQ[b] + R * R;
         oL[b + 1] = oL[b] + (int64_t)cdiv(R, CHOL_NB) * CHOL_NB * CHOL_NB;
@@ -859,8 +885,8 @@ void fp32_precondition(Ctx& C, const std::vector<PrecondJob>& jobs, bool floor, 
     std::vector<JacobiDescT<float>> jd(nb);
     for (int b = 0; b < nb; ++b) {
         const PrecondJob& j = jobs[b];
-        cd[b] = {j.A, j.R, j.L, j.lda, m32 + o32[b], Qraw + oQ[b]};
-        jd[b] = {m32 + o32[b], j.R, j.L + j.R, j.L, j.L + j.R, n32 + oR[b], floor ? f32 + b : nullptr};
+        cd[b] = {j.A, j.R, j.L, j.lda, m32 + o32[b], ld32[b], Qraw + oQ[b]};
+        jd[b] = {m32 + o32[b], j.R, ld32[b], j.L, j.L + j.R, n32 + oR[b], floor ? f32 + b : nullptr};
     }
     const CvtDesc* dcd = C.up(cd);
     const JacobiDescT<float>* djd = C.up(jd);
@@ -1494,9 +1520,8 @@ void mf_local_eigs(Ctx& C, amdd_handle* h, const double* X1, const std::vector<i
             if (h->nI[i] == 0) continue;
             pd.push_back({X1 + off_x[i], h->nt[i], h->nG[i] + h->nD[i], h->ni[i], h->nI[i], sig + h->off_om[i],
                           delta + i, Cc + oc[i], Bm + oc[i]});
-            // L_A (leading nI x nI block of the Cholesky factor of A_ii) enters
-            // full GEMMs: clear the rest of its rows
-            zu.push_back({Lb + h->off_sq[i], h->ni[i], 0, h->nI[i], h->nI[i], i});
+            // L_A enters full GEMMs: clear its upper triangle
+            zu.push_back({Lb + h->off_ii[i], h->nI[i], 0, h->nI[i], h->nI[i], i});
         }
         if (pd.empty()) return;
         auto a = C.up(pd);
@@ -1568,13 +1593,13 @@ void mf_local_eigs(Ctx& C, amdd_handle* h, const double* X1, const std::vector<i
             for (int q = 0; q < nq; ++q) {
                 if (r[q] == 0) continue;
                 const int i = todo[q], ni = h->ni[i], nI = n[q];
-                const double* LA = Lb + h->off_sq[i];
+                const double* LA = Lb + h->off_ii[i];
                 double* Y = Ybuf + q * stride;
                 double* W = Wbuf + q * wstride;
-                g1.push_back(gd(in + q * stride, ld, 0, LA, ni, 1, Y, ld, r[q], nI, nI, 1.0, 0.0, 0));
+                g1.push_back(gd(in + q * stride, ld, 0, LA, nI, 1, Y, ld, r[q], nI, nI, 1.0, 0.0, 0));
                 g2.push_back(gd(Y, ld, 0, Cc + oc[i], nI, 1, W, maxni, r[q], ni, nI, 1.0, 0.0, 0));
                 g3.push_back(gd(W, maxni, 0, Bm + oc[i], nI, 0, Y, ld, r[q], nI, ni, -1.0, 1.0, 0));
-                g4.push_back(gd(Y, ld, 0, LA, ni, 0, out + q * stride, ld, r[q], nI, nI, -1.0 / dl[i], 0.0, 0));
+                g4.push_back(gd(Y, ld, 0, LA, nI, 0, out + q * stride, ld, r[q], nI, nI, -1.0 / dl[i], 0.0, 0));
             }
             gemm(C, g1);
             gemm(C, g2);
@@ -1732,13 +1757,13 @@ std::vector<int> learned_eigvecs(Ctx& C, amdd_handle* h, const std::vector<int>&
         int maxn = 1;
         std::vector<GemmDescT<T>> g1, g2;
         for (int q = 0; q < np; ++q) {
-            const int i = partial[q], ni = h->ni[i];
-            zu[q] = {Lb + h->off_sq[i], ni, 0, n[q], n[q], i};
+            const int i = partial[q];
+            zu[q] = {Lb + h->off_ii[i], n[q], 0, n[q], n[q], i};
             maxn = std::max(maxn, n[q]);
             if (m[q] == 0) continue;
             g1.push_back(gd<T>(WtT + (int64_t)q * PROP_NO, PROP_NB, 0, BtT + off_b[q], n[q], 0, U0 + xoff[q], n[q], m[q],
                                n[q], PROP_NB, 1.0, 0.0, 0));
-            g2.push_back(gd<T>(U0 + xoff[q], n[q], 0, Lb + h->off_sq[i], ni, 0, X0 + xoff[q], n[q], m[q], n[q], n[q], 1.0,
+            g2.push_back(gd<T>(U0 + xoff[q], n[q], 0, Lb + h->off_ii[i], n[q], 0, X0 + xoff[q], n[q], m[q], n[q], n[q], 1.0,
                                0.0, 0));
         }
         {
@@ -1862,17 +1887,18 @@ struct FrontEntries {
     std::vector<int64_t> src, diag;
 };
 
-// Factors a matrix (the entries sp, or the dense lower triangle E of order nE in
-// the caller's order) in the plan's stages: each part's front collects its
+// Factors a matrix (the entries sp, or gathered from a dense lower triangle per
+// front, dense) in the plan's stages: each part's front collects its
 // entries and its children's Schur complements, a partial Cholesky eliminates the
 // interior, and the interior's inverse Ainv = Y^T Y (Y = L_II^{-1}) and W^T =
 // L_BI Y are kept for the solve.  All of this in FP64; with T = float (the local
 // solves of the mixed form) Ainv and W are rounded once at the end, so that the
 // solve carries only that rounding and its own FP32 sums (one-level apply on 24^3,
-// relative error 7e-8; with FP32 factors 4e-7 to 7e-7).
+// relative error 7e-8; with FP32 factors 4e-7 to 7e-7).  What a stage needs beside
+// the fronts (Y and W^T in FP64) is shared by the stages.
 template <typename T>
 void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& P, const FrontEntries* sp,
-                   const double* E, int64_t nE) {
+                   const std::vector<FrontSrc>& dense) {
     cudaStream_t s = h->s;
     const int nf = (int)P.fronts.size(), S = P.stages();
     std::vector<FrontDevT<double>> fd(nf);  // of the factorisation
@@ -1885,23 +1911,26 @@ void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& 
         oW[k + 1] = oW[k] + m * b;
         oL[k + 1] = oL[k] + (int64_t)cdiv(m, CHOL_NB) * CHOL_NB * CHOL_NB;
     }
+    // (at most 32768 fronts a launch: some kernels count the matrices in a
+    // 16-bit grid dimension)
+    std::vector<std::pair<int, int>> batches;
+    int64_t bA = 0, bW = 0, bL = 0;
+    for (int st = 0; st < S; ++st)
+        for (int k0 = P.stage_part[st]; k0 < P.stage_part[st + 1]; k0 += 32768) {
+            const int k1 = std::min(P.stage_part[st + 1], k0 + 32768);
+            batches.push_back({k0, k1});
+            bA = std::max(bA, oA[k1] - oA[k0]);
+            bW = std::max(bW, oW[k1] - oW[k0]);
+            bL = std::max(bL, oL[k1] - oL[k0]);
+        }
     constexpr bool f64 = std::is_same<T, double>::value;
     double* F = C.tnew<double>(oF[nf]);
-    double* Y = C.tnew<double>(oA[nf]);
-    double* linv = C.tnew<double>(oL[nf]);
+    double* linv = C.tnew<double>(bL);
     T* Aik = dnew<T>(h, oA[nf]);
     T* Wk = dnew<T>(h, oW[nf]);
     T* Wtk = dnew<T>(h, oW[nf]);
-    double *Ai, *W, *Wt;
-    if constexpr (f64) {
-        Ai = Aik;
-        W = Wk;
-        Wt = Wtk;
-    } else {
-        Ai = C.tnew<double>(oA[nf]);
-        W = C.tnew<double>(oW[nf]);
-        Wt = C.tnew<double>(oW[nf]);
-    }
+    double* Yb = f64 ? nullptr : C.tnew<double>(bA);  // Y and W^T of a batch (FP64: in Ainv's and W^T's place)
+    double* Wb = f64 ? nullptr : C.tnew<double>(bW);
     ck(cudaMemsetAsync(F, 0, oF[nf] * sizeof(double), s));
 
     // children of each front, with the maps between their boundary and its rows
@@ -1913,7 +1942,7 @@ void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& 
     std::vector<int32_t> at(P.n, -1);
     for (int k = 0; k < nf; ++k) {
         const Front& f = P.fronts[k];
-        fd[k] = {F + oF[k], Ai + oA[k], W + oW[k], f.m, f.nb, f.i0, f.b0, (int)ch.size(), 0};
+        fd[k] = {F + oF[k], nullptr, nullptr, f.m, f.nb, f.i0, f.b0, (int)ch.size(), 0};
         if (!kids[k].empty()) {
             for (int a = 0; a < f.m; ++a) at[f.i0 + a] = a;
             for (int b = 0; b < f.nb; ++b) at[P.bnd[f.b0 + b]] = f.m + b;
@@ -1999,72 +2028,78 @@ void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& 
     fs.down_rows = C.up(drow, true);
     fs.down_ptr = C.up(dptr, true);
     fs.refs = C.up(refs, true);
-    fs.v = dnew<T>(h, (size_t)MAXB * P.n);
-    fs.e = dnew<T>(h, (size_t)MAXB * P.n);
+    fs.v = dnew<T>(h, P.n);
+    fs.e = dnew<T>(h, P.n);
     fs.entries = (double)(oA[nf] + 2 * oW[nf]);
     const FrontChild* dch = C.up(ch);
     const int32_t* dmaps = C.up(maps);
 
-    for (int st = 0; st < S; ++st)
-        // (at most 32768 fronts a launch: some kernels count the matrices in a
-        // 16-bit grid dimension)
-        for (int k0 = P.stage_part[st]; k0 < P.stage_part[st + 1]; k0 += 32768) {
-            const int k1 = std::min(P.stage_part[st + 1], k0 + 32768);
-            int maxn = 1, maxm = 1;
-            bool add = false;
-            std::vector<CholDesc> cd;
-            std::vector<TrtriDesc> td;
-            std::vector<GemmDesc> ga, gw;
-            std::vector<double*> mats;
-            std::vector<int> mm;
-            std::vector<TransDesc> tr;
-            for (int k = k0; k < k1; ++k) {
-                const int m = P.fronts[k].m, b = P.fronts[k].nb, n = m + b;
-                maxn = std::max(maxn, n);
-                maxm = std::max(maxm, std::max(m, b));
-                add = add || !kids[k].empty();
-                cd.push_back({F + oF[k], n, n, m, nullptr, linv + oL[k]});
-                td.push_back({F + oF[k], Y + oA[k], linv + oL[k], m, n, m});
-                GemmDesc g = gd<double>(Y + oA[k], m, 1, Y + oA[k], m, 0, Ai + oA[k], m, m, m, m, 1.0, 0.0, 1);
-                g.kfrom_row = 1;
-                ga.push_back(g);
-                mats.push_back(Ai + oA[k]);
-                mm.push_back(m);
-                if (b > 0) {
-                    gw.push_back(gd<double>(F + oF[k] + (size_t)m * n, n, 0, Y + oA[k], m, 0, Wt + oW[k], m, b, m, m, 1.0,
-                                       0.0, 0));
-                    tr.push_back({Wt + oW[k], W + oW[k], b, m, m, b});
-                }
+    const FrontSrc* dsrc = sp ? nullptr : C.up(dense);
+    for (const auto& range : batches) {
+        const int k0 = range.first, k1 = range.second;
+        int maxn = 1, maxm = 1;
+        bool add = false;
+        std::vector<CholDesc> cd;
+        std::vector<TrtriDesc> td;
+        std::vector<GemmDesc> ga, gw;
+        std::vector<double*> mats;
+        std::vector<T*> keep;
+        std::vector<int> mm, ld;
+        std::vector<TransDescT<T>> tr;
+        for (int k = k0; k < k1; ++k) {
+            const int m = P.fronts[k].m, b = P.fronts[k].nb, n = m + b;
+            maxn = std::max(maxn, n);
+            maxm = std::max(maxm, std::max(m, b));
+            add = add || !kids[k].empty();
+            double *Yk, *Wt;
+            if constexpr (f64) {
+                Yk = Aik + oA[k];
+                Wt = Wtk + oW[k];
+            } else {
+                Yk = Yb + (oA[k] - oA[k0]);
+                Wt = Wb + (oW[k] - oW[k0]);
             }
-            if (!sp) {
-                PScope ps(h, PK_E_ASM, 0.0);
-                launch_front_gather(dfd + k0, k1 - k0, fs.bnd, fs.perm, E, nE, maxn, s);
-            }
-            if (add) {
-                PScope ps(h, PK_SMALL);
-                launch_front_extend_add(dfd + k0, k1 - k0, dch, dmaps, maxn, s);
-            }
-            chol_batched<double>(C, cd);
-            trtri_batched<double>(C, td);
-            gemm(C, ga);
-            gemm(C, gw);
-            {
-                auto a = C.up(mats);
-                auto b = C.up(mm);
-                PScope ps(h, PK_SMALL);
-                launch_mirror_lower<double>(a, b, b, (int)mats.size(), maxm, s);
-            }
-            if (!tr.empty()) {
-                auto t = C.up(tr);
-                PScope ps(h, PK_SMALL);
-                launch_transpose_rect(t, (int)tr.size(), maxm, s);
+            cd.push_back({F + oF[k], n, n, m, nullptr, linv + (oL[k] - oL[k0])});
+            td.push_back({F + oF[k], Yk, linv + (oL[k] - oL[k0]), m, n, m});
+            // Ainv comes first in place of L_II, which Y has replaced
+            GemmDesc g = gd<double>(Yk, m, 1, Yk, m, 0, F + oF[k], n, m, m, m, 1.0, 0.0, 1);
+            g.kfrom_row = 1;
+            ga.push_back(g);
+            mats.push_back(F + oF[k]);
+            keep.push_back(Aik + oA[k]);
+            mm.push_back(m);
+            ld.push_back(n);
+            if (b > 0) {
+                gw.push_back(gd<double>(F + oF[k] + (size_t)m * n, n, 0, Yk, m, 0, Wt, m, b, m, m, 1.0, 0.0, 0));
+                tr.push_back({Wtk + oW[k], Wk + oW[k], b, m, m, b});
             }
         }
-    if constexpr (!f64) {
-        PScope ps(h, PK_SMALL);
-        launch_convert<double, float>(Ai, Aik, oA[nf], s);
-        launch_convert<double, float>(W, Wk, oW[nf], s);
-        launch_convert<double, float>(Wt, Wtk, oW[nf], s);
+        if (!sp) {
+            PScope ps(h, PK_E_ASM, 0.0);
+            launch_front_gather(dfd + k0, dsrc + k0, k1 - k0, fs.bnd, fs.perm, maxn, s);
+        }
+        if (add) {
+            PScope ps(h, PK_SMALL);
+            launch_front_extend_add(dfd + k0, k1 - k0, dch, dmaps, maxn, s);
+        }
+        chol_batched<double>(C, cd);
+        trtri_batched<double>(C, td);
+        gemm(C, ga);
+        gemm(C, gw);
+        {
+            auto a = C.up(mats);
+            auto b = C.up(mm);
+            auto c = C.up(ld);
+            PScope ps(h, PK_SMALL);
+            launch_mirror_lower<double>(a, b, c, (int)mats.size(), maxm, s);
+            launch_convert_blocks<double, T>(a, c, C.up(keep), b, b, (int)mats.size(), maxm, s);
+        }
+        if (!tr.empty()) {
+            auto t = C.up(tr);
+            PScope ps(h, PK_SMALL);
+            if constexpr (!f64) launch_convert<double, float>(Wb, Wtk + oW[k0], oW[k1] - oW[k0], s);
+            launch_transpose_rect<T>(t, (int)tr.size(), maxm, s);
+        }
     }
 }
 
@@ -2258,8 +2293,17 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     h->off_om.assign(N + 1, 0);
     h->off_sq.assign(N + 1, 0);
     h->off_I.assign(N + 1, 0);
-    std::vector<int> ldx(N);  // leading dimensions of the X_i
-    std::vector<int64_t> off_x(N + 1, 0), off_m(N + 1, 0), off_ti(N + 1, 0), off_P(N + 1, 0), off_la(N + 1, 0),
+    // leading dimensions of the X_i: padded for the block-pair Jacobi in FP32 (rows beyond
+    // the shared memory of a cluster)
+    std::vector<int> ldx(N);
+    bool pad_x = false;
+    for (int i = 0; i < N && !s64; ++i) {
+        const int ni = (int)(Il[i].size() + Gl[i].size()), nt = ni + (int)Dl[i].size();
+        pad_x = pad_x || jacobi_beyond_cluster(ni, nt);
+    }
+    h->off_ii.assign(N + 1, 0);
+    std::vector<int64_t>& off_P = h->off_ii;
+    std::vector<int64_t> off_x(N + 1, 0), off_m(N + 1, 0), off_ti(N + 1, 0), off_la(N + 1, 0),
         off_lm(N + 1, 0);
     for (int i = 0; i < N; ++i) {
         const int a = (int)Il[i].size(), b = (int)Gl[i].size(), c = (int)Dl[i].size();
@@ -2272,7 +2316,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         h->off_om[i + 1] = h->off_om[i] + ni;
         h->off_sq[i + 1] = h->off_sq[i] + ni * ni;
         h->off_I[i + 1] = h->off_I[i] + a;
-        ldx[i] = s64 ? (int)nt : jacobi_ld((int)nt);
+        ldx[i] = pad_x ? jacobi_ld((int)nt) : (int)nt;
         off_x[i + 1] = off_x[i] + ni * ldx[i];
         off_m[i + 1] = off_m[i] + nt * nt;
         off_ti[i + 1] = off_ti[i] + (int64_t)a * 2 * a;
@@ -2294,7 +2338,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     // X_i = R_i A tilde R_i^T with columns ordered [G, D, I] (Eq. (Xi)).
     std::vector<int32_t> omega(h->sum_ni);
     std::vector<int64_t> pa_src, pa_dst, px_src, px_dst;
-    FrontEntries le;  // lower triangles of all A_ii (unknown: position in omega)
+    std::vector<int32_t> la_row, la_col;  // graph of all A_ii, lower triangles (positions in omega)
     {
         std::vector<int32_t> stamp(n, -1), posA(n, -1), posX(n, -1);
         for (int i = 0; i < N; ++i) {
@@ -2329,10 +2373,9 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                     if (posA[c] >= 0) {
                         pa_src.push_back(k);
                         pa_dst.push_back(h->off_sq[i] + (int64_t)a * ni + posA[c]);
-                        if (posA[c] <= a) {
-                            le.row.push_back((int32_t)(h->off_om[i] + a));
-                            le.col.push_back((int32_t)(h->off_om[i] + posA[c]));
-                            le.src.push_back(k);
+                        if (posA[c] < a) {
+                            la_row.push_back((int32_t)(h->off_om[i] + a));
+                            la_col.push_back((int32_t)(h->off_om[i] + posA[c]));
                         }
                     }
                     px_src.push_back(k);
@@ -2345,7 +2388,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     // ---- device buffers
     h->d_omega = C.up(omega, true);
     double* Araw = C.tnew<double>(h->sum_sq);
-    T* Lb = C.tnew<T>(h->sum_sq);
+    T* Lb = C.tnew<T>(off_P[N]);  // A_II, then its factor L_A
     double* Xp = C.tnew<double>(off_x[N]);
     // the matrix-free eigensolve (eig_solver 3) forms none of Abar_ii, its
     // Schur complement or T_i
@@ -2363,7 +2406,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     unsigned long long* rots = C.tnew<unsigned long long>(4 * N);
     ck(cudaMemsetAsync(rots, 0, 4 * N * sizeof(unsigned long long), s));
     TS* nrmT = C.tnew<TS>(h->sum_ni);
-    T* Yl = C.tnew<T>(h->sum_sq);  // L_A^{-1}, the leading nI x nI block of an ni x ni array
+    T* Yl = C.tnew<T>(off_P[N]);  // L_A^{-1}
     ck(cudaMemsetAsync(Araw, 0, h->sum_sq * sizeof(double), s));
     ck(cudaMemsetAsync(Xp, 0, off_x[N] * sizeof(double), s));
     {
@@ -2379,11 +2422,27 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             PScope ps(h, PK_GATHER, 0.0, 32.0 * px_src.size());
             launch_gather_values(sx, dx, (int64_t)px_src.size(), h->val, Xp, s);
         }
+        C.release(sa);
+        C.release(da);
+        C.release(sx);
+        C.release(dx);
     }
-    if constexpr (f64)
-        ck(cudaMemcpyAsync(Lb, Araw, h->sum_sq * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    else
-        launch_convert<double, float>(Araw, Lb, h->sum_sq, s);
+    {
+        std::vector<const double*> src(N);
+        std::vector<T*> dst(N);
+        int maxn = 1;
+        for (int i = 0; i < N; ++i) {
+            src[i] = Araw + h->off_sq[i];
+            dst[i] = Lb + off_P[i];
+            maxn = std::max(maxn, h->nI[i]);
+        }
+        auto a = C.up(src);
+        auto b = C.up(h->ni);
+        auto c = C.up(dst);
+        auto d = C.up(h->nI);
+        for (int i0 = 0; i0 < N; i0 += 32768)  // (a 16-bit grid dimension)
+            launch_convert_blocks<double, T>(a + i0, b + i0, c + i0, d + i0, d + i0, std::min(N - i0, 32768), maxn, s);
+    }
 
     // full selections: the basis diag(A_II)^{-1/2} keeps every block of E that
     // touches such a subdomain as sparse as A (and the separators of its
@@ -2597,7 +2656,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             std::vector<int32_t> aptr, adj;
             front_graph((int)base.size(), h->all_diag ? sp.row : ea, h->all_diag ? sp.col : eb, !h->all_diag, aptr, adj);
             const FrontPlan plan = plan_fronts(aptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO);
-            factor_fronts<double>(C, h, h->fs, plan, h->all_diag ? &sp : nullptr, E, nC);
+            factor_fronts<double>(C, h, h->fs, plan, h->all_diag ? &sp : nullptr,
+                                  std::vector<FrontSrc>(plan.fronts.size(), FrontSrc{E, nC, 0}));
             if (h->all_diag) h->fs.src = C.up(plan_globals(plan, Il), true);
         }
     };
@@ -2647,7 +2707,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             if (!h->sparse_local) {
                 std::vector<int32_t> ptr, adj, wt(h->sum_ni, 1), base(h->sum_ni), src(h->sum_ni);
                 std::iota(base.begin(), base.end(), 0);
-                front_graph((int)h->sum_ni, le.row, le.col, false, ptr, adj);
+                front_graph((int)h->sum_ni, la_row, la_col, false, ptr, adj);
                 const FrontPlan P = plan_fronts(ptr, adj, wt, base, FRONT_LEAF, FRONT_RATIO);
                 local_pos.resize(h->sum_ni);
                 for (int64_t k = 0; k < P.n; ++k) {
@@ -2655,7 +2715,14 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                     src[k] = omega[P.perm[k]];
                 }
                 FrontSolveT<T>& lf = local_fronts<T>(h);
-                factor_fronts<T>(C, h, lf, P, &le, nullptr, 0);
+                std::vector<FrontSrc> from;  // a part lies in one subdomain
+                from.reserve(P.fronts.size());
+                for (const Front& f : P.fronts) {
+                    const int i = (int)(std::upper_bound(h->off_om.begin(), h->off_om.end(), P.perm[f.i0]) -
+                                        h->off_om.begin()) - 1;
+                    from.push_back({Araw + h->off_sq[i], h->ni[i], h->off_om[i]});
+                }
+                factor_fronts<T>(C, h, lf, P, nullptr, from);
                 lf.src = C.up(src, true);
             }
             ck(cudaEventRecord(h->ev_spec_done, h->s));
@@ -2672,12 +2739,14 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         std::vector<CholDescT<T>> cd(N);
         std::vector<TrtriDescT<T>> td(N);
         for (int i = 0; i < N; ++i) {
-            const int ni = h->ni[i], nIi = h->nI[i];
-            cd[i] = {Lb + h->off_sq[i], nIi, ni, nIi, nullptr, linvA + off_la[i]};
-            td[i] = {Lb + h->off_sq[i], Yl + h->off_sq[i], linvA + off_la[i], nIi, ni, ni};
+            const int nIi = h->nI[i];
+            cd[i] = {Lb + off_P[i], nIi, nIi, nIi, nullptr, linvA + off_la[i]};
+            td[i] = {Lb + off_P[i], Yl + off_P[i], linvA + off_la[i], nIi, nIi, nIi};
         }
         chol_batched(C, cd);
         trtri_batched(C, td);
+        C.release(linvA);
+        if (!mf && h->eig_solver == 0 && !h->keep_prop) C.release(Lb);  // (L_A itself is for those eigensolvers)
     }
 
     // ---- (1b) sparse Cholesky factors of the A_ii in a nested-dissection order
@@ -2709,6 +2778,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         }
         fp32_precondition(C, pj, false, 40, sweeps + 2 * N, rots + 2 * N);
         gemm(C, g);
+        C.release(Xp);
+        C.release(Q);
         std::vector<JacobiDesc> jd(N);
         std::vector<double*> sp(N);
         int maxc = 1;
@@ -2731,6 +2802,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
     else {
         // FP32 splitting: one-sided Jacobi on the rows of X_i alone
         launch_convert<double, float>(Xp, X1, off_x[N], s);
+        C.release(Xp);
         std::vector<JacobiDescT<float>> jd(N);
         std::vector<double*> sp(N);
         int maxc = 1;
@@ -2808,7 +2880,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 mats[i] = S;
                 nn[i] = nIi;
                 ld[i] = nt;
-                const T* Y = Yl + h->off_sq[i];
+                const T* Y = Yl + off_P[i];
                 const T* Sl;
                 int lds;
                 if constexpr (std::is_same<T, TS>::value) {
@@ -2822,8 +2894,8 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 cdst[i] = Sc ? Sc + off_P[i] : nullptr;
                 cls[i] = nt;
                 cld[i] = nIi;
-                g1[i] = gd(Y, ni, 0, Sl, lds, 0, Pb + off_P[i], nIi, nIi, nIi, nIi, 1.0, 0.0, 0);
-                g2[i] = gd(Pb + off_P[i], nIi, 0, Y, ni, 1, TI + off_ti[i], 2 * nIi, nIi, nIi, nIi, 1.0, 0.0, 0);
+                g1[i] = gd(Y, nIi, 0, Sl, lds, 0, Pb + off_P[i], nIi, nIi, nIi, nIi, 1.0, 0.0, 0);
+                g2[i] = gd(Pb + off_P[i], nIi, 0, Y, nIi, 1, TI + off_ti[i], 2 * nIi, nIi, nIi, nIi, 1.0, 0.0, 0);
                 idd[i] = {nullptr, TI + off_ti[i] + nIi, nullptr, nIi, 0, 2 * nIi};
             }
             {
@@ -2931,10 +3003,10 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 std::vector<GemmDescT<T>> g1, g2;
                 for (int q = 0; q < nf; ++q) {
                     const int i = F[q], ni = h->ni[i], nIi = h->nI[i];
-                    const T* Y = Yl + h->off_sq[i];  // L_A^{-1}: leading nI x nI block of L_i^{-1}
+                    const T* Y = Yl + off_P[i];  // L_A^{-1}
                     const double dv = (double)dl[i];
-                    g1.push_back(gd<T>(WT + ow[q], nIi, 0, Y, ni, 1, P + ow[q], nIi, ni, nIi, nIi, 1.0, 0.0, 0));
-                    g1.push_back(gd<T>(Y, ni, 0, Y, ni, 1, TI + off_ti[i], 2 * nIi, nIi, nIi, nIi, dv, 0.0, 0));
+                    g1.push_back(gd<T>(WT + ow[q], nIi, 0, Y, nIi, 1, P + ow[q], nIi, ni, nIi, nIi, 1.0, 0.0, 0));
+                    g1.push_back(gd<T>(Y, nIi, 0, Y, nIi, 1, TI + off_ti[i], 2 * nIi, nIi, nIi, nIi, dv, 0.0, 0));
                     g2.push_back(gd<T>(P + ow[q], nIi, 1, P + ow[q], nIi, 0, TI + off_ti[i], 2 * nIi, nIi, nIi, ni, dv,
                                        1.0, 0));
                 }
@@ -3100,7 +3172,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             for (int i = 0; i < N; ++i) {
                 if (h->p[i] != h->nI[i] || h->p[i] == 0 || diag_basis) continue;
                 for (int k = 0; k < h->nI[i]; ++k) {
-                    ysrc.push_back(h->off_sq[i] + (int64_t)k * h->ni[i]);
+                    ysrc.push_back(off_P[i] + (int64_t)k * h->nI[i]);
                     ydst.push_back(h->off_zt[i] + (int64_t)k * h->nI[i]);
                     ylen.push_back(h->nI[i]);
                 }
@@ -3214,7 +3286,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
             if (!partial.empty()) {
                 std::vector<GemmDescT<T>> g;
                 for (int i : partial)
-                    g.push_back(gd<T>(Wsel + h->off_zt[i], h->nI[i], 0, Yl + h->off_sq[i], h->ni[i], 0,
+                    g.push_back(gd<T>(Wsel + h->off_zt[i], h->nI[i], 0, Yl + off_P[i], h->nI[i], 0,
                                       ZtT + h->off_zt[i], h->nI[i], h->p[i], h->nI[i], h->nI[i], 1.0, 0.0, 0));
                 gemm(C, g);
             }
@@ -3524,6 +3596,12 @@ void spmv_pq_h(amdd_handle* h) {
 // Buffers and descriptors of the batched path (MAXB right-hand sides), on first use.
 void ensure_multi(amdd_handle* h) {
     if (h->mb_cap >= MAXB) return;
+    auto batched = [&](auto& m, const auto& one) {
+        m = one;
+        if (one.n <= 0) return;
+        m.v = dnew<std::remove_pointer_t<decltype(m.v)>>(h, MAXB * one.n);
+        m.e = dnew<std::remove_pointer_t<decltype(m.e)>>(h, MAXB * one.n);
+    };
     const int64_t L = (int64_t)MAXB * h->sum_ni, V = (int64_t)MAXB * h->n, CC = (int64_t)MAXB * std::max<int64_t>(h->nC, 1);
     if (h->sparse_local || (h->nC > 0 && !h->all_diag)) h->d_m_rloc = dnew<double>(h, L);
     if (h->sparse_local) {
@@ -3534,9 +3612,12 @@ void ensure_multi(amdd_handle* h) {
             h->d_m_yloc32 = dnew<float>(h, L);
         }
     } else {
-        h->d_m_yloc = h->lfs.e;
-        h->d_m_yloc32 = h->lfs32.e;
+        batched(h->m_lfs, h->lfs);
+        batched(h->m_lfs32, h->lfs32);
+        h->d_m_yloc = h->m_lfs.e;
+        h->d_m_yloc32 = h->m_lfs32.e;
     }
+    batched(h->m_fs, h->fs);
     h->d_m_c = dnew<double>(h, CC);
     h->d_m_e = dnew<double>(h, CC);
     if (h->nC > 0) {
@@ -3591,7 +3672,7 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb, const DotAr
         side.run([&] {
             if (h->all_diag) {
                 PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
-                launch_front_solve<double>(h->fs, r, h->n, h->d_m_zc, h->n, nb, h->s);
+                launch_front_solve<double>(h->m_fs, r, h->n, h->d_m_zc, h->n, nb, h->s);
                 return;
             }
             const double zt = (double)h->sum_zt;
@@ -3601,16 +3682,16 @@ void apply_multi(amdd_handle* h, const double* r, double* z, int nb, const DotAr
             }
             {
                 PScope ps(h, PK_CSOLVE, 2.0 * h->fs.entries * nb, 8.0 * h->fs.entries + 48.0 * h->nC * nb);
-                launch_front_solve<double>(h->fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, h->s);
+                launch_front_solve<double>(h->m_fs, h->d_m_c, h->nC, h->d_m_e, h->nC, nb, h->s);
             }
             PScope ps(h, PK_GEMV, 2.0 * zt * nb, 8.0 * zt + (8.0 * h->nC + 8.0 * h->n) * nb);
             launch_gemv_rows_multi<double>(h->d_m_gv_zp, h->d_rd_zp, h->d_rl_zp, h->n_zp, nb, h->nC, h->n, h->s);
         });
     if (!h->sparse_local) {
         if (h->precision == 0)
-            front_local_solves<double>(h, h->lfs, r, nb);
+            front_local_solves<double>(h, h->m_lfs, r, nb);
         else
-            front_local_solves<float>(h, h->lfs32, r, nb);
+            front_local_solves<float>(h, h->m_lfs32, r, nb);
     } else if (h->precision == 0) {
         sparse_local_solves<double>(h, h->d_m_rloc, h->d_m_yloc, nb, L);
     } else {

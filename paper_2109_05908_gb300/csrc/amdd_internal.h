@@ -112,7 +112,8 @@ using JacobiDesc = JacobiDescT<double>;
 struct CvtDesc {
     const double* A;  // rows x L (lda)
     int rows, L, lda;
-    float* out32;     // rows x (L + rows)
+    float* out32;     // rows x (L + rows), ld32
+    int ld32;
     double* Q;        // rows x rows
 };
 
@@ -368,12 +369,15 @@ void launch_scatter_prolong(int64_t n, const int32_t* order_g, const int64_t* sc
                             int64_t ldzc = 0, int64_t ldz = 0, const double* r = nullptr,
                             const DotArgs* d = nullptr);
 // batched rectangular transposes: dst (cols x rows, leading dimension ldd) = src^T
-struct TransDesc {
-    const double* src;
-    double* dst;
+template <typename T>
+struct TransDescT {
+    const T* src;
+    T* dst;
     int rows, cols, lds, ldd;
 };
-void launch_transpose_rect(const TransDesc* d, int nmat, int maxdim, cudaStream_t s);
+using TransDesc = TransDescT<double>;
+template <typename T>
+void launch_transpose_rect(const TransDescT<T>* d, int nmat, int maxdim, cudaStream_t s);
 struct EPairRef {
     int i, j;          // block E_ij, i > j
     int64_t list_off;  // entries [list_off, list_off + list_len)
@@ -511,13 +515,18 @@ struct FrontSolveT {
     const int32_t* down_rows = nullptr;  // boundary unknowns of each stage's parts
     const int32_t* down_ptr = nullptr;   // their refs (one shared list, nrow + 1 pointers over all stages)
     const FrontRefT<T>* refs = nullptr;
-    T* v = nullptr;  // MAXB vectors of n each
+    T* v = nullptr;  // work and solution: as many vectors of n each as a solve is given
     T* e = nullptr;
     std::vector<int64_t> down_off, row_off;  // host: per stage
     double entries = 0.0;                    // host: stored entries (multiply-adds of one solve)
 };
-void launch_front_gather(const FrontDevT<double>* fr, int nfr, const int32_t* bnd, const int32_t* perm,
-                         const double* E, int64_t nE, int maxn, cudaStream_t s);
+// the dense matrix (lower triangle) that a front is gathered from: unknown u is its row u - off
+struct FrontSrc {
+    const double* A;
+    int64_t ld, off;
+};
+void launch_front_gather(const FrontDevT<double>* fr, const FrontSrc* src, int nfr, const int32_t* bnd,
+                         const int32_t* perm, int maxn, cudaStream_t s);
 // scale[k] = own[perm[k]] = 1 / sqrt(val[diag[k]]) (val 0 where diag[k] < 0), k < n
 void launch_front_scale(const double* val, const int64_t* diag, const int32_t* perm, double* scale, double* own,
                         int64_t n, cudaStream_t s);

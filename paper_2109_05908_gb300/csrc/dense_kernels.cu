@@ -896,13 +896,13 @@ void launch_row_maxnorm2(const JacobiDescT<T>* d, int nmat, T eps, T* out, cudaS
 template void launch_row_maxnorm2<float>(const JacobiDescT<float>*, int, float, float*, cudaStream_t);
 template void launch_row_maxnorm2<double>(const JacobiDescT<double>*, int, double, double*, cudaStream_t);
 
-// out32 (rows x (L + rows), ld L + rows) = [float(A) | I] for A rows x L (lda).
+// out32 (rows x (L + rows), ld32) = [float(A) | I] for A rows x L (lda).
 __global__ void to_f32_with_identity_kernel(const CvtDesc* __restrict__ descs) {
     const CvtDesc d = descs[blockIdx.y];
     const int w = d.L + d.rows;
     for (int r = blockIdx.x; r < d.rows; r += gridDim.x) {
         const double* a = d.A + (size_t)r * d.lda;
-        float* o = d.out32 + (size_t)r * w;
+        float* o = d.out32 + (size_t)r * d.ld32;
         for (int c = threadIdx.x; c < w; c += blockDim.x) o[c] = (c < d.L) ? (float)a[c] : (c - d.L == r ? 1.f : 0.f);
     }
 }
@@ -916,9 +916,8 @@ void launch_to_f32_with_identity(const CvtDesc* d, int nmat, int maxrows, cudaSt
 // Q64 (rows x rows) = double(right block of out32).
 __global__ void extract_q_kernel(const CvtDesc* __restrict__ descs) {
     const CvtDesc d = descs[blockIdx.y];
-    const int w = d.L + d.rows;
     for (int r = blockIdx.x; r < d.rows; r += gridDim.x) {
-        const float* o = d.out32 + (size_t)r * w + d.L;
+        const float* o = d.out32 + (size_t)r * d.ld32 + d.L;
         double* q = d.Q + (size_t)r * d.rows;
         for (int c = threadIdx.x; c < d.rows; c += blockDim.x) q[c] = (double)o[c];
     }
@@ -1106,15 +1105,16 @@ template void launch_mirror_lower<double>(double* const*, const int*, const int*
 
 // dst = src^T for a batch of rectangular matrices, 32 x 32 tiles through
 // shared memory (blockIdx.z = matrix)
-__global__ void transpose_rect_kernel(const TransDesc* __restrict__ descs) {
-    const TransDesc d = descs[blockIdx.z];
-    __shared__ double tile[32][33];
+template <typename T>
+__global__ void transpose_rect_kernel(const TransDescT<T>* __restrict__ descs) {
+    const TransDescT<T> d = descs[blockIdx.z];
+    __shared__ T tile[32][33];
     const int tr = (d.rows + 31) / 32, tc = (d.cols + 31) / 32;
     for (int t = blockIdx.x; t < tr * tc; t += gridDim.x) {
         const int r0 = (t / tc) * 32, c0 = (t % tc) * 32;
         for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
             const int r = e / 32, c = e % 32;
-            tile[r][c] = (r0 + r < d.rows && c0 + c < d.cols) ? d.src[(size_t)(r0 + r) * d.lds + c0 + c] : 0.0;
+            tile[r][c] = (r0 + r < d.rows && c0 + c < d.cols) ? d.src[(size_t)(r0 + r) * d.lds + c0 + c] : T(0);
         }
         __syncthreads();
         for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
@@ -1125,12 +1125,15 @@ __global__ void transpose_rect_kernel(const TransDesc* __restrict__ descs) {
     }
 }
 
-void launch_transpose_rect(const TransDesc* d, int nmat, int maxdim, cudaStream_t s) {
+template <typename T>
+void launch_transpose_rect(const TransDescT<T>* d, int nmat, int maxdim, cudaStream_t s) {
     if (nmat <= 0 || maxdim <= 0) return;
     const int t = (maxdim + 31) / 32;
     dim3 grid(min(t * t, 4096), 1, nmat);
-    transpose_rect_kernel<<<grid, 256, 0, s>>>(d);
+    transpose_rect_kernel<T><<<grid, 256, 0, s>>>(d);
 }
+template void launch_transpose_rect<float>(const TransDescT<float>*, int, int, cudaStream_t);
+template void launch_transpose_rect<double>(const TransDescT<double>*, int, int, cudaStream_t);
 
 // dst[i] = (To) src[i]
 template <typename Ti, typename To>
@@ -1170,6 +1173,8 @@ void launch_convert_blocks(const Ti* const* src, const int* lds, To* const* dst,
 }
 template void launch_convert_blocks<double, float>(const double* const*, const int*, float* const*, const int*,
                                                    const int*, int, int, cudaStream_t);
+template void launch_convert_blocks<double, double>(const double* const*, const int*, double* const*, const int*,
+                                                    const int*, int, int, cudaStream_t);
 
 // ------------------------------------------------------------------ tridiagonal eigenvalues
 // Householder reduction of a symmetric n x n matrix (full storage, updated in

@@ -59,31 +59,32 @@ __device__ __forceinline__ T lane_sum(T v) {
 
 }  // namespace
 
-// Lower triangle of the front of part p, columns of its interior, from the
-// dense lower triangle of E (subdomain order): F[r][c] = E[max][min] of the
-// two coarse unknowns.  F is zero on entry (its boundary block stays zero).
+// Lower triangle of the front of part p, columns of its interior, from the lower
+// triangle of its dense matrix A (E, or the A_ii of its subdomain): F[r][c] =
+// A[max][min] of the two unknowns.  F is zero on entry (its boundary block stays zero).
 __global__ void __launch_bounds__(256) front_gather_kernel(const FrontDevT<double>* __restrict__ fr,
+                                                           const FrontSrc* __restrict__ src,
                                                            const int32_t* __restrict__ bnd,
-                                                           const int32_t* __restrict__ perm,
-                                                           const double* __restrict__ E, int64_t nE) {
+                                                           const int32_t* __restrict__ perm) {
     const FrontDevT<double> f = fr[blockIdx.y];
+    const FrontSrc a = src[blockIdx.y];
     const int n = f.m + f.nb;
     for (int r = blockIdx.x; r < n; r += gridDim.x) {
-        const int64_t pr = perm[r < f.m ? f.i0 + r : bnd[f.b0 + r - f.m]];
+        const int64_t pr = perm[r < f.m ? f.i0 + r : bnd[f.b0 + r - f.m]] - a.off;
         double* row = f.F + (size_t)r * n;
         const int cend = min(r + 1, f.m);
         for (int c = threadIdx.x; c < cend; c += blockDim.x) {
-            const int64_t pc = perm[f.i0 + c];
-            row[c] = E[(pr > pc ? pr : pc) * nE + (pr > pc ? pc : pr)];
+            const int64_t pc = perm[f.i0 + c] - a.off;
+            row[c] = a.A[(pr > pc ? pr : pc) * a.ld + (pr > pc ? pc : pr)];
         }
     }
 }
 
-void launch_front_gather(const FrontDevT<double>* fr, int nfr, const int32_t* bnd, const int32_t* perm,
-                         const double* E, int64_t nE, int maxn, cudaStream_t s) {
+void launch_front_gather(const FrontDevT<double>* fr, const FrontSrc* src, int nfr, const int32_t* bnd,
+                         const int32_t* perm, int maxn, cudaStream_t s) {
     for (int k = 0; k < nfr; k += 32768)  // grid.y is 16 bits wide
         front_gather_kernel<<<dim3(maxn < 512 ? maxn : 512, nfr - k < 32768 ? nfr - k : 32768), 256, 0, s>>>(
-            fr + k, bnd, perm, E, nE);
+            fr + k, src + k, bnd, perm);
 }
 
 // Adds the Schur complements of the children of every front of a stage into it
