@@ -54,8 +54,7 @@ __device__ __forceinline__ void jb_pair(int g, int ir, int& p, int& q) {
 }
 
 // rotation of the pair [[a, g], [g, b]] as in jpi_rotation; false (cs = 1, sn = t = 0)
-// when the tests leave it.  sqrt and the quotient to within 2 units in the last
-// place: t only has to make the pair orthogonal to rounding, and cs, sn follow from t.
+// when the tests leave it
 __device__ __forceinline__ bool jb_rotation(float a, float b, float g, const JbTest& ts, float& cs, float& sn, float& t) {
     cs = 1.0f;
     sn = t = 0.0f;
@@ -64,9 +63,7 @@ __device__ __forceinline__ bool jb_rotation(float a, float b, float g, const JbT
           fabsf(g) > ts.rel * m))
         return false;
     const float dd = b - a, gg = g + g;
-    float h;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(h) : "f"(fmaf(dd, dd, gg * gg)));
-    t = copysignf(1.0f, dd) * __fdividef(gg, fabsf(dd) + h);
+    t = copysignf(1.0f, dd) * gg / (fabsf(dd) + sqrtf(fmaf(dd, dd, gg * gg)));
     const float x = fmaf(t, t, 1.0f);
     cs = rsqrtf(x);
     cs = fmaf(0.5f * cs, fmaf(-x * cs, cs, 1.0f), cs);  // one Newton step: rows keep their length to rounding
