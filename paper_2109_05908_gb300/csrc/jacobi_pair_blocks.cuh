@@ -64,9 +64,7 @@ __device__ __forceinline__ bool jb_rotation(float a, float b, float g, const JbT
         return false;
     const float dd = b - a, gg = g + g;
     t = copysignf(1.0f, dd) * gg / (fabsf(dd) + sqrtf(fmaf(dd, dd, gg * gg)));
-    const float x = fmaf(t, t, 1.0f);
-    cs = rsqrtf(x);
-    cs = fmaf(0.5f * cs, fmaf(-x * cs, cs, 1.0f), cs);  // one Newton step: rows keep their length to rounding
+    cs = jpi_rsqrt(fmaf(t, t, 1.0f));
     sn = cs * t;
     return true;
 }

@@ -54,7 +54,11 @@ __device__ __forceinline__ void jpi_pair(int k, int rr, int& p, int& q) {
     }
 }
 
-__device__ __forceinline__ float jpi_rsqrt(float x) { return rsqrtf(x); }
+// (FP32 with a Newton step: rsqrtf alone shortens the rows a little in every rotation)
+__device__ __forceinline__ float jpi_rsqrt(float x) {
+    const float r = rsqrtf(x);
+    return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
 __device__ __forceinline__ double jpi_rsqrt(double x) { return rsqrt(x); }
 
 __device__ __forceinline__ int jpi_gi(int x, int y) { return x < y ? x * JPI_LDG + y : y * JPI_LDG + x; }
