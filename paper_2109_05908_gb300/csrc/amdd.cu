@@ -3332,7 +3332,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
                 const int pi = h->p[i], nIi = h->nI[i];
                 tdz.push_back({h->d_Zt + h->off_zt[i], h->d_Zr + h->off_zt[i], pi, nIi, nIi, pi});
                 maxd = std::max(maxd, std::max(pi, nIi));
-                GemvDesc g{h->d_Zr + h->off_zt[i], nIi, pi, pi, 0, h->d_e + h->coff[i], h->d_zc + h->off_I[i]};
+                GemvDesc g{h->d_Zr + h->off_zt[i], nIi, pi, pi, h->d_e + h->coff[i], h->d_zc + h->off_I[i]};
                 for (int a = 0; a < nIi; ++a) {
                     rdz.push_back((int32_t)h->gv_zp_h.size());
                     rlz.push_back(a);
@@ -3352,7 +3352,7 @@ void do_setup(amdd_handle* h, const amdd_csr* A, const int32_t* d_part) {
         std::vector<int32_t> rdc, rlc;
         for (int i = 0; i < N; ++i) {
             if (h->d_Zt)
-                cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_rloc + h->off_om[i],
+                cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], h->d_rloc + h->off_om[i],
                          h->d_c + h->coff[i]};
             for (int k = 0; k < h->p[i] && !h->all_diag; ++k) {
                 rdc.push_back(i);
@@ -3627,7 +3627,7 @@ void ensure_multi(amdd_handle* h) {
     if (h->nC > 0 && !h->all_diag) {
         std::vector<GemvDesc> cr(h->N);
         for (int i = 0; i < h->N; ++i)
-            cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], 0, h->d_m_rloc + h->off_om[i],
+            cr[i] = {h->d_Zt + h->off_zt[i], h->p[i], h->nI[i], h->nI[i], h->d_m_rloc + h->off_om[i],
                      h->d_m_c + h->coff[i]};
         h->d_m_gv_c = dnew<GemvDesc>(h, h->N);
         ck(cudaMemcpyAsync(h->d_m_gv_c, cr.data(), h->N * sizeof(GemvDesc), cudaMemcpyHostToDevice, h->s));

@@ -133,14 +133,9 @@ using TridiagDesc = TridiagDescT<double>;
 template <typename T>
 struct GemvDescT {
     const T* M;
-    int rows, ncols, ld, mode;
+    int rows, ncols, ld;
     const T* x;
     T* y;
-    const T* b = nullptr;  // y[row] = b[row] + alpha * (M x)[row] when b is given
-    T alpha = T(1);
-    const int* cstart = nullptr;  // optional per-row first column (absolute, minus coff)
-    const int* cend = nullptr;    // optional per-row end column (absolute, minus coff)
-    int coff = 0;
 };
 using GemvDesc = GemvDescT<double>;
 
@@ -442,6 +437,14 @@ void launch_mlp_forward(const float* wb, const float* x, int n, float* q, cudaSt
 void launch_mlp_step(float* w, float* wb, float* m, float* v, int t, float lr, const float* x, const float* qt, int n,
                      float* grad, float* work, float* loss, cudaStream_t s);
 void launch_bf16_round(const float* W, float* Wb, int n, cudaStream_t s);
+// bfloat16 rounding of binary32: add 0x7FFF plus the lowest kept bit, keep
+// the top 16 bits (nearest, ties to even); NaN stays NaN.
+__device__ __forceinline__ float bf16_round(float x) {
+    if (x != x) return x;
+    unsigned u = __float_as_uint(x);
+    u = (u + 0x7FFFu + ((u >> 16) & 1u)) & 0xFFFF0000u;
+    return __uint_as_float(u);
+}
 
 template <typename T>
 struct RowsDesc {  // rows [r0, r1) of a row-major matrix (cols entries each)

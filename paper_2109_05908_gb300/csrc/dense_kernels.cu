@@ -1720,23 +1720,18 @@ __global__ void __launch_bounds__(256) gemv_rows_kernel(const GemvDescT<T>* __re
     if (w >= nrows) return;
     const GemvDescT<T> d = descs[row_desc[w]];
     const int r = row_local[w];
-    int c0 = 0, c1 = d.ncols;
-    if (d.mode == 1) c1 = min(r + 1, d.ncols);
-    if (d.mode == 2) c0 = r;
-    if (d.cstart) c0 = max(c0, d.cstart[r] - d.coff);
-    if (d.cend) c1 = min(c1, d.cend[r] - d.coff);
     const T* row = d.M + (size_t)r * d.ld;
     T s0 = T(0), s1 = T(0);
-    int c = c0 + lane;
-    for (; c + 32 < c1; c += 64) {
+    int c = lane;
+    for (; c + 32 < d.ncols; c += 64) {
         s0 = fma(row[c], d.x[c], s0);
         s1 = fma(row[c + 32], d.x[c + 32], s1);
     }
-    if (c < c1) s0 = fma(row[c], d.x[c], s0);
+    if (c < d.ncols) s0 = fma(row[c], d.x[c], s0);
     T s = s0 + s1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) d.y[r] = d.b ? fma(d.alpha, s, d.b[r]) : d.alpha * s;
+    if (lane == 0) d.y[r] = s;
 }
 
 template <typename T>
@@ -1747,11 +1742,10 @@ void launch_gemv_rows(const GemvDescT<T>* d, const int* row_desc, const int* row
     const int64_t blocks = (threads + 255) / 256;
     gemv_rows_kernel<T><<<(unsigned)blocks, 256, 0, s>>>(d, row_desc, row_local, nrows);
 }
-template void launch_gemv_rows<float>(const GemvDescT<float>*, const int*, const int*, int64_t, cudaStream_t);
 template void launch_gemv_rows<double>(const GemvDescT<double>*, const int*, const int*, int64_t, cudaStream_t);
 
-// One warp per row of a batch of row-major matrices (mode 0: all columns),
-// nb right-hand sides: y_k[row] = alpha (M x_k)[row].
+// One warp per row of a batch of row-major matrices, nb right-hand sides:
+// y_k[row] = (M x_k)[row].
 template <typename T>
 __global__ void __launch_bounds__(256) gemv_rows_multi_kernel(const GemvDescT<T>* __restrict__ descs,
                                                               const int* __restrict__ row_desc,
@@ -1777,7 +1771,7 @@ __global__ void __launch_bounds__(256) gemv_rows_multi_kernel(const GemvDescT<T>
         T v = acc[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && k < nb) d.y[k * ys + r] = d.alpha * v;
+        if (lane == 0 && k < nb) d.y[k * ys + r] = v;
     }
 }
 

@@ -215,15 +215,6 @@ void launch_krylov(const KrylovDesc* d, int nmat, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ MLP
-// bfloat16 rounding of binary32: add 0x7FFF plus the lowest kept bit, keep
-// the top 16 bits (nearest, ties to even); NaN stays NaN.
-__device__ __forceinline__ float bf16_round(float x) {
-    if (x != x) return x;
-    unsigned u = __float_as_uint(x);
-    u = (u + 0x7FFFu + ((u >> 16) & 1u)) & 0xFFFF0000u;
-    return __uint_as_float(u);
-}
-
 // X[b][f] = (feat[b][f] - mean[f]) / sd[f]
 __global__ void normalize_features_kernel(const float* __restrict__ feat, const float* __restrict__ mean,
                                           const float* __restrict__ sd, float* __restrict__ X, int n) {

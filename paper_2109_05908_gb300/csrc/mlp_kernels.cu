@@ -39,12 +39,6 @@ __device__ __forceinline__ void mlp_cp(float* dst, const float* src, int vec) {
 __device__ __forceinline__ void mlp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void mlp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-__device__ __forceinline__ float mlp_bf16_round(float x) {
-    const unsigned b = __float_as_uint(x);
-    if ((b & 0x7f800000u) == 0x7f800000u) return x;  // infinities and NaN as they are
-    return __uint_as_float((b + 0x7fffu + ((b >> 16) & 1u)) & 0xffff0000u);
-}
-
 // tile t of the 33: 0 W1; 1..8 W2 forward; 9..16 W3 forward; 17..24 W3 backward; 25..32 W2 backward
 __device__ __forceinline__ void mlp_issue(int t, const float* __restrict__ wb, float* buf, int vec) {
     if (t < 17) {  // 32 rows of 256, contiguous
@@ -306,7 +300,7 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(const float* __restrict
             v[t] = vt;
             const float w = W[t] - lr * (mt / c1) / (sqrtf(vt / c2) + eps);
             W[t] = w;
-            Wb[t] = mlp_bf16_round(w);
+            Wb[t] = bf16_round(w);
         }
     }
     if (blockIdx.x + 1 == gridDim.x) {  // a CTA of its own: the loss
