@@ -50,7 +50,7 @@ SVD_CLASSES = {"jacobi_f32": True, "jacobi_svd": False}
 # `bench.py --steps 1 --warmup 1 --plain-steps 1 --no-scale --no-variants` (dram__bytes_read.sum +
 # dram__bytes_write.sum summed over the class's launches of one step); reported as roofline.traffic only for the
 # workload it was taken on
-TRAFFIC_PER_STEP = {("jacobi_f32", "diffusion3d_24^3_sigma2_ch16_bfs16_256-2048_ov2_tau100"): 3.894e11}
+TRAFFIC_PER_STEP = {("jacobi_f32", "diffusion3d_24^3_sigma2_ch16_bfs16_256-2048_ov2_tau100"): 3.939e11}
 # TF32 / bf16 dense tensor rates (nominal 1.1 and 2.25 PFLOP/s); an FP32 product by the 3xTF32 split costs three
 # TF32 MMAs
 TF32_OVER_BF16 = 1.1 / 2.25

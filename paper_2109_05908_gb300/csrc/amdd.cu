@@ -2110,8 +2110,8 @@ void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& 
 // symbolic structure are rounding residues of exact zeros and are dropped), and
 // its entries compacted into columns.  With local_solver = 2 (automatic) the
 // factors are kept only when every subdomain's factor fits in shared memory and
-// holds at most a quarter of its dense triangle; otherwise the dense inverse
-// factors serve and nothing is kept.
+// holds at most a quarter of its dense triangle; otherwise substructuring
+// serves and nothing is kept.
 template <typename T>
 void build_sparse_local(Ctx& C, amdd_handle* h, const std::vector<int64_t>& rp, const std::vector<int32_t>& ci,
                         const std::vector<int32_t>& omega) {
@@ -3653,7 +3653,7 @@ void ensure_multi(amdd_handle* h) {
 }
 
 // z_k = M^{-1} r_k for nb <= MAXB right-hand sides (vectors n apart): every
-// factor, Z_i and L_E entry is read once per pass for all of them.
+// entry of the parts and of the Z_i is read once per pass for all of them.
 void apply_multi(amdd_handle* h, const double* r, double* z, int nb, const DotArgs& d = DotArgs{}) {
     if (h->next) {  // inexact coarse solves run one right-hand side at a time
         for (int k = 0; k < nb; ++k) apply_one(h, r + (size_t)k * h->n, z + (size_t)k * h->n);
