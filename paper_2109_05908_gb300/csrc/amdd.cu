@@ -1879,9 +1879,9 @@ void front_graph(int nv, const std::vector<int32_t>& a, const std::vector<int32_
     adj.resize(w);
 }
 
-// Lower-triangle entries of a matrix given through the CSR values of A: (row
-// unknown, column unknown, position in the values); with diag (position of each
-// unknown's diagonal entry) the matrix is scaled to unit diagonal on both sides.
+// Lower-triangle entries of a matrix given through the CSR values of A, scaled to unit
+// diagonal on both sides: (row unknown, column unknown, position in the values), and
+// the position of each unknown's diagonal entry.
 struct FrontEntries {
     std::vector<int32_t> row, col;
     std::vector<int64_t> src, diag;
@@ -2010,15 +2010,10 @@ void factor_fronts(Ctx& C, amdd_handle* h, FrontSolveT<T>& fs, const FrontPlan& 
             ea[e] = (int32_t)a;
             eb[e] = (int32_t)b;
         }
-        const double* scale = nullptr;
-        if (!sp->diag.empty()) {
-            double* sc = dnew<double>(h, P.n);
-            h->d_dsc = dnew<double>(h, P.n);
-            launch_front_scale(h->val, C.up(dg), fs.perm, sc, h->d_dsc, P.n, s);
-            scale = sc;
-        }
-        launch_front_scatter(h->val, C.up(sp->src), C.up(dst), C.up(ea), C.up(eb), scale, F, (int64_t)dst.size(),
-                                s);
+        double* scale = dnew<double>(h, P.n);
+        h->d_dsc = dnew<double>(h, P.n);
+        launch_front_scale(h->val, C.up(dg), fs.perm, scale, h->d_dsc, P.n, s);
+        launch_front_scatter(h->val, C.up(sp->src), C.up(dst), C.up(ea), C.up(eb), scale, F, (int64_t)dst.size(), s);
         fs.scale = scale;
     }
     fs.fr = C.up(fk, true);

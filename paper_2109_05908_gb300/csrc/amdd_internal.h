@@ -533,7 +533,7 @@ void launch_front_gather(const FrontDevT<double>* fr, const FrontSrc* src, int n
 // scale[k] = own[perm[k]] = 1 / sqrt(val[diag[k]]) (val 0 where diag[k] < 0), k < n
 void launch_front_scale(const double* val, const int64_t* diag, const int32_t* perm, double* scale, double* own,
                         int64_t n, cudaStream_t s);
-// F[dst[t]] = val[src[t]] (times scale[a[t]] scale[b[t]] when given), t < cnt
+// F[dst[t]] = val[src[t]] scale[a[t]] scale[b[t]], t < cnt
 void launch_front_scatter(const double* val, const int64_t* src, const int64_t* dst, const int32_t* a,
                           const int32_t* b, const double* scale, double* F, int64_t cnt, cudaStream_t s);
 void launch_front_extend_add(const FrontDevT<double>* fr, int nfr, const FrontChild* kids, const int32_t* maps,

@@ -147,8 +147,7 @@ __global__ void __launch_bounds__(256) front_scatter_kernel(const double* __rest
                                                             const double* __restrict__ scale, double* __restrict__ F,
                                                             int64_t cnt) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        const double v = val[src[t]];
-        F[dst[t]] = scale ? v * scale[b[t]] * scale[a[t]] : v;
+        F[dst[t]] = val[src[t]] * scale[b[t]] * scale[a[t]];
     }
 }
 
